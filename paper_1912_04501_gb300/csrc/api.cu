@@ -33,6 +33,7 @@ static void free_all(bie_ctx* c) {
     if (c->aux) cudaStreamSynchronize(c->aux);  // nothing of an application left in flight
     free_graph(c);
     free_precond(c);
+    free_fmm(c);
     void* ptrs[] = {c->cells, c->node_cell, c->body_cell, c->x, c->y, c->nx, c->ny, c->w, c->kap, c->owner, c->body,
                     c->tgt32, c->posdf, c->xw, c->yw, c->imc, c->bimg, c->ws.src32n, c->ws.src64u, c->next.yp,
                     c->next.ypf, c->glc, c->contour_part, c->bshape, c->near_ctr,
@@ -586,6 +587,7 @@ int bie_init_batch(bie_ctx** out, int32_t n_cells, const bie_cell* cells, const 
         rc = rc ? rc : up(c->next.ypf, ypf.data(), ypf.size() * sizeof(float2));
     }
     rc = rc ? rc : up(c->e2d, c->e2_0.data(), c->e2_0.size() * sizeof(double));
+    rc = rc ? rc : fmm_plan(c);
     rc = rc ? rc : build_near_items(c);
     rc = rc ? rc : build_dot_chunks(c);
     rc = rc ? rc : build_dirichlet_tables(c, 64);
@@ -875,7 +877,12 @@ int bie_set_state(bie_ctx* c, double t, const double* e2, const double* xc, cons
         const double e1[2] = {cl.e1[0], cl.e1[1]};
         cell_set_lattice(cl, e1, e2 + 2 * k);
     }
-    int rc = upload_cells(c, c->stream);
+    c->body_host = h;
+    const unsigned long long epoch = c->epoch;
+    int rc = fmm_plan(c);
+    if (rc) return rc;
+    if (c->epoch != epoch && (rc = build_near_items(c))) return rc;  // other boxes: the image sums' layout may change
+    rc = upload_cells(c, c->stream);
     if (rc) return rc;
     rc = upload_e2(c, c->e2d, current_e2(c), c->stream);
     if (rc) return rc;

@@ -474,102 +474,6 @@ k_near64(const int4* __restrict__ items, const Cell* __restrict__ cells, const d
     }
 }
 
-// ---------------------------------------------------------------------------
-// Near image sum in double-float arithmetic ("df64": every quantity is an
-// unevaluated sum hi + lo of two floats, ~48 significant bits) on the FP32
-// pipe.  GB300's FP64 pipe sustains about 1/100 of the FP32 pair rate, so the
-// FP64-accurate refinement residual runs here instead.  Error-free
-// transformations: TwoSum (6 FP32 ops) for sums, FMA-based TwoProd (2 ops)
-// for products, MUFU rcp refined by one FMA residual step for 1/r^2; the
-// difference r = x - y is formed exactly from both words (three TwoSums) and
-// r, r.n, r.q are renormalised before they are multiplied, so that the
-// dropped lo*lo cross terms stay at 2^-48; each source tile's sum is kept as
-// (TwoSum hi, float error) and folded into double accumulators.  About 140
-// FP32 instructions per pair; each term is accurate to ~1e-14 of the
-// kernel's scale |q| / |r| at any distance (the inputs carry 48 of double's
-// 53 bits).
-// ---------------------------------------------------------------------------
-struct __align__(16) SrcDF {
-    float xh, xl, yh, yl, qxh, qxl, qyh, qyl;
-};
-
-// (ah + al) * (bh + bl) -> (ph, pl), pl not renormalised
-__device__ __forceinline__ void df_mul(float ah, float al, float bh, float bl, float& ph, float& pl) {
-    ph = ah * bh;
-    pl = fmaf(ah, bh, -ph);
-    pl = fmaf(ah, bl, fmaf(al, bh, pl));
-}
-
-
-// The y-parts of a double-float pair, shared by every image with the same
-// r_y: r_y itself, its square (b + eb) and its products with n_y and q_y.
-struct DFy {
-    float ryh, ryl, b, eb, pn, en, pq, eq;
-};
-
-__device__ __forceinline__ DFy pair_df_y(float pyh, float pyl, float nyh, float nyl, const SrcDF& q) {
-    DFy y;
-    df_diff(pyh, pyl, q.yh, q.yl, y.ryh, y.ryl);
-    y.b = y.ryh * y.ryh;
-    y.eb = fmaf(y.ryh, y.ryh, -y.b);
-    y.eb = fmaf(y.ryh, y.ryl + y.ryl, y.eb);
-    df_mul(y.ryh, y.ryl, nyh, nyl, y.pn, y.en);
-    df_mul(y.ryh, y.ryl, q.qyh, q.qyl, y.pq, y.eq);
-    return y;
-}
-
-// One double-float pair of the near sum from its y-parts: target
-// x = pxh + pxl with normal x-component nx, source record q; the term c r,
-// c = (r.n / r^2)(r.q / r^2), r = p - y, is added to the tile accumulators
-// (TwoSum hi, float error).
-__device__ __forceinline__ void pair_df_x(float pxh, float pxl, float nxh, float nxl, const DFy& y, const SrcDF& q,
-                                          float& axh, float& axe, float& ayh, float& aye) {
-    float rxh, rxl, e;
-    const float ryh = y.ryh, ryl = y.ryl;
-    df_diff(pxh, pxl, q.xh, q.xl, rxh, rxl);
-    // r^2 (the 1e-30 floor absorbs the zero-distance self pair)
-    float a, ea, r2h, r2l;
-    a = rxh * rxh;
-    ea = fmaf(rxh, rxh, -a);
-    ea = fmaf(rxh, rxl + rxl, ea);
-    two_sum(a, y.b, r2h, e);
-    r2l = e + ea + y.eb;
-    r2h += 1e-30f;
-    // 1 / r^2
-    const float ih = rcp_approx(r2h);
-    float res = fmaf(-r2h, ih, 1.0f);
-    res = fmaf(-r2l, ih, res);
-    const float il = ih * res;
-    // r . n and r . q
-    float p1, e1, rnh, rnl, rqh, rql;
-    df_mul(rxh, rxl, nxh, nxl, p1, e1);
-    two_sum(p1, y.pn, rnh, e);
-    rnl = e + e1 + y.en;
-    fast2(rnh, rnl);  // r.n may cancel: renormalise before multiplying
-    df_mul(rxh, rxl, q.qxh, q.qxl, p1, e1);
-    two_sum(p1, y.pq, rqh, e);
-    rql = e + e1 + y.eq;
-    fast2(rqh, rql);
-    // c = (r.n / r^2) (r.q / r^2), term = c r
-    float uh, ul, vh, vl, ch, cl2, th, tl;
-    df_mul(rnh, rnl, ih, il, uh, ul);
-    df_mul(rqh, rql, ih, il, vh, vl);
-    df_mul(uh, ul, vh, vl, ch, cl2);
-    df_mul(ch, cl2, rxh, rxl, th, tl);
-    two_sum(axh, th, axh, e);
-    axe += e + tl;
-    df_mul(ch, cl2, ryh, ryl, th, tl);
-    two_sum(ayh, th, ayh, e);
-    aye += e + tl;
-}
-
-// One double-float pair with its own y-parts.
-__device__ __forceinline__ void pair_df(float pxh, float pxl, float pyh, float pyl, float nxh, float nxl, float nyh,
-                                        float nyl, const SrcDF& q, float& axh, float& axe, float& ayh, float& aye) {
-    const DFy y = pair_df_y(pyh, pyl, nyh, nyl, q);
-    pair_df_x(pxh, pxl, nxh, nxl, y, q, axh, axe, ayh, aye);
-}
-
 // a1 in one pass, one CTA per body: q = sigma w packed into whichever source
 // records the application needs (single-precision cell-centred, double,
 // double-float), and the body's force and torque moments F_b = sum q,
@@ -615,6 +519,21 @@ k_pack_moments(const double2* __restrict__ sigma, const double* __restrict__ x, 
     }
 }
 
+// ---------------------------------------------------------------------------
+// Near image sum in double-float arithmetic ("df64": every quantity is an
+// unevaluated sum hi + lo of two floats, ~48 significant bits) on the FP32
+// pipe.  GB300's FP64 pipe sustains about 1/100 of the FP32 pair rate, so the
+// FP64-accurate refinement residual runs here instead.  Error-free
+// transformations: TwoSum (6 FP32 ops) for sums, FMA-based TwoProd (2 ops)
+// for products, MUFU rcp refined by one FMA residual step for 1/r^2; the
+// difference r = x - y is formed exactly from both words (three TwoSums) and
+// r, r.n, r.q are renormalised before they are multiplied, so that the
+// dropped lo*lo cross terms stay at 2^-48; each source tile's sum is kept as
+// (TwoSum hi, float error) and folded into double accumulators.  About 140
+// FP32 instructions per pair; each term is accurate to ~1e-14 of the
+// kernel's scale |q| / |r| at any distance (the inputs carry 48 of double's
+// 53 bits).
+// ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kNearThreads, 4)
 k_near_df(const int4* __restrict__ items, const Cell* __restrict__ cells, const double* __restrict__ x,
           const double* __restrict__ y, const double* __restrict__ nx, const double* __restrict__ ny,
@@ -1386,7 +1305,17 @@ static void choose_splits(const std::vector<Cell>& cells, int tile, int slots, s
 // Items (cell, target tile, source split) for every precision; also sets each
 // cell's splits and partial offsets and uploads the cell table.
 // Items of one precision for the context's current single-precision shape.
-static int build_near_items_prec(bie_ctx* c, int prec) {
+// Cells whose near sums run by expansions (fmm.cu) have one partial per node
+// and no items, unless `direct`.
+static int build_near_items_prec(bie_ctx* c, int prec, bool direct = false) {
+    if (c->fmm[prec].on && !direct) {
+        for (Cell& cl : c->cells_h) {
+            cl.splits[prec] = 1;
+            cl.part_off[prec] = cl.node_off;
+        }
+        c->near[prec].count = 0;
+        return BIE_OK;
+    }
     const int tile = near_tile(c->shape32, prec, c->utilde);
     std::vector<int> splits;
     choose_splits(c->cells_h, tile, near_ctas_per_sm(c->shape32, prec, c->utilde) * c->sms, splits, c->srcmul);
@@ -1567,21 +1496,24 @@ static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, i
     const bool f32 = precision == BIE_MIXED;
     const bool df = precision == BIE_DF64;
     const int prec = f32 ? 0 : (df ? 2 : 1);
+    const bool fast = c->fmm[prec].on;  // the fast image sum packs its own sorted strengths
     if (part == 0) {
         if (&ws == &c->ws) c->ws_x = nullptr;  // the workspace is about to change
         if (c->utilde)
             k_pack_moments_u<<<c->nb, 256, 0, c->stream>>>(sg, c->x, c->y, c->w, c->body, c->body_cell, c->cells,
-                                                           c->imc, f32 ? ws.src32 : nullptr, f32 ? ws.src32n : nullptr,
-                                                           ws.src64, (!f32 && !df) ? ws.src64u : nullptr,
-                                                           df ? (SrcDF*)ws.srcdf : nullptr, ws.bodyF);
+                                                           c->imc, f32 && !fast ? ws.src32 : nullptr,
+                                                           f32 ? ws.src32n : nullptr, ws.src64,
+                                                           !f32 && !df && !fast ? ws.src64u : nullptr,
+                                                           df && !fast ? (SrcDF*)ws.srcdf : nullptr, ws.bodyF);
         else
             k_pack_moments<<<c->nb, 256, 0, c->stream>>>(sg, c->x, c->y, c->w, c->body, c->body_cell, c->cells,
                                                          f32 ? ws.src32 : nullptr, ws.src64,
-                                                         df ? (SrcDF*)ws.srcdf : nullptr, ws.bodyF);
+                                                         df && !fast ? (SrcDF*)ws.srcdf : nullptr, ws.bodyF);
         BIE_LAUNCH(c, "k_pack_moments");
         return BIE_OK;
     }
     if (part == 1) {
+        if (fast) return fmm_near(c, sigma, prec, ws);
         if (f32) return launch_near32(c, ws.src32, (float2*)ws.part);
         if (c->utilde) {
             if (df)
@@ -1630,6 +1562,7 @@ static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, i
 
 static int apply_impl(bie_ctx* c, const double* sigma, double* yout, int precision, Workspace& ws) {
     const int kind = precision == BIE_MIXED ? 0 : (precision == BIE_DF64 ? 2 : 1);
+    if (int rc = fmm_build(c, kind)) return rc;
     if (int rc = apply_part(c, 0, sigma, yout, precision, ws)) return rc;
     // part 2 on the auxiliary stream, overlapping the near sum
     BIE_CUDA(c, cudaEventRecord(c->aux_fork, c->stream));
@@ -1656,6 +1589,7 @@ static int apply_impl(bie_ctx* c, const double* sigma, double* yout, int precisi
 // beside it): the results are bit for bit those of the direct launches.
 static int apply_graph(bie_ctx* c, const double* sigma, double* yout) {
     auto& g = c->graph;
+    if (int rc = fmm_build(c, 0)) return rc;  // outside the captured work
     const size_t bytes = 2 * (size_t)c->N * sizeof(double);
     if (!g.in) {
         BIE_CUDA(c, cudaMalloc((void**)&g.in, bytes));
@@ -1754,7 +1688,7 @@ int autotune_near32(bie_ctx* c) {
     int rc = BIE_OK;
     for (int sh = 0; sh < kNear32Shapes && !rc; ++sh) {
         c->shape32 = sh;
-        if ((rc = build_near_items_prec(c, 0)) || (rc = upload_cells(c, c->stream))) break;
+        if ((rc = build_near_items_prec(c, 0, true)) || (rc = upload_cells(c, c->stream))) break;
         float t[3];
         for (int k = 0; k < 4 && !rc; ++k) {
             if (k > 0) rc = ck(cudaEventRecord(ev[0], c->stream), "cudaEventRecord");

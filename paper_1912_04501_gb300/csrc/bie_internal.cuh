@@ -77,6 +77,10 @@ constexpr int kNetMaxIn = 16;         // its maximum number of inputs per node
 constexpr int kNetFeatures = 13;      // node features of the warm start (features_device)
 constexpr int kMaxAug = 3;            // augmentation directions of the first GMRES cycle
 
+constexpr int kFmmP32 = 24;           // expansion orders of the fast image sum (fmm.cu): single precision
+constexpr int kFmmP64 = 56;           // and double
+constexpr int kFmmLevels = 12;
+
 // One unit cell of the batch (device table; the host keeps a mirror).
 struct Cell {
     double e1[2], e2[2], C[2];
@@ -150,6 +154,10 @@ struct Workspace {
     float* xif = nullptr;       // ncell x 2M the same in single precision
     double* T = nullptr;        // 2N traction before the pressure fix
     double* vpart = nullptr;    // nb x kVelSplits x 3 velocity partials
+    // fast image sum: sorted strengths, multipole and local expansions, and
+    // the last-child counters of the upward pass (zero between launches)
+    void *fsq = nullptr, *fmp = nullptr, *floc = nullptr;
+    unsigned* ftick = nullptr;
 };
 
 // Proxy least-squares fits (Sec. 6.1) of every cell for given lattices:
@@ -205,6 +213,44 @@ struct Solver {
     float* feat = nullptr;         // N x kNetFeatures node features
     float* pred = nullptr;         // N x 2 network output
     std::vector<bie_solve_info> cell_info;  // last solve, per cell
+};
+
+// Boxes of one cell in the fast image sum: a grid of gx x gy squares of side
+// h 2^l per level l (0 the finest), its corner at (ox, oy) from the cell centre.
+struct FmmCell {
+    double ox, oy, h, inv_h;
+    int nlev;
+    int gx[kFmmLevels], gy[kFmmLevels], off[kFmmLevels];  // off: the level's first box
+};
+
+// Node data the sorting reads.
+struct FmmGeom {
+    const double *x, *y, *xw, *yw;
+    const int *imc, *node_cell;
+};
+
+// Device view of the boxes: records sorted by leaf (targets are the sources
+// themselves, except with the doubled cell).
+struct FmmTree {
+    const FmmCell* cells = nullptr;
+    const int4* box = nullptr;     // nbox: (cell, level, x | y << 16, parent or -1); leaves first
+    int nbox = 0, nleaf = 0;
+    int *scount = nullptr, *tcount = nullptr;  // nbox: records in the box
+    int *sstart = nullptr, *tstart = nullptr;  // nleaf + 1: first sorted record
+    int *sperm = nullptr, *tperm = nullptr;    // sorted record -> record (sources: node, or 4 node + image)
+    float4 *spos = nullptr, *tpos = nullptr;   // sorted positions from the cell centre, double-float
+    double2 *spos64 = nullptr, *tpos64 = nullptr;  // and double
+};
+
+struct Fmm {
+    bool on = false;
+    FmmTree t;
+    FmmCell* cells = nullptr;
+    int4* box = nullptr;
+    int *cursor = nullptr, *leaf = nullptr, *raw = nullptr;  // sorting scratch
+    unsigned long long built = 0;      // geometry the records are sorted for (0: none)
+    size_t mp_bytes = 0, sq_bytes = 0; // expansions (each way) and sorted strengths
+    std::vector<void*> owned;
 };
 
 // Near-sum work list of one precision: one CTA per item (cell, tile, split).
@@ -273,6 +319,10 @@ struct bie_ctx {
     bie::NearItems near[3];     // 0 single precision, 1 double, 2 double-float
     int shape32 = 0;            // tile shape of the single-precision near sum (kNear32ShapeList)
     int* near_ctr = nullptr;    // work-queue counter of the persistent near sum (batches)
+    bie::Fmm fmm[3];            // fast image sum per precision (0 single, 1 double, 2 double-float)
+    void* fmm_tab[2] = {nullptr, nullptr};  // its constant matrices (single, double)
+    std::vector<double> fmm_rects;          // 4 x ncell: the rectangles its boxes cover
+    unsigned long long geometry = 0;        // bumped by build_geometry
     unsigned long long epoch = 0;  // bumped whenever a kernel argument of the operator application changes
     // contact-block right preconditioner (opts.precond, precond.cu)
     struct {
@@ -366,6 +416,12 @@ int close_apply(bie_ctx* c, const double* sigma, double* T);
 // pressure fix and rigid completion in two launches (close.cu)
 int assemble32(bie_ctx* c, const double* sigma, const Workspace& ws, double* yout);
 
+// fmm.cu --------------------------------------------------------------------
+int fmm_plan(bie_ctx* c);             // boxes for the bodies' current places (host mirror)
+int fmm_build(bie_ctx* c, int prec);  // sorts the current geometry if it is not
+int fmm_near(bie_ctx* c, const double* sigma, int prec, Workspace& ws);
+void free_fmm(bie_ctx* c);
+
 // apply.cu ------------------------------------------------------------------
 // near-sum work items (and partial offsets) for the current cell sizes
 int build_near_items(bie_ctx* c);
@@ -434,6 +490,88 @@ __device__ __forceinline__ void df_diff(float ph, float pl, float sh, float sl, 
     two_sum(s1, s2, h, e3);
     l = (e1 + e2) + e3;
     fast2(h, l);
+}
+
+// Double-float source record and pair of the near sums (apply.cu, fmm.cu).
+struct __align__(16) SrcDF {
+    float xh, xl, yh, yl, qxh, qxl, qyh, qyl;
+};
+
+// (ah + al) * (bh + bl) -> (ph, pl), pl not renormalised
+__device__ __forceinline__ void df_mul(float ah, float al, float bh, float bl, float& ph, float& pl) {
+    ph = ah * bh;
+    pl = fmaf(ah, bh, -ph);
+    pl = fmaf(ah, bl, fmaf(al, bh, pl));
+}
+
+
+// The y-parts of a double-float pair, shared by every image with the same
+// r_y: r_y itself, its square (b + eb) and its products with n_y and q_y.
+struct DFy {
+    float ryh, ryl, b, eb, pn, en, pq, eq;
+};
+
+__device__ __forceinline__ DFy pair_df_y(float pyh, float pyl, float nyh, float nyl, const SrcDF& q) {
+    DFy y;
+    df_diff(pyh, pyl, q.yh, q.yl, y.ryh, y.ryl);
+    y.b = y.ryh * y.ryh;
+    y.eb = fmaf(y.ryh, y.ryh, -y.b);
+    y.eb = fmaf(y.ryh, y.ryl + y.ryl, y.eb);
+    df_mul(y.ryh, y.ryl, nyh, nyl, y.pn, y.en);
+    df_mul(y.ryh, y.ryl, q.qyh, q.qyl, y.pq, y.eq);
+    return y;
+}
+
+// One double-float pair of the near sum from its y-parts: target
+// x = pxh + pxl with normal x-component nx, source record q; the term c r,
+// c = (r.n / r^2)(r.q / r^2), r = p - y, is added to the tile accumulators
+// (TwoSum hi, float error).
+__device__ __forceinline__ void pair_df_x(float pxh, float pxl, float nxh, float nxl, const DFy& y, const SrcDF& q,
+                                          float& axh, float& axe, float& ayh, float& aye) {
+    float rxh, rxl, e;
+    const float ryh = y.ryh, ryl = y.ryl;
+    df_diff(pxh, pxl, q.xh, q.xl, rxh, rxl);
+    // r^2 (the 1e-30 floor absorbs the zero-distance self pair)
+    float a, ea, r2h, r2l;
+    a = rxh * rxh;
+    ea = fmaf(rxh, rxh, -a);
+    ea = fmaf(rxh, rxl + rxl, ea);
+    two_sum(a, y.b, r2h, e);
+    r2l = e + ea + y.eb;
+    r2h += 1e-30f;
+    // 1 / r^2
+    const float ih = rcp_approx(r2h);
+    float res = fmaf(-r2h, ih, 1.0f);
+    res = fmaf(-r2l, ih, res);
+    const float il = ih * res;
+    // r . n and r . q
+    float p1, e1, rnh, rnl, rqh, rql;
+    df_mul(rxh, rxl, nxh, nxl, p1, e1);
+    two_sum(p1, y.pn, rnh, e);
+    rnl = e + e1 + y.en;
+    fast2(rnh, rnl);  // r.n may cancel: renormalise before multiplying
+    df_mul(rxh, rxl, q.qxh, q.qxl, p1, e1);
+    two_sum(p1, y.pq, rqh, e);
+    rql = e + e1 + y.eq;
+    fast2(rqh, rql);
+    // c = (r.n / r^2) (r.q / r^2), term = c r
+    float uh, ul, vh, vl, ch, cl2, th, tl;
+    df_mul(rnh, rnl, ih, il, uh, ul);
+    df_mul(rqh, rql, ih, il, vh, vl);
+    df_mul(uh, ul, vh, vl, ch, cl2);
+    df_mul(ch, cl2, rxh, rxl, th, tl);
+    two_sum(axh, th, axh, e);
+    axe += e + tl;
+    df_mul(ch, cl2, ryh, ryl, th, tl);
+    two_sum(ayh, th, ayh, e);
+    aye += e + tl;
+}
+
+// One double-float pair with its own y-parts.
+__device__ __forceinline__ void pair_df(float pxh, float pxl, float pyh, float pyl, float nxh, float nxl, float nyh,
+                                        float nyl, const SrcDF& q, float& axh, float& axe, float& ayh, float& aye) {
+    const DFy y = pair_df_y(pyh, pyl, nyh, nyl, q);
+    pair_df_x(pxh, pxl, nxh, nxl, y, q, axh, axe, ayh, aye);
 }
 
 // Packed pairs of floats (PTX .f32x2 on sm_100-family GPUs): one instruction

@@ -801,7 +801,9 @@ int build_dirichlet_tables(bie_ctx* c, int rho_max) {
 // terms with r formed exactly from double-float positions (then rounded to
 // single precision); the close-evaluation blocks are applied in single
 // precision (stored divided by the weights, acting on q = sigma w).
-// Everything but the final sums runs on the FP32 pipe.
+// Everything but the final sums runs on the FP32 pipe.  The fast image sum
+// (fmm.cu) already takes its near pairs from double-float positions, so after
+// it nothing is redone.
 //
 // With the doubled-cell periodizer (imc non-null) the near sum evaluated the
 // pair at the target's translate inside U (tgt32) against the source's image
@@ -834,6 +836,8 @@ struct Asm32 {
     const Cell* cells;
     const int* imc;
     const double* bodyF;
+    const float4* qsrc;  // per-node strengths q (z, w)
+    int redo;  // the near sum's own-body and close terms are to be redone (direct single-precision sum)
 };
 
 // T_i on every thread of the calling group of NL threads (a warp, NL = 32,
@@ -908,7 +912,7 @@ __device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane, d
         fx += c1 * rx - c0 * dx;
         fy += c1 * ry - c0 * dy;
     };
-    {
+    if (a.redo) {
         const int b = a.owner[i];
         const int nbn = (int)a.body[8 * b + 5], off = (int)a.body[8 * b + 6];
         const float4 p = shifted(4);
@@ -927,8 +931,8 @@ __device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane, d
             const float4 p = shifted(im);
 #pragma unroll 2
             for (int k = lane; k < nbn; k += NL) {
-                redo(off + k, im, p);
-                const float4 s = a.src32[a.imc ? 4 * (size_t)(off + k) : (size_t)(off + k)];  // q: the same in every record
+                if (a.redo) redo(off + k, im, p);
+                const float4 s = a.qsrc[off + k];
                 const float A = C[3 * k], B = C[3 * k + 1], D = C[3 * k + 2];
                 bx = fmaf(A, s.z, fmaf(B, s.w, bx));
                 by = fmaf(B, s.z, fmaf(D, s.w, by));
@@ -1037,6 +1041,8 @@ int assemble32(bie_ctx* c, const double* sigma, const Workspace& ws, double* you
     a.cells = c->cells;
     a.imc = c->utilde ? c->imc : nullptr;
     a.bodyF = ws.bodyF;
+    a.redo = !c->fmm[0].on;
+    a.qsrc = c->utilde ? ws.src32n : ws.src32;
     double* alpha = ws.T;  // the single-precision path keeps no T: its first ncell entries hold alpha
     k_alpha32<<<c->ncell, kAlphaThreads, 0, c->stream>>>(a, alpha);
     BIE_LAUNCH(c, "k_alpha32");

@@ -315,6 +315,7 @@ __global__ void k_body_img(const int* __restrict__ imc, const double* __restrict
 
 int build_geometry(bie_ctx* c) {
     ++c->epoch;  // node data and the adopted proxy fit (pointers swapped by a time step)
+    ++c->geometry;
     c->ws_x = nullptr;  // positions change: the workspace's sources are stale
     int bs = 256, gs = (c->N + bs - 1) / bs;
     int* gflag = c->cl.flags + 6 + 1;  // doubled-cell violations (read with the close pairs)
