@@ -594,11 +594,14 @@ int solve_device(bie_ctx* c, const double* b, double* x, bool use_guess, bie_sol
                 else res_prec = BIE_FP64;
             }
         }
-        for (int q = 0; q < nc; ++q)
-            if (beta[q] > 0.0)
-                atol[q] = (mixed && inner_prec == BIE_MIXED)
-                              ? std::max(c->opts.inner_tol * rn[q], 0.5 * tol * bnorm[q])
-                              : 0.5 * tol * bnorm[q];
+        for (int q = 0; q < nc; ++q) {
+            if (!(beta[q] > 0.0)) continue;
+            // a sweep whose inner tolerance would end within a factor of two of the
+            // final one goes on to it: a few iterations instead of another sweep
+            // (and its residual) for the last factor
+            const double last = 0.5 * tol * bnorm[q], inner = c->opts.inner_tol * rn[q];
+            atol[q] = mixed && inner_prec == BIE_MIXED && inner > 4.0 * last ? inner : last;
+        }
         if (!left || outer == max_outer) break;
         int napply = 0;
         if (mixed) {
