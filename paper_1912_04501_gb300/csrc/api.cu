@@ -36,14 +36,14 @@ static void free_all(bie_ctx* c) {
     free_fmm(c);
     void* ptrs[] = {c->cells, c->node_cell, c->body_cell, c->x, c->y, c->nx, c->ny, c->w, c->kap, c->owner, c->body,
                     c->tgt32, c->posdf, c->xw, c->yw, c->imc, c->bimg, c->ws.src32n, c->ws.src64u, c->next.yp,
-                    c->next.ypf, c->glc, c->contour_part, c->bshape, c->near_ctr,
+                    c->next.ypf, c->glc, c->contour_part, c->bshape, c->near_ctr, c->fin_chunks,
                     c->gl_s, c->A, c->beta, c->P, c->wall, c->e2d, c->next.A, c->next.beta, c->next.P,
                     c->next.wall, c->next.e2, c->yp, c->ypf, c->scal, c->ws.sigma, c->ws.out, c->ws.src64, c->ws.src32,
                     c->ws.srcdf, c->ws.bodyF, c->ws.part, c->ws.gpart, c->ws.gt, c->ws.dticket, c->sv.ticket, c->ws.xi, c->ws.xif, c->ws.T, c->ws.vpart, c->sv.V,
                     c->sv.w, c->sv.r, c->sv.x, c->sv.b, c->sv.d, c->sv.h, c->sv.fac, c->sv.dpart,
                     c->sv.chunks,
                     c->sv.cell_chunks, c->sv.sigma_prev, c->sv.sigma_prev2, c->sv.aug, c->sv.d2,
-                    c->sv.feat, c->sv.pred, c->cl.dmin, c->cl.dmin_prev, c->cl.ddir, c->cl.slots, c->cl.count, c->cl.pair_base, c->cl.pairs,
+                    c->sv.feat, c->sv.pred, c->cl.dmin, c->cl.dmin_prev, c->cl.ddir, c->cl.slots, c->cl.count, c->cl.pair_base, c->cl.pairs, c->cl.psum,
                     c->cl.blk_off, c->cl.blocks, c->cl.blocks32, c->cl.flags, c->cl.dtab, c->cl.dtab_off,
                     c->cl.bkd, c->cl.bcot, c->cl.bary, c->near[0].items,
                     c->near[1].items, c->near[2].items};
@@ -54,6 +54,7 @@ static void free_all(bie_ctx* c) {
     c->ev_pool.clear();
     if (c->next_done) cudaEventDestroy(c->next_done);
     if (c->aux_fork) cudaEventDestroy(c->aux_fork);
+    if (c->aux_up) cudaEventDestroy(c->aux_up);
     if (c->aux_join) cudaEventDestroy(c->aux_join);
     for (auto e : c->sv.ev)
         if (e) cudaEventDestroy(e);
@@ -461,6 +462,7 @@ int bie_init_batch(bie_ctx** out, int32_t n_cells, const bie_cell* cells, const 
     if (!rc) rc = cu(cudaEventCreateWithFlags(&c->next_done, cudaEventDisableTiming), "cudaEventCreate");
     if (!rc) rc = cu(cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking), "cudaStreamCreate");
     if (!rc) rc = cu(cudaEventCreateWithFlags(&c->aux_fork, cudaEventDisableTiming), "cudaEventCreate");
+    if (!rc) rc = cu(cudaEventCreateWithFlags(&c->aux_up, cudaEventDisableTiming), "cudaEventCreate");
     if (!rc) rc = cu(cudaEventCreateWithFlags(&c->aux_join, cudaEventDisableTiming), "cudaEventCreate");
     rc = rc ? rc : dalloc(c, &c->yp, nc * 2 * M);
     rc = rc ? rc : dalloc(c, &c->ypf, nc * M);
@@ -529,6 +531,7 @@ int bie_init_batch(bie_ctx** out, int32_t n_cells, const bie_cell* cells, const 
         rc = rc ? rc : dalloc(c, &c->cl.pair_base, (size_t)n + 1);
         rc = rc ? rc : dalloc(c, &c->cl.pairs, c->cl.cap_pairs);
         rc = rc ? rc : dalloc(c, &c->cl.blk_off, c->cl.cap_pairs);
+        rc = rc ? rc : dalloc(c, &c->cl.psum, c->cl.cap_pairs);
         rc = rc ? rc : dalloc(c, &c->cl.blocks, (size_t)c->cl.cap_doubles);
         rc = rc ? rc : dalloc(c, &c->cl.blocks32, (size_t)c->cl.cap_doubles);
         rc = rc ? rc : dalloc(c, &c->cl.flags, 10);

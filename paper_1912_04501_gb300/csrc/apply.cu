@@ -14,16 +14,15 @@
 //                   split, cell) (its last block per wall point forms
 //                   g~ = g0 - g, Sec. 6.2 step 3)
 //   k_xi            (auxiliary stream) xi = P g~ per (row, cell) (Sec. 6.2 step 3)
-// then, single precision (close.cu):
+// then (close.cu), after the direct single-precision sum:
 //   k_alpha32       alpha = -T_0 . n_0 per cell
 //   k_assemble32    per target: T = partials + on-curve diagonal + proxy traction
 //                   (step 4) + close evaluation (Sec. 6.3) with the own-body and
 //                   close pairs redone from positions differenced in double-float;
 //                   y = sigma/2 + T + alpha n + L sigma
-// or, FP64 and double-float:
-//   k_correct       T = sum of partials + on-curve diagonal + proxy traction (step 4)
-//   k_close_apply   close-evaluation correction (Sec. 6.3)
-//   k_finish        alpha = -T_0 . n_0 per cell;  y = sigma/2 + T + alpha n + L sigma
+// and after the others:
+//   k_finish        the same in one launch, nothing redone
+// The near sum itself runs by expansions where that is faster (fmm.cu).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -1118,17 +1117,31 @@ k_disc(const Src64* __restrict__ src64, const float4* __restrict__ src32, const 
 // to ~1/lam, so a plain double-precision product would add relative noise
 // ~1e-11 to the correction and put a floor under the GMRES residual).  xi is
 // also stored in single precision for the single-precision correction.
+// gimg: the discrepancy as k_side leaves it (six far images' parts and the
+// force per cell); otherwise gt holds g~.
 __global__ void __launch_bounds__(32)
-k_xi(const double* __restrict__ gt, int m, int M, const Cell* __restrict__ cells, const double* __restrict__ Pall,
-     double* __restrict__ xiall, float* __restrict__ xifall) {
+k_xi(const double* __restrict__ gt, const double* __restrict__ gimg, int m, int M, const Cell* __restrict__ cells,
+     const double* __restrict__ Pall, double* __restrict__ xiall, float* __restrict__ xifall) {
     const int lane = threadIdx.x, r = blockIdx.x, cidx = blockIdx.y;
     if (!cells[cidx].active) return;
     const int nv = 8 * m;
-    const double* d = gt + (size_t)cidx * nv;
+    const double* d = gimg ? nullptr : gt + (size_t)cidx * nv;
+    const double* gi = gimg ? gimg + (size_t)cidx * 7 * nv : nullptr;
+    const Cell& cl = cells[cidx];
     const double* P = Pall + (size_t)cidx * 2 * M * nv;
     double s = 0, e = 0;
     for (int cc = lane; cc < nv; cc += 32) {
-        const double a = P[(size_t)r * nv + cc], b = d[cc];
+        const double a = P[(size_t)r * nv + cc];
+        double b;
+        if (gi) {  // g~ = g0 - g from the far images' parts (k_side), as k_disc's last block forms it
+            const int L = cc < 4 * m, k = (cc % (4 * m)) / m, wp = (L ? 0 : m) + cc % m;
+            double g = 0;
+#pragma unroll
+            for (int im = 0; im < 6; ++im) g += gi[(size_t)im * nv + 4 * wp + k];
+            b = (k < 2 ? 0.0 : gi[6 * (size_t)nv + k - 2] / (2.0 * (L ? cl.l2 : cl.l1))) - g;
+        } else {
+            b = d[cc];
+        }
         const double p = a * b;
         const double pe = fma(a, b, -p);
         const double t = s + p;
@@ -1148,81 +1161,6 @@ k_xi(const double* __restrict__ gt, int m, int M, const Cell* __restrict__ cells
         xiall[(size_t)cidx * 2 * M + r] = s + e;
         xifall[(size_t)cidx * 2 * M + r] = (float)(s + e);
     }
-}
-
-// T = near partials + on-curve diagonal -(kappa/2pi) tau (tau . q) + proxy
-// traction, double-precision paths.  kCorrLanes lanes per target split the
-// near-sum partials and the proxies, then combine with shuffles (fixed order:
-// deterministic).
-__global__ void __launch_bounds__(256)
-k_correct(const double2* __restrict__ part, int prec, int N, const int* __restrict__ node_cell,
-          const Cell* __restrict__ cells, const double2* __restrict__ sigma, const double* __restrict__ x,
-          const double* __restrict__ y, const double* __restrict__ nx, const double* __restrict__ ny,
-          const double* __restrict__ w, const double* __restrict__ kap, const double* __restrict__ ypall,
-          const double* __restrict__ xiall, int M, double2* __restrict__ T) {
-    const int g = (blockIdx.x * blockDim.x + threadIdx.x) / kCorrLanes;
-    const int sub = threadIdx.x % kCorrLanes;
-    const int i = g < N ? g : N - 1;
-    const int cidx = node_cell[i];
-    const Cell& cl = cells[cidx];
-    double tx = 0, ty = 0;
-    const int splits = cl.splits[prec];
-    const long long base = cl.part_off[prec] + (i - cl.node_off);
-    for (int s = sub; s < splits; s += kCorrLanes) {
-        const double2 p = part[base + (long long)s * cl.n_nodes];
-        tx += p.x;
-        ty += p.y;
-    }
-    const double n0 = nx[i], n1 = ny[i];
-    const double* yp = ypall + (size_t)cidx * 2 * M;
-    const double* xi = xiall + (size_t)cidx * 2 * M;
-    const double X = x[i], Y = y[i];
-    double cx = 0, cy = 0;
-    for (int p = sub; p < M; p += kCorrLanes) {
-        const double rx = X - yp[2 * p], ry = Y - yp[2 * p + 1];
-        const double fx = xi[p], fy = xi[M + p];
-        const double inv = 1.0 / (rx * rx + ry * ry);
-        const double cc = ((rx * n0 + ry * n1) * inv) * ((rx * fx + ry * fy) * inv);
-        cx += cc * rx;
-        cy += cc * ry;
-    }
-    tx += -cx / kPi;
-    ty += -cy / kPi;
-#pragma unroll
-    for (int o = kCorrLanes / 2; o > 0; o >>= 1) {
-        tx += __shfl_xor_sync(0xffffffffu, tx, o);
-        ty += __shfl_xor_sync(0xffffffffu, ty, o);
-    }
-    if (sub != 0 || g >= N) return;
-    const double2 sg = sigma[i];
-    const double t0 = -n1, t1 = n0;  // unit tangent
-    const double qx = sg.x * w[i], qy = sg.y * w[i];
-    const double dg = -(kap[i] / (2.0 * kPi)) * (t0 * qx + t1 * qy);
-    T[i] = make_double2(tx + dg * t0, ty + dg * t1);
-}
-
-// The same for the single-precision path, on the FP32 pipe: the partials are
-// added with TwoSum compensation, the proxy traction uses the cell-centred
-// single-precision targets, proxies and strengths; only the per-target
-// results and the diagonal term are formed in double.
-__global__ void k_finish(const double2* __restrict__ T, const double2* __restrict__ sigma, int N,
-                         const double* __restrict__ x, const double* __restrict__ y,
-                         const double* __restrict__ nx, const double* __restrict__ ny,
-                         const int* __restrict__ owner, const double* __restrict__ body,
-                         const double* __restrict__ bodyF, const int* __restrict__ node_cell,
-                         const Cell* __restrict__ cells, double2* __restrict__ out) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const int i0 = cells[node_cell[i]].node_off;  // node 0 of the cell's first body
-    double2 T0 = T[i0];
-    double alpha = -(T0.x * nx[i0] + T0.y * ny[i0]);
-    int b = owner[i];
-    double xc = body[8 * b + 2], yc = body[8 * b + 3];
-    double Fx = bodyF[3 * b], Fy = bodyF[3 * b + 1], tq = bodyF[3 * b + 2];
-    double2 Ti = T[i], s = sigma[i];
-    double ox = 0.5 * s.x + Ti.x + alpha * nx[i] + Fx - (y[i] - yc) * tq;
-    double oy = 0.5 * s.y + Ti.y + alpha * ny[i] + Fy + (x[i] - xc) * tq;
-    out[i] = make_double2(ox, oy);
 }
 
 __global__ void k_rhs(const double* __restrict__ nx, const double* __restrict__ ny,
@@ -1463,7 +1401,12 @@ static_assert(kNear32Shapes == 5 && BIE_SHAPE_IS(0, 1, BIE_NEAR32_TPT, BIE_NEAR3
 // 2 wall discrepancy, proxy fit and correction, close evaluation, assembly.
 // a3 + a4: the wall discrepancy g~ of the packed sources and the proxy
 // strengths xi = P g~ on stream st (independent of the near sum)
-static int launch_disc_xi(bie_ctx* c, bool f32, Workspace& ws, cudaStream_t st) {
+static int launch_disc_xi(bie_ctx* c, bool f32, bool walls, Workspace& ws, cudaStream_t st) {
+    if (walls) {  // k_side has left the discrepancy's parts
+        k_xi<<<dim3(2 * c->M, c->ncell), 32, 0, st>>>(ws.gt, ws.gpart, c->m, c->M, c->cells, c->P, ws.xi, ws.xif);
+        BIE_LAUNCH(c, "k_xi");
+        return BIE_OK;
+    }
     const dim3 dgrid(2 * c->m, kDiscSplits, c->ncell);
     if (c->utilde) {
         if (f32)
@@ -1480,18 +1423,18 @@ static int launch_disc_xi(bie_ctx* c, bool f32, Workspace& ws, cudaStream_t st) 
                                                     ws.dticket, ws.gt, nullptr);
     }
     BIE_LAUNCH(c, "k_disc");
-    k_xi<<<dim3(2 * c->M, c->ncell), 32, 0, st>>>(ws.gt, c->m, c->M, c->cells, c->P, ws.xi, ws.xif);
+    k_xi<<<dim3(2 * c->M, c->ncell), 32, 0, st>>>(ws.gt, nullptr, c->m, c->M, c->cells, c->P, ws.xi, ws.xif);
     BIE_LAUNCH(c, "k_xi");
     return BIE_OK;
 }
 
 // One operator application in four parts: 0 packs the sources and body
 // moments, 1 is the near sum, 2 the wall discrepancy and proxy strengths
-// (independent of 1), 3 the assembly (traction, close evaluation, pressure
-// fix, rigid completion).
-static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, int precision, Workspace& ws) {
-    const int N = c->N;
-    const int bs = 256, gs = (N + bs - 1) / bs;
+// (independent of 1 after the direct sum, from its boxes' moments after the
+// fast one) and the close pairs' sums, 3 the assembly (traction, close
+// evaluation, pressure fix, rigid completion).
+static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, int precision, Workspace& ws,
+                      cudaStream_t st) {
     const double2* sg = reinterpret_cast<const double2*>(sigma);
     const bool f32 = precision == BIE_MIXED;
     const bool df = precision == BIE_DF64;
@@ -1500,20 +1443,23 @@ static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, i
     if (part == 0) {
         if (&ws == &c->ws) c->ws_x = nullptr;  // the workspace is about to change
         if (c->utilde)
-            k_pack_moments_u<<<c->nb, 256, 0, c->stream>>>(sg, c->x, c->y, c->w, c->body, c->body_cell, c->cells,
+            k_pack_moments_u<<<c->nb, 256, 0, st>>>(sg, c->x, c->y, c->w, c->body, c->body_cell, c->cells,
                                                            c->imc, f32 && !fast ? ws.src32 : nullptr,
                                                            f32 ? ws.src32n : nullptr, ws.src64,
                                                            !f32 && !df && !fast ? ws.src64u : nullptr,
                                                            df && !fast ? (SrcDF*)ws.srcdf : nullptr, ws.bodyF);
         else
-            k_pack_moments<<<c->nb, 256, 0, c->stream>>>(sg, c->x, c->y, c->w, c->body, c->body_cell, c->cells,
+            k_pack_moments<<<c->nb, 256, 0, st>>>(sg, c->x, c->y, c->w, c->body, c->body_cell, c->cells,
                                                          f32 ? ws.src32 : nullptr, ws.src64,
                                                          df && !fast ? (SrcDF*)ws.srcdf : nullptr, ws.bodyF);
         BIE_LAUNCH(c, "k_pack_moments");
         return BIE_OK;
     }
     if (part == 1) {
-        if (fast) return fmm_near(c, sigma, prec, ws);
+        if (fast) {
+            if (int rc = fmm_up(c, sigma, prec, ws)) return rc;
+            return fmm_across(c, prec, ws);
+        }
         if (f32) return launch_near32(c, ws.src32, (float2*)ws.part);
         if (c->utilde) {
             if (df)
@@ -1539,17 +1485,15 @@ static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, i
         }
         return BIE_OK;
     }
-    if (part == 2) return launch_disc_xi(c, f32, ws, c->stream);
-    if (f32) return assemble32(c, sigma, ws, yout);
-    double2* T = reinterpret_cast<double2*>(ws.T);
-    const int gsc = (N * kCorrLanes + 255) / 256;
-    k_correct<<<gsc, 256, 0, c->stream>>>((const double2*)ws.part, prec, N, c->node_cell, c->cells, sg, c->xw, c->yw,
-                                          c->nx, c->ny, c->w, c->kap, c->yp, ws.xi, c->M, T);
-    BIE_LAUNCH(c, "k_correct");
-    if (int rc = close_apply(c, sigma, ws.T)) return rc;
-    k_finish<<<gs, bs, 0, c->stream>>>(T, sg, N, c->x, c->y, c->nx, c->ny, c->owner, c->body, ws.bodyF, c->node_cell,
-                                       c->cells, reinterpret_cast<double2*>(yout));
-    BIE_LAUNCH(c, "k_finish");
+    if (part == 2) {
+        const bool walls = fast && c->fmm[prec].walls;
+        if (fast || !f32)
+            if (int rc = side(c, sigma, prec, walls, ws, st)) return rc;
+        return launch_disc_xi(c, f32, walls, ws, st);
+    }
+    if (f32 && !fast) return assemble32(c, sigma, ws, yout);
+    if (int rc = finish(c, sigma, prec, ws, yout)) return rc;
+    if (f32) return BIE_OK;
     // an FP64-class application over every cell leaves the double-precision
     // sources, body moments and proxy strengths of sigma in the workspace
     if (&ws == &c->ws) {
@@ -1563,23 +1507,43 @@ static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, i
 static int apply_impl(bie_ctx* c, const double* sigma, double* yout, int precision, Workspace& ws) {
     const int kind = precision == BIE_MIXED ? 0 : (precision == BIE_DF64 ? 2 : 1);
     if (int rc = fmm_build(c, kind)) return rc;
-    if (int rc = apply_part(c, 0, sigma, yout, precision, ws)) return rc;
+    const auto record = [](cudaEvent_t e, cudaStream_t from, cudaStream_t to) {
+        const cudaError_t rc = cudaEventRecord(e, from);
+        return rc == cudaSuccess ? cudaStreamWaitEvent(to, e, 0) : rc;
+    };
+    if (c->fmm[kind].on) {
+        // everything but the image sum on the auxiliary stream: the pack at once,
+        // the walls and close pairs once the boxes' moments are there
+        BIE_CUDA(c, record(c->aux_fork, c->stream, c->aux));
+        if (int rc = prof_begin(c, kind)) return rc;
+        if (int rc = fmm_up(c, sigma, kind, ws)) return rc;
+        BIE_CUDA(c, cudaEventRecord(c->aux_up, c->stream));
+        if (int rc = apply_part(c, 0, sigma, yout, precision, ws, c->aux)) return rc;
+        BIE_CUDA(c, cudaStreamWaitEvent(c->aux, c->aux_up, 0));
+        if (int rc = apply_part(c, 2, sigma, yout, precision, ws, c->aux)) return rc;
+        BIE_CUDA(c, cudaEventRecord(c->aux_join, c->aux));
+        if (int rc = fmm_across(c, kind, ws)) return rc;
+        if (int rc = prof_end(c)) return rc;
+        BIE_CUDA(c, cudaStreamWaitEvent(c->stream, c->aux_join, 0));
+        return apply_part(c, 3, sigma, yout, precision, ws, c->stream);
+    }
+    if (int rc = apply_part(c, 0, sigma, yout, precision, ws, c->stream)) return rc;
     // part 2 on the auxiliary stream, overlapping the near sum
-    BIE_CUDA(c, cudaEventRecord(c->aux_fork, c->stream));
-    BIE_CUDA(c, cudaStreamWaitEvent(c->aux, c->aux_fork, 0));
-    if (int rc = launch_disc_xi(c, precision == BIE_MIXED, ws, c->aux)) return rc;
+    BIE_CUDA(c, record(c->aux_fork, c->stream, c->aux));
+    if (int rc = apply_part(c, 2, sigma, yout, precision, ws, c->aux)) return rc;
     BIE_CUDA(c, cudaEventRecord(c->aux_join, c->aux));
     if (int rc = prof_begin(c, kind)) return rc;
-    if (int rc = apply_part(c, 1, sigma, yout, precision, ws)) return rc;
+    if (int rc = apply_part(c, 1, sigma, yout, precision, ws, c->stream)) return rc;
     if (int rc = prof_end(c)) return rc;
     BIE_CUDA(c, cudaStreamWaitEvent(c->stream, c->aux_join, 0));
-    return apply_part(c, 3, sigma, yout, precision, ws);
+    return apply_part(c, 3, sigma, yout, precision, ws, c->stream);
 }
 
 // The single-precision application replayed from CUDA graphs (opts.graph):
 // the parts of apply_part are captured once per epoch (any change of their
 // arguments: geometry, proxy fit, close pairs, work items) as three graphs
-// (pack with the wall discrepancy and proxy strengths; near sum; assembly)
+// (pack; near sum; assembly, the wall discrepancy and proxy strengths with the
+// first or the last)
 // with fixed input and output buffers, on a stream of the context's own (the
 // caller's stream may be the legacy default stream, which cannot capture).
 // Each application copies sigma in, replays the graphs on the context's
@@ -1611,10 +1575,13 @@ static int apply_graph(bie_ctx* c, const double* sigma, double* yout) {
             cudaGraph_t graph = nullptr;
             e = cudaStreamBeginCapture(g.capture, cudaStreamCaptureModeThreadLocal);
             if (e != cudaSuccess) break;
-            // graphs: pack + wall discrepancy and proxy strengths; near sum; assembly
+            // graphs: pack; near sum; assembly, with the wall discrepancy and proxy
+            // strengths in the first, or (they read the fast sum's moments) the third
             static constexpr int kFirst[3] = {0, 1, 3};
-            rc = apply_part(c, kFirst[part], g.in, g.out, BIE_MIXED, c->ws);
-            if (!rc && part == 0) rc = apply_part(c, 2, g.in, g.out, BIE_MIXED, c->ws);
+            const bool last = c->fmm[0].on;
+            if (part == 2 && last) rc = apply_part(c, 2, g.in, g.out, BIE_MIXED, c->ws, c->stream);
+            if (!rc) rc = apply_part(c, kFirst[part], g.in, g.out, BIE_MIXED, c->ws, c->stream);
+            if (!rc && part == 0 && !last) rc = apply_part(c, 2, g.in, g.out, BIE_MIXED, c->ws, c->stream);
             e = cudaStreamEndCapture(g.capture, &graph);
             if (!rc && e == cudaSuccess) e = cudaGraphInstantiate(&g.exec[part], graph, 0);
             if (graph) cudaGraphDestroy(graph);
@@ -1851,7 +1818,7 @@ int fp64_moments_and_xi(bie_ctx* c, const double* sigma, bool reuse_ws) {
                 c->ws.src64, nullptr, c->cells, c->m, c->wall, c->ws.bodyF, c->ws.gpart, c->ws.dticket, c->ws.gt,
                 nullptr);
         BIE_LAUNCH(c, "k_disc");
-        k_xi<<<dim3(2 * c->M, c->ncell), 32, 0, c->stream>>>(c->ws.gt, c->m, c->M, c->cells, c->P, c->ws.xi,
+        k_xi<<<dim3(2 * c->M, c->ncell), 32, 0, c->stream>>>(c->ws.gt, nullptr, c->m, c->M, c->cells, c->P, c->ws.xi,
                                                                c->ws.xif);
         BIE_LAUNCH(c, "k_xi");
     }

@@ -51,11 +51,13 @@ extern "C" int bie_apply_static(bie_ctx* c, const double* sigma, double* out) {
     const size_t b_tk = round256(nc * 2 * c->m * sizeof(unsigned int));
     const size_t b_T = round256(2 * N * sizeof(double));
     const Fmm& fm = c->fmm[0];
+    const size_t b_ps = fm.on ? round256((size_t)c->cl.npairs * sizeof(float2)) : 0;
     const size_t b_fsq = fm.on ? round256(fm.sq_bytes) : 0;
     const size_t b_fmp = fm.on ? round256(fm.mp_bytes) : 0;
+    const size_t b_floc = fm.on ? round256(fm.loc_bytes) : 0;
     const size_t b_ftk = fm.on ? round256(fm.t.nbox * sizeof(unsigned)) : 0;
     const size_t need = b_src32 + b_src32n + b_src64 + b_part + b_body + b_gpart + b_xi + b_xif + b_gt + b_tk + b_T +
-                        b_fsq + 2 * b_fmp + b_ftk;
+                        b_ps + b_fsq + b_fmp + b_floc + b_ftk;
     if (need > BIE_STATIC_SCRATCH_BYTES)
         return fail(c, BIE_EINVAL, "bie_apply_static: this context needs " + std::to_string(need) +
                                        " bytes of scratch; the static array holds " +
@@ -103,12 +105,14 @@ extern "C" int bie_apply_static(bie_ctx* c, const double* sigma, double* out) {
     ws.T = reinterpret_cast<double*>(base + o);
     o += b_T;
     if (fm.on) {
+        if (b_ps) ws.psum = base + o;
+        o += b_ps;
         ws.fsq = base + o;
         o += b_fsq;
         ws.fmp = base + o;
         o += b_fmp;
         ws.floc = base + o;
-        o += b_fmp;
+        o += b_floc;
         ws.ftick = reinterpret_cast<unsigned*>(base + o);
         BIE_CUDA(c, cudaMemsetAsync(ws.ftick, 0, b_ftk, c->stream));
     }

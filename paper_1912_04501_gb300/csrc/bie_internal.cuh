@@ -60,11 +60,11 @@ constexpr Near32Shape kNear32ShapeList[kNear32Shapes] = {
 static_assert(kNear32Shapes == BIE_NEAR32_SHAPES, "shape count of the public header");
 constexpr int kNear32CompChunk = 2048;  // splits with more sources use compensated tile accumulation
 constexpr int kDiscSplits = 8;        // source splits per wall point of the wall-discrepancy kernel
-constexpr int kCorrLanes = 8;         // lanes per target in k_correct (a power of two <= 32)
 constexpr int kVelSplits = 8;         // source splits per body in the velocity extraction
 constexpr int kDotChunk = 256;        // vector entries per partial dot product (chunks never span cells)
 constexpr int kMaxProxy = 256;
 constexpr int kMaxColl = 128;
+constexpr int kFinNodes = 128;        // nodes per CTA of the assembly (chunks never span cells)
 constexpr int kCloseSlots = 8;        // close body images per target node
 constexpr int kMaxRho = 4096;         // largest fine-rule factor of the close evaluation (a power of two)
 constexpr int kCloseAccNodes = 4096;  // source nodes per CTA of k_close_blocks (shared accumulators)
@@ -78,7 +78,7 @@ constexpr int kNetFeatures = 13;      // node features of the warm start (featur
 constexpr int kMaxAug = 3;            // augmentation directions of the first GMRES cycle
 
 constexpr int kFmmP32 = 24;           // expansion orders of the fast image sum (fmm.cu): single precision
-constexpr int kFmmP64 = 56;           // and double
+constexpr int kFmmP64 = 48;           // and double
 constexpr int kFmmLevels = 12;
 
 // One unit cell of the batch (device table; the host keeps a mirror).
@@ -112,6 +112,7 @@ struct Close {
                                   //  smallest gap below min_gap (8 bytes), largest rho, doubled-cell
                                   //  violations (bit 0: a node beyond the doubled cell, bit 1: a close
                                   //  pair's body image not wholly among its nodes' images), block doubles (8 bytes)]
+    double2* psum = nullptr;      // cap_pairs: the pairs' sums of one application
     int cap_pairs = 0;
     long long cap_doubles = 0;
     bool grow = true;             // storage grows on demand (no close_capacity given)
@@ -147,15 +148,16 @@ struct Workspace {
     double* bodyF = nullptr;    // 3 nb  (F_x, F_y, tau) per body
     void* part = nullptr;       // near-sum partials (see Cell::part_off)
     size_t part_bytes = 0;
-    double* gpart = nullptr;    // ncell x kDiscSplits x 8m discrepancy partials
+    double* gpart = nullptr;    // ncell x kDiscSplits x 8m discrepancy partials (by expansions: 6 images, and the force)
     double* gt = nullptr;       // ncell x 8m  g~ = g0 - g
     unsigned int* dticket = nullptr;  // ncell x 2m last-block counters of k_disc (zero between launches)
     double* xi = nullptr;       // ncell x 2M proxy strengths
     float* xif = nullptr;       // ncell x 2M the same in single precision
-    double* T = nullptr;        // 2N traction before the pressure fix
+    double* T = nullptr;        // 2N; alpha per cell (k_alpha32)
     double* vpart = nullptr;    // nb x kVelSplits x 3 velocity partials
     // fast image sum: sorted strengths, multipole and local expansions, and
     // the last-child counters of the upward pass (zero between launches)
+    void* psum = nullptr;       // close pairs' sums (null: Close::psum)
     void *fsq = nullptr, *fmp = nullptr, *floc = nullptr;
     unsigned* ftick = nullptr;
 };
@@ -221,6 +223,7 @@ struct FmmCell {
     double ox, oy, h, inv_h;
     int nlev;
     int gx[kFmmLevels], gy[kFmmLevels], off[kFmmLevels];  // off: the level's first box
+    int wall;  // level whose boxes the walls' far images are well away from
 };
 
 // Node data the sorting reads.
@@ -235,6 +238,7 @@ struct FmmTree {
     const FmmCell* cells = nullptr;
     const int4* box = nullptr;     // nbox: (cell, level, x | y << 16, parent or -1); leaves first
     int nbox = 0, nleaf = 0;
+    float4* centre = nullptr;      // nleaf: leaf centres from the cell centre, double-float
     int *scount = nullptr, *tcount = nullptr;  // nbox: records in the box
     int *sstart = nullptr, *tstart = nullptr;  // nleaf + 1: first sorted record
     int *sperm = nullptr, *tperm = nullptr;    // sorted record -> record (sources: node, or 4 node + image)
@@ -247,9 +251,11 @@ struct Fmm {
     FmmTree t;
     FmmCell* cells = nullptr;
     int4* box = nullptr;
+    bool walls = false;                // the wall discrepancy runs by expansions too
     int *cursor = nullptr, *leaf = nullptr, *raw = nullptr;  // sorting scratch
     unsigned long long built = 0;      // geometry the records are sorted for (0: none)
-    size_t mp_bytes = 0, sq_bytes = 0; // expansions (each way) and sorted strengths
+    int shares = 1;                    // CTAs a box's list is split over
+    size_t mp_bytes = 0, loc_bytes = 0, sq_bytes = 0;  // multipole and local expansions, sorted strengths
     std::vector<void*> owned;
 };
 
@@ -308,7 +314,7 @@ struct bie_ctx {
     // the wall discrepancy and proxy strengths of an application run on this
     // stream while the near sum runs on the context's stream (direct launches)
     cudaStream_t aux = nullptr;
-    cudaEvent_t aux_fork = nullptr, aux_join = nullptr;
+    cudaEvent_t aux_fork = nullptr, aux_up = nullptr, aux_join = nullptr;
     double* yp = nullptr;       // ncell x M x 2 proxy points of the current fit
     float2* ypf = nullptr;      // ncell x M proxy points minus the cell centre (single precision)
     double* scal = nullptr;     // 3 nb + ncell + 8: velocities, rotation rates, mu_eff
@@ -318,9 +324,11 @@ struct bie_ctx {
     bie::Close cl;
     bie::NearItems near[3];     // 0 single precision, 1 double, 2 double-float
     int shape32 = 0;            // tile shape of the single-precision near sum (kNear32ShapeList)
+    int4* fin_chunks = nullptr; // n_fin: (cell, first node, end node, 0)
+    int n_fin = 0;
     int* near_ctr = nullptr;    // work-queue counter of the persistent near sum (batches)
     bie::Fmm fmm[3];            // fast image sum per precision (0 single, 1 double, 2 double-float)
-    void* fmm_tab[2] = {nullptr, nullptr};  // its constant matrices (single, double)
+    void* fmm_tab[3] = {};      // its constant matrices
     std::vector<double> fmm_rects;          // 4 x ncell: the rectangles its boxes cover
     unsigned long long geometry = 0;        // bumped by build_geometry
     unsigned long long epoch = 0;  // bumped whenever a kernel argument of the operator application changes
@@ -408,18 +416,20 @@ int build_precond(bie_ctx* c);                             // opts.precond: cont
 int precond_apply(bie_ctx* c, const double* v, double* z); // z = M^-1 v
 void free_precond(bie_ctx* c);
 void free_graph(bie_ctx* c);
-// T += C sigma; with src32 (the single-precision path's packed sources) the
-// own-body and close pairs of the single-precision near sum are also redone
-// with positions differenced in double precision
-int close_apply(bie_ctx* c, const double* sigma, double* T);
-// the single-precision application's assembly: traction, close evaluation,
-// pressure fix and rigid completion in two launches (close.cu)
+// assembly of an application: traction, close evaluation, pressure fix and
+// rigid completion; after the direct single-precision sum (with the own-body
+// and close pairs redone) and after the other sums
 int assemble32(bie_ctx* c, const double* sigma, const Workspace& ws, double* yout);
+int finish(bie_ctx* c, const double* sigma, int prec, const Workspace& ws, double* yout);
 
 // fmm.cu --------------------------------------------------------------------
 int fmm_plan(bie_ctx* c);             // boxes for the bodies' current places (host mirror)
 int fmm_build(bie_ctx* c, int prec);  // sorts the current geometry if it is not
-int fmm_near(bie_ctx* c, const double* sigma, int prec, Workspace& ws);
+int fmm_up(bie_ctx* c, const double* sigma, int prec, Workspace& ws);     // moments of every box
+int fmm_across(bie_ctx* c, int prec, Workspace& ws);                      // partials of every target from them
+// on stream st: the wall discrepancy from the boxes' moments (walls true) and
+// the close pairs' sums of sigma
+int side(bie_ctx* c, const double* sigma, int prec, bool walls, Workspace& ws, cudaStream_t st);
 void free_fmm(bie_ctx* c);
 
 // apply.cu ------------------------------------------------------------------
@@ -460,6 +470,15 @@ __device__ __forceinline__ float rcp_approx(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
+}
+
+// 1 / x by the hardware's approximation (20 bits) and one step of the cubic
+// iteration r <- r (1 + e + e^2), e = 1 - x r
+__device__ __forceinline__ double rcp64(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
 // Error-free sum: s + e == a + b exactly (Knuth's TwoSum, 6 operations).
@@ -574,6 +593,69 @@ __device__ __forceinline__ void pair_df(float pxh, float pxl, float pyh, float p
     pair_df_x(pxh, pxl, nxh, nxl, y, q, axh, axe, ayh, aye);
 }
 
+// Double-float arithmetic (an unevaluated sum of two floats, ~48 bits) with the
+// operators the expansions need, so that the double-float application runs on
+// the FP32 pipe throughout: a multiply-add is 13 FP32 instructions, and GB300's
+// FP64 pipe issues one DFMA in the time of 64 of them.
+struct df {
+    float h, l;
+    df() = default;
+    __host__ __device__ df(float a, float b) : h(a), l(b) {}
+    __host__ __device__ df(float a) : h(a), l(0.f) {}
+    __host__ __device__ df(int a) : h((float)a), l(0.f) {}  // |a| < 2^24
+    __host__ __device__ df(double a) : h((float)a), l((float)(a - (double)(float)a)) {}
+};
+__device__ __forceinline__ df operator-(df a) { return df(-a.h, -a.l); }
+__device__ __forceinline__ df operator+(df a, df b) {
+    float s, e;
+    two_sum(a.h, b.h, s, e);
+    e += a.l + b.l;
+    fast2(s, e);
+    return df(s, e);
+}
+__device__ __forceinline__ df operator-(df a, df b) { return a + (-b); }
+__device__ __forceinline__ df operator*(df a, df b) {
+    float p = a.h * b.h;
+    float e = fmaf(a.h, b.h, -p);
+    e = fmaf(a.h, b.l, fmaf(a.l, b.h, e));
+    fast2(p, e);
+    return df(p, e);
+}
+// a b + c, the sum not renormalised (c an accumulator: its low part stays a
+// few roundings of the high part)
+__device__ __forceinline__ df fma_(df a, df b, df c) {
+    const float p = a.h * b.h;
+    float e = fmaf(a.h, b.h, -p);
+    e = fmaf(a.h, b.l, fmaf(a.l, b.h, e));
+    float s, t;
+    two_sum(c.h, p, s, t);
+    return df(s, c.l + (t + e));
+}
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ df renorm(df a) {
+    fast2(a.h, a.l);
+    return a;
+}
+__device__ __forceinline__ float renorm(float a) { return a; }
+__device__ __forceinline__ double renorm(double a) { return a; }
+__device__ __forceinline__ df ldcg(const df* p) {
+    const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+    return df(v.x, v.y);
+}
+__device__ __forceinline__ float ldcg(const float* p) { return __ldcg(p); }
+__device__ __forceinline__ double ldcg(const double* p) { return __ldcg(p); }
+__device__ __forceinline__ double to_double(df a) { return (double)a.h + (double)a.l; }
+__device__ __forceinline__ double to_double(double a) { return a; }
+__device__ __forceinline__ double to_double(float a) { return a; }
+
+__device__ __forceinline__ float rcp(float a) { return rcp_approx(a); }
+__device__ __forceinline__ double rcp(double a) { return rcp64(a); }
+__device__ __forceinline__ df rcp(df a) {  // MUFU reciprocal and one residual step
+    const float i = rcp_approx(a.h);
+    const float e = fmaf(-a.l, i, fmaf(-a.h, i, 1.0f));
+    return renorm(df(i, i * e));
+}
 // Packed pairs of floats (PTX .f32x2 on sm_100-family GPUs): one instruction
 // performs the same round-to-nearest operation on both halves, so results are
 // bit-identical to the scalar operations, with half the issue slots.

@@ -589,40 +589,6 @@ k_close_blocks_bary(const int4* __restrict__ pairs, const long long* __restrict_
     }
 }
 
-// One warp per target: T_i += sum over its pairs of C sigma_b (slot order).
-__global__ void k_close_apply(const int* __restrict__ pair_base, const int4* __restrict__ pairs,
-                              const long long* __restrict__ blk_off, const double* __restrict__ blocks,
-                              const double* __restrict__ body, const double2* __restrict__ sigma, int N,
-                              double2* __restrict__ T) {
-    int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (wid >= N) return;
-    int p0 = pair_base[wid], p1 = pair_base[wid + 1];
-    if (p0 == p1) return;
-    double tx = 0, ty = 0;
-    for (int p = p0; p < p1; ++p) {
-        int b = pairs[p].y;
-        int nbn = (int)body[8 * b + 5], off = (int)body[8 * b + 6];
-        const double* C = blocks + blk_off[p];
-        double ax = 0, ay = 0;
-        for (int k = lane; k < nbn; k += 32) {
-            double2 s = sigma[off + k];
-            double A = C[3 * k], B = C[3 * k + 1], D = C[3 * k + 2];
-            ax = fma(A, s.x, fma(B, s.y, ax));
-            ay = fma(B, s.x, fma(D, s.y, ay));
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            ax += __shfl_xor_sync(0xffffffffu, ax, o);
-            ay += __shfl_xor_sync(0xffffffffu, ay, o);
-        }
-        tx += ax;
-        ty += ay;
-    }
-    if (lane == 0) {
-        double2 t = T[wid];
-        T[wid] = make_double2(t.x + tx, t.y + ty);
-    }
-}
-
 // Replace *p by a fresh device array of count elements (the old contents are
 // not kept).
 template <typename T>
@@ -700,6 +666,7 @@ int build_close(bie_ctx* c) {
             const int cap = h[0] + h[0] / 4 + 16;
             int rc = regrow(c, &c->cl.pairs, cap);
             rc = rc ? rc : regrow(c, &c->cl.blk_off, cap);
+            rc = rc ? rc : regrow(c, &c->cl.psum, cap);
             if (rc) return rc;
             c->cl.cap_pairs = cap;
         }
@@ -782,8 +749,9 @@ int build_dirichlet_tables(bie_ctx* c, int rho_max) {
     return BIE_OK;
 }
 
-// Single-precision assembly (a5 + a6 + a7 of one application), one warp
-// per target: the traction T_i is summed from
+// Assembly after the direct single-precision sum (a5 + a6 + a7 of one
+// application; the fast sum needs no redo and takes k_finish), one warp per
+// target: the traction T_i is summed from
 //   - the target's near-sum partials (one per source split, TwoSum per lane),
 //   - the proxy traction sum_p G^t(x_i, y_p; n_i) xi_p (single precision),
 //   - the on-curve diagonal -(kappa_i / 2 pi) tau_i (tau_i . q_i),
@@ -801,9 +769,7 @@ int build_dirichlet_tables(bie_ctx* c, int rho_max) {
 // terms with r formed exactly from double-float positions (then rounded to
 // single precision); the close-evaluation blocks are applied in single
 // precision (stored divided by the weights, acting on q = sigma w).
-// Everything but the final sums runs on the FP32 pipe.  The fast image sum
-// (fmm.cu) already takes its near pairs from double-float positions, so after
-// it nothing is redone.
+// Everything but the final sums runs on the FP32 pipe.
 //
 // With the doubled-cell periodizer (imc non-null) the near sum evaluated the
 // pair at the target's translate inside U (tgt32) against the source's image
@@ -836,8 +802,6 @@ struct Asm32 {
     const Cell* cells;
     const int* imc;
     const double* bodyF;
-    const float4* qsrc;  // per-node strengths q (z, w)
-    int redo;  // the near sum's own-body and close terms are to be redone (direct single-precision sum)
 };
 
 // T_i on every thread of the calling group of NL threads (a warp, NL = 32,
@@ -912,7 +876,7 @@ __device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane, d
         fx += c1 * rx - c0 * dx;
         fy += c1 * ry - c0 * dy;
     };
-    if (a.redo) {
+    {
         const int b = a.owner[i];
         const int nbn = (int)a.body[8 * b + 5], off = (int)a.body[8 * b + 6];
         const float4 p = shifted(4);
@@ -931,8 +895,8 @@ __device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane, d
             const float4 p = shifted(im);
 #pragma unroll 2
             for (int k = lane; k < nbn; k += NL) {
-                if (a.redo) redo(off + k, im, p);
-                const float4 s = a.qsrc[off + k];
+                redo(off + k, im, p);
+                const float4 s = a.src32[a.imc ? 4 * (size_t)(off + k) : (size_t)(off + k)];  // q: the same in every record
                 const float A = C[3 * k], B = C[3 * k + 1], D = C[3 * k + 2];
                 bx = fmaf(A, s.z, fmaf(B, s.w, bx));
                 by = fmaf(B, s.z, fmaf(D, s.w, by));
@@ -1041,8 +1005,6 @@ int assemble32(bie_ctx* c, const double* sigma, const Workspace& ws, double* you
     a.cells = c->cells;
     a.imc = c->utilde ? c->imc : nullptr;
     a.bodyF = ws.bodyF;
-    a.redo = !c->fmm[0].on;
-    a.qsrc = c->utilde ? ws.src32n : ws.src32;
     double* alpha = ws.T;  // the single-precision path keeps no T: its first ncell entries hold alpha
     k_alpha32<<<c->ncell, kAlphaThreads, 0, c->stream>>>(a, alpha);
     BIE_LAUNCH(c, "k_alpha32");
@@ -1053,15 +1015,209 @@ int assemble32(bie_ctx* c, const double* sigma, const Workspace& ws, double* you
     return BIE_OK;
 }
 
-int close_apply(bie_ctx* c, const double* sigma, double* T) {
-    if (c->cl.npairs == 0) return BIE_OK;
-    const int bs = 256;
-    const int gs = (int)((32LL * c->N + bs - 1) / bs);
-    k_close_apply<<<gs, bs, 0, c->stream>>>(c->cl.pair_base, c->cl.pairs, c->cl.blk_off, c->cl.blocks, c->body,
-                                           reinterpret_cast<const double2*>(sigma), c->N,
-                                           reinterpret_cast<double2*>(T));
-    BIE_LAUNCH(c, "k_close_apply");
+// ---------------------------------------------------------------------------
+// Assembly after the fast image sum (single precision) and after every FP64 or
+// double-float sum: T_i = partials + proxy traction + on-curve diagonal + close
+// pairs' sums (k_side), y_i = sigma_i / 2 + T_i + alpha n_i + F_b +
+// (x_i - x^c)^perp tau_b.  One thread per node, a CTA per chunk of one cell's
+// nodes: the double-precision epilogue then costs one instruction per 32 nodes.
+// (A warp per node spent 340 us on it at 102400 nodes, the FP64 pipe issuing a
+// warp instruction every 16 cycles whatever its active lanes.)  The proxies'
+// traction is single precision, double or double-float as the sum's.  alpha =
+// -T(x_1) . n_1 of the cell: each chunk sums T at the cell's first node again
+// (one warp), which is cheaper than a launch of its own.
+// ---------------------------------------------------------------------------
+template <typename R>
+struct Finish {
+    const int4* chunks;
+    int prec, M, use_pairs;
+    const void* part;  // float2, or double2
+    const double* yp;
+    const float2* ypf;  // from the cell centre
+    const double* xi;
+    const float* xif;
+    const int* pair_base;
+    const void* psum;  // per close pair: float2, or double2
+    const double2* sigma;
+    const float4* tgt32;
+    const double *xw, *yw, *x, *y, *nx, *ny, *w, *kap;
+    const int* owner;
+    const double *body, *bodyF;
+    const Cell* cells;
+};
+
+template <typename R>
+struct R2 {
+    R x, y;
+};
+
+// Partials first, first + step, ... and the same proxies' traction at node i.
+template <typename R>
+__device__ __forceinline__ void finish_sum(const Finish<R>& a, const Cell& cl, int i, int first, int step,
+                                           const R2<R>* yp, const R2<R>* xi, double& tx, double& ty) {
+    const long long at = cl.part_off[a.prec] + (i - cl.node_off);
+    const int splits = cl.splits[a.prec];
+    R X, Y, n0, n1;
+    if constexpr (sizeof(R) == 4) {
+        const float2* pp = reinterpret_cast<const float2*>(a.part) + at;
+        float hx = 0, lx = 0, hy = 0, ly = 0;
+        for (int s = first; s < splits; s += step) {
+            const float2 p = pp[(long long)s * cl.n_nodes];
+            float e;
+            two_sum(hx, p.x, hx, e);
+            lx += e;
+            two_sum(hy, p.y, hy, e);
+            ly += e;
+        }
+        tx = (double)hx + (double)lx;
+        ty = (double)hy + (double)ly;
+        const float4 tv = a.tgt32[i];
+        X = tv.x;
+        Y = tv.y;
+        n0 = tv.z;
+        n1 = tv.w;
+    } else {
+        const double2* pp = reinterpret_cast<const double2*>(a.part) + at;
+        tx = ty = 0;
+#pragma unroll 4
+        for (int s = first; s < splits; s += step) {
+            const double2 p = pp[(long long)s * cl.n_nodes];
+            tx += p.x;
+            ty += p.y;
+        }
+        X = R(a.xw[i] - cl.C[0]);
+        Y = R(a.yw[i] - cl.C[1]);
+        n0 = R(a.nx[i]);
+        n1 = R(a.ny[i]);
+    }
+    R cx(0), cy(0);
+#pragma unroll 2
+    for (int p = first; p < a.M; p += step) {
+        const R2<R> q = yp[p], f = xi[p];
+        const R rx = X - q.x, ry = Y - q.y;
+        const R inv = rcp(renorm(fma_(rx, rx, ry * ry)));
+        const R cc = (renorm(fma_(rx, n0, ry * n1)) * inv) * (renorm(fma_(rx, f.x, ry * f.y)) * inv);
+        cx = fma_(cc, rx, cx);
+        cy = fma_(cc, ry, cy);
+    }
+    const double c = -1.0 / kPi;
+    tx += c * to_double(cx);
+    ty += c * to_double(cy);
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kFinNodes)
+k_finish(Finish<R> a, double2* __restrict__ out) {
+    __shared__ R2<R> s_yp[kMaxProxy], s_xi[kMaxProxy];
+    __shared__ double s_t0[2];
+    const int t = threadIdx.x, wid = t >> 5, lane = t & 31;
+    const int4 ch = a.chunks[blockIdx.x];
+    const Cell& cl = a.cells[ch.x];
+    const int i0 = ch.y, i1 = ch.z, head = cl.node_off;
+    for (int p = t; p < a.M; p += kFinNodes) {
+        if constexpr (sizeof(R) == 4) {
+            const float2 q = a.ypf[(size_t)ch.x * a.M + p];
+            const float* xi = a.xif + (size_t)ch.x * 2 * a.M;
+            s_yp[p] = R2<R>{q.x, q.y};
+            s_xi[p] = R2<R>{xi[p], xi[a.M + p]};
+        } else {
+            const double* q = a.yp + ((size_t)ch.x * a.M + p) * 2;
+            const double* xi = a.xi + (size_t)ch.x * 2 * a.M;
+            s_yp[p] = R2<R>{R(q[0] - cl.C[0]), R(q[1] - cl.C[1])};
+            s_xi[p] = R2<R>{R(xi[p]), R(xi[a.M + p])};
+        }
+    }
+    __syncthreads();
+    // on-curve diagonal -(kappa / 2 pi) tau (tau . q), and the node's close pairs in order
+    auto own_terms = [&](int i, double n0, double n1, double2 sg, double& tx, double& ty) {
+        const double t0 = -n1, t1 = n0;
+        const double dg = -(a.kap[i] / (2.0 * kPi)) * (t0 * (sg.x * a.w[i]) + t1 * (sg.y * a.w[i]));
+        tx += dg * t0;
+        ty += dg * t1;
+        if (!a.use_pairs) return;
+        const int p1 = a.pair_base[i + 1];
+        for (int p = a.pair_base[i]; p < p1; ++p) {
+            if constexpr (sizeof(R) == 4) {
+                const float2 v = reinterpret_cast<const float2*>(a.psum)[p];
+                tx += (double)v.x;
+                ty += (double)v.y;
+            } else {
+                const double2 v = reinterpret_cast<const double2*>(a.psum)[p];
+                tx += v.x;
+                ty += v.y;
+            }
+        }
+    };
+    if (wid == 3) {  // T at the cell's first node
+        double tx, ty;
+        finish_sum(a, cl, head, lane, 32, s_yp, s_xi, tx, ty);
+        for (int s = 16; s > 0; s >>= 1) {
+            tx += __shfl_xor_sync(0xffffffffu, tx, s);
+            ty += __shfl_xor_sync(0xffffffffu, ty, s);
+        }
+        if (lane == 0) {
+            own_terms(head, a.nx[head], a.ny[head], a.sigma[head], tx, ty);
+            s_t0[0] = tx;
+            s_t0[1] = ty;
+        }
+    }
+    const int i = i0 + t;
+    double tx = 0, ty = 0, n0 = 0, n1 = 0;
+    double2 sg = make_double2(0.0, 0.0);
+    if (i < i1) {
+        finish_sum(a, cl, i, 0, 1, s_yp, s_xi, tx, ty);
+        n0 = a.nx[i];
+        n1 = a.ny[i];
+        sg = a.sigma[i];
+        own_terms(i, n0, n1, sg, tx, ty);
+    }
+    __syncthreads();
+    if (i >= i1) return;
+    const double al = -(s_t0[0] * a.nx[head] + s_t0[1] * a.ny[head]);
+    const int b = a.owner[i];
+    const double* bd = a.body + 8 * b;
+    const double tq = a.bodyF[3 * b + 2];
+    out[i] = make_double2(0.5 * sg.x + tx + al * n0 + a.bodyF[3 * b] - (a.y[i] - bd[3]) * tq,
+                          0.5 * sg.y + ty + al * n1 + a.bodyF[3 * b + 1] + (a.x[i] - bd[2]) * tq);
+}
+
+template <typename R>
+static int finish_launch(bie_ctx* c, const double* sigma, int prec, const Workspace& ws, double* yout) {
+    Finish<R> a;
+    a.chunks = c->fin_chunks;
+    a.prec = prec;
+    a.M = c->M;
+    a.use_pairs = c->cl.npairs > 0 ? 1 : 0;
+    a.part = ws.part;
+    a.yp = c->yp;
+    a.ypf = c->ypf;
+    a.xi = ws.xi;
+    a.xif = ws.xif;
+    a.pair_base = c->cl.pair_base;
+    a.psum = ws.psum ? ws.psum : c->cl.psum;
+    a.sigma = reinterpret_cast<const double2*>(sigma);
+    a.tgt32 = c->tgt32;
+    a.xw = c->xw;
+    a.yw = c->yw;
+    a.x = c->x;
+    a.y = c->y;
+    a.nx = c->nx;
+    a.ny = c->ny;
+    a.w = c->w;
+    a.kap = c->kap;
+    a.owner = c->owner;
+    a.body = c->body;
+    a.bodyF = ws.bodyF;
+    a.cells = c->cells;
+    k_finish<R><<<c->n_fin, kFinNodes, 0, c->stream>>>(a, reinterpret_cast<double2*>(yout));
+    BIE_LAUNCH(c, "k_finish");
     return BIE_OK;
+}
+
+int finish(bie_ctx* c, const double* sigma, int prec, const Workspace& ws, double* yout) {
+    return prec == 0 ? finish_launch<float>(c, sigma, prec, ws, yout)
+                     : (prec == 1 ? finish_launch<double>(c, sigma, prec, ws, yout)
+                                  : finish_launch<df>(c, sigma, prec, ws, yout));
 }
 
 }  // namespace bie

@@ -22,19 +22,24 @@
 // triples whose parents are near (every far triple at the top) pass by
 // expansions; near triples of the finest level are evaluated pair by pair.
 // Truncation: worst case (two box corners) 0.547^P, typically 1e-2 of that:
-// P = 24 in single precision, P = 56 in double.
+// P = 24 in single precision, P = 48 in double.
 //
-// What bounds it.  Single precision: the pair sum (about 20 instructions per
-// pair, a few hundred pairs per target), then latency; double: the FP64 pipe in
-// the translations (two DFMA per SM and cycle).  Whole applications on GB300,
-// direct sum before and this now: single precision 32.8 -> 0.60 ms on the
-// 400-ellipse cell (102400 nodes), 0.94 -> 0.20 ms at 16000 nodes, 0.21 ->
-// 0.15 ms at 6400; double-float 338 -> 6.6 ms at 102400; FP64 12.2 -> 1.55 ms
-// at 6400.  The single-precision application's error against 64 bits falls
-// (8.6e-7 -> 2.0e-7 at 6400 nodes): near pairs are differenced exactly.
+// Three arithmetics: float, double, and double-float (df, bie_internal.cuh) for
+// the double-float application, all of it on the FP32 pipe.
+//
+// What bounds it.  Single precision: latency up to some 10^4 nodes, then the
+// pair sum (about 20 instructions per pair, a few hundred pairs per target);
+// double: the FP64 pipe in the translations (a warp DFMA per 19 cycles and SM).
+// Whole applications on GB300, direct sum before and this now: single precision
+// 32.8 -> 0.20 ms on the 400-ellipse cell (102400 nodes), 0.94 -> 0.105 ms at
+// 16000 nodes, 0.21 -> 0.092 ms at 6400; double-float 340 -> 1.12 ms at 102400;
+// FP64 12.2 -> 0.86 ms at 6400.  The single-precision application's error
+// against 64 bits falls (4.2e-7 -> 1.2e-7 at 6400 nodes): near pairs are
+// differenced exactly.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "bie_internal.cuh"
@@ -42,10 +47,14 @@
 namespace bie {
 
 template <typename R>
-struct __align__(sizeof(R) * 2) C2 {
+struct __align__(8) C2 {
     R x, y;
 };
-// coefficient pair: (a, e) of one order
+template <>
+struct __align__(16) C2<double> {
+    double x, y;
+};
+// coefficient pair of one order: (a, e)
 template <typename R>
 struct __align__(16) V4 {
     R x, y, z, w;
@@ -53,28 +62,79 @@ struct __align__(16) V4 {
 
 template <typename R>
 __device__ __forceinline__ C2<R> cmul(C2<R> a, C2<R> b) {
-    return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
+    return {renorm(fma_(a.x, b.x, -(a.y * b.y))), renorm(fma_(a.x, b.y, a.y * b.x))};
 }
 template <typename R>
-__device__ __forceinline__ R fma_(R a, R b, R c) {
-    return fma(a, b, c);
+__device__ __forceinline__ C2<R> czero() {
+    return {R(0), R(0)};
 }
-// z^n, 0 <= n < 64, by repeated squaring
 template <typename R>
-__device__ __forceinline__ C2<R> cpow(C2<R> z, int n) {
+__device__ __forceinline__ V4<R> vzero() {
+    return {R(0), R(0), R(0), R(0)};
+}
+// s += c v
+template <typename R>
+__device__ __forceinline__ void axpy(V4<R>& s, R c, const V4<R>& v) {
+    s.x = fma_(c, v.x, s.x);
+    s.y = fma_(c, v.y, s.y);
+    s.z = fma_(c, v.z, s.z);
+    s.w = fma_(c, v.w, s.w);
+}
+// acc += p s (both series by one complex power)
+template <typename R>
+__device__ __forceinline__ void add_scaled(V4<R>& acc, C2<R> p, const V4<R>& s) {
+    const R sx = renorm(s.x), sy = renorm(s.y), sz = renorm(s.z), sw = renorm(s.w);
+    acc.x = fma_(p.x, sx, fma_(-p.y, sy, acc.x));
+    acc.y = fma_(p.x, sy, fma_(p.y, sx, acc.y));
+    acc.z = fma_(p.x, sz, fma_(-p.y, sw, acc.z));
+    acc.w = fma_(p.x, sw, fma_(p.y, sz, acc.w));
+}
+template <typename R>
+__device__ __forceinline__ V4<R> scaled(C2<R> p, C2<R> a, C2<R> e) {
+    const C2<R> va = cmul(p, a), ve = cmul(p, e);
+    return {va.x, va.y, ve.x, ve.y};
+}
+template <typename R>
+__device__ __forceinline__ V4<R> vadd(const V4<R>& a, const V4<R>& b) {
+    return {a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w};
+}
+
+// Powers z^k, 0 <= k < 64, from three small tables (radix 4, 4, 4): entries
+// 0..2 z, z^2, z^3; 3..5 z^4, z^8, z^12; 6..8 z^16, z^32, z^48.
+constexpr int kPowTab = 9;
+template <typename R>
+__device__ __forceinline__ void pow_table(C2<R> z, C2<R>* t) {
+    t[0] = z;
+    t[1] = cmul(z, z);
+    t[2] = cmul(t[1], z);
+    t[3] = cmul(t[1], t[1]);
+    t[4] = cmul(t[3], t[3]);
+    t[5] = cmul(t[4], t[3]);
+    t[6] = cmul(t[4], t[4]);
+    t[7] = cmul(t[6], t[6]);
+    t[8] = cmul(t[7], t[6]);
+}
+template <typename R>
+__device__ __forceinline__ C2<R> pow_at(const C2<R>* t, int k) {
+    const int a = k & 3, b = (k >> 2) & 3, c = k >> 4;
     C2<R> r{R(1), R(0)};
-#pragma unroll
-    for (int b = 0; b < 6; ++b) {
-        if ((n >> b) & 1) r = cmul(r, z);
-        z = cmul(z, z);
-    }
+    if (a) r = t[a - 1];
+    if (b) r = cmul(r, t[2 + b]);
+    if (c) r = cmul(r, t[5 + c]);
     return r;
 }
+
+// storage type <-> arithmetic: strengths (double in memory for double)
 template <typename R>
-__device__ __forceinline__ C2<R> cinv(C2<R> z) {
-    const R s = R(1) / (z.x * z.x + z.y * z.y);
-    return {z.x * s, -z.y * s};
-}
+struct FmmTypes {
+    static constexpr int P = kFmmP64;
+};
+template <>
+struct FmmTypes<float> {
+    static constexpr int P = kFmmP32;
+};
+constexpr int kFmmItems = 96;  // orders x groups of sources or entries per warp: three per lane
+static_assert(kFmmItems % kFmmP32 == 0 && kFmmItems % kFmmP64 == 0, "items");
 
 __host__ __device__ inline int fmm_ix(int4 b) { return b.z & 0xffff; }
 __host__ __device__ inline int fmm_iy(int4 b) { return (b.z >> 16) & 0xffff; }
@@ -187,62 +247,83 @@ __device__ __forceinline__ C2<float> fmm_local(float4 p, float4 c, float inv_h) 
     return {((p.x - c.x) + (p.y - c.y)) * inv_h, ((p.z - c.z) + (p.w - c.w)) * inv_h};
 }
 
-__device__ __forceinline__ double2 fmm_centre(const FmmCell& f, int level, int ix, int iy) {
+__host__ __device__ inline double2 fmm_centre(const FmmCell& f, int level, int ix, int iy) {
     const double H = f.h * (1 << level);
     return make_double2(f.ox + (ix + 0.5) * H, f.oy + (iy + 0.5) * H);
 }
 
-// One warp per leaf: gathers the strengths q = sigma w of the box's sources in
-// sorted order (sq, or sqdf as double-float pairs) and sums their moments (lane
-// k: orders k and k + 32; eta^k = eta^(k % 4) (eta^4)^(k / 4) from two small
-// tables per source); the last child of a parent to finish forms the parent's
-// moments, and so on up.
-template <typename R, int P>
+// Constant tables of one precision (host: fmm_tables): the matrix C(k + l, l)
+// [k][l], the binomials C(m, k) [k][m], and for a child at (+-1/4, +-1/4) of its
+// parent delta^m and (1 / (2 delta))^k.
+template <typename R>
+struct FmmTab {
+    const R *hankel, *binom;
+    const C2<R>*dpow, *gpow;  // [quadrant][order]
+};
+
+template <typename R>
+__device__ __forceinline__ C2<R> fmm_offset(const FmmTree& t, int s, double2 c, float4 cf, double inv_h);
+template <>
+__device__ __forceinline__ C2<float> fmm_offset<float>(const FmmTree& t, int s, double2 c, float4 cf, double inv_h) {
+    return fmm_local(t.spos[s], cf, (float)inv_h);
+}
+template <>
+__device__ __forceinline__ C2<double> fmm_offset<double>(const FmmTree& t, int s, double2 c, float4 cf, double inv_h) {
+    const double2 p = t.spos64[s];
+    return {(p.x - c.x) * inv_h, (p.y - c.y) * inv_h};
+}
+template <>
+__device__ __forceinline__ C2<df> fmm_offset<df>(const FmmTree& t, int s, double2 c, float4 cf, double inv_h) {
+    const double2 p = t.spos64[s];
+    return {df((p.x - c.x) * inv_h), df((p.y - c.y) * inv_h)};
+}
+
+// One CTA per leaf: gathers the strengths q = sigma w of the box's sources in
+// sorted order and sums their moments.  A warp takes 32 sources at a time; a
+// lane sums three (order, group of sources) items, eta^k = eta^(k % 4)
+// (eta^4)^(k / 4) from two small tables per source.  The CTA of a parent's last
+// child forms the parent's moments, a warp per child, and so on up.
+template <typename R>
 __global__ void __launch_bounds__(128)
 k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ sigma, const double* __restrict__ w,
-         int shift, C2<R>* __restrict__ sq, float4* __restrict__ sqdf, V4<R>* __restrict__ mp, unsigned* __restrict__ ticket,
-         const R* __restrict__ binom) {
-    constexpr int ROWS = (P + 31) / 32, HI = (P + 3) / 4;
-    __shared__ __align__(16) C2<R> s_lo[4][4][33], s_hi[4][HI][33], s_q[4][32], s_s[4][32];
-    static_assert(P * sizeof(V4<R>) <= HI * 33 * sizeof(C2<R>), "translation buffer");
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int b = blockIdx.x * 4 + wid;
-    if (b >= t.nleaf) return;
+         int shift, C2<R>* __restrict__ sq, V4<R>* __restrict__ mp, unsigned* __restrict__ ticket, FmmTab<R> tab) {
+    constexpr int P = FmmTypes<R>::P, G = kFmmItems / P, PER = 32 / G, HI = P / 4;
+    struct Tables {
+        C2<R> lo[4][4][33], hi[4][HI][33], q[4][32], s[4][32];
+    };
+    __shared__ __align__(16) Tables sh;
+    __shared__ bool s_last;
+    auto& s_lo = sh.lo;
+    auto& s_hi = sh.hi;
+    auto& s_q = sh.q;
+    auto& s_s = sh.s;
+    // the tables' space holds the warps' sums (6 numbers per item), then the
+    // children's translated series
+    R* s_sum = reinterpret_cast<R*>(&sh);
+    static_assert(4 * kFmmItems * 6 * sizeof(R) <= sizeof(Tables), "sums");
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    const int b = blockIdx.x;
     int4 bx = t.box[b];
     const FmmCell& f = t.cells[bx.x];
     if (!cells[bx.x].active) return;
     const int s0 = t.sstart[b], s1 = t.sstart[b + 1];
     if (s1 > s0) {
-        const double2 c = fmm_centre(f, 0, fmm_ix(bx), fmm_iy(bx));
-        float4 cf;
-        split_df(c.x, cf.x, cf.y);
-        split_df(c.y, cf.z, cf.w);
-        // real moments of q_x and q_y (complex each) and of s = q conj(eta)
-        C2<R> X[ROWS], Y[ROWS], D[ROWS];
+        const double2 c = sizeof(R) == 4 ? make_double2(0.0, 0.0) : fmm_centre(f, 0, fmm_ix(bx), fmm_iy(bx));
+        const float4 cf = t.centre[b];
+        // per item the moments of q_x and q_y and of s = q conj(eta)
+        C2<R> X[3], Y[3], D[3];
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r) X[r] = Y[r] = D[r] = {R(0), R(0)};
-        for (int k0 = s0; k0 < s1; k0 += 32) {
+        for (int r = 0; r < 3; ++r) X[r] = Y[r] = D[r] = czero<R>();
+        for (int k0 = s0 + 32 * wid; k0 < s1; k0 += 128) {
             const int s = k0 + lane, cnt = min(32, s1 - k0);
-            C2<R> eta{R(0), R(0)}, q{R(0), R(0)};
+            C2<R> eta = czero<R>(), q = czero<R>();
             if (lane < cnt) {
-                if constexpr (sizeof(R) == 4) {
-                    eta = fmm_local(t.spos[s], cf, (float)f.inv_h);
-                } else {
-                    const double2 p = t.spos64[s];
-                    eta = {(p.x - c.x) * f.inv_h, (p.y - c.y) * f.inv_h};
-                }
+                eta = fmm_offset<R>(t, s, c, cf, f.inv_h);
                 const int i = t.sperm[s] >> shift;
                 const double2 sg = sigma[i];
                 const double wi = w[i];
-                q = {(R)(sg.x * wi), (R)(sg.y * wi)};
-                if (sqdf) {
-                    float4 v;
-                    split_df((double)q.x, v.x, v.y);
-                    split_df((double)q.y, v.z, v.w);
-                    sqdf[s] = v;
-                } else {
-                    sq[s] = q;
-                }
+                q = {R(sg.x * wi), R(sg.y * wi)};
+                sq[s] = q;
             }
             const C2<R> e2 = cmul(eta, eta), e4 = cmul(e2, e2);
             __syncwarp();
@@ -257,15 +338,15 @@ k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ 
                 h = cmul(h, e4);
             }
             s_q[wid][lane] = q;
-            s_s[wid][lane] = {q.x * eta.x + q.y * eta.y, q.y * eta.x - q.x * eta.y};
+            s_s[wid][lane] = {fma_(q.x, eta.x, q.y * eta.y), fma_(q.y, eta.x, -(q.x * eta.y))};
             __syncwarp();
-            for (int j = 0; j < cnt; ++j) {
-                const C2<R> qj = s_q[wid][j], sj = s_s[wid][j], lo = s_lo[wid][lane & 3][j];
+            for (int j = 0; j < PER; ++j) {
 #pragma unroll
-                for (int r = 0; r < ROWS; ++r) {
-                    const int a = (lane >> 2) + 8 * r;
-                    if (a < HI) {
-                        const C2<R> pw = cmul(lo, s_hi[wid][a][j]);
+                for (int r = 0; r < 3; ++r) {
+                    const int it = lane + 32 * r, k = it % P, js = (it / P) * PER + j;
+                    if (js < cnt) {
+                        const C2<R> qj = s_q[wid][js], sj = s_s[wid][js];
+                        const C2<R> pw = cmul(s_lo[wid][k & 3][js], s_hi[wid][k >> 2][js]);
                         X[r].x = fma_(qj.x, pw.x, X[r].x);
                         X[r].y = fma_(qj.x, pw.y, X[r].y);
                         Y[r].x = fma_(qj.y, pw.x, Y[r].x);
@@ -275,94 +356,93 @@ k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ 
                     }
                 }
             }
+            __syncwarp();
         }
-        // a = X + i Y, b = X - i Y, e_k = b_k - k d_{k-1}
-        C2<R> carry{R(0), R(0)};
+        __syncthreads();
+        // the sums of 4 warps x G groups, in order; number n of order k at n P + k
+        R* mine = s_sum + (size_t)wid * kFmmItems * 6;
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
-            const int k = lane + 32 * r;
-            C2<R> d{__shfl_up_sync(0xffffffffu, D[r].x, 1), __shfl_up_sync(0xffffffffu, D[r].y, 1)};
-            if (lane == 0) d = carry;
-            carry = {__shfl_sync(0xffffffffu, D[r].x, 31), __shfl_sync(0xffffffffu, D[r].y, 31)};
-            if (k < P)
-                mp[(size_t)b * P + k] = {X[r].x - Y[r].y, X[r].y + Y[r].x, X[r].x + Y[r].y - R(k) * d.x,
-                                         X[r].y - Y[r].x - R(k) * d.y};
+        for (int r = 0; r < 3; ++r) {
+            const int it = lane + 32 * r;
+            const R v[6] = {X[r].x, X[r].y, Y[r].x, Y[r].y, D[r].x, D[r].y};
+#pragma unroll
+            for (int n = 0; n < 6; ++n) mine[n * kFmmItems + it] = renorm(v[n]);
+        }
+        __syncthreads();
+        for (int e = tid; e < 6 * P; e += 128) {
+            const int n = e / P, k = e % P;
+            R v = s_sum[n * kFmmItems + k];
+            for (int g = 1; g < 4 * G; ++g)
+                v = v + s_sum[(size_t)(g / G) * kFmmItems * 6 + n * kFmmItems + (g % G) * P + k];
+            // only this thread reads (n, k) of warp 0's group 0 below this line's write
+            s_sum[n * kFmmItems + k] = v;
+        }
+        __syncthreads();
+        // a = X + i Y, b = X - i Y, e_k = b_k - k d_{k-1}
+        if (tid < P) {
+            const int k = tid;
+            const R xx = s_sum[k], xy = s_sum[kFmmItems + k], yx = s_sum[2 * kFmmItems + k],
+                    yy = s_sum[3 * kFmmItems + k];
+            R dx(0), dy(0);
+            if (k) {
+                dx = s_sum[4 * kFmmItems + k - 1];
+                dy = s_sum[5 * kFmmItems + k - 1];
+            }
+            mp[(size_t)b * P + k] = {xx - yy, xy + yx, (xx + yy) - R(k) * dx, (xy - yx) - R(k) * dy};
         }
     }
-    // parents (a warp's power table is free now: it holds the translated series)
-    V4<R>* s_v = reinterpret_cast<V4<R>*>(&s_hi[wid][0][0]);
+    // parents: the series translated from the four children, a warp each
+    V4<R>* s_v = reinterpret_cast<V4<R>*>(&sh);  // [4][P] scaled, then [4][P] translated
+    static_assert(8 * P * sizeof(V4<R>) <= sizeof(Tables), "series");
     for (int level = 0; bx.w >= 0; ++level) {
         const int parent = bx.w;
         const int px = fmm_ix(t.box[parent]), py = fmm_iy(t.box[parent]);
         const int nx = min(2, f.gx[level] - 2 * px), ny = min(2, f.gy[level] - 2 * py);
         __threadfence();
-        __syncwarp();
-        unsigned old = 0;
-        if (lane == 0) old = atomicAdd(ticket + parent, 1u);
-        old = __shfl_sync(0xffffffffu, old, 0);
-        if (old != (unsigned)(nx * ny) - 1) return;
+        __syncthreads();
+        if (tid == 0) s_last = atomicAdd(ticket + parent, 1u) == (unsigned)(nx * ny) - 1;
+        __syncthreads();
+        if (!s_last) return;
         __threadfence();
-        if (lane == 0) ticket[parent] = 0u;
-        V4<R> acc[ROWS];
-#pragma unroll
-        for (int r = 0; r < ROWS; ++r) acc[r] = {R(0), R(0), R(0), R(0)};
-        for (int q = 0; q < nx * ny; ++q) {
-            const int jx = q % nx, jy = q / nx;
-            const int child = f.off[level] + (2 * py + jy) * f.gx[level] + 2 * px + jx;
-            if (t.scount[child] == 0) continue;
-            const C2<R> dl{jx ? R(0.25) : R(-0.25), jy ? R(0.25) : R(-0.25)};
-            // child's unit is half the parent's: v_k = a_k (1/2)^k delta^-k = a_k (1 / (2 delta))^k
-            const C2<R> g = cinv(C2<R>{2 * dl.x, 2 * dl.y});
-            C2<R> carry{R(0), R(0)};
-            __syncwarp();
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                const int k = lane + 32 * r;
-                V4<R> m{R(0), R(0), R(0), R(0)};
-                if (k < P) {
-                    const R* src = reinterpret_cast<const R*>(mp + (size_t)child * P + k);
-                    m = {__ldcg(src), __ldcg(src + 1), __ldcg(src + 2), __ldcg(src + 3)};
+        if (tid == 0) ticket[parent] = 0u;
+        bx = t.box[parent];
+        if (t.scount[parent] == 0) continue;
+        const int jx = wid & 1, jy = wid >> 1;
+        const int child = f.off[level] + (2 * py + jy) * f.gx[level] + 2 * px + jx;
+        const bool have = jx < nx && jy < ny && t.scount[child] > 0;
+        V4<R>* v = s_v + wid * P;
+        V4<R>* o = s_v + (4 + wid) * P;
+        if (have) {
+            // child's unit is half the parent's: v_k = a_k (1 / (2 delta))^k; with
+            // delta = (+-1/2, +-1/2) in the child's unit, e_k - conj(delta) k a_{k-1}
+            const R hx(jx ? 0.5 : -0.5), hy(jy ? 0.5 : -0.5);
+            for (int k = lane; k < P; k += 32) {
+                const R* src = reinterpret_cast<const R*>(mp + (size_t)child * P + k);
+                const C2<R> a{ldcg(src), ldcg(src + 1)};
+                C2<R> e{ldcg(src + 2), ldcg(src + 3)};
+                if (k) {
+                    const R pax = ldcg(src - 4), pay = ldcg(src - 3);
+                    e.x = e.x - R(k) * fma_(hx, pax, hy * pay);
+                    e.y = e.y - R(k) * fma_(hx, pay, -(hy * pax));
                 }
-                C2<R> pa{__shfl_up_sync(0xffffffffu, m.x, 1), __shfl_up_sync(0xffffffffu, m.y, 1)};
-                if (lane == 0) pa = carry;
-                carry = {__shfl_sync(0xffffffffu, m.x, 31), __shfl_sync(0xffffffffu, m.y, 31)};
-                // e_k - conj(delta) k a_{k-1}, delta in the child's unit: 2 dl
-                m.z -= R(2 * k) * (dl.x * pa.x + dl.y * pa.y);
-                m.w -= R(2 * k) * (dl.x * pa.y - dl.y * pa.x);
-                const C2<R> pg = cpow(g, k);
-                if (k < P) {
-                    const C2<R> va = cmul(pg, C2<R>{m.x, m.y}), ve = cmul(pg, C2<R>{m.z, m.w});
-                    s_v[k] = {va.x, va.y, ve.x, ve.y};
-                }
+                v[k] = scaled(tab.gpow[wid * P + k], a, e);
             }
             __syncwarp();
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                const int m = lane + 32 * r;
-                if (m < P) {
-                    V4<R> s{R(0), R(0), R(0), R(0)};
-                    for (int k = 0; k <= m; ++k) {
-                        const R cb = binom[(size_t)k * P + m];  // C(m, k)
-                        const V4<R> v = s_v[k];
-                        s.x = fma_(cb, v.x, s.x);
-                        s.y = fma_(cb, v.y, s.y);
-                        s.z = fma_(cb, v.z, s.z);
-                        s.w = fma_(cb, v.w, s.w);
-                    }
-                    const C2<R> pd = cpow(dl, m);
-                    const C2<R> ra = cmul(pd, C2<R>{s.x, s.y}), re = cmul(pd, C2<R>{s.z, s.w});
-                    acc[r].x += ra.x;
-                    acc[r].y += ra.y;
-                    acc[r].z += re.x;
-                    acc[r].w += re.y;
-                }
+            for (int m = lane; m < P; m += 32) {
+                V4<R> s = vzero<R>();
+                for (int k = 0; k <= m; ++k) axpy(s, tab.binom[(size_t)k * P + m], v[k]);  // C(m, k)
+                V4<R> r = vzero<R>();
+                add_scaled(r, tab.dpow[wid * P + m], s);
+                o[m] = r;
             }
         }
-        if (t.scount[parent] > 0)
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r)
-                if (lane + 32 * r < P) mp[(size_t)parent * P + lane + 32 * r] = acc[r];
-        bx = t.box[parent];
+        if (!have)
+            for (int m = lane; m < P; m += 32) o[m] = vzero<R>();
+        __syncthreads();
+        if (tid < P) {
+            const V4<R>* q = s_v + 4 * P + tid;
+            mp[(size_t)parent * P + tid] = vadd(vadd(q[0], q[P]), vadd(q[2 * P], q[3 * P]));
+        }
     }
 }
 
@@ -370,25 +450,44 @@ k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ 
 // across: local expansion of every target box from the far boxes whose
 // parents are near
 // ---------------------------------------------------------------------------
-// Boxes ix and jx (under a shift of s sides) near in one coordinate: centres
-// closer than two sides.  One expression everywhere, so that a level's far
-// list, its children's and the pair sum's rows partition the pairs exactly.
-__device__ __forceinline__ bool fmm_close(int ix, int jx, double s) { return fabs((double)(ix - jx) - s) < 2.0 - 1e-9; }
+// Which boxes are near is decided in whole numbers: an image shift is rounded
+// to 2^-16 of a leaf side (kFmmBits), and boxes ix and jx of a level (unit
+// 2^(kFmmBits + level)) are near in one coordinate when their centres under the
+// shift are less than two units apart.  The same numbers at every level make a
+// level's far list, its children's and the pair sum's rows partition the pairs
+// exactly; the FP64 pipe, which took 6000 cycles per box to list its far boxes,
+// is left to the sums.
+constexpr int kFmmBits = 16;
+__device__ __forceinline__ bool fmm_close(int ix, int jx, int s, int level) {
+    return abs(((ix - jx) << (kFmmBits + level)) - s) < (2 << (kFmmBits + level));
+}
+// the first of the (at most four) boxes near ix
+__device__ __forceinline__ int fmm_first(int ix, int s, int level) { return ix - 1 + ((-s) >> (kFmmBits + level)); }
+__device__ __forceinline__ int fmm_shift(double s, double inv_h) { return __double2int_rn(s * inv_h * (1 << kFmmBits)); }
 constexpr int kFmmList = 512;            // far boxes listed at a time
+constexpr int kFmmShares = 4;            // most CTAs a box's list is split over
 
-// One CTA per target box (all levels).  Its threads scan the candidate (box,
-// image) pairs, compact the far ones into shared memory in a fixed order, and
-// the warps translate them in turn (lane l: orders l and l + 32).
-template <typename R, int P>
+// One CTA per (target box of any level, share of its list).  Its threads scan
+// the candidate (box, image) pairs and compact the far ones into shared memory
+// in a fixed order; the warps translate them in turn.  Single precision: an
+// entry per warp and step, lane l holding order l and its row of the matrix.
+// Double: two entries per warp and step, three (entry, order) items per lane.
+// The shares' sums are separate (slot blockIdx.y of loc): without shares the
+// longest lists (90 boxes, at the coarse levels) held up the launch.
+template <typename R>
 __global__ void __launch_bounds__(128)
 k_fmm_m2l(FmmTree t, const Cell* __restrict__ cells, int nimg, const V4<R>* __restrict__ mp, V4<R>* __restrict__ loc,
-          const R* __restrict__ hankel) {
-    constexpr int ROWS = (P + 31) / 32;
-    __shared__ int s_src[kFmmList];
-    __shared__ C2<R> s_z[kFmmList];
-    __shared__ V4<R> s_v[4][P];
+          FmmTab<R> tab) {
+    constexpr int P = FmmTypes<R>::P;
+    constexpr bool F32 = sizeof(R) == 4;
+    constexpr int ENT = F32 ? 1 : 2, ITEMS = F32 ? 1 : 3;
+    __shared__ int2 s_far[kFmmList];  // box; offsets from it + 2^12 (13 bits each) and the image
+    __shared__ int2 s_shift[9];
+    __shared__ C2<R> s_tab[4][F32 ? 32 : 16][kPowTab], s_z[4][F32 ? 32 : 16];
+    __shared__ V4<R> s_v[4][ENT][P + (F32 ? 0 : 1)];
     __shared__ int s_n[4];
     const int b = blockIdx.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int share = blockIdx.y, shares = gridDim.y;
     if (t.tcount[b] == 0) return;
     const int4 bx = t.box[b];
     const FmmCell& f = t.cells[bx.x];
@@ -396,27 +495,28 @@ k_fmm_m2l(FmmTree t, const Cell* __restrict__ cells, int nimg, const V4<R>* __re
     if (!cl.active) return;
     const int level = bx.y, ix = fmm_ix(bx), iy = fmm_iy(bx);
     const bool top = level == f.nlev - 1;
-    const int gx = f.gx[level], gy = f.gy[level];
-    const double H = f.h * (1 << level), inv = 1.0 / H;
+    const int gx = f.gx[level], gy = f.gy[level], off = f.off[level];
     const int per = top ? gx * gy : 64;
-    V4<R> acc[ROWS];
+    if (threadIdx.x < 9)
+        s_shift[threadIdx.x] = make_int2(fmm_shift(cl.sx[threadIdx.x], f.inv_h), fmm_shift(cl.sy[threadIdx.x], f.inv_h));
+    __syncthreads();
+    V4<R> acc[ITEMS];
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) acc[r] = {R(0), R(0), R(0), R(0)};
-    R row[sizeof(R) == 4 ? P : 1];  // single precision: lane l's row of the matrix in registers
-    if constexpr (sizeof(R) == 4) {
+    for (int r = 0; r < ITEMS; ++r) acc[r] = vzero<R>();
+    R row[F32 ? P : 1];  // single precision: lane l's row of the matrix in registers
+    if constexpr (F32) {
 #pragma unroll
-        for (int k = 0; k < P; ++k) row[k] = lane < P ? hankel[(size_t)k * P + lane] : R(0);
+        for (int k = 0; k < P; ++k) row[k] = lane < P ? tab.hankel[(size_t)k * P + lane] : R(0);
     }
-    int listed = 0;
+    int listed = 0;  // far boxes of all shares since the last translation
     const int ncand = per * nimg;
     for (int q0 = 0; q0 < ncand; q0 += 128) {
         const int q = q0 + threadIdx.x;
         bool far = false;
-        int src = 0;
-        double zx = 0, zy = 0;
+        int2 entry2 = make_int2(0, 0);
         if (q < ncand) {
             const int im = nimg == 1 ? 4 : q / per, e = nimg == 1 ? q : q % per;
-            const double sx = cl.sx[im] * inv, sy = cl.sy[im] * inv;  // sides of this level
+            const int2 sh = s_shift[im];
             int jx, jy;
             bool ok = true;
             if (top) {
@@ -425,17 +525,16 @@ k_fmm_m2l(FmmTree t, const Cell* __restrict__ cells, int nimg, const V4<R>* __re
             } else {
                 // children of the (up to 4 x 4) near parents
                 const int kx = ix >> 1, ky = iy >> 1;
-                const int px = (int)floor(kx - 0.5 * sx - 2.0) + 1 + (e & 7) / 2;
-                const int py = (int)floor(ky - 0.5 * sy - 2.0) + 1 + (e >> 3) / 2;
-                ok = fmm_close(kx, px, 0.5 * sx) && fmm_close(ky, py, 0.5 * sy);
+                const int px = fmm_first(kx, sh.x, level + 1) + (e & 7) / 2;
+                const int py = fmm_first(ky, sh.y, level + 1) + (e >> 3) / 2;
+                ok = fmm_close(kx, px, sh.x, level + 1) && fmm_close(ky, py, sh.y, level + 1);
                 jx = 2 * px + (e & 1);
                 jy = 2 * py + ((e >> 3) & 1);
             }
             if (ok && jx >= 0 && jx < gx && jy >= 0 && jy < gy) {
-                zx = (ix - jx) - sx;
-                zy = (iy - jy) - sy;
-                src = f.off[level] + jy * gx + jx;
-                far = !(fmm_close(ix, jx, sx) && fmm_close(iy, jy, sy)) && t.scount[src] > 0;
+                const int src = off + jy * gx + jx;
+                far = !(fmm_close(ix, jx, sh.x, level) && fmm_close(iy, jy, sh.y, level)) && t.scount[src] > 0;
+                entry2 = make_int2(src, (ix - jx + 4096) | ((iy - jy + 4096) << 13) | (im << 26));
             }
         }
         const unsigned m = __ballot_sync(0xffffffffu, far);
@@ -446,108 +545,126 @@ k_fmm_m2l(FmmTree t, const Cell* __restrict__ cells, int nimg, const V4<R>* __re
             if (k < wid) at += s_n[k];
             all += s_n[k];
         }
-        if (far) {
-            at += __popc(m & ((1u << lane) - 1));
-            s_src[at] = src;
-            s_z[at] = {(R)zx, (R)zy};
+        at += __popc(m & ((1u << lane) - 1));
+        if (far && at % shares == share) {
+            s_far[at / shares] = entry2;
         }
         __syncthreads();
         listed = all;
         if (listed <= kFmmList - 128 && q0 + 128 < ncand) continue;
-        V4<R> nxt[ROWS];
-        auto fetch = [&](int e) {
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                const int k = lane + 32 * r;
-                nxt[r] = {R(0), R(0), R(0), R(0)};
-                if (e < listed && k < P) nxt[r] = mp[(size_t)s_src[e] * P + k];
-            }
-        };
-        fetch(wid);
-        for (int e = wid; e < listed; e += 4) {
-            const C2<R> z = s_z[e], u = cinv(z);
-            C2<R> pw[ROWS], carry{R(0), R(0)};
-            V4<R> m4[ROWS];
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) m4[r] = nxt[r];
-            fetch(e + 4);
-            pw[0] = cpow(u, lane);
-            if constexpr (ROWS > 1) {
-                C2<R> u32 = u;
-#pragma unroll
-                for (int k = 0; k < 5; ++k) u32 = cmul(u32, u32);
-                pw[1] = cmul(pw[0], u32);
-            }
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                const int k = lane + 32 * r;
-                C2<R> pa{__shfl_up_sync(0xffffffffu, m4[r].x, 1), __shfl_up_sync(0xffffffffu, m4[r].y, 1)};
-                if (lane == 0) pa = carry;
-                carry = {__shfl_sync(0xffffffffu, m4[r].x, 31), __shfl_sync(0xffffffffu, m4[r].y, 31)};
-                // e_k + conj(z0) k a_{k-1}
-                const C2<R> ev{m4[r].z + R(k) * (z.x * pa.x + z.y * pa.y), m4[r].w + R(k) * (z.x * pa.y - z.y * pa.x)};
-                const C2<R> pu = cmul(pw[r], u);
-                const C2<R> va = cmul(pu, C2<R>{m4[r].x, m4[r].y}), ve = cmul(pu, ev);
-                if (k < P) s_v[wid][k] = {va.x, va.y, ve.x, ve.y};
+        const int mine = (listed - share + shares - 1) / shares;  // this share's entries
+        constexpr int GRP = F32 ? 32 : 16;  // entries whose power tables a warp holds
+        for (int g0 = 0; g0 * 4 < mine; g0 += GRP) {
+            // the warp's entries of this group: e = (g0 + n) 4 + wid (single), or
+            // consecutive pairs (double)
+            const int stepn = ENT == 1 ? 1 : 2;
+            auto entry = [&](int n) { return ENT == 1 ? (g0 + n) * 4 + wid : ((g0 + n) / 2 * 4 + wid) * 2 + (n & 1); };
+            __syncwarp();
+            if (lane < GRP && entry(lane) < mine) {
+                // target centre minus source centre in sides, its inverse's powers
+                const int at2 = s_far[entry(lane)].y;
+                const double inv = f.inv_h / (1 << level);
+                const double x = (double)((at2 & 8191) - 4096) - cl.sx[at2 >> 26] * inv;
+                const double y = (double)(((at2 >> 13) & 8191) - 4096) - cl.sy[at2 >> 26] * inv;
+                s_z[wid][lane] = {R(x), R(y)};
+                C2<R> u;
+                if constexpr (F32) {
+                    const float fx = (float)x, fy = (float)y, sc = 1.f / (fx * fx + fy * fy);
+                    u = {fx * sc, -fy * sc};
+                } else {
+                    const double sc = rcp64(x * x + y * y);
+                    u = {R(x * sc), R(-y * sc)};
+                }
+                pow_table(u, s_tab[wid][lane]);
             }
             __syncwarp();
-            V4<R> s[ROWS];
+            if constexpr (F32) {
+                V4<R> nxt = vzero<R>();
+                const int e0 = entry(0);
+                if (e0 < mine && lane < P) nxt = mp[(size_t)s_far[e0].x * P + lane];
+                for (int n = 0; n < GRP && entry(n) < mine; ++n) {
+                    const C2<R> z = s_z[wid][n];
+                    const V4<R> m4 = nxt;
+                    const int en = entry(n + 1);
+                    if (n + 1 < GRP && en < mine && lane < P) nxt = mp[(size_t)s_far[en].x * P + lane];
+                    const C2<R> u = s_tab[wid][n][0];
+                    C2<R> pw = pow_at(s_tab[wid][n], lane);
+                    C2<R> pa{__shfl_up_sync(0xffffffffu, m4.x, 1), __shfl_up_sync(0xffffffffu, m4.y, 1)};
+                    if (lane == 0) pa = czero<R>();
+                    // e_k + conj(z0) k a_{k-1}
+                    const C2<R> ev{m4.z + R(lane) * (z.x * pa.x + z.y * pa.y),
+                                   m4.w + R(lane) * (z.x * pa.y - z.y * pa.x)};
+                    if (lane < P) s_v[wid][0][lane] = scaled(pw, C2<R>{m4.x, m4.y}, ev);
+                    __syncwarp();
+                    V4<R> s = vzero<R>();
 #pragma unroll
-            for (int r = 0; r < ROWS; ++r) s[r] = {R(0), R(0), R(0), R(0)};
-            if constexpr (sizeof(R) == 4) {
-#pragma unroll
-                for (int k = 0; k < P; ++k) {
-                    const V4<R> v = s_v[wid][k];
-                    s[0].x = fma_(row[k], v.x, s[0].x);
-                    s[0].y = fma_(row[k], v.y, s[0].y);
-                    s[0].z = fma_(row[k], v.z, s[0].z);
-                    s[0].w = fma_(row[k], v.w, s[0].w);
+                    for (int k = 0; k < P; ++k) axpy(s, row[k], s_v[wid][0][k]);
+                    __syncwarp();
+                    pw = cmul(pw, u);
+                    if (lane & 1) pw = {-pw.x, -pw.y};
+                    add_scaled(acc[0], pw, s);
                 }
             } else {
-#pragma unroll 4
-                for (int k = 0; k < P; ++k) {
-                    const V4<R> v = s_v[wid][k];
+                for (int n = 0; n < GRP && entry(n) < mine; n += stepn) {
+                    C2<R> pw[ITEMS];
 #pragma unroll
-                    for (int r = 0; r < ROWS; ++r) {
-                        const int l = lane + 32 * r;
-                        const R c = l < P ? __ldg(hankel + (size_t)k * P + l) : R(0);
-                        s[r].x = fma_(c, v.x, s[r].x);
-                        s[r].y = fma_(c, v.y, s[r].y);
-                        s[r].z = fma_(c, v.z, s[r].z);
-                        s[r].w = fma_(c, v.w, s[r].w);
+                    for (int r = 0; r < ITEMS; ++r) {
+                        const int it = lane + 32 * r, en = it / P, k = it % P, e = entry(n + en);
+                        V4<R> v = vzero<R>();
+                        pw[r] = czero<R>();
+                        if (e < mine) {
+                            const V4<R>* src4 = mp + (size_t)s_far[e].x * P + k;
+                            const V4<R> m4 = *src4;
+                            C2<R> ev{m4.z, m4.w};
+                            if (k) {
+                                const C2<R> z = s_z[wid][n + en];
+                                const R pax = src4[-1].x, pay = src4[-1].y;
+                                ev.x = ev.x + R(k) * fma_(z.x, pax, z.y * pay);
+                                ev.y = ev.y + R(k) * fma_(z.x, pay, -(z.y * pax));
+                            }
+                            pw[r] = pow_at(s_tab[wid][n + en], k);
+                            v = scaled(pw[r], C2<R>{m4.x, m4.y}, ev);
+                            pw[r] = cmul(pw[r], s_tab[wid][n + en][0]);
+                            if (k & 1) pw[r] = {-pw[r].x, -pw[r].y};
+                        }
+                        s_v[wid][en][k] = v;
                     }
-                }
-            }
-            __syncwarp();
-            const R sg = (lane & 1) ? R(-1) : R(1);  // (-1)^l, l = lane or lane + 32
+                    __syncwarp();
+                    V4<R> s[ITEMS];
 #pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                const C2<R> pl{sg * pw[r].x, sg * pw[r].y};
-                const C2<R> ra = cmul(pl, C2<R>{s[r].x, s[r].y}), re = cmul(pl, C2<R>{s[r].z, s[r].w});
-                acc[r].x += ra.x;
-                acc[r].y += ra.y;
-                acc[r].z += re.x;
-                acc[r].w += re.y;
+                    for (int r = 0; r < ITEMS; ++r) s[r] = vzero<R>();
+#pragma unroll 2
+                    for (int k = 0; k < P; ++k) {
+#pragma unroll
+                        for (int r = 0; r < ITEMS; ++r) {
+                            const int it = lane + 32 * r;
+                            axpy(s[r], tab.hankel[(size_t)k * P + it % P], s_v[wid][it / P][k]);
+                        }
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int r = 0; r < ITEMS; ++r) add_scaled(acc[r], pw[r], s[r]);
+                }
             }
         }
         listed = 0;
         __syncthreads();
     }
-    // the warps' sums, in warp order
+    // the warps' sums, in order
+    V4<R>* flat = &s_v[wid][0][0];
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r)
-        if (lane + 32 * r < P) s_v[wid][lane + 32 * r] = acc[r];
+    for (int r = 0; r < ITEMS; ++r) {
+        const int it = lane + 32 * r;
+        if (it < ENT * P) flat[it] = V4<R>{renorm(acc[r].x), renorm(acc[r].y), renorm(acc[r].z), renorm(acc[r].w)};
+    }
     __syncthreads();
     for (int k = threadIdx.x; k < P; k += 128) {
-        V4<R> s = s_v[0][k];
+        V4<R> s = vzero<R>();
 #pragma unroll
-        for (int q = 1; q < 4; ++q) {
-            s.x += s_v[q][k].x;
-            s.y += s_v[q][k].y;
-            s.z += s_v[q][k].z;
-            s.w += s_v[q][k].w;
-        }
-        loc[(size_t)b * P + k] = s;
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int en = 0; en < ENT; ++en) s = vadd(s, (&s_v[q][0][0])[en * P + k]);
+        loc[((size_t)share * t.nbox + b) * P + k] = s;
     }
 }
 
@@ -563,105 +680,114 @@ struct FmmRange {
 constexpr int kFmmRanges = 36;  // 9 images x 4 rows
 
 // The local expansion of a leaf with its ancestors' moved to its centre, in
-// s_l[0]: warp w moves levels w, w + 4, ... (level 0 is the leaf's own); every
-// thread of the 128 takes part.
-template <typename R, int P>
+// s_l[0] (the shares of k_fmm_m2l added on the way): warp w moves levels w,
+// w + 4, ... (level 0 is the leaf's own); every thread of the 128 takes part.
+template <typename R>
 __device__ __forceinline__ void fmm_local_to_leaf(const FmmTree& t, const FmmCell& f, int4 bx, const V4<R>* loc,
-                                                  const R* binom, V4<R> (*s_l)[P], int wid, int lane) {
+                                                  int shares, const FmmTab<R>& tab, V4<R> (*s_l)[FmmTypes<R>::P],
+                                                  C2<R> (*s_pw)[2][kPowTab], int wid, int lane) {
+    constexpr int P = FmmTypes<R>::P, ROWS = (P + 31) / 32;
     V4<R>* s_v = s_l[wid];
-    constexpr int ROWS = (P + 31) / 32;
     V4<R> acc[ROWS];
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) acc[r] = {R(0), R(0), R(0), R(0)};
+    for (int r = 0; r < ROWS; ++r) acc[r] = vzero<R>();
     for (int level = wid; level < f.nlev; level += 4) {
         const int jx = fmm_ix(bx) >> level, jy = fmm_iy(bx) >> level;
-        const int b = f.off[level] + jy * f.gx[level] + jx;
-        const V4<R>* src = loc + (size_t)b * P;
+        const V4<R>* src = loc + (size_t)(f.off[level] + jy * f.gx[level] + jx) * P;
+        auto get = [&](int l) {
+            V4<R> m = src[l];
+            for (int q = 1; q < shares; ++q) m = vadd(m, src[(size_t)q * t.nbox * P + l]);
+            return m;
+        };
         if (level == 0) {
 #pragma unroll
             for (int r = 0; r < ROWS; ++r)
-                if (lane + 32 * r < P) acc[r] = src[lane + 32 * r];
+                if (lane + 32 * r < P) acc[r] = get(lane + 32 * r);
             continue;
         }
-        // leaf centre minus ancestor centre, in the ancestor's unit
-        const R u = R(1) / R(1 << level);
-        const C2<R> d{(R(fmm_ix(bx)) + R(0.5)) * u - (R(jx) + R(0.5)), (R(fmm_iy(bx)) + R(0.5)) * u - (R(jy) + R(0.5))};
+        // leaf centre minus ancestor centre, in the ancestor's unit (exact)
+        const float u = 1.f / (1 << level);
+        const float dx = (fmm_ix(bx) + 0.5f) * u - (jx + 0.5f), dy = (fmm_iy(bx) + 0.5f) * u - (jy + 0.5f);
+        const C2<R>*pd = s_pw[wid][0], *pg = s_pw[wid][1];  // powers of delta and of 2^-level / delta
         __syncwarp();
-        C2<R> next_a{R(0), R(0)};
+        if (lane < 2) {
+            const R i2 = lane ? R(double(u) / ((double)dx * dx + (double)dy * dy)) : R(1);
+            pow_table(C2<R>{R(dx) * i2, R(lane ? -dy : dy) * i2}, s_pw[wid][lane]);
+        }
+        __syncwarp();
 #pragma unroll
-        for (int r = ROWS - 1; r >= 0; --r) {
+        for (int r = 0; r < ROWS; ++r) {
             const int l = lane + 32 * r;
-            V4<R> m{R(0), R(0), R(0), R(0)};
-            if (l < P) m = src[l];
-            C2<R> na{__shfl_down_sync(0xffffffffu, m.x, 1), __shfl_down_sync(0xffffffffu, m.y, 1)};
-            if (lane == 31) na = next_a;
-            next_a = {__shfl_sync(0xffffffffu, m.x, 0), __shfl_sync(0xffffffffu, m.y, 0)};
-            // e_l - conj(d) (l + 1) a_{l+1}
-            m.z -= R(l + 1) * (d.x * na.x + d.y * na.y);
-            m.w -= R(l + 1) * (d.x * na.y - d.y * na.x);
-            const C2<R> pd = cpow(d, l);
             if (l < P) {
-                const C2<R> va = cmul(pd, C2<R>{m.x, m.y}), ve = cmul(pd, C2<R>{m.z, m.w});
-                s_v[l] = {va.x, va.y, ve.x, ve.y};
+                const V4<R> m = get(l);
+                C2<R> e{m.z, m.w};
+                if (l + 1 < P) {  // e_l - conj(d) (l + 1) a_{l+1}
+                    const V4<R> n = get(l + 1);
+                    e.x = e.x - R(l + 1) * fma_(R(dx), n.x, R(dy) * n.y);
+                    e.y = e.y - R(l + 1) * fma_(R(dx), n.y, -(R(dy) * n.x));
+                }
+                s_v[l] = scaled(pow_at(pd, l), C2<R>{m.x, m.y}, e);
             }
         }
         __syncwarp();
-        const C2<R> g = cinv(d);
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
             const int m = lane + 32 * r;
-            V4<R> s{R(0), R(0), R(0), R(0)};
-            if (m < P)
-                for (int l = m; l < P; ++l) {
-                    const R cb = binom[(size_t)m * P + l];  // C(l, m)
-                    const V4<R> v = s_v[l];
-                    s.x = fma_(cb, v.x, s.x);
-                    s.y = fma_(cb, v.y, s.y);
-                    s.z = fma_(cb, v.z, s.z);
-                    s.w = fma_(cb, v.w, s.w);
-                }
-            // to the leaf's unit: 2^-level per order and one more for the field's own scale
-            C2<R> pg = cpow(C2<R>{g.x * u, g.y * u}, m);
-            pg = {pg.x * u, pg.y * u};
-            const C2<R> ra = cmul(pg, C2<R>{s.x, s.y}), re = cmul(pg, C2<R>{s.z, s.w});
-            acc[r].x += ra.x;
-            acc[r].y += ra.y;
-            acc[r].z += re.x;
-            acc[r].w += re.y;
+            if (m < P) {
+                V4<R> s = vzero<R>();
+                for (int l = m; l < P; ++l) axpy(s, tab.binom[(size_t)m * P + l], s_v[l]);  // C(l, m)
+                // to the leaf's unit: 2^-level per order and one more for the field's own scale
+                C2<R> p = pow_at(pg, m);
+                p = {p.x * R(u), p.y * R(u)};
+                add_scaled(acc[r], p, s);
+            }
         }
+        __syncwarp();
     }
     __syncwarp();
 #pragma unroll
     for (int r = 0; r < ROWS; ++r)
-        if (lane + 32 * r < P) s_v[lane + 32 * r] = acc[r];
+        if (lane + 32 * r < P)
+            s_v[lane + 32 * r] = V4<R>{renorm(acc[r].x), renorm(acc[r].y), renorm(acc[r].z), renorm(acc[r].w)};
     __syncthreads();
-    for (int k = threadIdx.x; k < P; k += 128) {
-        V4<R> s = s_l[0][k];
-#pragma unroll
-        for (int q = 1; q < 4; ++q) {
-            s.x += s_l[q][k].x;
-            s.y += s_l[q][k].y;
-            s.z += s_l[q][k].z;
-            s.w += s_l[q][k].w;
-        }
-        s_l[0][k] = s;
-    }
+    for (int k = threadIdx.x; k < P; k += 128) s_l[0][k] = vadd(vadd(s_l[0][k], s_l[1][k]), vadd(s_l[2][k], s_l[3][k]));
     __syncthreads();
 }
 
-// Traction of the local expansion at W (leaf units) with normal n, times 4 pi h
-template <typename R, int P>
-__device__ __forceinline__ C2<R> fmm_local_at(const V4<R>* c, C2<R> W, R nx, R ny) {
-    C2<R> A{R(0), R(0)}, dA{R(0), R(0)}, E{R(0), R(0)};
-    for (int l = P - 1; l >= 0; --l) {
+// Traction, times 4 pi h, of the local expansion's orders r, r + STEP, ... at W
+// (leaf units) with normal n; the STEP residues add up to the whole.
+template <typename R, int STEP>
+__device__ __forceinline__ C2<R> fmm_local_at(const V4<R>* c, C2<R> W, int r, R nx, R ny) {
+    constexpr int P = FmmTypes<R>::P;
+    static_assert(P % STEP == 0, "residues");
+    C2<R> S = W;  // W^STEP
+#pragma unroll
+    for (int k = 1; k < STEP; k <<= 1) S = cmul(S, S);
+    // sums over l = r + STEP j of a_l, l a_l and e_l: A and E times W^r, and A'
+    // times W^(r - 1) (r = 0: its j = 0 term is nil, the rest times W^(STEP - 1))
+    C2<R> A = czero<R>(), B = czero<R>(), E = czero<R>();
+    auto step = [&](C2<R>& a, R vx, R vy) {
+        a = {renorm(fma_(a.x, S.x, fma_(-a.y, S.y, vx))), renorm(fma_(a.x, S.y, fma_(a.y, S.x, vy)))};
+    };
+#pragma unroll 2
+    for (int l = P - STEP + r; l >= 0; l -= STEP) {
         const V4<R> v = c[l];
-        dA = {fma_(dA.x, W.x, fma_(-dA.y, W.y, A.x)), fma_(dA.x, W.y, fma_(dA.y, W.x, A.y))};
-        A = {fma_(A.x, W.x, fma_(-A.y, W.y, v.x)), fma_(A.x, W.y, fma_(A.y, W.x, v.y))};
-        E = {fma_(E.x, W.x, fma_(-E.y, W.y, v.z)), fma_(E.x, W.y, fma_(E.y, W.x, v.w))};
+        const R fl(l);
+        step(A, v.x, v.y);
+        if (l) step(B, fl * v.x, fl * v.y);
+        step(E, v.z, v.w);
+    }
+    if constexpr (STEP > 1) {
+        C2<R> p{R(1), R(0)}, pb{R(1), R(0)};
+        for (int k = 0; k < r; ++k) p = cmul(p, W);
+        for (int k = 1; k < (r ? r : STEP); ++k) pb = cmul(pb, W);
+        A = cmul(A, p);
+        E = cmul(E, p);
+        B = cmul(B, pb);
     }
     // F = E - conj(W) A';  -(2 n Re A + conj(n F))
-    const C2<R> F{E.x - (W.x * dA.x + W.y * dA.y), E.y - (W.x * dA.y - W.y * dA.x)};
-    return {-(2 * nx * A.x + nx * F.x - ny * F.y), -(2 * ny * A.x - (nx * F.y + ny * F.x))};
+    const C2<R> F{E.x - fma_(W.x, B.x, W.y * B.y), E.y - fma_(W.x, B.y, -(W.y * B.x))};
+    return {-(R(2) * nx * A.x + nx * F.x - ny * F.y), -(R(2) * ny * A.x - (nx * F.y + ny * F.x))};
 }
 
 // Near rows of a leaf's targets, compacted in (image, row) order by warp 0.
@@ -673,13 +799,13 @@ __device__ __forceinline__ int fmm_ranges(const FmmTree& t, const FmmCell& f, co
         FmmRange r{0, 0, 0};
         if (q < 4 * nimg) {
             r.im = nimg == 1 ? 4 : q >> 2;
-            const double sx = cl.sx[r.im] * f.inv_h, sy = cl.sy[r.im] * f.inv_h;
+            const int sx = fmm_shift(cl.sx[r.im], f.inv_h), sy = fmm_shift(cl.sy[r.im], f.inv_h);
             const int ix = fmm_ix(bx), iy = fmm_iy(bx);
-            const int jy = (int)floor(iy - sy - 2.0) + 1 + (q & 3);
-            if (fmm_close(iy, jy, sy) && jy >= 0 && jy < f.gy[0]) {
-                int x0 = (int)floor(ix - sx - 2.0) + 1, x1 = x0 + 3;
-                if (!fmm_close(ix, x0, sx)) ++x0;
-                if (!fmm_close(ix, x1, sx)) --x1;
+            const int jy = fmm_first(iy, sy, 0) + (q & 3);
+            if (fmm_close(iy, jy, sy, 0) && jy >= 0 && jy < f.gy[0]) {
+                int x0 = fmm_first(ix, sx, 0), x1 = x0 + 3;
+                if (!fmm_close(ix, x0, sx, 0)) ++x0;
+                if (!fmm_close(ix, x1, sx, 0)) --x1;
                 x0 = max(x0, 0);
                 x1 = min(x1, f.gx[0] - 1);
                 if (x0 <= x1) {
@@ -702,10 +828,11 @@ __device__ __forceinline__ int fmm_ranges(const FmmTree& t, const FmmCell& f, co
 // later pass has to redo near pairs.
 __global__ void __launch_bounds__(128, 6)
 k_fmm_down32(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<float>* __restrict__ sq,
-             const V4<float>* __restrict__ loc, const float* __restrict__ binom, const float4* __restrict__ tgt32,
+             const V4<float>* __restrict__ loc, int shares, FmmTab<float> tab, const float4* __restrict__ tgt32,
              int n0, int n1, float2* __restrict__ part) {
     constexpr int P = kFmmP32;
     __shared__ V4<float> s_l[4][P];
+    __shared__ C2<float> s_pw[4][2][kPowTab];
     __shared__ FmmRange s_r[kFmmRanges];
     __shared__ int s_nr;
     __shared__ float4 s_p[4][32];
@@ -722,12 +849,9 @@ k_fmm_down32(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<float
         const int n = fmm_ranges(t, f, cl, bx, nimg, s_r, lane);
         if (lane == 0) s_nr = n;
     }
-    fmm_local_to_leaf<float, P>(t, f, bx, loc, binom, s_l, wid, lane);
+    fmm_local_to_leaf<float>(t, f, bx, loc, shares, tab, s_l, s_pw, wid, lane);
     const int nr = s_nr;
-    const double2 c = fmm_centre(f, 0, fmm_ix(bx), fmm_iy(bx));
-    float4 cf;
-    split_df(c.x, cf.x, cf.y);
-    split_df(c.y, cf.z, cf.w);
+    const float4 cf = t.centre[b];
     const float inv_h = (float)f.inv_h;
     for (int k0 = t0 + 64 * blockIdx.y; k0 < t1; k0 += 64 * gridDim.y) {
         const bool two = t1 - k0 > 32;  // uniform: the second target of every lane
@@ -805,7 +929,7 @@ k_fmm_down32(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<float
                     sy += s_acc[q][lane + 32 * wid].y;
                 }
                 const C2<float> W = fmm_local(pt, cf, inv_h);
-                const C2<float> F = fmm_local_at<float, P>(s_l[0], W, wid ? nx[1] : nx[0], wid ? ny[1] : ny[0]);
+                const C2<float> F = fmm_local_at<float, 1>(s_l[0], W, 0, wid ? nx[1] : nx[0], wid ? ny[1] : ny[0]);
                 const float g = (float)(1.0 / (4.0 * kPi)) * inv_h, cp = (float)(-1.0 / kPi);
                 part[cl.part_off[0] + (nd - cl.node_off)] = make_float2(fmaf(cp, sx, g * F.x), fmaf(cp, sy, g * F.y));
             }
@@ -813,30 +937,23 @@ k_fmm_down32(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<float
     }
 }
 
-// 1 / x by the hardware's approximation (20 bits) and one step of the cubic
-// iteration r <- r (1 + e + e^2), e = 1 - x r
-__device__ __forceinline__ double rcp64(double x) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-
-// Double precision (DF: the pairs in double-float arithmetic on the FP32 pipe).
-// One CTA per (leaf, tile share): four warps share a tile of 32 targets and
-// split the near sources.
-template <bool DF>
+// Double precision, native or double-float (everything but the last sums).  One
+// CTA per (leaf, tile share): four warps share a tile of 32 targets and split
+// the near sources, then four lanes per target split the local expansion.
+template <typename R>
 __global__ void __launch_bounds__(128, 4)
-k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<double>* __restrict__ sq,
-             const float4* __restrict__ sqdf, const V4<double>* __restrict__ loc, const double* __restrict__ binom,
-             const double* __restrict__ nxv, const double* __restrict__ nyv, int prec, int n0, int n1,
-             double2* __restrict__ part) {
-    constexpr int P = kFmmP64;
-    __shared__ V4<double> s_l[4][P];
+k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<R>* __restrict__ sq,
+             const V4<R>* __restrict__ loc, int shares, FmmTab<R> tab, const double* __restrict__ nxv,
+             const double* __restrict__ nyv, int prec, int n0, int n1, double2* __restrict__ part) {
+    constexpr int P = FmmTypes<R>::P;
+    constexpr bool DF = std::is_same<R, df>::value;
+    __shared__ V4<R> s_l[4][P];
+    __shared__ C2<R> s_pw[4][2][kPowTab];
     __shared__ FmmRange s_r[kFmmRanges];
     __shared__ int s_nr;
     __shared__ double2 s_p[4][32], s_q[4][32];  // double-float: a float4 each
-    __shared__ double2 s_acc[4][32];
+    __shared__ double2 s_acc[4][32], s_t[32], s_n[32];
+    __shared__ int s_node[32];
     const int b = blockIdx.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t0 = t.tstart[b], t1 = t.tstart[b + 1];
     if (t0 + 32 * (int)blockIdx.y >= t1) return;
@@ -848,7 +965,7 @@ k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<doubl
         const int n = fmm_ranges(t, f, cl, bx, nimg, s_r, lane);
         if (lane == 0) s_nr = n;
     }
-    fmm_local_to_leaf<double, P>(t, f, bx, loc, binom, s_l, wid, lane);
+    fmm_local_to_leaf<R>(t, f, bx, loc, shares, tab, s_l, s_pw, wid, lane);
     const int nr = s_nr;
     const double2 c = fmm_centre(f, 0, fmm_ix(bx), fmm_iy(bx));
     for (int k0 = t0 + 32 * blockIdx.y; k0 < t1; k0 += 32 * gridDim.y) {
@@ -887,10 +1004,10 @@ k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<doubl
                 if (lane < cnt) {
                     if constexpr (DF) {
                         *reinterpret_cast<float4*>(&s_p[wid][lane]) = t.spos[s];
-                        *reinterpret_cast<float4*>(&s_q[wid][lane]) = sqdf[s];
+                        *reinterpret_cast<float4*>(&s_q[wid][lane]) = reinterpret_cast<const float4*>(sq)[s];
                     } else {
                         s_p[wid][lane] = t.spos64[s];
-                        s_q[wid][lane] = make_double2(sq[s].x, sq[s].y);
+                        s_q[wid][lane] = reinterpret_cast<const double2*>(sq)[s];
                     }
                 }
                 __syncwarp();
@@ -898,6 +1015,7 @@ k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<doubl
                     // chunk sums as (TwoSum high part, float error), folded into
                     // double after every chunk
                     float axh = 0, axe = 0, ayh = 0, aye = 0;
+#pragma unroll 2
                     for (int j = 0; j < cnt; ++j) {
                         const float4 sp = *reinterpret_cast<const float4*>(&s_p[wid][j]);
                         const float4 ss = *reinterpret_cast<const float4*>(&s_q[wid][j]);
@@ -920,21 +1038,172 @@ k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<doubl
                 }
             }
         }
-        __syncthreads();
+        __syncthreads();  // also: the previous tile's targets have been read
         s_acc[wid][lane] = make_double2(ax, ay);
-        __syncthreads();
-        if (wid == 0 && node >= 0) {
-            double sx = 0, sy = 0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                sx += s_acc[q][lane].x;
-                sy += s_acc[q][lane].y;
-            }
-            const C2<double> W{(p.x - c.x) * f.inv_h, (p.y - c.y) * f.inv_h};
-            const C2<double> F = fmm_local_at<double, P>(s_l[0], W, nx, ny);
-            const double g = f.inv_h / (4.0 * kPi), cp = -1.0 / kPi;
-            part[cl.part_off[prec] + (node - cl.node_off)] = make_double2(fma(cp, sx, g * F.x), fma(cp, sy, g * F.y));
+        if (wid == 0) {
+            s_t[lane] = make_double2((p.x - c.x) * f.inv_h, (p.y - c.y) * f.inv_h);
+            s_n[lane] = make_double2(nx, ny);
+            s_node[lane] = node;
         }
+        __syncthreads();
+        const int q = threadIdx.x >> 2, res = threadIdx.x & 3, nd = s_node[q];
+        double fx = 0, fy = 0;
+        if (nd >= 0) {
+            const C2<R> F = fmm_local_at<R, 4>(s_l[0], C2<R>{R(s_t[q].x), R(s_t[q].y)}, res, R(s_n[q].x),
+                                               R(s_n[q].y));
+            const double g = f.inv_h / (4.0 * kPi), cp = -1.0 / kPi;
+            fx = fma(cp, s_acc[res][q].x, g * to_double(F.x));
+            fy = fma(cp, s_acc[res][q].y, g * to_double(F.y));
+        }
+        fx += __shfl_xor_sync(0xffffffffu, fx, 1);
+        fy += __shfl_xor_sync(0xffffffffu, fy, 1);
+        fx += __shfl_xor_sync(0xffffffffu, fx, 2);
+        fy += __shfl_xor_sync(0xffffffffu, fy, 2);
+        if (nd >= 0 && res == 0) part[cl.part_off[prec] + (nd - cl.node_off)] = make_double2(fx, fy);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// beside the sum (auxiliary stream): wall discrepancy and close pairs
+// ---------------------------------------------------------------------------
+// The wall discrepancy (Sec. 6.2 step 2, the far-image form of k_disc) from the
+// moments of the boxes of one level: the six far images of a wall point lie a
+// cell away from every box, so the series converge by 0.3 per order or better.
+// With u = 1 / W, W = (p - c) / H, per box
+//   velocity   4 pi mu u = -a_0 log|w| + (sum_{k>0} a_k u^k / k + conj(sum_{k>0} e_k u^k / k)
+//                          + conj(conj(W) A) + a_0) / 2,
+//   traction  -4 pi H T = 2 n Re A + conj(n (E - conj(W) A')).
+// The single-layer sum took 12 N (4 m) kernel evaluations with a logarithm
+// each: 3.5 ms of the FP64 pipe at 102400 nodes, 0.23 ms at 6400.
+template <typename R>
+__device__ __forceinline__ void wall_box(const V4<R>* mp, C2<R> W, double ln_w, R n0, R n1, const R* inv_k, double* v) {
+    constexpr int P = FmmTypes<R>::P;
+    const R s = rcp(fma_(W.x, W.x, W.y * W.y));
+    const C2<R> u{renorm(W.x * s), renorm(-(W.y * s))};
+    C2<R> A = czero<R>(), B = czero<R>(), E = czero<R>(), L = czero<R>(), M = czero<R>();
+    auto step = [&](C2<R>& a, R vx, R vy) {
+        a = {renorm(fma_(a.x, u.x, fma_(-a.y, u.y, vx))), renorm(fma_(a.x, u.y, fma_(a.y, u.x, vy)))};
+    };
+    for (int k = P - 1; k > 0; --k) {
+        const V4<R> m = mp[k];
+        const R k1(k + 1), ik = inv_k[k];
+        step(A, m.x, m.y);
+        step(B, k1 * m.x, k1 * m.y);
+        step(E, m.z, m.w);
+        step(L, ik * m.x, ik * m.y);
+        step(M, ik * m.z, ik * m.w);
+    }
+    const V4<R> m = mp[0];
+    step(A, m.x, m.y);
+    step(B, m.x, m.y);
+    step(E, m.z, m.w);
+    L = cmul(L, u);
+    M = cmul(M, u);
+    A = cmul(A, u);
+    E = cmul(E, u);
+    B = cmul(cmul(B, u), u);  // -A'
+    // F = E - conj(W) A'
+    const C2<R> F{E.x + fma_(W.x, B.x, W.y * B.y), E.y + fma_(W.x, B.y, -(W.y * B.x))};
+    // conj(conj(W) A) = W conj(A)
+    const R wx = fma_(W.x, A.x, W.y * A.y), wy = fma_(W.y, A.x, -(W.x * A.y));
+    v[0] = 0.5 * to_double(L.x + M.x + wx + m.x) - ln_w * to_double(m.x);
+    v[1] = 0.5 * to_double(L.y - M.y + wy + m.y) - ln_w * to_double(m.y);
+    v[2] = -to_double(R(2) * n0 * A.x + (n0 * F.x - n1 * F.y));
+    v[3] = -to_double(R(2) * n1 * A.x - (n0 * F.y + n1 * F.x));
+}
+constexpr int kWallImages = 6;
+
+// One warp per task: first (cell, wall point, far image), writing
+// gpart[((cell 7) + image) 8m + 4 wp + component]; then one per cell for its
+// total force (slot 6); then the close pairs (Sec. 6.3), C_p sigma into psum[p].
+template <typename R, typename B>
+__global__ void __launch_bounds__(128)
+k_side(FmmTree t, const Cell* __restrict__ cells, int ncell, int m, int walls, const V4<R>* __restrict__ mp,
+       const double* __restrict__ wall, const double* __restrict__ bodyF, double* __restrict__ gpart, int npairs,
+       const int4* __restrict__ pairs, const int* __restrict__ node_cell, const long long* __restrict__ blk_off,
+       const B* __restrict__ blocks, const double* __restrict__ body, const double2* __restrict__ sigma,
+       const double* __restrict__ w, void* __restrict__ psum) {
+    constexpr int P = FmmTypes<R>::P;
+    __shared__ R s_inv[P];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int task = blockIdx.x * 4 + wid;
+    if (walls) {
+        for (int k = threadIdx.x; k < P; k += 128) s_inv[k] = R(k ? 1.0 / k : 0.0);
+        __syncthreads();
+        const int per = 2 * m * kWallImages + 1;
+        if (task < ncell * per) {
+            const int ci = task / per, q = task % per;
+            const Cell& cl = cells[ci];
+            if (!cl.active) return;
+            double* gp = gpart + (size_t)ci * 7 * 8 * m;
+            double v[4] = {0, 0, 0, 0};
+            if (q == per - 1) {
+                for (int b = cl.body_off + lane; b < cl.body_off + cl.n_bodies; b += 32) {
+                    v[0] += bodyF[3 * b];
+                    v[1] += bodyF[3 * b + 1];
+                }
+            } else {
+                const int wp = q / kWallImages, im = q % kWallImages;
+                const FmmCell& f = t.cells[ci];
+                const int lv = f.wall, n = f.gx[lv] * f.gy[lv];
+                const double H = f.h * (1 << lv);
+                const double* wt = wall + ((size_t)ci * 2 * m + wp) * kWallStride;
+                const double px = wt[2 * im] - cl.C[0], py = wt[2 * im + 1] - cl.C[1];
+                const R n0(wt[12]), n1(wt[13]);
+                for (int e = lane; e < n; e += 32) {
+                    const int b = f.off[lv] + e;
+                    if (t.scount[b] == 0) continue;
+                    const double2 c = fmm_centre(f, lv, e % f.gx[lv], e / f.gx[lv]);
+                    const double wx = px - c.x, wy = py - c.y;
+                    double o[4];
+                    wall_box<R>(mp + (size_t)b * P, C2<R>{R(wx / H), R(wy / H)}, 0.5 * log(wx * wx + wy * wy), n0, n1,
+                                s_inv, o);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) v[k] += o[k];
+                }
+                const double sg = im < 3 ? 1.0 : -1.0;
+                const double cu = sg / (4.0 * kPi * cl.mu), ct = sg / (4.0 * kPi * H);
+                v[0] *= cu;
+                v[1] *= cu;
+                v[2] *= ct;
+                v[3] *= ct;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+            if (q == per - 1) {
+                if (lane < 2) gp[6 * 8 * (size_t)m + lane] = lane ? v[1] : v[0];
+            } else if (lane < 4) {
+                const int wp = q / kWallImages, im = q % kWallImages;
+                gp[(size_t)im * 8 * m + 4 * wp + lane] = lane == 0 ? v[0] : (lane == 1 ? v[1] : (lane == 2 ? v[2] : v[3]));
+            }
+            return;
+        }
+        task -= ncell * per;
+    }
+    if (task >= npairs) return;
+    const int4 pr = pairs[task];
+    if (!cells[node_cell[pr.x]].active) return;
+    const int n = (int)body[8 * pr.y + 5], off = (int)body[8 * pr.y + 6];
+    const B* C = blocks + blk_off[task];
+    B bx = 0, by = 0;
+#pragma unroll 4
+    for (int j = lane; j < n; j += 32) {
+        const double2 sg = sigma[off + j];
+        // single precision: blocks act on q = sigma w
+        const double wj = sizeof(B) == 4 ? w[off + j] : 1.0;
+        const B sx = sizeof(B) == 4 ? (B)(sg.x * wj) : (B)sg.x, sy = sizeof(B) == 4 ? (B)(sg.y * wj) : (B)sg.y;
+        const B a = C[3 * j], b = C[3 * j + 1], d = C[3 * j + 2];
+        bx = fma(a, sx, fma(b, sy, bx));
+        by = fma(b, sx, fma(d, sy, by));
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        bx += __shfl_xor_sync(0xffffffffu, bx, o);
+        by += __shfl_xor_sync(0xffffffffu, by, o);
+    }
+    if (lane == 0) {
+        if constexpr (sizeof(B) == 4) reinterpret_cast<float2*>(psum)[task] = make_float2(bx, by);
+        else reinterpret_cast<double2*>(psum)[task] = make_double2(bx, by);
     }
 }
 
@@ -954,8 +1223,8 @@ k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<doubl
 // leaves of side h.  Rates per precision (0 single, 1 double, 2 double-float):
 // a direct pair, a pair of the fast sum's leaves, a translation.
 static constexpr double kDirectPair[3] = {0.345e-12, 31.7e-12, 3.57e-12};
-static constexpr double kLeafPair[3] = {1.0e-12, 25e-12, 4.5e-12};
-static constexpr double kTranslate[3] = {0.5e-9, 26e-9, 26e-9};
+static constexpr double kLeafPair[3] = {1.2e-12, 25e-12, 5e-12};
+static constexpr double kTranslate[3] = {0.7e-9, 26e-9, 7e-9};
 static constexpr double kFmmFixed[3] = {12e-6, 20e-6, 20e-6};
 
 struct FmmPlanCell {
@@ -1038,10 +1307,25 @@ void free_fmm(bie_ctx* c) {
     c->ws.ftick = nullptr;
 }
 
+// Table sizes in numbers of R: hankel, binom, then the child powers.
 template <typename R>
-static int fmm_tables(bie_ctx* c, int P, void** out) {
-    // [C(k + l, l)], [k][l]; then [C(m, k)], [k][m] (0 for k > m)
-    std::vector<R> t(2 * (size_t)P * P);
+static FmmTab<R> fmm_tab(const bie_ctx* c, int prec) {
+    constexpr int P = FmmTypes<R>::P;
+    const R* h = (const R*)c->fmm_tab[prec];
+    const C2<R>* pw = (const C2<R>*)(h + 2 * P * P);
+    return FmmTab<R>{h, h + P * P, pw, pw + 4 * P};
+}
+
+static df to_df(long double v) { return df((float)v, (float)(v - (long double)(float)v)); }
+
+template <typename R>
+static int fmm_tables(bie_ctx* c, int prec) {
+    constexpr int P = FmmTypes<R>::P;
+    std::vector<R> t(2 * (size_t)P * P + 16 * P);
+    auto put = [&](size_t k, long double v) {
+        if constexpr (std::is_same<R, df>::value) t[k] = to_df(v);
+        else t[k] = (R)v;
+    };
     std::vector<std::vector<long double>> b(2 * P, std::vector<long double>(2 * P, 0.0L));
     for (int n = 0; n < 2 * P; ++n) {
         b[n][0] = 1;
@@ -1049,12 +1333,56 @@ static int fmm_tables(bie_ctx* c, int P, void** out) {
     }
     for (int k = 0; k < P; ++k)
         for (int l = 0; l < P; ++l) {
-            t[(size_t)k * P + l] = (R)b[k + l][l];
-            t[(size_t)(P + k) * P + l] = (R)b[l][k];
+            put((size_t)k * P + l, b[k + l][l]);
+            put((size_t)(P + k) * P + l, b[l][k]);
         }
-    BIE_CUDA(c, cudaMalloc(out, t.size() * sizeof(R)));
-    BIE_CUDA(c, cudaMemcpy(*out, t.data(), t.size() * sizeof(R), cudaMemcpyHostToDevice));
+    for (int q = 0; q < 4; ++q) {
+        // delta = (+-1/4, +-1/4); 1 / (2 delta) = (+-1, -+1)
+        const long double dx = q & 1 ? 0.25L : -0.25L, dy = q >> 1 ? 0.25L : -0.25L;
+        long double d[2] = {1, 0}, g[2] = {1, 0};
+        for (int k = 0; k < P; ++k) {
+            const size_t o = 2 * (size_t)P * P + 2 * ((size_t)q * P + k);
+            put(o, d[0]);
+            put(o + 1, d[1]);
+            put(o + 8 * P, g[0]);
+            put(o + 8 * P + 1, g[1]);
+            const long double nd[2] = {d[0] * dx - d[1] * dy, d[0] * dy + d[1] * dx};
+            const long double ex = 4 * dx, ey = -4 * dy;
+            const long double ng[2] = {g[0] * ex - g[1] * ey, g[0] * ey + g[1] * ex};
+            d[0] = nd[0];
+            d[1] = nd[1];
+            g[0] = ng[0];
+            g[1] = ng[1];
+        }
+    }
+    BIE_CUDA(c, cudaMalloc(&c->fmm_tab[prec], t.size() * sizeof(R)));
+    BIE_CUDA(c, cudaMemcpy(c->fmm_tab[prec], t.data(), t.size() * sizeof(R), cudaMemcpyHostToDevice));
     return BIE_OK;
+}
+
+// The largest box side from whose corners the walls' far images are so far that
+// the moments converge there by a factor of 0.3 per order (24 orders reach
+// 3e-13) or 0.45 (48 orders, 2e-17); <= 0: none.  The images of L and R lie on the
+// lines lattice coordinate s = +-3/2, those of D and U on t = +-3/2; nodes lie
+// within a bounding radius of their centres.
+static double fmm_wall_side(const bie_ctx* c, int k, int prec) {
+    const Cell& cl = c->cells_h[k];
+    const double det = cl.e1[0] * cl.e2[1] - cl.e1[1] * cl.e2[0];
+    double R = 0, far = 0.5;  // bounding radius; largest |s|, |t| of a centre
+    for (int b = cl.body_off; b < cl.body_off + cl.n_bodies; ++b) {
+        const double* h = &c->body_host[8 * (size_t)b];
+        R = std::max(R, std::max(h[0], h[1]));
+        const double px = h[2] - cl.C[0], py = h[3] - cl.C[1];
+        far = std::max(far, std::max(std::fabs(px * cl.e2[1] - py * cl.e2[0]), std::fabs(cl.e1[0] * py - cl.e1[1] * px)) /
+                                std::fabs(det));
+    }
+    // perpendicular spacing of the lattice lines; a sheared cell's e2 lengthens
+    // to (e1 / 2, e2_y) at most
+    double e2x = std::fabs(cl.e2[0]);
+    if (cl.e1[1] == 0.0) e2x = std::max(e2x, 0.5 * std::fabs(cl.e1[0]));
+    const double l2 = std::hypot(e2x, cl.e2[1]), l1 = std::hypot(cl.e1[0], cl.e1[1]);
+    const double d = (1.5 - far) * std::fabs(det) / std::max(l1, l2) - R;
+    return (prec == 0 ? 0.3 : 0.45) * d * std::sqrt(2.0);
 }
 
 // Boxes of every precision whose near sums run faster this way.  Called when
@@ -1086,7 +1414,7 @@ int fmm_plan(bie_ctx* c) {
     std::vector<double> per(c->nb);
     for (int b = 0; b < c->nb; ++b) per[b] = body_perimeter(c, b);
     const int N = c->N, nsrc = N * c->srcmul;
-    size_t mp_bytes = 0, sq_bytes = 0;
+    size_t mp_bytes = 0, loc_bytes = 0, sq_bytes = 0;
     int max_box = 0;
     for (int prec = 0; prec < 3; ++prec) {
         Fmm& f = c->fmm[prec];
@@ -1100,10 +1428,13 @@ int fmm_plan(bie_ctx* c) {
             // leaf side: the modelled best of a geometric ladder, with at most
             // one box per 8 source records (64 at least)
             const double most = std::max(64.0, cl.n_nodes * (double)c->srcmul / 8);
+            const double wall = fmm_wall_side(c, k, prec);
             double best = INFINITY, bh = 0;
             for (int j = 0; j < 48; ++j) {
                 const double h = std::sqrt(rc.area) * std::pow(2.0, -0.25 * j);
                 if (std::ceil(rc.w / h) * std::ceil(rc.ht / h) * 1.34 + 8 > most) break;
+                if (wall > 0 && h > wall) continue;
+                if (std::ceil(rc.w / h) > 4000 || std::ceil(rc.ht / h) > 4000) break;
                 const double t = fmm_cost(c, cl, per, rc.area, h, prec);
                 if (t < best) {
                     best = t;
@@ -1129,10 +1460,15 @@ int fmm_plan(bie_ctx* c) {
                 fc.gy[fc.nlev] = (fc.gy[fc.nlev - 1] + 1) / 2;
                 ++fc.nlev;
             }
+            fc.wall = -1;
+            for (int l = 0; l < fc.nlev; ++l)
+                if (bh * (1 << l) <= wall) fc.wall = l;
             fc.off[0] = (int)nleaf;
             nleaf += (long long)fc.gx[0] * fc.gy[0];
         }
         f.on = t_fast < t_direct && nleaf < (1 << 26);
+        f.walls = f.on && !c->utilde;
+        for (const FmmCell& fc : cells) f.walls = f.walls && fc.wall >= 0;
         if (!f.on) continue;
         // leaves of all cells first, then the coarser levels cell by cell
         nbox = nleaf;
@@ -1164,6 +1500,7 @@ int fmm_plan(bie_ctx* c) {
         t.nbox = (int)nbox;
         int rc = get(&f.cells, cells.size() * sizeof(FmmCell));
         rc = rc ? rc : get(&f.box, box.size() * sizeof(int4));
+        rc = rc ? rc : get(&t.centre, nleaf * sizeof(float4));
         rc = rc ? rc : get(&t.scount, nbox * sizeof(int));
         rc = rc ? rc : get(&t.sstart, (nleaf + 1) * sizeof(int));
         rc = rc ? rc : get(&t.sperm, nsrc * sizeof(int));
@@ -1189,23 +1526,36 @@ int fmm_plan(bie_ctx* c) {
         if (rc) return rc;
         BIE_CUDA(c, cudaMemcpy(f.cells, cells.data(), cells.size() * sizeof(FmmCell), cudaMemcpyHostToDevice));
         BIE_CUDA(c, cudaMemcpy(f.box, box.data(), box.size() * sizeof(int4), cudaMemcpyHostToDevice));
+        std::vector<float4> centre(nleaf);
+        for (long long b = 0; b < nleaf; ++b) {
+            const double2 p = fmm_centre(cells[box[b].x], 0, fmm_ix(box[b]), fmm_iy(box[b]));
+            centre[b].x = (float)p.x;
+            centre[b].y = (float)(p.x - (double)centre[b].x);
+            centre[b].z = (float)p.y;
+            centre[b].w = (float)(p.y - (double)centre[b].z);
+        }
+        BIE_CUDA(c, cudaMemcpy(t.centre, centre.data(), centre.size() * sizeof(float4), cudaMemcpyHostToDevice));
         t.cells = f.cells;
         t.box = f.box;
         f.built = 0;
-        if (!c->fmm_tab[dbl]) {
-            rc = dbl ? fmm_tables<double>(c, kFmmP64, &c->fmm_tab[1]) : fmm_tables<float>(c, kFmmP32, &c->fmm_tab[0]);
-            if (rc) return rc;
-        }
+        rc = prec == 0 ? fmm_tables<float>(c, prec)
+                       : (prec == 1 ? fmm_tables<double>(c, prec) : fmm_tables<df>(c, prec));
+        if (rc) return rc;
         f.mp_bytes = (size_t)nbox * (dbl ? kFmmP64 * sizeof(V4<double>) : kFmmP32 * sizeof(V4<float>));
+        // lists split into shares until the boxes (about half of them occupied)
+        // fill the SMs four times over
+        f.shares = std::max(1, std::min(kFmmShares, (int)(8LL * c->sms / std::max(1LL, nbox))));
+        f.loc_bytes = f.mp_bytes * f.shares;
         f.sq_bytes = (size_t)nsrc * (dbl ? sizeof(double2) : sizeof(float2));
         mp_bytes = std::max(mp_bytes, f.mp_bytes);
+        loc_bytes = std::max(loc_bytes, f.loc_bytes);
         sq_bytes = std::max(sq_bytes, f.sq_bytes);
         max_box = std::max(max_box, (int)nbox);
     }
     if (max_box) {
         BIE_CUDA(c, cudaMalloc(&c->ws.fsq, sq_bytes + 16));
         BIE_CUDA(c, cudaMalloc(&c->ws.fmp, mp_bytes + 16));
-        BIE_CUDA(c, cudaMalloc(&c->ws.floc, mp_bytes + 16));
+        BIE_CUDA(c, cudaMalloc(&c->ws.floc, loc_bytes + 16));
         BIE_CUDA(c, cudaMalloc((void**)&c->ws.ftick, max_box * sizeof(unsigned)));
         BIE_CUDA(c, cudaMemset(c->ws.ftick, 0, max_box * sizeof(unsigned)));
     }
@@ -1238,49 +1588,65 @@ int fmm_build(bie_ctx* c, int prec) {
     return BIE_OK;
 }
 
-// The near sum's partials (one split per cell) of sigma in ws.part.
-int fmm_near(bie_ctx* c, const double* sigma, int prec, Workspace& ws) {
-    Fmm& f = c->fmm[prec];
-    const FmmTree& t = f.t;
-    const int nimg = c->utilde ? 1 : 9, shift = c->utilde ? 2 : 0;
-    const double2* sg = reinterpret_cast<const double2*>(sigma);
-    const int n0 = c->shard.on ? c->shard.n0 : 0, n1 = c->shard.on ? c->shard.n1 : c->N;
-    const dim3 down(t.nleaf, 2);
-    if (prec == 0) {
-        const float* tab = (const float*)c->fmm_tab[0];
-        const float* bin = tab + kFmmP32 * kFmmP32;
-        k_fmm_up<float, kFmmP32><<<(t.nleaf + 3) / 4, 128, 0, c->stream>>>(
-            t, c->cells, sg, c->w, shift, (C2<float>*)ws.fsq, nullptr, (V4<float>*)ws.fmp, ws.ftick, bin);
-        BIE_LAUNCH(c, "k_fmm_up");
-        k_fmm_m2l<float, kFmmP32><<<t.nbox, 128, 0, c->stream>>>(t, c->cells, nimg, (const V4<float>*)ws.fmp,
-                                                               (V4<float>*)ws.floc, tab);
-        BIE_LAUNCH(c, "k_fmm_m2l");
-        k_fmm_down32<<<down, 128, 0, c->stream>>>(t, c->cells, nimg, (const C2<float>*)ws.fsq,
-                                                  (const V4<float>*)ws.floc, bin, c->tgt32, n0, n1,
-                                                  (float2*)ws.part);
-        BIE_LAUNCH(c, "k_fmm_down32");
-        return BIE_OK;
-    }
-    const double* tab = (const double*)c->fmm_tab[1];
-    const double* bin = tab + kFmmP64 * kFmmP64;
-    const bool df = prec == 2;
-    k_fmm_up<double, kFmmP64><<<(t.nleaf + 3) / 4, 128, 0, c->stream>>>(
-        t, c->cells, sg, c->w, shift, (C2<double>*)ws.fsq, df ? (float4*)ws.fsq : nullptr, (V4<double>*)ws.fmp,
-        ws.ftick, bin);
+template <typename R>
+static int up_launch(bie_ctx* c, const double* sigma, int prec, Workspace& ws) {
+    const FmmTree& t = c->fmm[prec].t;
+    k_fmm_up<R><<<t.nleaf, 128, 0, c->stream>>>(t, c->cells, reinterpret_cast<const double2*>(sigma), c->w,
+                                                c->utilde ? 2 : 0, (C2<R>*)ws.fsq, (V4<R>*)ws.fmp, ws.ftick,
+                                                fmm_tab<R>(c, prec));
     BIE_LAUNCH(c, "k_fmm_up");
-    k_fmm_m2l<double, kFmmP64><<<t.nbox, 128, 0, c->stream>>>(t, c->cells, nimg, (const V4<double>*)ws.fmp,
-                                                            (V4<double>*)ws.floc, tab);
-    BIE_LAUNCH(c, "k_fmm_m2l");
-    if (df)
-        k_fmm_down64<true><<<down, 128, 0, c->stream>>>(t, c->cells, nimg, nullptr, (const float4*)ws.fsq,
-                                                        (const V4<double>*)ws.floc, bin, c->nx, c->ny, prec, n0, n1,
-                                                        (double2*)ws.part);
-    else
-        k_fmm_down64<false><<<down, 128, 0, c->stream>>>(t, c->cells, nimg, (const C2<double>*)ws.fsq, nullptr,
-                                                         (const V4<double>*)ws.floc, bin, c->nx, c->ny, prec, n0, n1,
-                                                         (double2*)ws.part);
-    BIE_LAUNCH(c, "k_fmm_down64");
     return BIE_OK;
+}
+
+int fmm_up(bie_ctx* c, const double* sigma, int prec, Workspace& ws) {
+    return prec == 0 ? up_launch<float>(c, sigma, prec, ws)
+                     : (prec == 1 ? up_launch<double>(c, sigma, prec, ws) : up_launch<df>(c, sigma, prec, ws));
+}
+
+template <typename R>
+static int across_launch(bie_ctx* c, int prec, Workspace& ws) {
+    const Fmm& f = c->fmm[prec];
+    const FmmTree& t = f.t;
+    const FmmTab<R> tab = fmm_tab<R>(c, prec);
+    const int nimg = c->utilde ? 1 : 9;
+    const int n0 = c->shard.on ? c->shard.n0 : 0, n1 = c->shard.on ? c->shard.n1 : c->N;
+    const V4<R>* loc = (const V4<R>*)ws.floc;
+    k_fmm_m2l<R><<<dim3(t.nbox, f.shares), 128, 0, c->stream>>>(t, c->cells, nimg, (const V4<R>*)ws.fmp,
+                                                                (V4<R>*)ws.floc, tab);
+    BIE_LAUNCH(c, "k_fmm_m2l");
+    const dim3 down(t.nleaf, 2);
+    if constexpr (sizeof(R) == 4)
+        k_fmm_down32<<<down, 128, 0, c->stream>>>(t, c->cells, nimg, (const C2<float>*)ws.fsq, loc, f.shares, tab,
+                                                  c->tgt32, n0, n1, (float2*)ws.part);
+    else
+        k_fmm_down64<R><<<down, 128, 0, c->stream>>>(t, c->cells, nimg, (const C2<R>*)ws.fsq, loc, f.shares, tab,
+                                                     c->nx, c->ny, prec, n0, n1, (double2*)ws.part);
+    BIE_LAUNCH(c, "k_fmm_down");
+    return BIE_OK;
+}
+
+int fmm_across(bie_ctx* c, int prec, Workspace& ws) {
+    return prec == 0 ? across_launch<float>(c, prec, ws)
+                     : (prec == 1 ? across_launch<double>(c, prec, ws) : across_launch<df>(c, prec, ws));
+}
+
+template <typename R, typename B>
+static int side_launch(bie_ctx* c, const double* sigma, int prec, bool walls, const B* blocks, Workspace& ws,
+                       cudaStream_t st) {
+    const long long tasks = (walls ? (long long)c->ncell * (2 * c->m * kWallImages + 1) : 0) + c->cl.npairs;
+    if (tasks == 0) return BIE_OK;
+    k_side<R, B><<<(unsigned)((tasks + 3) / 4), 128, 0, st>>>(
+        c->fmm[prec].t, c->cells, c->ncell, c->m, walls ? 1 : 0, (const V4<R>*)ws.fmp, c->wall, ws.bodyF, ws.gpart,
+        c->cl.npairs, c->cl.pairs, c->node_cell, c->cl.blk_off, blocks, c->body,
+        reinterpret_cast<const double2*>(sigma), c->w, ws.psum ? ws.psum : c->cl.psum);
+    BIE_LAUNCH(c, "k_side");
+    return BIE_OK;
+}
+
+int side(bie_ctx* c, const double* sigma, int prec, bool walls, Workspace& ws, cudaStream_t st) {
+    if (prec == 0) return side_launch<float>(c, sigma, prec, walls, c->cl.blocks32, ws, st);
+    return prec == 1 ? side_launch<double>(c, sigma, prec, walls, c->cl.blocks, ws, st)
+                     : side_launch<df>(c, sigma, prec, walls, c->cl.blocks, ws, st);
 }
 
 }  // namespace bie

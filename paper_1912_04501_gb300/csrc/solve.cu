@@ -49,6 +49,14 @@ int build_dot_chunks(bie_ctx* c) {
         for (int e = e0; e < e1; e += kDotChunk) ch.push_back(make_int4(ci, e, std::min(e1, e + kDotChunk), 0));
         cc[ci].y = (int)ch.size() - cc[ci].x;
     }
+    std::vector<int4> fin;  // the assembly's chunks of nodes
+    for (int ci = 0; ci < c->ncell; ++ci) {
+        const int n0 = c->cells_h[ci].node_off, n1 = n0 + c->cells_h[ci].n_nodes;
+        for (int i = n0; i < n1; i += kFinNodes) fin.push_back(make_int4(ci, i, std::min(n1, i + kFinNodes), 0));
+    }
+    c->n_fin = (int)fin.size();
+    BIE_CUDA(c, cudaMalloc((void**)&c->fin_chunks, fin.size() * sizeof(int4)));
+    BIE_CUDA(c, cudaMemcpy(c->fin_chunks, fin.data(), fin.size() * sizeof(int4), cudaMemcpyHostToDevice));
     c->sv.nchunks = (int)ch.size();
     BIE_CUDA(c, cudaMalloc((void**)&c->sv.chunks, ch.size() * sizeof(int4)));
     BIE_CUDA(c, cudaMalloc((void**)&c->sv.cell_chunks, cc.size() * sizeof(int2)));
