@@ -54,7 +54,6 @@ static void free_all(bie_ctx* c) {
     c->ev_pool.clear();
     if (c->next_done) cudaEventDestroy(c->next_done);
     if (c->aux_fork) cudaEventDestroy(c->aux_fork);
-    if (c->aux_up) cudaEventDestroy(c->aux_up);
     if (c->aux_join) cudaEventDestroy(c->aux_join);
     for (auto e : c->sv.ev)
         if (e) cudaEventDestroy(e);
@@ -462,7 +461,6 @@ int bie_init_batch(bie_ctx** out, int32_t n_cells, const bie_cell* cells, const 
     if (!rc) rc = cu(cudaEventCreateWithFlags(&c->next_done, cudaEventDisableTiming), "cudaEventCreate");
     if (!rc) rc = cu(cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking), "cudaStreamCreate");
     if (!rc) rc = cu(cudaEventCreateWithFlags(&c->aux_fork, cudaEventDisableTiming), "cudaEventCreate");
-    if (!rc) rc = cu(cudaEventCreateWithFlags(&c->aux_up, cudaEventDisableTiming), "cudaEventCreate");
     if (!rc) rc = cu(cudaEventCreateWithFlags(&c->aux_join, cudaEventDisableTiming), "cudaEventCreate");
     rc = rc ? rc : dalloc(c, &c->yp, nc * 2 * M);
     rc = rc ? rc : dalloc(c, &c->ypf, nc * M);

@@ -31,34 +31,6 @@
 
 namespace bie {
 
-__device__ inline double warp_sum_d(double v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-__device__ inline double block_sum_d(double v, double* red) {
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    v = warp_sum_d(v);
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        double s = lane < nw ? red[lane] : 0.0;
-        s = warp_sum_d(s);
-        if (lane == 0) red[32] = s;
-    }
-    __syncthreads();
-    double r = red[32];
-    __syncthreads();
-    return r;
-}
-
-
-// Knuth's TwoSum: s + e == a + b exactly
-
-// ---------------------------------------------------------------------------
-
-
 // Work item of a near-sum launch: cell, target tile and source split.  The
 // tile covers `tile` targets of the cell; the split covers the cell's sources
 // [split * chunk, (split + 1) * chunk), chunk = ceil(N_cell / splits).
@@ -1117,31 +1089,17 @@ k_disc(const Src64* __restrict__ src64, const float4* __restrict__ src32, const 
 // to ~1/lam, so a plain double-precision product would add relative noise
 // ~1e-11 to the correction and put a floor under the GMRES residual).  xi is
 // also stored in single precision for the single-precision correction.
-// gimg: the discrepancy as k_side leaves it (six far images' parts and the
-// force per cell); otherwise gt holds g~.
 __global__ void __launch_bounds__(32)
-k_xi(const double* __restrict__ gt, const double* __restrict__ gimg, int m, int M, const Cell* __restrict__ cells,
-     const double* __restrict__ Pall, double* __restrict__ xiall, float* __restrict__ xifall) {
+k_xi(const double* __restrict__ gt, int m, int M, const Cell* __restrict__ cells, const double* __restrict__ Pall,
+     double* __restrict__ xiall, float* __restrict__ xifall) {
     const int lane = threadIdx.x, r = blockIdx.x, cidx = blockIdx.y;
     if (!cells[cidx].active) return;
     const int nv = 8 * m;
-    const double* d = gimg ? nullptr : gt + (size_t)cidx * nv;
-    const double* gi = gimg ? gimg + (size_t)cidx * 7 * nv : nullptr;
-    const Cell& cl = cells[cidx];
+    const double* d = gt + (size_t)cidx * nv;
     const double* P = Pall + (size_t)cidx * 2 * M * nv;
     double s = 0, e = 0;
     for (int cc = lane; cc < nv; cc += 32) {
-        const double a = P[(size_t)r * nv + cc];
-        double b;
-        if (gi) {  // g~ = g0 - g from the far images' parts (k_side), as k_disc's last block forms it
-            const int L = cc < 4 * m, k = (cc % (4 * m)) / m, wp = (L ? 0 : m) + cc % m;
-            double g = 0;
-#pragma unroll
-            for (int im = 0; im < 6; ++im) g += gi[(size_t)im * nv + 4 * wp + k];
-            b = (k < 2 ? 0.0 : gi[6 * (size_t)nv + k - 2] / (2.0 * (L ? cl.l2 : cl.l1))) - g;
-        } else {
-            b = d[cc];
-        }
+        const double a = P[(size_t)r * nv + cc], b = d[cc];
         const double p = a * b;
         const double pe = fma(a, b, -p);
         const double t = s + p;
@@ -1401,12 +1359,7 @@ static_assert(kNear32Shapes == 5 && BIE_SHAPE_IS(0, 1, BIE_NEAR32_TPT, BIE_NEAR3
 // 2 wall discrepancy, proxy fit and correction, close evaluation, assembly.
 // a3 + a4: the wall discrepancy g~ of the packed sources and the proxy
 // strengths xi = P g~ on stream st (independent of the near sum)
-static int launch_disc_xi(bie_ctx* c, bool f32, bool walls, Workspace& ws, cudaStream_t st) {
-    if (walls) {  // k_side has left the discrepancy's parts
-        k_xi<<<dim3(2 * c->M, c->ncell), 32, 0, st>>>(ws.gt, ws.gpart, c->m, c->M, c->cells, c->P, ws.xi, ws.xif);
-        BIE_LAUNCH(c, "k_xi");
-        return BIE_OK;
-    }
+static int launch_disc_xi(bie_ctx* c, bool f32, Workspace& ws, cudaStream_t st) {
     const dim3 dgrid(2 * c->m, kDiscSplits, c->ncell);
     if (c->utilde) {
         if (f32)
@@ -1423,16 +1376,18 @@ static int launch_disc_xi(bie_ctx* c, bool f32, bool walls, Workspace& ws, cudaS
                                                     ws.dticket, ws.gt, nullptr);
     }
     BIE_LAUNCH(c, "k_disc");
-    k_xi<<<dim3(2 * c->M, c->ncell), 32, 0, st>>>(ws.gt, nullptr, c->m, c->M, c->cells, c->P, ws.xi, ws.xif);
+    k_xi<<<dim3(2 * c->M, c->ncell), 32, 0, st>>>(ws.gt, c->m, c->M, c->cells, c->P, ws.xi, ws.xif);
     BIE_LAUNCH(c, "k_xi");
     return BIE_OK;
 }
 
 // One operator application in four parts: 0 packs the sources and body
 // moments, 1 is the near sum, 2 the wall discrepancy and proxy strengths
-// (independent of 1 after the direct sum, from its boxes' moments after the
-// fast one) and the close pairs' sums, 3 the assembly (traction, close
-// evaluation, pressure fix, rigid completion).
+// (independent of 1) and, but for the single-precision assembly, the close
+// pairs' sums, 3 the assembly (traction, close evaluation, pressure fix, rigid
+// completion).  After the fast image sum (fmm.cu) part 0 is its first launch and
+// 1 its second and third, which do the rest of 0 and 2 besides; where the walls
+// do not run by expansions, part 2 is theirs alone.
 static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, int precision, Workspace& ws,
                       cudaStream_t st) {
     const double2* sg = reinterpret_cast<const double2*>(sigma);
@@ -1442,24 +1397,21 @@ static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, i
     const bool fast = c->fmm[prec].on;  // the fast image sum packs its own sorted strengths
     if (part == 0) {
         if (&ws == &c->ws) c->ws_x = nullptr;  // the workspace is about to change
+        if (fast) return fmm_up(c, sigma, prec, ws);
         if (c->utilde)
             k_pack_moments_u<<<c->nb, 256, 0, st>>>(sg, c->x, c->y, c->w, c->body, c->body_cell, c->cells,
-                                                           c->imc, f32 && !fast ? ws.src32 : nullptr,
-                                                           f32 ? ws.src32n : nullptr, ws.src64,
-                                                           !f32 && !df && !fast ? ws.src64u : nullptr,
-                                                           df && !fast ? (SrcDF*)ws.srcdf : nullptr, ws.bodyF);
+                                                           c->imc, f32 ? ws.src32 : nullptr, f32 ? ws.src32n : nullptr,
+                                                           ws.src64, (!f32 && !df) ? ws.src64u : nullptr,
+                                                           df ? (SrcDF*)ws.srcdf : nullptr, ws.bodyF);
         else
             k_pack_moments<<<c->nb, 256, 0, st>>>(sg, c->x, c->y, c->w, c->body, c->body_cell, c->cells,
                                                          f32 ? ws.src32 : nullptr, ws.src64,
-                                                         df && !fast ? (SrcDF*)ws.srcdf : nullptr, ws.bodyF);
+                                                         df ? (SrcDF*)ws.srcdf : nullptr, ws.bodyF);
         BIE_LAUNCH(c, "k_pack_moments");
         return BIE_OK;
     }
     if (part == 1) {
-        if (fast) {
-            if (int rc = fmm_up(c, sigma, prec, ws)) return rc;
-            return fmm_across(c, prec, ws);
-        }
+        if (fast) return fmm_across(c, sigma, prec, ws);
         if (f32) return launch_near32(c, ws.src32, (float2*)ws.part);
         if (c->utilde) {
             if (df)
@@ -1486,10 +1438,10 @@ static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, i
         return BIE_OK;
     }
     if (part == 2) {
-        const bool walls = fast && c->fmm[prec].walls;
-        if (fast || !f32)
-            if (int rc = side(c, sigma, prec, walls, ws, st)) return rc;
-        return launch_disc_xi(c, f32, walls, ws, st);
+        if (fast && c->fmm[prec].walls) return BIE_OK;
+        if (!fast && !f32)
+            if (int rc = close_pairs(c, sigma, prec, ws, st)) return rc;
+        return launch_disc_xi(c, f32, ws, st);
     }
     if (f32 && !fast) return assemble32(c, sigma, ws, yout);
     if (int rc = finish(c, sigma, prec, ws, yout)) return rc;
@@ -1507,29 +1459,17 @@ static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, i
 static int apply_impl(bie_ctx* c, const double* sigma, double* yout, int precision, Workspace& ws) {
     const int kind = precision == BIE_MIXED ? 0 : (precision == BIE_DF64 ? 2 : 1);
     if (int rc = fmm_build(c, kind)) return rc;
-    const auto record = [](cudaEvent_t e, cudaStream_t from, cudaStream_t to) {
-        const cudaError_t rc = cudaEventRecord(e, from);
-        return rc == cudaSuccess ? cudaStreamWaitEvent(to, e, 0) : rc;
-    };
-    if (c->fmm[kind].on) {
-        // everything but the image sum on the auxiliary stream: the pack at once,
-        // the walls and close pairs once the boxes' moments are there
-        BIE_CUDA(c, record(c->aux_fork, c->stream, c->aux));
+    if (c->fmm[kind].walls) {  // four launches, one after the other
+        if (int rc = apply_part(c, 0, sigma, yout, precision, ws, c->stream)) return rc;
         if (int rc = prof_begin(c, kind)) return rc;
-        if (int rc = fmm_up(c, sigma, kind, ws)) return rc;
-        BIE_CUDA(c, cudaEventRecord(c->aux_up, c->stream));
-        if (int rc = apply_part(c, 0, sigma, yout, precision, ws, c->aux)) return rc;
-        BIE_CUDA(c, cudaStreamWaitEvent(c->aux, c->aux_up, 0));
-        if (int rc = apply_part(c, 2, sigma, yout, precision, ws, c->aux)) return rc;
-        BIE_CUDA(c, cudaEventRecord(c->aux_join, c->aux));
-        if (int rc = fmm_across(c, kind, ws)) return rc;
+        if (int rc = apply_part(c, 1, sigma, yout, precision, ws, c->stream)) return rc;
         if (int rc = prof_end(c)) return rc;
-        BIE_CUDA(c, cudaStreamWaitEvent(c->stream, c->aux_join, 0));
         return apply_part(c, 3, sigma, yout, precision, ws, c->stream);
     }
     if (int rc = apply_part(c, 0, sigma, yout, precision, ws, c->stream)) return rc;
     // part 2 on the auxiliary stream, overlapping the near sum
-    BIE_CUDA(c, record(c->aux_fork, c->stream, c->aux));
+    BIE_CUDA(c, cudaEventRecord(c->aux_fork, c->stream));
+    BIE_CUDA(c, cudaStreamWaitEvent(c->aux, c->aux_fork, 0));
     if (int rc = apply_part(c, 2, sigma, yout, precision, ws, c->aux)) return rc;
     BIE_CUDA(c, cudaEventRecord(c->aux_join, c->aux));
     if (int rc = prof_begin(c, kind)) return rc;
@@ -1542,8 +1482,7 @@ static int apply_impl(bie_ctx* c, const double* sigma, double* yout, int precisi
 // The single-precision application replayed from CUDA graphs (opts.graph):
 // the parts of apply_part are captured once per epoch (any change of their
 // arguments: geometry, proxy fit, close pairs, work items) as three graphs
-// (pack; near sum; assembly, the wall discrepancy and proxy strengths with the
-// first or the last)
+// (pack with the wall discrepancy and proxy strengths; near sum; assembly)
 // with fixed input and output buffers, on a stream of the context's own (the
 // caller's stream may be the legacy default stream, which cannot capture).
 // Each application copies sigma in, replays the graphs on the context's
@@ -1575,13 +1514,10 @@ static int apply_graph(bie_ctx* c, const double* sigma, double* yout) {
             cudaGraph_t graph = nullptr;
             e = cudaStreamBeginCapture(g.capture, cudaStreamCaptureModeThreadLocal);
             if (e != cudaSuccess) break;
-            // graphs: pack; near sum; assembly, with the wall discrepancy and proxy
-            // strengths in the first, or (they read the fast sum's moments) the third
+            // graphs: pack + wall discrepancy and proxy strengths; near sum; assembly
             static constexpr int kFirst[3] = {0, 1, 3};
-            const bool last = c->fmm[0].on;
-            if (part == 2 && last) rc = apply_part(c, 2, g.in, g.out, BIE_MIXED, c->ws, c->stream);
-            if (!rc) rc = apply_part(c, kFirst[part], g.in, g.out, BIE_MIXED, c->ws, c->stream);
-            if (!rc && part == 0 && !last) rc = apply_part(c, 2, g.in, g.out, BIE_MIXED, c->ws, c->stream);
+            rc = apply_part(c, kFirst[part], g.in, g.out, BIE_MIXED, c->ws, c->stream);
+            if (!rc && part == 0) rc = apply_part(c, 2, g.in, g.out, BIE_MIXED, c->ws, c->stream);
             e = cudaStreamEndCapture(g.capture, &graph);
             if (!rc && e == cudaSuccess) e = cudaGraphInstantiate(&g.exec[part], graph, 0);
             if (graph) cudaGraphDestroy(graph);
@@ -1818,7 +1754,7 @@ int fp64_moments_and_xi(bie_ctx* c, const double* sigma, bool reuse_ws) {
                 c->ws.src64, nullptr, c->cells, c->m, c->wall, c->ws.bodyF, c->ws.gpart, c->ws.dticket, c->ws.gt,
                 nullptr);
         BIE_LAUNCH(c, "k_disc");
-        k_xi<<<dim3(2 * c->M, c->ncell), 32, 0, c->stream>>>(c->ws.gt, nullptr, c->m, c->M, c->cells, c->P, c->ws.xi,
+        k_xi<<<dim3(2 * c->M, c->ncell), 32, 0, c->stream>>>(c->ws.gt, c->m, c->M, c->cells, c->P, c->ws.xi,
                                                                c->ws.xif);
         BIE_LAUNCH(c, "k_xi");
     }

@@ -232,13 +232,26 @@ struct FmmGeom {
     const int *imc, *node_cell;
 };
 
+// The sources of a near row of boxes are contiguous: a range of sorted records
+// under one image shift.
+struct FmmRange {
+    int s0, s1, im;
+};
+constexpr int kFmmRanges = 36;  // at most per leaf: 9 images x 4 rows
+constexpr int kFmmFar = 576;    // far boxes per box at most: 9 images x 64 children of near parents
+
 // Device view of the boxes: records sorted by leaf (targets are the sources
 // themselves, except with the doubled cell).
 struct FmmTree {
     const FmmCell* cells = nullptr;
     const int4* box = nullptr;     // nbox: (cell, level, x | y << 16, parent or -1); leaves first
     int nbox = 0, nleaf = 0;
-    float4* centre = nullptr;      // nleaf: leaf centres from the cell centre, double-float
+    float4* centre = nullptr;      // nbox: centres from the cell centre, double-float
+    int4* grid = nullptr;          // nbox: (first box of the level, its width, 0, 0)
+    int *far = nullptr, *nfar = nullptr;        // per box: the boxes to translate from (box | image << 28)
+    FmmRange* near = nullptr;      // per leaf: the near rows of sources
+    int* nnear = nullptr;
+    float4* shift = nullptr;       // 9 per cell: image shifts in leaf sides, float pairs
     int *scount = nullptr, *tcount = nullptr;  // nbox: records in the box
     int *sstart = nullptr, *tstart = nullptr;  // nleaf + 1: first sorted record
     int *sperm = nullptr, *tperm = nullptr;    // sorted record -> record (sources: node, or 4 node + image)
@@ -256,7 +269,8 @@ struct Fmm {
     unsigned long long built = 0;      // geometry the records are sorted for (0: none)
     int shares = 1;                    // CTAs a box's list is split over
     size_t mp_bytes = 0, loc_bytes = 0, sq_bytes = 0;  // multipole and local expansions, sorted strengths
-    std::vector<void*> owned;
+    void* arena = nullptr;             // holds all of the above
+    void* tables = nullptr;            // constant matrices (FmmTab), in the arena
 };
 
 // Near-sum work list of one precision: one CTA per item (cell, tile, split).
@@ -314,7 +328,7 @@ struct bie_ctx {
     // the wall discrepancy and proxy strengths of an application run on this
     // stream while the near sum runs on the context's stream (direct launches)
     cudaStream_t aux = nullptr;
-    cudaEvent_t aux_fork = nullptr, aux_up = nullptr, aux_join = nullptr;
+    cudaEvent_t aux_fork = nullptr, aux_join = nullptr;
     double* yp = nullptr;       // ncell x M x 2 proxy points of the current fit
     float2* ypf = nullptr;      // ncell x M proxy points minus the cell centre (single precision)
     double* scal = nullptr;     // 3 nb + ncell + 8: velocities, rotation rates, mu_eff
@@ -324,11 +338,11 @@ struct bie_ctx {
     bie::Close cl;
     bie::NearItems near[3];     // 0 single precision, 1 double, 2 double-float
     int shape32 = 0;            // tile shape of the single-precision near sum (kNear32ShapeList)
-    int4* fin_chunks = nullptr; // n_fin: (cell, first node, end node, 0)
+    int4* fin_chunks = nullptr; // n_fin: (cell, first node, end node, the cell's first)
     int n_fin = 0;
     int* near_ctr = nullptr;    // work-queue counter of the persistent near sum (batches)
     bie::Fmm fmm[3];            // fast image sum per precision (0 single, 1 double, 2 double-float)
-    void* fmm_tab[3] = {};      // its constant matrices
+    void* fmm_ws = nullptr;     // its part of the workspace
     std::vector<double> fmm_rects;          // 4 x ncell: the rectangles its boxes cover
     unsigned long long geometry = 0;        // bumped by build_geometry
     unsigned long long epoch = 0;  // bumped whenever a kernel argument of the operator application changes
@@ -422,15 +436,43 @@ void free_graph(bie_ctx* c);
 int assemble32(bie_ctx* c, const double* sigma, const Workspace& ws, double* yout);
 int finish(bie_ctx* c, const double* sigma, int prec, const Workspace& ws, double* yout);
 
+// Sum over the block; every thread receives the result.  red: 33 doubles.
+__device__ inline double warp_sum_d(double v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ inline double block_sum_d(double v, double* red) {
+    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    v = warp_sum_d(v);
+    __syncthreads();
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        double s = lane < nw ? red[lane] : 0.0;
+        s = warp_sum_d(s);
+        if (lane == 0) red[32] = s;
+    }
+    __syncthreads();
+    double r = red[32];
+    __syncthreads();
+    return r;
+}
+
 // fmm.cu --------------------------------------------------------------------
 int fmm_plan(bie_ctx* c);             // boxes for the bodies' current places (host mirror)
 int fmm_build(bie_ctx* c, int prec);  // sorts the current geometry if it is not
-int fmm_up(bie_ctx* c, const double* sigma, int prec, Workspace& ws);     // moments of every box
-int fmm_across(bie_ctx* c, int prec, Workspace& ws);                      // partials of every target from them
-// on stream st: the wall discrepancy from the boxes' moments (walls true) and
-// the close pairs' sums of sigma
-int side(bie_ctx* c, const double* sigma, int prec, bool walls, Workspace& ws, cudaStream_t st);
+int fmm_up(bie_ctx* c, const double* sigma, int prec, Workspace& ws);      // moments of every box, and of every body
+// partials of every target from them; the close pairs' sums and, with
+// Fmm::walls, the wall discrepancy and the proxy strengths
+int fmm_across(bie_ctx* c, const double* sigma, int prec, Workspace& ws);
+int close_pairs(bie_ctx* c, const double* sigma, int prec, Workspace& ws, cudaStream_t st);  // the pairs alone
 void free_fmm(bie_ctx* c);
+
+// whether an application's launches follow one another in one stream with nothing
+// between them
+inline bool fmm_chained(const bie_ctx* c, int prec) {
+    return c->fmm[prec].walls && !c->prof && c->stream != c->graph.capture;
+}
 
 // apply.cu ------------------------------------------------------------------
 // near-sum work items (and partial offsets) for the current cell sizes
@@ -464,6 +506,32 @@ int features_device(bie_ctx* c, float* X);
 int solve_device(bie_ctx* c, const double* b, double* x, bool use_guess, bie_solve_info* info,
                  const double* U = nullptr, int nu = 0, bool recycle_second = false);
 int build_dot_chunks(bie_ctx* c);
+
+// The second to fourth launches of a fast application start while the one before
+// still runs (programmatic stream serialisation): they read what only the geometry
+// decides, then wait here for the whole of it and its memory.  Every CTA passes
+// pdl_wait before it ends or reads or writes what an earlier launch touches, and
+// the next launch is let go only after the wait, so at most two overlap.  What the
+// earlier launch writes is not read through const __restrict__ pointers.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// With `early`, a launch that may begin before the one ahead of it in the stream
+// has ended (it waits in the kernel: pdl_wait).
+template <typename... A>
+inline cudaError_t launch_after(bool early, void (*k)(A...), unsigned grid, unsigned block, cudaStream_t st,
+                                typename std::common_type<A>::type... a) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, a...);
+}
 
 // small device math shared by the kernels --------------------------------------
 __device__ __forceinline__ float rcp_approx(float x) {

@@ -1030,7 +1030,7 @@ int assemble32(bie_ctx* c, const double* sigma, const Workspace& ws, double* you
 template <typename R>
 struct Finish {
     const int4* chunks;
-    int prec, M, use_pairs;
+    int prec, M, use_pairs, single;
     const void* part;  // float2, or double2
     const double* yp;
     const float2* ypf;  // from the cell centre
@@ -1051,58 +1051,58 @@ struct R2 {
     R x, y;
 };
 
-// Partials first, first + step, ... and the same proxies' traction at node i.
+// Traction of proxies first, first + step, ... at (X, Y) with normal n: four
+// independent sums, so that their chains overlap.
 template <typename R>
-__device__ __forceinline__ void finish_sum(const Finish<R>& a, const Cell& cl, int i, int first, int step,
-                                           const R2<R>* yp, const R2<R>* xi, double& tx, double& ty) {
-    const long long at = cl.part_off[a.prec] + (i - cl.node_off);
-    const int splits = cl.splits[a.prec];
-    R X, Y, n0, n1;
-    if constexpr (sizeof(R) == 4) {
-        const float2* pp = reinterpret_cast<const float2*>(a.part) + at;
-        float hx = 0, lx = 0, hy = 0, ly = 0;
-        for (int s = first; s < splits; s += step) {
-            const float2 p = pp[(long long)s * cl.n_nodes];
-            float e;
-            two_sum(hx, p.x, hx, e);
-            lx += e;
-            two_sum(hy, p.y, hy, e);
-            ly += e;
+__device__ __forceinline__ void proxy_sum(int M, int first, int step, const R2<R>* yp, const R2<R>* xi, R X, R Y, R n0,
+                                          R n1, double& tx, double& ty) {
+    R cx[4] = {R(0), R(0), R(0), R(0)}, cy[4] = {R(0), R(0), R(0), R(0)};
+    auto one = [&](int p, int u) {
+        const R2<R> q = yp[p], f = xi[p];
+        const R rx = X - q.x, ry = Y - q.y;
+        const R inv = rcp(renorm(fma_(rx, rx, ry * ry)));
+        const R cc = (renorm(fma_(rx, n0, ry * n1)) * inv) * (renorm(fma_(rx, f.x, ry * f.y)) * inv);
+        cx[u] = fma_(cc, rx, cx[u]);
+        cy[u] = fma_(cc, ry, cy[u]);
+    };
+    int p = first;
+    for (; p + 3 * step < M; p += 4 * step) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) one(p + u * step, u);
+    }
+    for (; p < M; p += step) one(p, 0);
+    const double c = -1.0 / kPi;
+    tx = c * to_double((cx[0] + cx[1]) + (cx[2] + cx[3]));
+    ty = c * to_double((cy[0] + cy[1]) + (cy[2] + cy[3]));
+}
+
+// The near sum's partials first, first + step, ... of node i.
+template <typename R>
+__device__ __forceinline__ void partial_sum(const Finish<R>& a, const Cell& cl, int i, int first, int step, double& tx,
+                                            double& ty) {
+    if (a.single) {  // after the fast sum: one per node, in node order
+        if (first) return;
+        if constexpr (sizeof(R) == 4) {
+            const float2 p = reinterpret_cast<const float2*>(a.part)[i];
+            tx += (double)p.x;
+            ty += (double)p.y;
+        } else {
+            const double2 p = reinterpret_cast<const double2*>(a.part)[i];
+            tx += p.x;
+            ty += p.y;
         }
-        tx = (double)hx + (double)lx;
-        ty = (double)hy + (double)ly;
-        const float4 tv = a.tgt32[i];
-        X = tv.x;
-        Y = tv.y;
-        n0 = tv.z;
-        n1 = tv.w;
-    } else {
-        const double2* pp = reinterpret_cast<const double2*>(a.part) + at;
-        tx = ty = 0;
+        return;
+    }
+    if constexpr (sizeof(R) == 8) {
+        const double2* pp = reinterpret_cast<const double2*>(a.part) + cl.part_off[a.prec] + (i - cl.node_off);
+        const int splits = cl.splits[a.prec];
 #pragma unroll 4
         for (int s = first; s < splits; s += step) {
             const double2 p = pp[(long long)s * cl.n_nodes];
             tx += p.x;
             ty += p.y;
         }
-        X = R(a.xw[i] - cl.C[0]);
-        Y = R(a.yw[i] - cl.C[1]);
-        n0 = R(a.nx[i]);
-        n1 = R(a.ny[i]);
     }
-    R cx(0), cy(0);
-#pragma unroll 2
-    for (int p = first; p < a.M; p += step) {
-        const R2<R> q = yp[p], f = xi[p];
-        const R rx = X - q.x, ry = Y - q.y;
-        const R inv = rcp(renorm(fma_(rx, rx, ry * ry)));
-        const R cc = (renorm(fma_(rx, n0, ry * n1)) * inv) * (renorm(fma_(rx, f.x, ry * f.y)) * inv);
-        cx = fma_(cc, rx, cx);
-        cy = fma_(cc, ry, cy);
-    }
-    const double c = -1.0 / kPi;
-    tx += c * to_double(cx);
-    ty += c * to_double(cy);
 }
 
 template <typename R>
@@ -1112,31 +1112,59 @@ k_finish(Finish<R> a, double2* __restrict__ out) {
     __shared__ double s_t0[2];
     const int t = threadIdx.x, wid = t >> 5, lane = t & 31;
     const int4 ch = a.chunks[blockIdx.x];
+    const int i0 = ch.y, i1 = ch.z, head = ch.w;
     const Cell& cl = a.cells[ch.x];
-    const int i0 = ch.y, i1 = ch.z, head = cl.node_off;
+    // what only the geometry and the density decide, before the wait
+    const int i = min(i0 + t, i1 - 1);
+    const double2 sg = a.sigma[i];
+    const double n0 = a.nx[i], n1 = a.ny[i], wi = a.w[i], ki = a.kap[i], xi_ = a.x[i], yi = a.y[i];
+    const int b = a.owner[i];
+    const int p0 = a.use_pairs ? a.pair_base[i] : 0, p1 = a.use_pairs ? a.pair_base[i + 1] : 0;
+    const double xc = a.body[8 * b + 2], yc = a.body[8 * b + 3];
+    R X, Y, m0, m1;
+    auto place = [&](int node, R& px, R& py, R& q0, R& q1) {
+        if constexpr (sizeof(R) == 4) {
+            const float4 tv = a.tgt32[node];
+            px = tv.x;
+            py = tv.y;
+            q0 = tv.z;
+            q1 = tv.w;
+        } else {
+            px = R(a.xw[node] - cl.C[0]);
+            py = R(a.yw[node] - cl.C[1]);
+            q0 = R(a.nx[node]);
+            q1 = R(a.ny[node]);
+        }
+    };
+    place(i, X, Y, m0, m1);
+    const double h0 = a.nx[head], h1 = a.ny[head];
     for (int p = t; p < a.M; p += kFinNodes) {
         if constexpr (sizeof(R) == 4) {
             const float2 q = a.ypf[(size_t)ch.x * a.M + p];
-            const float* xi = a.xif + (size_t)ch.x * 2 * a.M;
             s_yp[p] = R2<R>{q.x, q.y};
-            s_xi[p] = R2<R>{xi[p], xi[a.M + p]};
         } else {
             const double* q = a.yp + ((size_t)ch.x * a.M + p) * 2;
-            const double* xi = a.xi + (size_t)ch.x * 2 * a.M;
             s_yp[p] = R2<R>{R(q[0] - cl.C[0]), R(q[1] - cl.C[1])};
+        }
+    }
+    pdl_wait();
+    for (int p = t; p < a.M; p += kFinNodes) {
+        if constexpr (sizeof(R) == 4) {
+            const float* xi = a.xif + (size_t)ch.x * 2 * a.M;
+            s_xi[p] = R2<R>{xi[p], xi[a.M + p]};
+        } else {
+            const double* xi = a.xi + (size_t)ch.x * 2 * a.M;
             s_xi[p] = R2<R>{R(xi[p]), R(xi[a.M + p])};
         }
     }
+    const double F0 = a.bodyF[3 * b], F1 = a.bodyF[3 * b + 1], tq = a.bodyF[3 * b + 2];
     __syncthreads();
     // on-curve diagonal -(kappa / 2 pi) tau (tau . q), and the node's close pairs in order
-    auto own_terms = [&](int i, double n0, double n1, double2 sg, double& tx, double& ty) {
-        const double t0 = -n1, t1 = n0;
-        const double dg = -(a.kap[i] / (2.0 * kPi)) * (t0 * (sg.x * a.w[i]) + t1 * (sg.y * a.w[i]));
-        tx += dg * t0;
-        ty += dg * t1;
-        if (!a.use_pairs) return;
-        const int p1 = a.pair_base[i + 1];
-        for (int p = a.pair_base[i]; p < p1; ++p) {
+    auto own_terms = [&](double k, double w, double q0, double q1, double2 s, int pa, int pb, double& tx, double& ty) {
+        const double dg = -(k / (2.0 * kPi)) * (-q1 * (s.x * w) + q0 * (s.y * w));
+        tx -= dg * q1;
+        ty += dg * q0;
+        for (int p = pa; p < pb; ++p) {
             if constexpr (sizeof(R) == 4) {
                 const float2 v = reinterpret_cast<const float2*>(a.psum)[p];
                 tx += (double)v.x;
@@ -1150,35 +1178,29 @@ k_finish(Finish<R> a, double2* __restrict__ out) {
     };
     if (wid == 3) {  // T at the cell's first node
         double tx, ty;
-        finish_sum(a, cl, head, lane, 32, s_yp, s_xi, tx, ty);
+        R hx, hy, g0, g1;
+        place(head, hx, hy, g0, g1);
+        proxy_sum(a.M, lane, 32, s_yp, s_xi, hx, hy, g0, g1, tx, ty);
+        partial_sum(a, cl, head, lane, 32, tx, ty);
         for (int s = 16; s > 0; s >>= 1) {
             tx += __shfl_xor_sync(0xffffffffu, tx, s);
             ty += __shfl_xor_sync(0xffffffffu, ty, s);
         }
         if (lane == 0) {
-            own_terms(head, a.nx[head], a.ny[head], a.sigma[head], tx, ty);
+            own_terms(a.kap[head], a.w[head], h0, h1, a.sigma[head], a.use_pairs ? a.pair_base[head] : 0,
+                      a.use_pairs ? a.pair_base[head + 1] : 0, tx, ty);
             s_t0[0] = tx;
             s_t0[1] = ty;
         }
     }
-    const int i = i0 + t;
-    double tx = 0, ty = 0, n0 = 0, n1 = 0;
-    double2 sg = make_double2(0.0, 0.0);
-    if (i < i1) {
-        finish_sum(a, cl, i, 0, 1, s_yp, s_xi, tx, ty);
-        n0 = a.nx[i];
-        n1 = a.ny[i];
-        sg = a.sigma[i];
-        own_terms(i, n0, n1, sg, tx, ty);
-    }
+    double tx, ty;
+    proxy_sum(a.M, 0, 1, s_yp, s_xi, X, Y, m0, m1, tx, ty);
+    partial_sum(a, cl, i, 0, 1, tx, ty);
+    own_terms(ki, wi, n0, n1, sg, p0, p1, tx, ty);
     __syncthreads();
-    if (i >= i1) return;
-    const double al = -(s_t0[0] * a.nx[head] + s_t0[1] * a.ny[head]);
-    const int b = a.owner[i];
-    const double* bd = a.body + 8 * b;
-    const double tq = a.bodyF[3 * b + 2];
-    out[i] = make_double2(0.5 * sg.x + tx + al * n0 + a.bodyF[3 * b] - (a.y[i] - bd[3]) * tq,
-                          0.5 * sg.y + ty + al * n1 + a.bodyF[3 * b + 1] + (a.x[i] - bd[2]) * tq);
+    if (i0 + t >= i1) return;
+    const double al = -(s_t0[0] * h0 + s_t0[1] * h1);
+    out[i] = make_double2(0.5 * sg.x + tx + al * n0 + F0 - (yi - yc) * tq, 0.5 * sg.y + ty + al * n1 + F1 + (xi_ - xc) * tq);
 }
 
 template <typename R>
@@ -1188,6 +1210,7 @@ static int finish_launch(bie_ctx* c, const double* sigma, int prec, const Worksp
     a.prec = prec;
     a.M = c->M;
     a.use_pairs = c->cl.npairs > 0 ? 1 : 0;
+    a.single = c->fmm[prec].on ? 1 : 0;
     a.part = ws.part;
     a.yp = c->yp;
     a.ypf = c->ypf;
@@ -1209,8 +1232,8 @@ static int finish_launch(bie_ctx* c, const double* sigma, int prec, const Worksp
     a.body = c->body;
     a.bodyF = ws.bodyF;
     a.cells = c->cells;
-    k_finish<R><<<c->n_fin, kFinNodes, 0, c->stream>>>(a, reinterpret_cast<double2*>(yout));
-    BIE_LAUNCH(c, "k_finish");
+    BIE_CUDA(c, launch_after(fmm_chained(c, prec), k_finish<R>, c->n_fin, kFinNodes, c->stream, a, reinterpret_cast<double2*>(yout)));
+    ++c->launches;
     return BIE_OK;
 }
 

@@ -257,7 +257,7 @@ __host__ __device__ inline double2 fmm_centre(const FmmCell& f, int level, int i
 // parent delta^m and (1 / (2 delta))^k.
 template <typename R>
 struct FmmTab {
-    const R *hankel, *binom;
+    const R *hankel, *binom, *binomt;  // binomt: [k][m] = C(k, m)
     const C2<R>*dpow, *gpow;  // [quadrant][order]
 };
 
@@ -278,15 +278,64 @@ __device__ __forceinline__ C2<df> fmm_offset<df>(const FmmTree& t, int s, double
     return {df((p.x - c.x) * inv_h), df((p.y - c.y) * inv_h)};
 }
 
-// One CTA per leaf: gathers the strengths q = sigma w of the box's sources in
-// sorted order and sums their moments.  A warp takes 32 sources at a time; a
+// One CTA per box.  Boxes of at most kFmmDirect sources (every leaf) sum their
+// moments from the sources, rows of leaves at a time; a leaf's CTA also gathers
+// the strengths q = sigma w in sorted order.  A warp takes 32 sources at a time; a
 // lane sums three (order, group of sources) items, eta^k = eta^(k % 4)
-// (eta^4)^(k / 4) from two small tables per source.  The CTA of a parent's last
-// child forms the parent's moments, a warp per child, and so on up.
+// (eta^4)^(k / 4) from two small tables per source.  Larger boxes' moments come
+// from their children's, a warp per child, in the CTA of the last child to finish,
+// and so on up: each such level waits for the one below (some 3 us), which is why
+// only boxes too large to sum in that time do it (single precision; the double
+// sums cost more, so their line is lower).
+// The CTAs past the boxes form the bodies' moments (F_b, tau_b), one body each,
+// with the per-node records that velocities and the direct walls read.
+struct FmmBodies {
+    const double *x, *y, *body;
+    const int* body_cell;
+    float4* src32;   // cell-centred, or null
+    Src64* src64;    // or null
+    double* bodyF;
+};
+
+__device__ void fmm_body(const FmmBodies& p, int b, const Cell* cells, const double2* sigma, const double* w) {
+    __shared__ double red[33];
+    const double* bd = p.body + 8 * b;
+    const double xc = bd[2], yc = bd[3];
+    const int n = (int)bd[5], off = (int)bd[6];
+    const Cell& cl = cells[p.body_cell[b]];
+    double fx = 0, fy = 0, tq = 0;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        const int i = off + k;
+        const double2 sg = sigma[i];
+        const double wi = w[i], X = p.x[i], Y = p.y[i];
+        const double qx = sg.x * wi, qy = sg.y * wi;
+        fx += qx;
+        fy += qy;
+        tq += -(Y - yc) * qx + (X - xc) * qy;
+        if (p.src32) p.src32[i] = make_float4((float)(X - cl.C[0]), (float)(Y - cl.C[1]), (float)qx, (float)qy);
+        if (p.src64) p.src64[i] = Src64{X, Y, qx, qy};
+    }
+    fx = block_sum_d(fx, red);
+    fy = block_sum_d(fy, red);
+    tq = block_sum_d(tq, red);
+    if (threadIdx.x == 0) {
+        p.bodyF[3 * b] = fx;
+        p.bodyF[3 * b + 1] = fy;
+        p.bodyF[3 * b + 2] = tq;
+    }
+}
+
+// Measured (whole application, us): single precision at 6400 / 102400 nodes 64.4 /
+// 167 with 128, 67.1 / 170 with 512, 80.9 / 188 with 2048; double-float 270 / 1119
+// with 64, 262 / 1132 with 256, 278 / 1178 with 512.
+template <typename R>
+constexpr int kFmmDirect = sizeof(R) == 4 ? 128 : 256;
+
 template <typename R>
 __global__ void __launch_bounds__(128)
 k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ sigma, const double* __restrict__ w,
-         int shift, C2<R>* __restrict__ sq, V4<R>* __restrict__ mp, unsigned* __restrict__ ticket, FmmTab<R> tab) {
+         int shift, C2<R>* __restrict__ sq, V4<R>* __restrict__ mp, unsigned* __restrict__ ticket, FmmTab<R> tab,
+         FmmBodies bodies) {
     constexpr int P = FmmTypes<R>::P, G = kFmmItems / P, PER = 32 / G, HI = P / 4;
     struct Tables {
         C2<R> lo[4][4][33], hi[4][HI][33], q[4][32], s[4][32];
@@ -301,29 +350,46 @@ k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ 
     // children's translated series
     R* s_sum = reinterpret_cast<R*>(&sh);
     static_assert(4 * kFmmItems * 6 * sizeof(R) <= sizeof(Tables), "sums");
+    pdl_trigger();
+    if ((int)blockIdx.x >= t.nbox) {
+        fmm_body(bodies, blockIdx.x - t.nbox, cells, sigma, w);
+        return;
+    }
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    constexpr int kDirect = kFmmDirect<R>;
     const int b = blockIdx.x;
     int4 bx = t.box[b];
+    const int total = t.scount[b];
+    if (bx.y > 0 && total > kDirect) return;  // from its children
     const FmmCell& f = t.cells[bx.x];
     if (!cells[bx.x].active) return;
-    const int s0 = t.sstart[b], s1 = t.sstart[b + 1];
-    if (s1 > s0) {
-        const double2 c = sizeof(R) == 4 ? make_double2(0.0, 0.0) : fmm_centre(f, 0, fmm_ix(bx), fmm_iy(bx));
-        const float4 cf = t.centre[b];
+    const int lv0 = bx.y;
+    if (total > 0) {
+        const double2 c = sizeof(R) == 4 ? make_double2(0.0, 0.0) : fmm_centre(f, lv0, fmm_ix(bx), fmm_iy(bx));
+        const float4 cf = sizeof(R) == 4 ? t.centre[b] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const double inv_h = f.inv_h / (1 << lv0);
         // per item the moments of q_x and q_y and of s = q conj(eta)
         C2<R> X[3], Y[3], D[3];
 #pragma unroll
         for (int r = 0; r < 3; ++r) X[r] = Y[r] = D[r] = czero<R>();
-        for (int k0 = s0 + 32 * wid; k0 < s1; k0 += 128) {
+        // the rows of leaves in turn, chunks of 32 sources dealt to the warps
+        const int gx0 = f.gx[0], x0 = fmm_ix(bx) << lv0, x1 = min(gx0, x0 + (1 << lv0)), y0 = fmm_iy(bx) << lv0,
+                  y1 = min(f.gy[0], y0 + (1 << lv0)), off0 = f.off[0];
+        int turn = 0;
+        for (int y = y0; y < y1; ++y) {
+        const int s0 = t.sstart[off0 + y * gx0 + x0], s1 = t.sstart[off0 + y * gx0 + x1];
+        const int first = (wid - turn) & 3;
+        turn += (s1 - s0 + 31) >> 5;
+        for (int k0 = s0 + 32 * first; k0 < s1; k0 += 128) {
             const int s = k0 + lane, cnt = min(32, s1 - k0);
             C2<R> eta = czero<R>(), q = czero<R>();
             if (lane < cnt) {
-                eta = fmm_offset<R>(t, s, c, cf, f.inv_h);
+                eta = fmm_offset<R>(t, s, c, cf, inv_h);
                 const int i = t.sperm[s] >> shift;
                 const double2 sg = sigma[i];
                 const double wi = w[i];
                 q = {R(sg.x * wi), R(sg.y * wi)};
-                sq[s] = q;
+                if (lv0 == 0) sq[s] = q;
             }
             const C2<R> e2 = cmul(eta, eta), e4 = cmul(e2, e2);
             __syncwarp();
@@ -357,6 +423,7 @@ k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ 
                 }
             }
             __syncwarp();
+        }
         }
         __syncthreads();
         // the sums of 4 warps x G groups, in order; number n of order k at n P + k
@@ -394,8 +461,9 @@ k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ 
     // parents: the series translated from the four children, a warp each
     V4<R>* s_v = reinterpret_cast<V4<R>*>(&sh);  // [4][P] scaled, then [4][P] translated
     static_assert(8 * P * sizeof(V4<R>) <= sizeof(Tables), "series");
-    for (int level = 0; bx.w >= 0; ++level) {
+    for (int level = lv0; bx.w >= 0; ++level) {
         const int parent = bx.w;
+        if (t.scount[parent] <= kDirect) return;  // summed by its own CTA
         const int px = fmm_ix(t.box[parent]), py = fmm_iy(t.box[parent]);
         const int nx = min(2, f.gx[level] - 2 * px), ny = min(2, f.gy[level] - 2 * py);
         __threadfence();
@@ -406,7 +474,6 @@ k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ 
         __threadfence();
         if (tid == 0) ticket[parent] = 0u;
         bx = t.box[parent];
-        if (t.scount[parent] == 0) continue;
         const int jx = wid & 1, jy = wid >> 1;
         const int child = f.off[level] + (2 * py + jy) * f.gx[level] + 2 * px + jx;
         const bool have = jx < nx && jy < ny && t.scount[child] > 0;
@@ -430,7 +497,10 @@ k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ 
             __syncwarp();
             for (int m = lane; m < P; m += 32) {
                 V4<R> s = vzero<R>();
-                for (int k = 0; k <= m; ++k) axpy(s, tab.binom[(size_t)k * P + m], v[k]);  // C(m, k)
+                // C(m, k), 0 for k > m: whole rows keep the loads in flight
+                const int rows = m < 32 ? min(P, 32) : P;
+#pragma unroll 8
+                for (int k = 0; k < rows; ++k) axpy(s, tab.binom[(size_t)k * P + m], v[k]);
                 V4<R> r = vzero<R>();
                 add_scaled(r, tab.dpow[wid * P + m], s);
                 o[m] = r;
@@ -444,6 +514,209 @@ k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ 
             mp[(size_t)parent * P + tid] = vadd(vadd(q[0], q[P]), vadd(q[2 * P], q[3 * P]));
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// beside the translations: wall discrepancy and close pairs
+// ---------------------------------------------------------------------------
+// The wall discrepancy (Sec. 6.2 step 2, the far-image form of k_disc) from the
+// moments of the boxes of one level: the six far images of a wall point lie a
+// cell away from every box, so the series converge by 0.3 per order or better.
+// With u = 1 / W, W = (p - c) / H, per box
+//   velocity   4 pi mu u = -a_0 log|w| + (sum_{k>0} a_k u^k / k + conj(sum_{k>0} e_k u^k / k)
+//                          + conj(conj(W) A) + a_0) / 2,
+//   traction  -4 pi H T = 2 n Re A + conj(n (E - conj(W) A')).
+// The single-layer sum took 12 N (4 m) kernel evaluations with a logarithm
+// each: 3.5 ms of the FP64 pipe at 102400 nodes, 0.23 ms at 6400.
+// the sums' type: float, or double (double-float too)
+template <typename R>
+struct WallReal {
+    typedef double T;
+};
+template <>
+struct WallReal<float> {
+    typedef float T;
+};
+template <typename S, typename R>
+__device__ __forceinline__ S to_real(R a) {
+    return (S)to_double(a);
+}
+template <>
+__device__ __forceinline__ float to_real<float, float>(float a) {
+    return a;
+}
+
+template <typename R>
+__device__ __forceinline__ void wall_box(const V4<R>* mp, C2<R> W, typename WallReal<R>::T ln_w, R n0, R n1,
+                                         const R* inv_k, typename WallReal<R>::T* v) {
+    typedef typename WallReal<R>::T S;
+    constexpr int P = FmmTypes<R>::P;
+    const R s = rcp(fma_(W.x, W.x, W.y * W.y));
+    const C2<R> u{renorm(W.x * s), renorm(-(W.y * s))};
+    C2<R> A = czero<R>(), B = czero<R>(), E = czero<R>(), L = czero<R>(), M = czero<R>();
+    auto step = [&](C2<R>& a, R vx, R vy) {
+        a = {renorm(fma_(a.x, u.x, fma_(-a.y, u.y, vx))), renorm(fma_(a.x, u.y, fma_(a.y, u.x, vy)))};
+    };
+    for (int k = P - 1; k > 0; --k) {
+        const V4<R> m = mp[k];
+        const R k1(k + 1), ik = inv_k[k];
+        step(A, m.x, m.y);
+        step(B, k1 * m.x, k1 * m.y);
+        step(E, m.z, m.w);
+        step(L, ik * m.x, ik * m.y);
+        step(M, ik * m.z, ik * m.w);
+    }
+    const V4<R> m = mp[0];
+    step(A, m.x, m.y);
+    step(B, m.x, m.y);
+    step(E, m.z, m.w);
+    L = cmul(L, u);
+    M = cmul(M, u);
+    A = cmul(A, u);
+    E = cmul(E, u);
+    B = cmul(cmul(B, u), u);  // -A'
+    // F = E - conj(W) A'
+    const C2<R> F{E.x + fma_(W.x, B.x, W.y * B.y), E.y + fma_(W.x, B.y, -(W.y * B.x))};
+    // conj(conj(W) A) = W conj(A)
+    const R wx = fma_(W.x, A.x, W.y * A.y), wy = fma_(W.y, A.x, -(W.x * A.y));
+    v[0] = S(0.5) * to_real<S>(L.x + M.x + wx + m.x) - ln_w * to_real<S>(m.x);
+    v[1] = S(0.5) * to_real<S>(L.y - M.y + wy + m.y) - ln_w * to_real<S>(m.y);
+    v[2] = -to_real<S>(R(2) * n0 * A.x + (n0 * F.x - n1 * F.y));
+    v[3] = -to_real<S>(R(2) * n1 * A.x - (n0 * F.y + n1 * F.x));
+}
+constexpr int kWallImages = 6;
+
+// One warp per task: first (cell, wall point, far image), writing
+// gpart[((cell 7) + image) 8m + 4 wp + component]; then one per cell for its
+// total force (slot 6); then the close pairs (Sec. 6.3), C_p sigma into psum[p].
+struct SideArgs {
+    int ncell, m, walls, npairs, ctas;  // ctas: four tasks each
+    const double *wall, *bodyF;
+    double* gpart;
+    const int4* pairs;
+    const int* node_cell;
+    const long long* blk_off;
+    const void* blocks;  // float (single precision: on q = sigma w), or double
+    const double* body;
+    const double2* sigma;
+    const double* w;
+    void* psum;
+};
+
+// B: the blocks' type
+template <typename B>
+__device__ __forceinline__ void close_pair(const SideArgs& a, const Cell* cells, int p, int lane) {
+    const int4 pr = a.pairs[p];
+    if (!cells[a.node_cell[pr.x]].active) return;
+    const int n = (int)a.body[8 * pr.y + 5], off = (int)a.body[8 * pr.y + 6];
+    const B* C = reinterpret_cast<const B*>(a.blocks) + a.blk_off[p];
+    B bx = 0, by = 0;
+#pragma unroll 4
+    for (int j = lane; j < n; j += 32) {
+        const double2 sg = a.sigma[off + j];
+        B sx = (B)sg.x, sy = (B)sg.y;
+        if constexpr (sizeof(B) == 4) {
+            const float wj = (float)a.w[off + j];
+            sx *= wj;
+            sy *= wj;
+        }
+        const B c0 = C[3 * j], c1 = C[3 * j + 1], c2 = C[3 * j + 2];
+        bx = fma(c0, sx, fma(c1, sy, bx));
+        by = fma(c1, sx, fma(c2, sy, by));
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        bx += __shfl_xor_sync(0xffffffffu, bx, o);
+        by += __shfl_xor_sync(0xffffffffu, by, o);
+    }
+    if (lane) return;
+    if constexpr (sizeof(B) == 4) reinterpret_cast<float2*>(a.psum)[p] = make_float2(bx, by);
+    else reinterpret_cast<double2*>(a.psum)[p] = make_double2(bx, by);
+}
+
+template <typename B>
+__global__ void __launch_bounds__(128) k_close_pairs(SideArgs a, const Cell* __restrict__ cells) {
+    const int p = blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (p < a.npairs) close_pair<B>(a, cells, p, threadIdx.x & 31);
+}
+
+template <typename R>
+__device__ void side_tasks(const SideArgs& a, const FmmTree& t, const Cell* cells, const V4<R>* mp, int cta) {
+    constexpr int P = FmmTypes<R>::P;
+    typedef typename WallReal<R>::T S;
+    __shared__ R s_inv[P];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int task = cta * 4 + wid;
+    if (a.walls) {
+        for (int k = threadIdx.x; k < P; k += 128) s_inv[k] = R(k ? 1.0 / k : 0.0);
+        __syncthreads();
+        const int per = 2 * a.m * kWallImages + 1;
+        if (task < a.ncell * per) {
+            const int ci = task / per, q = task % per;
+            const Cell& cl = cells[ci];
+            if (!cl.active) return;
+            double* gp = a.gpart + (size_t)ci * 7 * 8 * a.m;
+            if (q == per - 1) {
+                double fx = 0, fy = 0;
+                for (int b = cl.body_off + lane; b < cl.body_off + cl.n_bodies; b += 32) {
+                    fx += a.bodyF[3 * b];
+                    fy += a.bodyF[3 * b + 1];
+                }
+                fx = warp_sum_d(fx);
+                fy = warp_sum_d(fy);
+                if (lane < 2) gp[6 * 8 * (size_t)a.m + lane] = lane ? fy : fx;
+                return;
+            }
+            const int wp = q / kWallImages, im = q % kWallImages;
+            const FmmCell& f = t.cells[ci];
+            const int lv = f.wall, gx = f.gx[lv], n = gx * f.gy[lv];
+            const double* wt = a.wall + ((size_t)ci * 2 * a.m + wp) * kWallStride;
+            S v[4] = {0, 0, 0, 0};
+            if constexpr (sizeof(R) == 4) {  // cell-centred single precision
+                const float* wf = reinterpret_cast<const float*>(wt + 16);
+                const float H = (float)f.h * (1 << lv), iH = 1.f / H;
+                const float px = wf[2 * im] - (float)f.ox, py = wf[2 * im + 1] - (float)f.oy, n0 = wf[12], n1 = wf[13];
+                const float lh = logf(H);
+                for (int e = lane; e < n; e += 32) {
+                    const int b = f.off[lv] + e;
+                    if (t.scount[b] == 0) continue;
+                    const C2<R> W{fmaf(px, iH, -(e % gx + 0.5f)), fmaf(py, iH, -(e / gx + 0.5f))};
+                    float o[4];
+                    wall_box<R>(mp + (size_t)b * P, W, 0.5f * logf(W.x * W.x + W.y * W.y) + lh, n0, n1, s_inv, o);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) v[k] += o[k];
+                }
+            } else {
+                const double H = f.h * (1 << lv), iH = f.inv_h / (1 << lv);
+                const double px = wt[2 * im] - cl.C[0] - f.ox, py = wt[2 * im + 1] - cl.C[1] - f.oy;
+                const double lh = log(H);
+                const R n0(wt[12]), n1(wt[13]);
+                for (int e = lane; e < n; e += 32) {
+                    const int b = f.off[lv] + e;
+                    if (t.scount[b] == 0) continue;
+                    const double wx = fma(px, iH, -(e % gx + 0.5)), wy = fma(py, iH, -(e / gx + 0.5));
+                    double o[4];
+                    wall_box<R>(mp + (size_t)b * P, C2<R>{R(wx), R(wy)}, 0.5 * log(wx * wx + wy * wy) + lh, n0, n1,
+                                s_inv, o);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) v[k] += o[k];
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+            if (lane < 4) {
+                const double sg = im < 3 ? 1.0 : -1.0;
+                const double g = lane < 2 ? sg / (4.0 * kPi * cl.mu) : sg * f.inv_h / (4.0 * kPi * (1 << lv));
+                gp[(size_t)im * 8 * a.m + 4 * wp + lane] =
+                    g * (double)(lane == 0 ? v[0] : (lane == 1 ? v[1] : (lane == 2 ? v[2] : v[3])));
+            }
+            return;
+        }
+        task -= a.ncell * per;
+    }
+    if (task >= a.npairs) return;
+    if constexpr (sizeof(R) == 4) close_pair<float>(a, cells, task, lane);
+    else close_pair<double>(a, cells, task, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -464,56 +737,81 @@ __device__ __forceinline__ bool fmm_close(int ix, int jx, int s, int level) {
 // the first of the (at most four) boxes near ix
 __device__ __forceinline__ int fmm_first(int ix, int s, int level) { return ix - 1 + ((-s) >> (kFmmBits + level)); }
 __device__ __forceinline__ int fmm_shift(double s, double inv_h) { return __double2int_rn(s * inv_h * (1 << kFmmBits)); }
-constexpr int kFmmList = 512;            // far boxes listed at a time
 constexpr int kFmmShares = 4;            // most CTAs a box's list is split over
 
-// One CTA per (target box of any level, share of its list).  Its threads scan
-// the candidate (box, image) pairs and compact the far ones into shared memory
-// in a fixed order; the warps translate them in turn.  Single precision: an
-// entry per warp and step, lane l holding order l and its row of the matrix.
-// Double: two entries per warp and step, three (entry, order) items per lane.
-// The shares' sums are separate (slot blockIdx.y of loc): without shares the
-// longest lists (90 boxes, at the coarse levels) held up the launch.
-template <typename R>
+// Near rows of a leaf's targets, compacted in (image, row) order by one warp.
+__device__ __forceinline__ int fmm_ranges(const FmmTree& t, const FmmCell& f, const int2* shift, int4 bx, int nimg,
+                                          FmmRange* out, int lane) {
+    int n = 0;
+    for (int q0 = 0; q0 < 4 * nimg; q0 += 32) {
+        const int q = q0 + lane;
+        FmmRange r{0, 0, 0};
+        if (q < 4 * nimg) {
+            r.im = nimg == 1 ? 4 : q >> 2;
+            const int sx = shift[r.im].x, sy = shift[r.im].y;
+            const int ix = fmm_ix(bx), iy = fmm_iy(bx);
+            const int jy = fmm_first(iy, sy, 0) + (q & 3);
+            if (fmm_close(iy, jy, sy, 0) && jy >= 0 && jy < f.gy[0]) {
+                int x0 = fmm_first(ix, sx, 0), x1 = x0 + 3;
+                if (!fmm_close(ix, x0, sx, 0)) ++x0;
+                if (!fmm_close(ix, x1, sx, 0)) --x1;
+                x0 = max(x0, 0);
+                x1 = min(x1, f.gx[0] - 1);
+                if (x0 <= x1) {
+                    const int row = f.off[0] + jy * f.gx[0];
+                    r.s0 = t.sstart[row + x0];
+                    r.s1 = t.sstart[row + x1 + 1];
+                }
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, r.s1 > r.s0);
+        if (r.s1 > r.s0) out[n + __popc(m & ((1u << lane) - 1))] = r;
+        n += __popc(m);
+    }
+    return n;
+}
+
+// Per geometry and box: the far boxes to translate from (box | image << 28, in a
+// fixed order; at most 9 images x 64 children of near parents, and 9 x 16 at the
+// top) and, for a leaf, its near rows (ranges of sorted records); per cell the
+// image shifts in leaf sides as float pairs.
 __global__ void __launch_bounds__(128)
-k_fmm_m2l(FmmTree t, const Cell* __restrict__ cells, int nimg, const V4<R>* __restrict__ mp, V4<R>* __restrict__ loc,
-          FmmTab<R> tab) {
-    constexpr int P = FmmTypes<R>::P;
-    constexpr bool F32 = sizeof(R) == 4;
-    constexpr int ENT = F32 ? 1 : 2, ITEMS = F32 ? 1 : 3;
-    __shared__ int2 s_far[kFmmList];  // box; offsets from it + 2^12 (13 bits each) and the image
+k_fmm_lists(FmmTree t, const Cell* __restrict__ cells, int nimg) {
     __shared__ int2 s_shift[9];
-    __shared__ C2<R> s_tab[4][F32 ? 32 : 16][kPowTab], s_z[4][F32 ? 32 : 16];
-    __shared__ V4<R> s_v[4][ENT][P + (F32 ? 0 : 1)];
     __shared__ int s_n[4];
     const int b = blockIdx.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int share = blockIdx.y, shares = gridDim.y;
-    if (t.tcount[b] == 0) return;
     const int4 bx = t.box[b];
     const FmmCell& f = t.cells[bx.x];
     const Cell& cl = cells[bx.x];
-    if (!cl.active) return;
     const int level = bx.y, ix = fmm_ix(bx), iy = fmm_iy(bx);
     const bool top = level == f.nlev - 1;
     const int gx = f.gx[level], gy = f.gy[level], off = f.off[level];
-    const int per = top ? gx * gy : 64;
-    if (threadIdx.x < 9)
-        s_shift[threadIdx.x] = make_int2(fmm_shift(cl.sx[threadIdx.x], f.inv_h), fmm_shift(cl.sy[threadIdx.x], f.inv_h));
-    __syncthreads();
-    V4<R> acc[ITEMS];
-#pragma unroll
-    for (int r = 0; r < ITEMS; ++r) acc[r] = vzero<R>();
-    R row[F32 ? P : 1];  // single precision: lane l's row of the matrix in registers
-    if constexpr (F32) {
-#pragma unroll
-        for (int k = 0; k < P; ++k) row[k] = lane < P ? tab.hankel[(size_t)k * P + lane] : R(0);
+    if (threadIdx.x < 9) {
+        const double sx = cl.sx[threadIdx.x], sy = cl.sy[threadIdx.x];
+        s_shift[threadIdx.x] = make_int2(fmm_shift(sx, f.inv_h), fmm_shift(sy, f.inv_h));
+        if (top && ix == 0 && iy == 0) {
+            float4 v;
+            split_df(sx * f.inv_h, v.x, v.y);
+            split_df(sy * f.inv_h, v.z, v.w);
+            t.shift[9 * bx.x + threadIdx.x] = v;
+        }
     }
-    int listed = 0;  // far boxes of all shares since the last translation
-    const int ncand = per * nimg;
+    __syncthreads();
+    if (t.tcount[b] == 0) {
+        if (threadIdx.x == 0) t.nfar[b] = 0;
+        if (threadIdx.x == 0 && level == 0) t.nnear[b] = 0;
+        return;
+    }
+    if (level == 0 && wid == 0) {
+        const int n = fmm_ranges(t, f, s_shift, bx, nimg, t.near + (size_t)b * kFmmRanges, lane);
+        if (lane == 0) t.nnear[b] = n;
+    }
+    const int per = top ? gx * gy : 64, ncand = per * nimg;
+    int listed = 0;
     for (int q0 = 0; q0 < ncand; q0 += 128) {
         const int q = q0 + threadIdx.x;
         bool far = false;
-        int2 entry2 = make_int2(0, 0);
+        int entry = 0;
         if (q < ncand) {
             const int im = nimg == 1 ? 4 : q / per, e = nimg == 1 ? q : q % per;
             const int2 sh = s_shift[im];
@@ -534,25 +832,67 @@ k_fmm_m2l(FmmTree t, const Cell* __restrict__ cells, int nimg, const V4<R>* __re
             if (ok && jx >= 0 && jx < gx && jy >= 0 && jy < gy) {
                 const int src = off + jy * gx + jx;
                 far = !(fmm_close(ix, jx, sh.x, level) && fmm_close(iy, jy, sh.y, level)) && t.scount[src] > 0;
-                entry2 = make_int2(src, (ix - jx + 4096) | ((iy - jy + 4096) << 13) | (im << 26));
+                entry = src | (im << 28);
             }
         }
         const unsigned m = __ballot_sync(0xffffffffu, far);
         if (lane == 0) s_n[wid] = __popc(m);
         __syncthreads();
-        int at = listed, all = listed;
+        int at = listed;
         for (int k = 0; k < 4; ++k) {
             if (k < wid) at += s_n[k];
-            all += s_n[k];
+            listed += s_n[k];
         }
-        at += __popc(m & ((1u << lane) - 1));
-        if (far && at % shares == share) {
-            s_far[at / shares] = entry2;
-        }
+        if (far) t.far[(size_t)b * kFmmFar + at + __popc(m & ((1u << lane) - 1))] = entry;
         __syncthreads();
-        listed = all;
-        if (listed <= kFmmList - 128 && q0 + 128 < ncand) continue;
-        const int mine = (listed - share + shares - 1) / shares;  // this share's entries
+    }
+    if (threadIdx.x == 0) t.nfar[b] = listed;
+}
+
+// The first CTAs take the side tasks above.  Then one CTA per (target box of any
+// level, share of its list): its warps translate the listed boxes in turn.
+// Single precision: an entry per warp and step, lane l holding order l and its
+// row of the matrix.  Double: two entries per warp and step, three (entry, order)
+// items per lane.  The shares' sums are separate (one slot of loc each): without
+// shares the longest lists (90 boxes, at the coarse levels) held up the launch.
+template <typename R>
+__global__ void __launch_bounds__(128)
+k_fmm_m2l(FmmTree t, const Cell* cells, int nimg, const V4<R>* mp, V4<R>* loc, FmmTab<R> tab, int shares,
+          SideArgs side) {
+    constexpr int P = FmmTypes<R>::P;
+    constexpr bool F32 = sizeof(R) == 4;
+    constexpr int ENT = F32 ? 1 : 2, ITEMS = F32 ? 1 : 3;
+    __shared__ C2<R> s_tab[4][F32 ? 32 : 16][kPowTab], s_z[4][F32 ? 32 : 16];
+    __shared__ V4<R> s_v[4][ENT][P + (F32 ? 0 : 1)];
+    __shared__ int s_src[4][F32 ? 32 : 16];
+    if ((int)blockIdx.x < side.ctas) {
+        pdl_wait();
+        pdl_trigger();
+        side_tasks<R>(side, t, cells, mp, blockIdx.x);
+        return;
+    }
+    const int id = blockIdx.x - side.ctas, b = id / shares, share = id % shares;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int4 bx = t.box[b];
+    const Cell& cl = cells[bx.x];
+    if (t.tcount[b] == 0 || !cl.active) {
+        pdl_wait();
+        return;
+    }
+    const int4 grid = t.grid[b];  // (first box of the level, its width, ...)
+    const int* far = t.far + (size_t)b * kFmmFar;
+    const int mine = (t.nfar[b] - share + shares - 1) / shares;  // this share's entries
+    const int level = bx.y, ix = fmm_ix(bx), iy = fmm_iy(bx), off = grid.x, gx = grid.y;
+    V4<R> acc[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) acc[r] = vzero<R>();
+    R row[F32 ? P : 1];  // single precision: lane l's row of the matrix in registers
+    if constexpr (F32) {
+#pragma unroll
+        for (int k = 0; k < P; ++k) row[k] = lane < P ? tab.hankel[(size_t)k * P + lane] : R(0);
+    }
+    if (mine <= 0) pdl_wait();
+    {
         constexpr int GRP = F32 ? 32 : 16;  // entries whose power tables a warp holds
         for (int g0 = 0; g0 * 4 < mine; g0 += GRP) {
             // the warp's entries of this group: e = (g0 + n) 4 + wid (single), or
@@ -562,31 +902,42 @@ k_fmm_m2l(FmmTree t, const Cell* __restrict__ cells, int nimg, const V4<R>* __re
             __syncwarp();
             if (lane < GRP && entry(lane) < mine) {
                 // target centre minus source centre in sides, its inverse's powers
-                const int at2 = s_far[entry(lane)].y;
-                const double inv = f.inv_h / (1 << level);
-                const double x = (double)((at2 & 8191) - 4096) - cl.sx[at2 >> 26] * inv;
-                const double y = (double)(((at2 >> 13) & 8191) - 4096) - cl.sy[at2 >> 26] * inv;
-                s_z[wid][lane] = {R(x), R(y)};
+                const int v = far[entry(lane) * shares + share], src = v & 0xfffffff, im = (unsigned)v >> 28;
+                const int jy = (src - off) / gx, jx = src - off - jy * gx;
+                s_src[wid][lane] = src;
+                const float4 sh = t.shift[9 * bx.x + im];  // leaf sides
+                R x, y;
+                if constexpr (F32) {
+                    const float iu = 1.f / (1 << level);
+                    x = (((float)((ix - jx) << level) - sh.x) - sh.y) * iu;
+                    y = (((float)((iy - jy) << level) - sh.z) - sh.w) * iu;
+                } else {
+                    const double inv = t.cells[bx.x].inv_h / (1 << level);
+                    x = R((ix - jx) - cl.sx[im] * inv);
+                    y = R((iy - jy) - cl.sy[im] * inv);
+                }
+                s_z[wid][lane] = {x, y};
                 C2<R> u;
                 if constexpr (F32) {
-                    const float fx = (float)x, fy = (float)y, sc = 1.f / (fx * fx + fy * fy);
-                    u = {fx * sc, -fy * sc};
+                    const float sc = 1.f / (x * x + y * y);
+                    u = {x * sc, -y * sc};
                 } else {
-                    const double sc = rcp64(x * x + y * y);
-                    u = {R(x * sc), R(-y * sc)};
+                    const double dx = to_double(x), dy = to_double(y), sc = rcp64(dx * dx + dy * dy);
+                    u = {R(dx * sc), R(-dy * sc)};
                 }
                 pow_table(u, s_tab[wid][lane]);
             }
             __syncwarp();
+            pdl_wait();
+            pdl_trigger();
             if constexpr (F32) {
                 V4<R> nxt = vzero<R>();
-                const int e0 = entry(0);
-                if (e0 < mine && lane < P) nxt = mp[(size_t)s_far[e0].x * P + lane];
+                if (entry(0) < mine && lane < P) nxt = mp[(size_t)s_src[wid][0] * P + lane];
                 for (int n = 0; n < GRP && entry(n) < mine; ++n) {
                     const C2<R> z = s_z[wid][n];
                     const V4<R> m4 = nxt;
                     const int en = entry(n + 1);
-                    if (n + 1 < GRP && en < mine && lane < P) nxt = mp[(size_t)s_far[en].x * P + lane];
+                    if (n + 1 < GRP && en < mine && lane < P) nxt = mp[(size_t)s_src[wid][n + 1] * P + lane];
                     const C2<R> u = s_tab[wid][n][0];
                     C2<R> pw = pow_at(s_tab[wid][n], lane);
                     C2<R> pa{__shfl_up_sync(0xffffffffu, m4.x, 1), __shfl_up_sync(0xffffffffu, m4.y, 1)};
@@ -613,7 +964,7 @@ k_fmm_m2l(FmmTree t, const Cell* __restrict__ cells, int nimg, const V4<R>* __re
                         V4<R> v = vzero<R>();
                         pw[r] = czero<R>();
                         if (e < mine) {
-                            const V4<R>* src4 = mp + (size_t)s_far[e].x * P + k;
+                            const V4<R>* src4 = mp + (size_t)s_src[wid][n + en] * P + k;
                             const V4<R> m4 = *src4;
                             C2<R> ev{m4.z, m4.w};
                             if (k) {
@@ -647,8 +998,6 @@ k_fmm_m2l(FmmTree t, const Cell* __restrict__ cells, int nimg, const V4<R>* __re
                 }
             }
         }
-        listed = 0;
-        __syncthreads();
     }
     // the warps' sums, in order
     V4<R>* flat = &s_v[wid][0][0];
@@ -672,13 +1021,6 @@ k_fmm_m2l(FmmTree t, const Cell* __restrict__ cells, int nimg, const V4<R>* __re
 // down: at every target, the ancestors' expansions moved to its leaf and the
 // near boxes pair by pair
 // ---------------------------------------------------------------------------
-// The sources of a near row of boxes are contiguous: a range of sorted records
-// under one image shift.
-struct FmmRange {
-    int s0, s1, im;
-};
-constexpr int kFmmRanges = 36;  // 9 images x 4 rows
-
 // The local expansion of a leaf with its ancestors' moved to its centre, in
 // s_l[0] (the shares of k_fmm_m2l added on the way): warp w moves levels w,
 // w + 4, ... (level 0 is the leaf's own); every thread of the 128 takes part.
@@ -735,7 +1077,9 @@ __device__ __forceinline__ void fmm_local_to_leaf(const FmmTree& t, const FmmCel
             const int m = lane + 32 * r;
             if (m < P) {
                 V4<R> s = vzero<R>();
-                for (int l = m; l < P; ++l) axpy(s, tab.binom[(size_t)m * P + l], s_v[l]);  // C(l, m)
+                // C(l, m), 0 for l < m: whole rows keep the loads in flight
+#pragma unroll 8
+                for (int l = r ? 32 : 0; l < P; ++l) axpy(s, tab.binomt[(size_t)l * P + m], s_v[l]);
                 // to the leaf's unit: 2^-level per order and one more for the field's own scale
                 C2<R> p = pow_at(pg, m);
                 p = {p.x * R(u), p.y * R(u)};
@@ -790,91 +1134,118 @@ __device__ __forceinline__ C2<R> fmm_local_at(const V4<R>* c, C2<R> W, int r, R 
     return {-(R(2) * nx * A.x + nx * F.x - ny * F.y), -(R(2) * ny * A.x - (nx * F.y + ny * F.x))};
 }
 
-// Near rows of a leaf's targets, compacted in (image, row) order by warp 0.
-__device__ __forceinline__ int fmm_ranges(const FmmTree& t, const FmmCell& f, const Cell& cl, int4 bx, int nimg,
-                                          FmmRange* out, int lane) {
-    int n = 0;
-    for (int q0 = 0; q0 < 4 * nimg; q0 += 32) {
-        const int q = q0 + lane;
-        FmmRange r{0, 0, 0};
-        if (q < 4 * nimg) {
-            r.im = nimg == 1 ? 4 : q >> 2;
-            const int sx = fmm_shift(cl.sx[r.im], f.inv_h), sy = fmm_shift(cl.sy[r.im], f.inv_h);
-            const int ix = fmm_ix(bx), iy = fmm_iy(bx);
-            const int jy = fmm_first(iy, sy, 0) + (q & 3);
-            if (fmm_close(iy, jy, sy, 0) && jy >= 0 && jy < f.gy[0]) {
-                int x0 = fmm_first(ix, sx, 0), x1 = x0 + 3;
-                if (!fmm_close(ix, x0, sx, 0)) ++x0;
-                if (!fmm_close(ix, x1, sx, 0)) --x1;
-                x0 = max(x0, 0);
-                x1 = min(x1, f.gx[0] - 1);
-                if (x0 <= x1) {
-                    const int row = f.off[0] + jy * f.gx[0];
-                    r.s0 = t.sstart[row + x0];
-                    r.s1 = t.sstart[row + x1 + 1];
-                }
-            }
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, r.s1 > r.s0);
-        if (r.s1 > r.s0) out[n + __popc(m & ((1u << lane) - 1))] = r;
-        n += __popc(m);
+// xi = P g~ (Sec. 6.2 step 3) by the CTAs in front of the leaves', four rows of P
+// each: the CTA gathers g~ = g0 - g from the far images' parts (side_tasks), a
+// warp takes a row by compensated products and sums (Ogita, Rump & Oishi's
+// Dot2, as k_xi, which says why).
+struct XiArgs {
+    int m, M, ctas, per_cell;  // ctas in all, per cell
+    const double *gpart, *P;
+    double* xi;
+    float* xif;
+};
+__device__ void xi_rows(const XiArgs& a, const Cell* cells, int cta) {
+    __shared__ double d[8 * kMaxColl];
+    const int ci = cta / a.per_cell, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int r = (cta % a.per_cell) * 4 + wid, nv = 8 * a.m;
+    const Cell& cl = cells[ci];
+    if (!cl.active) return;
+    const double* gp = a.gpart + (size_t)ci * 7 * nv;
+    for (int cc = threadIdx.x; cc < nv; cc += 128) {
+        const bool L = cc < 4 * a.m;
+        const int k = (cc % (4 * a.m)) / a.m, wp = (L ? 0 : a.m) + cc % a.m;
+        double g = 0;
+#pragma unroll
+        for (int im = 0; im < kWallImages; ++im) g += gp[(size_t)im * nv + 4 * wp + k];
+        d[cc] = (k < 2 ? 0.0 : gp[kWallImages * (size_t)nv + k - 2] / (2.0 * (L ? cl.l2 : cl.l1))) - g;
     }
-    return n;
+    __syncthreads();
+    if (r >= 2 * a.M) return;
+    const double* P = a.P + ((size_t)ci * 2 * a.M + r) * nv;
+    double s = 0, e = 0;
+    for (int cc = lane; cc < nv; cc += 32) {
+        const double x = P[cc], y = d[cc], p = x * y, pe = fma(x, y, -p), u = s + p, z = u - s;
+        e += pe + ((s - (u - z)) + (p - z));
+        s = u;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const double s2 = __shfl_xor_sync(0xffffffffu, s, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
+        const double u = s + s2, z = u - s;
+        e = e + e2 + ((s - (u - z)) + (s2 - z));
+        s = u;
+    }
+    if (lane == 0) {
+        a.xi[(size_t)ci * 2 * a.M + r] = s + e;
+        a.xif[(size_t)ci * 2 * a.M + r] = (float)(s + e);
+    }
 }
 
-// Single precision.  One CTA per (leaf, tile share): four warps share the
-// tile's 64 targets (two per lane) and split the near sources; the double-
-// float positions make every difference exact to single precision, so no
+// Lanes per target of a tile of n <= 32 targets: a short tile's spare lanes take
+// every g-th source (leaves hold some 10 to 60 targets, so half the lanes would
+// otherwise idle).
+__device__ __forceinline__ int fmm_split(int n) { return n > 16 ? 1 : (n > 8 ? 2 : (n > 4 ? 4 : 8)); }
+
+// Single precision.  One CTA per (leaf, tile share): four warps share a tile of 64
+// targets, two per lane (a source read from shared memory then serves two pairs:
+// 72 us against 83 with one target per lane at 102400 nodes), and split the near
+// sources; a tile of at most 32 splits them over its spare lanes too.  The
+// double-float positions make every difference exact to single precision, so no
 // later pass has to redo near pairs.
 __global__ void __launch_bounds__(128, 6)
-k_fmm_down32(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<float>* __restrict__ sq,
-             const V4<float>* __restrict__ loc, int shares, FmmTab<float> tab, const float4* __restrict__ tgt32,
-             int n0, int n1, float2* __restrict__ part) {
+k_fmm_down32(FmmTree t, const Cell* cells, int nimg, const C2<float>* sq, const V4<float>* loc, int shares, FmmTab<float> tab, const float4* __restrict__ tgt32,
+             int n0, int n1, float2* __restrict__ part, XiArgs xi, int tiles) {
     constexpr int P = kFmmP32;
     __shared__ V4<float> s_l[4][P];
     __shared__ C2<float> s_pw[4][2][kPowTab];
-    __shared__ FmmRange s_r[kFmmRanges];
-    __shared__ int s_nr;
     __shared__ float4 s_p[4][32];
     __shared__ float2 s_q[4][32];
     __shared__ float2 s_acc[4][64];
-    const int b = blockIdx.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if ((int)blockIdx.x < xi.ctas) {
+        pdl_wait();
+        pdl_trigger();
+        xi_rows(xi, cells, blockIdx.x);
+        return;
+    }
+    const int id = blockIdx.x - xi.ctas, b = id / tiles, tile = id % tiles;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t0 = t.tstart[b], t1 = t.tstart[b + 1];
-    if (t0 + 64 * (int)blockIdx.y >= t1) return;
     const int4 bx = t.box[b];
     const FmmCell& f = t.cells[bx.x];
     const Cell& cl = cells[bx.x];
-    if (!cl.active) return;
-    if (wid == 0) {
-        const int n = fmm_ranges(t, f, cl, bx, nimg, s_r, lane);
-        if (lane == 0) s_nr = n;
+    if (t0 + 64 * tile >= t1 || !cl.active) {
+        pdl_wait();
+        return;
     }
-    fmm_local_to_leaf<float>(t, f, bx, loc, shares, tab, s_l, s_pw, wid, lane);
-    const int nr = s_nr;
+    const FmmRange* near = t.near + (size_t)b * kFmmRanges;
+    const int nr = t.nnear[b];
     const float4 cf = t.centre[b];
     const float inv_h = (float)f.inv_h;
-    for (int k0 = t0 + 64 * blockIdx.y; k0 < t1; k0 += 64 * gridDim.y) {
-        const bool two = t1 - k0 > 32;  // uniform: the second target of every lane
+    pdl_wait();
+    pdl_trigger();
+    fmm_local_to_leaf<float>(t, f, bx, loc, shares, tab, s_l, s_pw, wid, lane);
+    for (int k0 = t0 + 64 * tile; k0 < t1; k0 += 64 * tiles) {
+        const int n = min(64, t1 - k0);
+        const bool two = n > 32;
+        const int g = two ? 1 : fmm_split(n), per = 32 / g, sub = lane / per;
         float4 p[2];
         float nx[2], ny[2], ax[2] = {0.f, 0.f}, ay[2] = {0.f, 0.f};
-        int node[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            const int k = k0 + lane + 32 * q;
-            node[q] = k < t1 ? t.tperm[k] : -1;
-            if (node[q] >= 0 && (node[q] < n0 || node[q] >= n1) && node[q] != cl.node_off) node[q] = -1;
+            const int k = k0 + lane % per + 32 * q;
+            int node = k < t1 && (q == 0 || two) ? t.tperm[k] : -1;
+            if (node >= 0 && (node < n0 || node >= n1) && node != cl.node_off) node = -1;
             p[q] = make_float4(1e4f, 0.f, 1e4f, 0.f);
             nx[q] = ny[q] = 0.f;
-            if (node[q] >= 0) {
+            if (node >= 0) {
                 p[q] = t.tpos[k];
-                const float4 tv = tgt32[node[q]];
+                const float4 tv = tgt32[node];
                 nx[q] = tv.z;
                 ny[q] = tv.w;
             }
         }
         int turn = 0;
         for (int r = 0; r < nr; ++r) {
-            const FmmRange rg = s_r[r];
+            const FmmRange rg = near[r];
             const int chunks = (rg.s1 - rg.s0 + 31) >> 5;
             const int first = (wid - turn) & 3;
             turn += chunks;
@@ -910,30 +1281,33 @@ k_fmm_down32(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<float
                     }
                 } else {
 #pragma unroll 4
-                    for (int j = 0; j < cnt; ++j) pair(0, s_p[wid][j], s_q[wid][j]);
+                    for (int j = sub; j < cnt; j += g) pair(0, s_p[wid][j], s_q[wid][j]);
                 }
             }
         }
-        __syncthreads();
+        for (int o = per; o < 32; o <<= 1) {
+            ax[0] += __shfl_xor_sync(0xffffffffu, ax[0], o);
+            ay[0] += __shfl_xor_sync(0xffffffffu, ay[0], o);
+        }
+        __syncthreads();  // the previous tile's sums have been read
         s_acc[wid][lane] = make_float2(ax[0], ay[0]);
         s_acc[wid][lane + 32] = make_float2(ax[1], ay[1]);
         __syncthreads();
-        if (wid < 2) {  // warp 0 finishes the first 32 targets, warp 1 the others
-            const int nd = wid ? node[1] : node[0];
-            const float4 pt = wid ? p[1] : p[0];
-            if (nd >= 0) {
-                float sx = 0.f, sy = 0.f;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    sx += s_acc[q][lane + 32 * wid].x;
-                    sy += s_acc[q][lane + 32 * wid].y;
-                }
-                const C2<float> W = fmm_local(pt, cf, inv_h);
-                const C2<float> F = fmm_local_at<float, 1>(s_l[0], W, 0, wid ? nx[1] : nx[0], wid ? ny[1] : ny[0]);
-                const float g = (float)(1.0 / (4.0 * kPi)) * inv_h, cp = (float)(-1.0 / kPi);
-                part[cl.part_off[0] + (nd - cl.node_off)] = make_float2(fmaf(cp, sx, g * F.x), fmaf(cp, sy, g * F.y));
-            }
+        // two lanes per target split the local expansion and the warps' sums
+        const int q = threadIdx.x >> 1, res = threadIdx.x & 1, kq = k0 + q;
+        int nd = q < n ? t.tperm[kq] : -1;
+        if (nd >= 0 && (nd < n0 || nd >= n1) && nd != cl.node_off) nd = -1;
+        float fx = 0.f, fy = 0.f;
+        if (nd >= 0) {
+            const float4 tv = tgt32[nd];
+            const C2<float> F = fmm_local_at<float, 2>(s_l[0], fmm_local(t.tpos[kq], cf, inv_h), res, tv.z, tv.w);
+            const float gl = (float)(1.0 / (4.0 * kPi)) * inv_h, cp = (float)(-1.0 / kPi);
+            fx = fmaf(cp, s_acc[res][q].x + s_acc[res + 2][q].x, gl * F.x);
+            fy = fmaf(cp, s_acc[res][q].y + s_acc[res + 2][q].y, gl * F.y);
         }
+        fx += __shfl_xor_sync(0xffffffffu, fx, 1);
+        fy += __shfl_xor_sync(0xffffffffu, fy, 1);
+        if (nd >= 0 && res == 0) part[cl.part_off[0] + (nd - cl.node_off)] = make_float2(fx, fy);
     }
 }
 
@@ -942,34 +1316,40 @@ k_fmm_down32(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<float
 // the near sources, then four lanes per target split the local expansion.
 template <typename R>
 __global__ void __launch_bounds__(128, 4)
-k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<R>* __restrict__ sq,
-             const V4<R>* __restrict__ loc, int shares, FmmTab<R> tab, const double* __restrict__ nxv,
-             const double* __restrict__ nyv, int prec, int n0, int n1, double2* __restrict__ part) {
+k_fmm_down64(FmmTree t, const Cell* cells, int nimg, const C2<R>* sq, const V4<R>* loc, int shares, FmmTab<R> tab, const double* __restrict__ nxv,
+             const double* __restrict__ nyv, int prec, int n0, int n1, double2* __restrict__ part,
+             XiArgs xi, int tiles) {
     constexpr int P = FmmTypes<R>::P;
     constexpr bool DF = std::is_same<R, df>::value;
     __shared__ V4<R> s_l[4][P];
     __shared__ C2<R> s_pw[4][2][kPowTab];
-    __shared__ FmmRange s_r[kFmmRanges];
-    __shared__ int s_nr;
     __shared__ double2 s_p[4][32], s_q[4][32];  // double-float: a float4 each
     __shared__ double2 s_acc[4][32], s_t[32], s_n[32];
     __shared__ int s_node[32];
-    const int b = blockIdx.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if ((int)blockIdx.x < xi.ctas) {
+        pdl_wait();
+        pdl_trigger();
+        xi_rows(xi, cells, blockIdx.x);
+        return;
+    }
+    const int id = blockIdx.x - xi.ctas, b = id / tiles, tile = id % tiles;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t0 = t.tstart[b], t1 = t.tstart[b + 1];
-    if (t0 + 32 * (int)blockIdx.y >= t1) return;
     const int4 bx = t.box[b];
     const FmmCell& f = t.cells[bx.x];
     const Cell& cl = cells[bx.x];
-    if (!cl.active) return;
-    if (wid == 0) {
-        const int n = fmm_ranges(t, f, cl, bx, nimg, s_r, lane);
-        if (lane == 0) s_nr = n;
+    if (t0 + 32 * tile >= t1 || !cl.active) {
+        pdl_wait();
+        return;
     }
+    const FmmRange* near = t.near + (size_t)b * kFmmRanges;
+    const int nr = t.nnear[b];
+    pdl_wait();
+    pdl_trigger();
     fmm_local_to_leaf<R>(t, f, bx, loc, shares, tab, s_l, s_pw, wid, lane);
-    const int nr = s_nr;
     const double2 c = fmm_centre(f, 0, fmm_ix(bx), fmm_iy(bx));
-    for (int k0 = t0 + 32 * blockIdx.y; k0 < t1; k0 += 32 * gridDim.y) {
-        const int k = k0 + lane;
+    for (int k0 = t0 + 32 * tile; k0 < t1; k0 += 32 * tiles) {
+        const int n = min(32, t1 - k0), g = fmm_split(n), per = 32 / g, sub = lane / per, k = k0 + lane % per;
         int node = k < t1 ? t.tperm[k] : -1;
         if (node >= 0 && (node < n0 || node >= n1) && node != cl.node_off) node = -1;
         double2 p = make_double2(1e4, 1e4);
@@ -987,7 +1367,7 @@ k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<R>* _
         double ax = 0, ay = 0;
         int turn = 0;
         for (int r = 0; r < nr; ++r) {
-            const FmmRange rg = s_r[r];
+            const FmmRange rg = near[r];
             const int chunks = (rg.s1 - rg.s0 + 31) >> 5;
             const int first = (wid - turn) & 3;
             turn += chunks;
@@ -1016,7 +1396,7 @@ k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<R>* _
                     // double after every chunk
                     float axh = 0, axe = 0, ayh = 0, aye = 0;
 #pragma unroll 2
-                    for (int j = 0; j < cnt; ++j) {
+                    for (int j = sub; j < cnt; j += g) {
                         const float4 sp = *reinterpret_cast<const float4*>(&s_p[wid][j]);
                         const float4 ss = *reinterpret_cast<const float4*>(&s_q[wid][j]);
                         pair_df(pxh, pxl, pyh, pyl, nxh, nxl, nyh, nyl,
@@ -1026,7 +1406,7 @@ k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<R>* _
                     ay += (double)ayh + (double)aye;
                 } else {
 #pragma unroll 2
-                    for (int j = 0; j < cnt; ++j) {
+                    for (int j = sub; j < cnt; j += g) {
                         const double2 sp = s_p[wid][j], ss = s_q[wid][j];
                         const double dx = px - sp.x, dy = py - sp.y;
                         const double inv = rcp64(fma(dx, dx, fma(dy, dy, 1e-300)));
@@ -1038,12 +1418,16 @@ k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<R>* _
                 }
             }
         }
+        for (int o = per; o < 32; o <<= 1) {
+            ax += __shfl_xor_sync(0xffffffffu, ax, o);
+            ay += __shfl_xor_sync(0xffffffffu, ay, o);
+        }
         __syncthreads();  // also: the previous tile's targets have been read
         s_acc[wid][lane] = make_double2(ax, ay);
         if (wid == 0) {
             s_t[lane] = make_double2((p.x - c.x) * f.inv_h, (p.y - c.y) * f.inv_h);
             s_n[lane] = make_double2(nx, ny);
-            s_node[lane] = node;
+            s_node[lane] = lane < per ? node : -1;
         }
         __syncthreads();
         const int q = threadIdx.x >> 2, res = threadIdx.x & 3, nd = s_node[q];
@@ -1060,150 +1444,6 @@ k_fmm_down64(FmmTree t, const Cell* __restrict__ cells, int nimg, const C2<R>* _
         fx += __shfl_xor_sync(0xffffffffu, fx, 2);
         fy += __shfl_xor_sync(0xffffffffu, fy, 2);
         if (nd >= 0 && res == 0) part[cl.part_off[prec] + (nd - cl.node_off)] = make_double2(fx, fy);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// beside the sum (auxiliary stream): wall discrepancy and close pairs
-// ---------------------------------------------------------------------------
-// The wall discrepancy (Sec. 6.2 step 2, the far-image form of k_disc) from the
-// moments of the boxes of one level: the six far images of a wall point lie a
-// cell away from every box, so the series converge by 0.3 per order or better.
-// With u = 1 / W, W = (p - c) / H, per box
-//   velocity   4 pi mu u = -a_0 log|w| + (sum_{k>0} a_k u^k / k + conj(sum_{k>0} e_k u^k / k)
-//                          + conj(conj(W) A) + a_0) / 2,
-//   traction  -4 pi H T = 2 n Re A + conj(n (E - conj(W) A')).
-// The single-layer sum took 12 N (4 m) kernel evaluations with a logarithm
-// each: 3.5 ms of the FP64 pipe at 102400 nodes, 0.23 ms at 6400.
-template <typename R>
-__device__ __forceinline__ void wall_box(const V4<R>* mp, C2<R> W, double ln_w, R n0, R n1, const R* inv_k, double* v) {
-    constexpr int P = FmmTypes<R>::P;
-    const R s = rcp(fma_(W.x, W.x, W.y * W.y));
-    const C2<R> u{renorm(W.x * s), renorm(-(W.y * s))};
-    C2<R> A = czero<R>(), B = czero<R>(), E = czero<R>(), L = czero<R>(), M = czero<R>();
-    auto step = [&](C2<R>& a, R vx, R vy) {
-        a = {renorm(fma_(a.x, u.x, fma_(-a.y, u.y, vx))), renorm(fma_(a.x, u.y, fma_(a.y, u.x, vy)))};
-    };
-    for (int k = P - 1; k > 0; --k) {
-        const V4<R> m = mp[k];
-        const R k1(k + 1), ik = inv_k[k];
-        step(A, m.x, m.y);
-        step(B, k1 * m.x, k1 * m.y);
-        step(E, m.z, m.w);
-        step(L, ik * m.x, ik * m.y);
-        step(M, ik * m.z, ik * m.w);
-    }
-    const V4<R> m = mp[0];
-    step(A, m.x, m.y);
-    step(B, m.x, m.y);
-    step(E, m.z, m.w);
-    L = cmul(L, u);
-    M = cmul(M, u);
-    A = cmul(A, u);
-    E = cmul(E, u);
-    B = cmul(cmul(B, u), u);  // -A'
-    // F = E - conj(W) A'
-    const C2<R> F{E.x + fma_(W.x, B.x, W.y * B.y), E.y + fma_(W.x, B.y, -(W.y * B.x))};
-    // conj(conj(W) A) = W conj(A)
-    const R wx = fma_(W.x, A.x, W.y * A.y), wy = fma_(W.y, A.x, -(W.x * A.y));
-    v[0] = 0.5 * to_double(L.x + M.x + wx + m.x) - ln_w * to_double(m.x);
-    v[1] = 0.5 * to_double(L.y - M.y + wy + m.y) - ln_w * to_double(m.y);
-    v[2] = -to_double(R(2) * n0 * A.x + (n0 * F.x - n1 * F.y));
-    v[3] = -to_double(R(2) * n1 * A.x - (n0 * F.y + n1 * F.x));
-}
-constexpr int kWallImages = 6;
-
-// One warp per task: first (cell, wall point, far image), writing
-// gpart[((cell 7) + image) 8m + 4 wp + component]; then one per cell for its
-// total force (slot 6); then the close pairs (Sec. 6.3), C_p sigma into psum[p].
-template <typename R, typename B>
-__global__ void __launch_bounds__(128)
-k_side(FmmTree t, const Cell* __restrict__ cells, int ncell, int m, int walls, const V4<R>* __restrict__ mp,
-       const double* __restrict__ wall, const double* __restrict__ bodyF, double* __restrict__ gpart, int npairs,
-       const int4* __restrict__ pairs, const int* __restrict__ node_cell, const long long* __restrict__ blk_off,
-       const B* __restrict__ blocks, const double* __restrict__ body, const double2* __restrict__ sigma,
-       const double* __restrict__ w, void* __restrict__ psum) {
-    constexpr int P = FmmTypes<R>::P;
-    __shared__ R s_inv[P];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int task = blockIdx.x * 4 + wid;
-    if (walls) {
-        for (int k = threadIdx.x; k < P; k += 128) s_inv[k] = R(k ? 1.0 / k : 0.0);
-        __syncthreads();
-        const int per = 2 * m * kWallImages + 1;
-        if (task < ncell * per) {
-            const int ci = task / per, q = task % per;
-            const Cell& cl = cells[ci];
-            if (!cl.active) return;
-            double* gp = gpart + (size_t)ci * 7 * 8 * m;
-            double v[4] = {0, 0, 0, 0};
-            if (q == per - 1) {
-                for (int b = cl.body_off + lane; b < cl.body_off + cl.n_bodies; b += 32) {
-                    v[0] += bodyF[3 * b];
-                    v[1] += bodyF[3 * b + 1];
-                }
-            } else {
-                const int wp = q / kWallImages, im = q % kWallImages;
-                const FmmCell& f = t.cells[ci];
-                const int lv = f.wall, n = f.gx[lv] * f.gy[lv];
-                const double H = f.h * (1 << lv);
-                const double* wt = wall + ((size_t)ci * 2 * m + wp) * kWallStride;
-                const double px = wt[2 * im] - cl.C[0], py = wt[2 * im + 1] - cl.C[1];
-                const R n0(wt[12]), n1(wt[13]);
-                for (int e = lane; e < n; e += 32) {
-                    const int b = f.off[lv] + e;
-                    if (t.scount[b] == 0) continue;
-                    const double2 c = fmm_centre(f, lv, e % f.gx[lv], e / f.gx[lv]);
-                    const double wx = px - c.x, wy = py - c.y;
-                    double o[4];
-                    wall_box<R>(mp + (size_t)b * P, C2<R>{R(wx / H), R(wy / H)}, 0.5 * log(wx * wx + wy * wy), n0, n1,
-                                s_inv, o);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) v[k] += o[k];
-                }
-                const double sg = im < 3 ? 1.0 : -1.0;
-                const double cu = sg / (4.0 * kPi * cl.mu), ct = sg / (4.0 * kPi * H);
-                v[0] *= cu;
-                v[1] *= cu;
-                v[2] *= ct;
-                v[3] *= ct;
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-            if (q == per - 1) {
-                if (lane < 2) gp[6 * 8 * (size_t)m + lane] = lane ? v[1] : v[0];
-            } else if (lane < 4) {
-                const int wp = q / kWallImages, im = q % kWallImages;
-                gp[(size_t)im * 8 * m + 4 * wp + lane] = lane == 0 ? v[0] : (lane == 1 ? v[1] : (lane == 2 ? v[2] : v[3]));
-            }
-            return;
-        }
-        task -= ncell * per;
-    }
-    if (task >= npairs) return;
-    const int4 pr = pairs[task];
-    if (!cells[node_cell[pr.x]].active) return;
-    const int n = (int)body[8 * pr.y + 5], off = (int)body[8 * pr.y + 6];
-    const B* C = blocks + blk_off[task];
-    B bx = 0, by = 0;
-#pragma unroll 4
-    for (int j = lane; j < n; j += 32) {
-        const double2 sg = sigma[off + j];
-        // single precision: blocks act on q = sigma w
-        const double wj = sizeof(B) == 4 ? w[off + j] : 1.0;
-        const B sx = sizeof(B) == 4 ? (B)(sg.x * wj) : (B)sg.x, sy = sizeof(B) == 4 ? (B)(sg.y * wj) : (B)sg.y;
-        const B a = C[3 * j], b = C[3 * j + 1], d = C[3 * j + 2];
-        bx = fma(a, sx, fma(b, sy, bx));
-        by = fma(b, sx, fma(d, sy, by));
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        bx += __shfl_xor_sync(0xffffffffu, bx, o);
-        by += __shfl_xor_sync(0xffffffffu, by, o);
-    }
-    if (lane == 0) {
-        if constexpr (sizeof(B) == 4) reinterpret_cast<float2*>(psum)[task] = make_float2(bx, by);
-        else reinterpret_cast<double2*>(psum)[task] = make_double2(bx, by);
     }
 }
 
@@ -1293,16 +1533,11 @@ static FmmPlanCell fmm_rect(const bie_ctx* c, int k) {
 
 void free_fmm(bie_ctx* c) {
     for (Fmm& f : c->fmm) {
-        for (void* p : f.owned)
-            if (p) cudaFree(p);
+        if (f.arena) cudaFree(f.arena);
         f = Fmm{};
     }
-    for (void*& p : c->fmm_tab) {
-        if (p) cudaFree(p);
-        p = nullptr;
-    }
-    for (void* p : {c->ws.fsq, c->ws.fmp, c->ws.floc, (void*)c->ws.ftick})
-        if (p) cudaFree(p);
+    if (c->fmm_ws) cudaFree(c->fmm_ws);
+    c->fmm_ws = nullptr;
     c->ws.fsq = c->ws.fmp = c->ws.floc = nullptr;
     c->ws.ftick = nullptr;
 }
@@ -1311,17 +1546,20 @@ void free_fmm(bie_ctx* c) {
 template <typename R>
 static FmmTab<R> fmm_tab(const bie_ctx* c, int prec) {
     constexpr int P = FmmTypes<R>::P;
-    const R* h = (const R*)c->fmm_tab[prec];
-    const C2<R>* pw = (const C2<R>*)(h + 2 * P * P);
-    return FmmTab<R>{h, h + P * P, pw, pw + 4 * P};
+    const R* h = (const R*)c->fmm[prec].tables;
+    const C2<R>* pw = (const C2<R>*)(h + 3 * P * P);
+    return FmmTab<R>{h, h + P * P, h + 2 * P * P, pw, pw + 4 * P};
 }
 
 static df to_df(long double v) { return df((float)v, (float)(v - (long double)(float)v)); }
 
 template <typename R>
-static int fmm_tables(bie_ctx* c, int prec) {
+static constexpr size_t kTableSize = (3 * (size_t)FmmTypes<R>::P * FmmTypes<R>::P + 16 * FmmTypes<R>::P) * sizeof(R);
+
+template <typename R>
+static void fmm_tables(void* out) {
     constexpr int P = FmmTypes<R>::P;
-    std::vector<R> t(2 * (size_t)P * P + 16 * P);
+    R* t = (R*)out;
     auto put = [&](size_t k, long double v) {
         if constexpr (std::is_same<R, df>::value) t[k] = to_df(v);
         else t[k] = (R)v;
@@ -1335,13 +1573,14 @@ static int fmm_tables(bie_ctx* c, int prec) {
         for (int l = 0; l < P; ++l) {
             put((size_t)k * P + l, b[k + l][l]);
             put((size_t)(P + k) * P + l, b[l][k]);
+            put((size_t)(2 * P + l) * P + k, b[l][k]);
         }
     for (int q = 0; q < 4; ++q) {
         // delta = (+-1/4, +-1/4); 1 / (2 delta) = (+-1, -+1)
         const long double dx = q & 1 ? 0.25L : -0.25L, dy = q >> 1 ? 0.25L : -0.25L;
         long double d[2] = {1, 0}, g[2] = {1, 0};
         for (int k = 0; k < P; ++k) {
-            const size_t o = 2 * (size_t)P * P + 2 * ((size_t)q * P + k);
+            const size_t o = 3 * (size_t)P * P + 2 * ((size_t)q * P + k);
             put(o, d[0]);
             put(o + 1, d[1]);
             put(o + 8 * P, g[0]);
@@ -1355,9 +1594,6 @@ static int fmm_tables(bie_ctx* c, int prec) {
             g[1] = ng[1];
         }
     }
-    BIE_CUDA(c, cudaMalloc(&c->fmm_tab[prec], t.size() * sizeof(R)));
-    BIE_CUDA(c, cudaMemcpy(c->fmm_tab[prec], t.data(), t.size() * sizeof(R), cudaMemcpyHostToDevice));
-    return BIE_OK;
 }
 
 // The largest box side from whose corners the walls' far images are so far that
@@ -1466,7 +1702,7 @@ int fmm_plan(bie_ctx* c) {
             fc.off[0] = (int)nleaf;
             nleaf += (long long)fc.gx[0] * fc.gy[0];
         }
-        f.on = t_fast < t_direct && nleaf < (1 << 26);
+        f.on = (t_fast < t_direct || BIE_FMM == 2) && nleaf < (1 << 26);
         f.walls = f.on && !c->utilde;
         for (const FmmCell& fc : cells) f.walls = f.walls && fc.wall >= 0;
         if (!f.on) continue;
@@ -1477,7 +1713,33 @@ int fmm_plan(bie_ctx* c) {
                 fc.off[l] = (int)nbox;
                 nbox += (long long)fc.gx[l] * fc.gy[l];
             }
-        std::vector<int4> box(nbox);
+        // one block: what the host writes first (cells, boxes, leaf centres, tables)
+        const bool dbl = prec != 0;
+        size_t total = 0;
+        auto place = [&](size_t bytes) {
+            const size_t at = total;
+            total += (bytes + 255) & ~(size_t)255;
+            return at;
+        };
+        const size_t tab_bytes = prec == 0 ? kTableSize<float> : (prec == 1 ? kTableSize<double> : kTableSize<df>);
+        const size_t o_cells = place(cells.size() * sizeof(FmmCell)), o_box = place(nbox * sizeof(int4)),
+                     o_centre = place(nbox * sizeof(float4)), o_grid = place(nbox * sizeof(int4)), o_tab = place(tab_bytes), written = total;
+        const size_t o_scount = place(nbox * sizeof(int)), o_sstart = place((nleaf + 1) * sizeof(int)),
+                     o_sperm = place(nsrc * sizeof(int)), o_cursor = place(nleaf * sizeof(int)),
+                     o_leaf = place(nsrc * sizeof(int)), o_raw = place(nsrc * sizeof(int)),
+                     o_spos = prec != 1 ? place(nsrc * sizeof(float4)) : 0,
+                     o_spos64 = dbl ? place(nsrc * sizeof(double2)) : 0;
+        const size_t o_far = place((size_t)nbox * kFmmFar * sizeof(int)), o_nfar = place(nbox * sizeof(int)),
+                     o_near = place((size_t)nleaf * kFmmRanges * sizeof(FmmRange)), o_nnear = place(nleaf * sizeof(int)),
+                     o_shift = place(9 * cells.size() * sizeof(float4));
+        const bool ut = c->utilde;
+        const size_t o_tcount = ut ? place(nbox * sizeof(int)) : 0, o_tstart = ut ? place((nleaf + 1) * sizeof(int)) : 0,
+                     o_tperm = ut ? place(N * sizeof(int)) : 0,
+                     o_tpos = ut ? place(N * (dbl ? sizeof(double2) : sizeof(float4))) : 0;
+        BIE_CUDA(c, cudaMalloc(&f.arena, total));
+        std::vector<unsigned char> host(written);
+        std::memcpy(&host[o_cells], cells.data(), cells.size() * sizeof(FmmCell));
+        int4* box = (int4*)&host[o_box];
         for (int k = 0; k < c->ncell; ++k) {
             const FmmCell& fc = cells[k];
             for (int l = 0; l < fc.nlev; ++l)
@@ -1487,60 +1749,51 @@ int fmm_plan(bie_ctx* c) {
                             make_int4(k, l, x | (y << 16),
                                       l + 1 < fc.nlev ? fc.off[l + 1] + (y / 2) * fc.gx[l + 1] + x / 2 : -1);
         }
-        const bool dbl = prec != 0;
-        auto get = [&](void* pp, size_t bytes) -> int {
-            void* p = nullptr;
-            BIE_CUDA(c, cudaMalloc(&p, bytes + 16));
-            f.owned.push_back(p);
-            std::memcpy(pp, &p, sizeof p);
-            return BIE_OK;
-        };
-        FmmTree& t = f.t;
-        t.nleaf = (int)nleaf;
-        t.nbox = (int)nbox;
-        int rc = get(&f.cells, cells.size() * sizeof(FmmCell));
-        rc = rc ? rc : get(&f.box, box.size() * sizeof(int4));
-        rc = rc ? rc : get(&t.centre, nleaf * sizeof(float4));
-        rc = rc ? rc : get(&t.scount, nbox * sizeof(int));
-        rc = rc ? rc : get(&t.sstart, (nleaf + 1) * sizeof(int));
-        rc = rc ? rc : get(&t.sperm, nsrc * sizeof(int));
-        rc = rc ? rc : get(&f.cursor, nleaf * sizeof(int));
-        rc = rc ? rc : get(&f.leaf, nsrc * sizeof(int));
-        rc = rc ? rc : get(&f.raw, nsrc * sizeof(int));
-        if (prec != 1) rc = rc ? rc : get(&t.spos, nsrc * sizeof(float4));
-        if (dbl) rc = rc ? rc : get(&t.spos64, nsrc * sizeof(double2));
-        t.tcount = t.scount;
-        t.tstart = t.sstart;
-        t.tperm = t.sperm;
-        t.tpos = t.spos;
-        t.tpos64 = t.spos64;
-        if (c->utilde) {
-            t.tpos = nullptr;
-            t.tpos64 = nullptr;
-            rc = rc ? rc : get(&t.tcount, nbox * sizeof(int));
-            rc = rc ? rc : get(&t.tstart, (nleaf + 1) * sizeof(int));
-            rc = rc ? rc : get(&t.tperm, N * sizeof(int));
-            if (!dbl) rc = rc ? rc : get(&t.tpos, N * sizeof(float4));
-            if (dbl) rc = rc ? rc : get(&t.tpos64, N * sizeof(double2));
-        }
-        if (rc) return rc;
-        BIE_CUDA(c, cudaMemcpy(f.cells, cells.data(), cells.size() * sizeof(FmmCell), cudaMemcpyHostToDevice));
-        BIE_CUDA(c, cudaMemcpy(f.box, box.data(), box.size() * sizeof(int4), cudaMemcpyHostToDevice));
-        std::vector<float4> centre(nleaf);
-        for (long long b = 0; b < nleaf; ++b) {
-            const double2 p = fmm_centre(cells[box[b].x], 0, fmm_ix(box[b]), fmm_iy(box[b]));
+        float4* centre = (float4*)&host[o_centre];
+        int4* grid = (int4*)&host[o_grid];
+        for (long long b = 0; b < nbox; ++b) {
+            const FmmCell& fc = cells[box[b].x];
+            grid[b] = make_int4(fc.off[box[b].y], fc.gx[box[b].y], 0, 0);
+            const double2 p = fmm_centre(fc, box[b].y, fmm_ix(box[b]), fmm_iy(box[b]));
             centre[b].x = (float)p.x;
             centre[b].y = (float)(p.x - (double)centre[b].x);
             centre[b].z = (float)p.y;
             centre[b].w = (float)(p.y - (double)centre[b].z);
         }
-        BIE_CUDA(c, cudaMemcpy(t.centre, centre.data(), centre.size() * sizeof(float4), cudaMemcpyHostToDevice));
-        t.cells = f.cells;
-        t.box = f.box;
+        if (prec == 0) fmm_tables<float>(&host[o_tab]);
+        else if (prec == 1) fmm_tables<double>(&host[o_tab]);
+        else fmm_tables<df>(&host[o_tab]);
+        BIE_CUDA(c, cudaMemcpy(f.arena, host.data(), written, cudaMemcpyHostToDevice));
+        unsigned char* a = (unsigned char*)f.arena;
+        FmmTree& t = f.t;
+        t.nleaf = (int)nleaf;
+        t.nbox = (int)nbox;
+        t.cells = f.cells = (FmmCell*)(a + o_cells);
+        t.box = f.box = (int4*)(a + o_box);
+        t.centre = (float4*)(a + o_centre);
+        t.grid = (int4*)(a + o_grid);
+        t.far = (int*)(a + o_far);
+        t.nfar = (int*)(a + o_nfar);
+        t.near = (FmmRange*)(a + o_near);
+        t.nnear = (int*)(a + o_nnear);
+        t.shift = (float4*)(a + o_shift);
+        f.tables = a + o_tab;
+        t.tcount = t.scount = (int*)(a + o_scount);
+        t.tstart = t.sstart = (int*)(a + o_sstart);
+        t.tperm = t.sperm = (int*)(a + o_sperm);
+        f.cursor = (int*)(a + o_cursor);
+        f.leaf = (int*)(a + o_leaf);
+        f.raw = (int*)(a + o_raw);
+        t.tpos = t.spos = prec != 1 ? (float4*)(a + o_spos) : nullptr;
+        t.tpos64 = t.spos64 = dbl ? (double2*)(a + o_spos64) : nullptr;
+        if (ut) {
+            t.tcount = (int*)(a + o_tcount);
+            t.tstart = (int*)(a + o_tstart);
+            t.tperm = (int*)(a + o_tperm);
+            t.tpos = dbl ? nullptr : (float4*)(a + o_tpos);
+            t.tpos64 = dbl ? (double2*)(a + o_tpos) : nullptr;
+        }
         f.built = 0;
-        rc = prec == 0 ? fmm_tables<float>(c, prec)
-                       : (prec == 1 ? fmm_tables<double>(c, prec) : fmm_tables<df>(c, prec));
-        if (rc) return rc;
         f.mp_bytes = (size_t)nbox * (dbl ? kFmmP64 * sizeof(V4<double>) : kFmmP32 * sizeof(V4<float>));
         // lists split into shares until the boxes (about half of them occupied)
         // fill the SMs four times over
@@ -1553,11 +1806,15 @@ int fmm_plan(bie_ctx* c) {
         max_box = std::max(max_box, (int)nbox);
     }
     if (max_box) {
-        BIE_CUDA(c, cudaMalloc(&c->ws.fsq, sq_bytes + 16));
-        BIE_CUDA(c, cudaMalloc(&c->ws.fmp, mp_bytes + 16));
-        BIE_CUDA(c, cudaMalloc(&c->ws.floc, loc_bytes + 16));
-        BIE_CUDA(c, cudaMalloc((void**)&c->ws.ftick, max_box * sizeof(unsigned)));
-        BIE_CUDA(c, cudaMemset(c->ws.ftick, 0, max_box * sizeof(unsigned)));
+        auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+        const size_t tick = up(max_box * sizeof(unsigned));
+        BIE_CUDA(c, cudaMalloc(&c->fmm_ws, tick + up(sq_bytes) + up(mp_bytes) + up(loc_bytes)));
+        unsigned char* a = (unsigned char*)c->fmm_ws;
+        c->ws.ftick = (unsigned*)a;
+        c->ws.fsq = a + tick;
+        c->ws.fmp = a + tick + up(sq_bytes);
+        c->ws.floc = a + tick + up(sq_bytes) + up(mp_bytes);
+        BIE_CUDA(c, cudaMemset(c->ws.ftick, 0, tick));
     }
     return BIE_OK;
 }
@@ -1584,16 +1841,23 @@ int fmm_build(bie_ctx* c, int prec) {
                                                   set ? t.tpos : t.spos, set ? t.tpos64 : t.spos64);
         BIE_LAUNCH(c, "k_fmm_sort");
     }
+    k_fmm_lists<<<t.nbox, 128, 0, c->stream>>>(t, c->cells, c->utilde ? 1 : 9);
+    BIE_LAUNCH(c, "k_fmm_lists");
     f.built = c->geometry;
     return BIE_OK;
 }
 
 template <typename R>
 static int up_launch(bie_ctx* c, const double* sigma, int prec, Workspace& ws) {
-    const FmmTree& t = c->fmm[prec].t;
-    k_fmm_up<R><<<t.nleaf, 128, 0, c->stream>>>(t, c->cells, reinterpret_cast<const double2*>(sigma), c->w,
-                                                c->utilde ? 2 : 0, (C2<R>*)ws.fsq, (V4<R>*)ws.fmp, ws.ftick,
-                                                fmm_tab<R>(c, prec));
+    const Fmm& f = c->fmm[prec];
+    // the per-node records: the direct walls' (single precision, or double), and
+    // for velocities_device after a double-precision application
+    FmmBodies p{c->x, c->y, c->body, c->body_cell, nullptr, nullptr, ws.bodyF};
+    if (!f.walls && prec == 0) p.src32 = c->utilde ? ws.src32n : ws.src32;
+    if (!f.walls || prec != 0) p.src64 = ws.src64;
+    k_fmm_up<R><<<f.t.nbox + c->nb, 128, 0, c->stream>>>(f.t, c->cells, reinterpret_cast<const double2*>(sigma), c->w,
+                                                          c->utilde ? 2 : 0, (C2<R>*)ws.fsq, (V4<R>*)ws.fmp, ws.ftick,
+                                                          fmm_tab<R>(c, prec), p);
     BIE_LAUNCH(c, "k_fmm_up");
     return BIE_OK;
 }
@@ -1603,50 +1867,67 @@ int fmm_up(bie_ctx* c, const double* sigma, int prec, Workspace& ws) {
                      : (prec == 1 ? up_launch<double>(c, sigma, prec, ws) : up_launch<df>(c, sigma, prec, ws));
 }
 
+static SideArgs side_args(bie_ctx* c, const double* sigma, int prec, bool walls, Workspace& ws) {
+    SideArgs a;
+    a.ncell = c->ncell;
+    a.m = c->m;
+    a.walls = walls ? 1 : 0;
+    a.npairs = c->cl.npairs;
+    const long long tasks = (walls ? (long long)c->ncell * (2 * c->m * kWallImages + 1) : 0) + a.npairs;
+    a.ctas = (int)((tasks + 3) / 4);
+    a.wall = c->wall;
+    a.bodyF = ws.bodyF;
+    a.gpart = ws.gpart;
+    a.pairs = c->cl.pairs;
+    a.node_cell = c->node_cell;
+    a.blk_off = c->cl.blk_off;
+    a.blocks = prec == 0 ? (const void*)c->cl.blocks32 : (const void*)c->cl.blocks;
+    a.body = c->body;
+    a.sigma = reinterpret_cast<const double2*>(sigma);
+    a.w = c->w;
+    a.psum = ws.psum ? ws.psum : c->cl.psum;
+    return a;
+}
+
+int close_pairs(bie_ctx* c, const double* sigma, int prec, Workspace& ws, cudaStream_t st) {
+    const SideArgs a = side_args(c, sigma, prec, false, ws);
+    if (a.npairs == 0) return BIE_OK;
+    if (prec == 0) k_close_pairs<float><<<a.ctas, 128, 0, st>>>(a, c->cells);
+    else k_close_pairs<double><<<a.ctas, 128, 0, st>>>(a, c->cells);
+    BIE_LAUNCH(c, "k_close_pairs");
+    return BIE_OK;
+}
+
 template <typename R>
-static int across_launch(bie_ctx* c, int prec, Workspace& ws) {
+static int across_launch(bie_ctx* c, const double* sigma, int prec, Workspace& ws) {
     const Fmm& f = c->fmm[prec];
     const FmmTree& t = f.t;
     const FmmTab<R> tab = fmm_tab<R>(c, prec);
-    const int nimg = c->utilde ? 1 : 9;
+    const int nimg = c->utilde ? 1 : 9, tiles = 2;
     const int n0 = c->shard.on ? c->shard.n0 : 0, n1 = c->shard.on ? c->shard.n1 : c->N;
     const V4<R>* loc = (const V4<R>*)ws.floc;
-    k_fmm_m2l<R><<<dim3(t.nbox, f.shares), 128, 0, c->stream>>>(t, c->cells, nimg, (const V4<R>*)ws.fmp,
-                                                                (V4<R>*)ws.floc, tab);
-    BIE_LAUNCH(c, "k_fmm_m2l");
-    const dim3 down(t.nleaf, 2);
+    const SideArgs side = side_args(c, sigma, prec, f.walls, ws);
+    const bool early = fmm_chained(c, prec);
+    BIE_CUDA(c, launch_after(early, k_fmm_m2l<R>, side.ctas + t.nbox * f.shares, 128, c->stream, t, c->cells, nimg,
+                             (const V4<R>*)ws.fmp, (V4<R>*)ws.floc, tab, f.shares, side));
+    ++c->launches;
+    XiArgs xi{c->m, c->M, 0, (2 * c->M + 3) / 4, ws.gpart, c->P, ws.xi, ws.xif};
+    if (f.walls) xi.ctas = xi.per_cell * c->ncell;
+    const unsigned down = xi.ctas + t.nleaf * tiles;
     if constexpr (sizeof(R) == 4)
-        k_fmm_down32<<<down, 128, 0, c->stream>>>(t, c->cells, nimg, (const C2<float>*)ws.fsq, loc, f.shares, tab,
-                                                  c->tgt32, n0, n1, (float2*)ws.part);
+        BIE_CUDA(c, launch_after(early, k_fmm_down32, down, 128, c->stream, t, c->cells, nimg, (const C2<float>*)ws.fsq, loc,
+                                 f.shares, tab, c->tgt32, n0, n1, (float2*)ws.part, xi, tiles));
     else
-        k_fmm_down64<R><<<down, 128, 0, c->stream>>>(t, c->cells, nimg, (const C2<R>*)ws.fsq, loc, f.shares, tab,
-                                                     c->nx, c->ny, prec, n0, n1, (double2*)ws.part);
-    BIE_LAUNCH(c, "k_fmm_down");
+        BIE_CUDA(c, launch_after(early, k_fmm_down64<R>, down, 128, c->stream, t, c->cells, nimg, (const C2<R>*)ws.fsq, loc,
+                                 f.shares, tab, c->nx, c->ny, prec, n0, n1, (double2*)ws.part, xi, tiles));
+    ++c->launches;
     return BIE_OK;
 }
 
-int fmm_across(bie_ctx* c, int prec, Workspace& ws) {
-    return prec == 0 ? across_launch<float>(c, prec, ws)
-                     : (prec == 1 ? across_launch<double>(c, prec, ws) : across_launch<df>(c, prec, ws));
-}
-
-template <typename R, typename B>
-static int side_launch(bie_ctx* c, const double* sigma, int prec, bool walls, const B* blocks, Workspace& ws,
-                       cudaStream_t st) {
-    const long long tasks = (walls ? (long long)c->ncell * (2 * c->m * kWallImages + 1) : 0) + c->cl.npairs;
-    if (tasks == 0) return BIE_OK;
-    k_side<R, B><<<(unsigned)((tasks + 3) / 4), 128, 0, st>>>(
-        c->fmm[prec].t, c->cells, c->ncell, c->m, walls ? 1 : 0, (const V4<R>*)ws.fmp, c->wall, ws.bodyF, ws.gpart,
-        c->cl.npairs, c->cl.pairs, c->node_cell, c->cl.blk_off, blocks, c->body,
-        reinterpret_cast<const double2*>(sigma), c->w, ws.psum ? ws.psum : c->cl.psum);
-    BIE_LAUNCH(c, "k_side");
-    return BIE_OK;
-}
-
-int side(bie_ctx* c, const double* sigma, int prec, bool walls, Workspace& ws, cudaStream_t st) {
-    if (prec == 0) return side_launch<float>(c, sigma, prec, walls, c->cl.blocks32, ws, st);
-    return prec == 1 ? side_launch<double>(c, sigma, prec, walls, c->cl.blocks, ws, st)
-                     : side_launch<df>(c, sigma, prec, walls, c->cl.blocks, ws, st);
+int fmm_across(bie_ctx* c, const double* sigma, int prec, Workspace& ws) {
+    return prec == 0 ? across_launch<float>(c, sigma, prec, ws)
+                     : (prec == 1 ? across_launch<double>(c, sigma, prec, ws)
+                                  : across_launch<df>(c, sigma, prec, ws));
 }
 
 }  // namespace bie

@@ -52,7 +52,7 @@ int build_dot_chunks(bie_ctx* c) {
     std::vector<int4> fin;  // the assembly's chunks of nodes
     for (int ci = 0; ci < c->ncell; ++ci) {
         const int n0 = c->cells_h[ci].node_off, n1 = n0 + c->cells_h[ci].n_nodes;
-        for (int i = n0; i < n1; i += kFinNodes) fin.push_back(make_int4(ci, i, std::min(n1, i + kFinNodes), 0));
+        for (int i = n0; i < n1; i += kFinNodes) fin.push_back(make_int4(ci, i, std::min(n1, i + kFinNodes), n0));
     }
     c->n_fin = (int)fin.size();
     BIE_CUDA(c, cudaMalloc((void**)&c->fin_chunks, fin.size() * sizeof(int4)));
