@@ -516,17 +516,29 @@ int build_dot_chunks(bie_ctx* c);
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// The two halves of a cluster's barrier: what a thread wrote before it arrives is
+// seen by the cluster's threads that have waited.
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // With `early`, a launch that may begin before the one ahead of it in the stream
 // has ended (it waits in the kernel: pdl_wait).
 template <typename... A>
-inline cudaError_t launch_after(bool early, void (*k)(A...), unsigned grid, unsigned block, cudaStream_t st,
+inline cudaError_t launch_after(bool early, void (*k)(A...), dim3 grid, unsigned block, unsigned shm, cudaStream_t st,
                                 typename std::common_type<A>::type... a) {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = shm;
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = early ? 1 : 0;

@@ -15,10 +15,13 @@
 //     D(tau) = sin(N_b tau / 2) cot(tau / 2) / N_b.
 // G^t applied to q is c r (r . q) with c = -(r . n)/(pi r^4), so each C_k is
 // a symmetric 2 x 2 matrix: three doubles (A, B, D) per node.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <utility>
 #include <vector>
+
+#include <cooperative_groups.h>
 
 #include "bie_internal.cuh"
 
@@ -50,6 +53,10 @@ __global__ void k_body_h(const double* __restrict__ w, double* __restrict__ body
 // With the doubled-cell periodizer (imc non-null) a pair is valid only when
 // the body image, seen from the target's translate inside U, is among the
 // images of every node of the body (bimg); otherwise bit 1 of *gflag is set.
+// Bound by the FP32 pipe: the bodies' images in single precision, tiles of bodies in
+// shared memory, and in double only what is near (102400 nodes of 400 bodies: 16.2 ms
+// with every distance in double, 0.83 so).
+constexpr int kDetectTile = 128;
 __global__ void k_close_detect(const double* __restrict__ x, const double* __restrict__ y,
                                const int* __restrict__ owner, const double* __restrict__ body,
                                const int* __restrict__ node_cell, const Cell* __restrict__ cells, int N,
@@ -58,33 +65,71 @@ __global__ void k_close_detect(const double* __restrict__ x, const double* __res
                                unsigned long long* __restrict__ gap_min, int* __restrict__ rho_max,
                                float* __restrict__ dmin, float2* __restrict__ ddir, const int* __restrict__ imc,
                                const int4* __restrict__ bimg, int* __restrict__ gflag,
-                               const double* __restrict__ bshape) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const Cell& sh = cells[node_cell[i]];
+                               const double* __restrict__ bshape, const float4* __restrict__ posdf) {
+    __shared__ float4 s_body[kDetectTile];  // centre from the cell's, reach, 0
+    const int i0 = blockIdx.x * blockDim.x, i = min(i0 + (int)threadIdx.x, N - 1);
+    const bool in = i0 + (int)threadIdx.x < N;
+    const int mine = node_cell[i];
+    const Cell& sh = cells[mine];
+    const float tx = posdf[i].x, ty = posdf[i].z, ta = fabsf(tx) + fabsf(ty);
     const int wi = imc ? img_wrap(imc[i]) : 4;  // the target's translate into U
     double X = x[i], Y = y[i];
     int own = owner[i];
     int c = 0;
     double dbest = INFINITY, dirx = 0, diry = 0;  // nearest other curve (or own periodic image)
-    for (int b = sh.body_off; b < sh.body_off + sh.n_bodies; ++b) {
+    // the cells of this CTA's targets (their nodes are consecutive), bodies in tiles
+    const int c1 = node_cell[min(i0 + (int)blockDim.x, N) - 1];
+    for (int cell = node_cell[i0]; cell <= c1; ++cell)
+    for (int b0 = cells[cell].body_off; b0 < cells[cell].body_off + cells[cell].n_bodies; b0 += kDetectTile) {
+    const int nt = min(kDetectTile, cells[cell].body_off + cells[cell].n_bodies - b0);
+    __syncthreads();
+    for (int q = threadIdx.x; q < nt; q += blockDim.x) {
+        const double* bd = body + 8 * (b0 + q);
+        const float bx = (float)(bd[2] - cells[cell].C[0]), by = (float)(bd[3] - cells[cell].C[1]);
+        const double reach = fmax(bd[0], bd[1]) + fmax(close_factor * bd[7], gap_lim);
+        s_body[q] = make_float4(bx, by, (float)reach * 1.00001f + 1e-6f * (fabsf(bx) + fabsf(by)), 0.f);
+    }
+    __syncthreads();
+    if (!in || mine != cell) continue;
+    for (int b = b0; b < b0 + nt; ++b) {
+        const float4 sb = s_body[b - b0];
         const double* bd = body + 8 * b;
-        double R = fmax(bd[0], bd[1]);
-        double hb = bd[7];
-        double zone = close_factor * hb;
-        double lim = fmax(zone, gap_lim);
-        int n = (int)bd[5], off = (int)bd[6];
         for (int im = 0; im < 9; ++im) {
             if (b == own && im == 4) continue;  // zero shift of the own body
+            // far bodies in single precision (their centre's distance, with more than
+            // its rounding errors to spare)
+            const float ux = (tx - sb.x) - sh.sxf[im], uy = (ty - sb.y) - sh.syf[im];
+            const float reach = sb.z + 1e-6f * (ta + fabsf(sh.sxf[im]) + fabsf(sh.syf[im]));
+            if (ux * ux + uy * uy > reach * reach) continue;
+            const double R = fmax(bd[0], bd[1]), hb = bd[7];
+            const double zone = close_factor * hb, lim = fmax(zone, gap_lim);
+            const int n = (int)bd[5], off = (int)bd[6];
             double cx = bd[2] + sh.sx[im], cy = bd[3] + sh.sy[im];
             double dc = sqrt((X - cx) * (X - cx) + (Y - cy) * (Y - cy));
             if (dc - R > lim) continue;
+            // the nearest node: over all of them in single precision, from exact
+            // differences of the double-float positions, then in double over the
+            // four on each side of that one
+            float pxh, pxl, pyh, pyl;
+            split_df(X - sh.sx[im] - sh.C[0], pxh, pxl);
+            split_df(Y - sh.sy[im] - sh.C[1], pyh, pyl);
+            float ebest = INFINITY;
+            int k0 = 0;
+            for (int k = 0; k < n; ++k) {
+                const float4 q = posdf[off + k];
+                const float dx = (pxh - q.x) + (pxl - q.y), dy = (pyh - q.z) + (pyl - q.w), e = dx * dx + dy * dy;
+                if (e < ebest) { ebest = e; k0 = k; }
+            }
+            // (all of them where the squares leave single precision's range)
+            const int side = ebest > 1e-30f && ebest < 1e30f ? min(4, n / 2) : n / 2;
             double d2 = 1e300;
             int kbest = 0;
-            for (int k = 0; k < n; ++k) {
+            for (int u = -side; u <= side; ++u) {
+                int k = k0 + u;
+                k += k < 0 ? n : (k >= n ? -n : 0);
                 double dx = X - (x[off + k] + sh.sx[im]), dy = Y - (y[off + k] + sh.sy[im]);
                 double e = dx * dx + dy * dy;
-                if (e < d2) { d2 = e; kbest = k; }
+                if (e < d2 || (e == d2 && k < kbest)) { d2 = e; kbest = k; }
             }
             if (sqrt(d2) >= lim) continue;
             // distance to the exact curve and local node spacing at the closest
@@ -163,6 +208,8 @@ __global__ void k_close_detect(const double* __restrict__ x, const double* __res
             ++c;
         }
     }
+    }
+    if (!in) return;
     if (c > kmax) {
         atomicMax(overflow, c);
         c = kmax;
@@ -249,47 +296,69 @@ __global__ void k_dirichlet(double* __restrict__ tab, int n, int rho_max) {
 
 constexpr int kCloseChunk = 2048;  // fine nodes staged in shared memory at a time
 
-// One CTA per close pair and range of kCloseAccNodes source nodes
-// (blockIdx.y).  The fine grid (rho N_b nodes) is streamed through shared
-// memory in chunks; warp w accumulates C_k for k = k0 + w, k0 + w + 8, ...
-// with its lanes on consecutive fine nodes (coalesced table and shared
-// reads).  Dynamic shared memory: 3 kCloseChunk + 3 min(N_b, kCloseAccNodes)
-// doubles.
-__global__ void __launch_bounds__(256)
-k_close_blocks(const int4* __restrict__ pairs, const long long* __restrict__ blk_off,
-               const double* __restrict__ x, const double* __restrict__ y,
-               const double* __restrict__ nx, const double* __restrict__ ny,
-               const double* __restrict__ w, const double* __restrict__ body,
-               const int* __restrict__ node_cell, const Cell* __restrict__ cells,
-               const double* __restrict__ dtab, const long long* __restrict__ dtab_off,
-               double* __restrict__ blocks, float* __restrict__ blocks32, const double* __restrict__ bshape) {
-    extern __shared__ double sm[];
+// Blocks of one close pair and range of kCloseAccNodes source nodes
+// (blockIdx.y).  The fine grid is streamed through shared memory in chunks;
+// warp w accumulates C_k for k = k0 + w, k0 + w + 8, ... with its lanes on
+// consecutive fine nodes (coalesced table and shared reads).  D is 1 at its own
+// node and 0 at the others: the fine nodes that are nodes contribute their own
+// term alone, and the sums run over the (rho - 1) N_b between them (half of them
+// at rho = 2, which most pairs have).  Bound by the FP64 pipe: 3 fma per node and
+// fine node.  A pair with more than kCloseHeavy of these is shared by a cluster of
+// kCloseCtas CTAs, each with its part of the fine nodes and the sums added through
+// distributed shared memory: one CTA for such a pair left the other SMs idle (two
+// bodies of 512 nodes 2e-3 apart: 3.6 ms, 1.7 so).  Dynamic shared memory:
+// 3 kCloseChunk + 3 min(N_b, kCloseAccNodes) doubles.
+constexpr long long kCloseHeavy = 1 << 17;
+constexpr int kCloseCtas = 8;
+
+struct BlockArgs {
+    const int4* pairs;
+    const long long* blk_off;
+    const double *x, *y, *nx, *ny, *w, *body;
+    const int* node_cell;
+    const Cell* cells;
+    const double* dtab;
+    const long long* dtab_off;
+    double* blocks;
+    float* blocks32;
+    const double* bshape;
+};
+
+__device__ inline bool close_heavy(const BlockArgs& g, int4 pr) {
+    const int n = (int)g.body[8 * pr.y + 5];
+    return (long long)(pr.w - 1) * n * n > kCloseHeavy;
+}
+
+template <int NC>
+__device__ void close_block(const BlockArgs& g, int pair, int4 pr, double* sm) {
+    namespace cg = cooperative_groups;
     double* sa = sm;
     double* sb = sm + kCloseChunk;
     double* sd = sm + 2 * kCloseChunk;
     double* acc = sm + 3 * kCloseChunk;
-    int4 pr = pairs[blockIdx.x];
-    int i = pr.x, b = pr.y, im = pr.z, rho = pr.w;
-    const Cell& sh = cells[node_cell[i]];
-    const double* bd = body + 8 * b;
-    double a = bd[0], bb = bd[1], xc = bd[2] + sh.sx[im], yc = bd[3] + sh.sy[im], th = bd[4];
-    int nbn = (int)bd[5], off = (int)bd[6];
-    int nf = rho * nbn;
-    const double* dir = dtab + dtab_off[b] + (long long)nbn * (rho - 2);
-    double X = x[i], Y = y[i], n0 = nx[i], n1 = ny[i];
+    const int rank = NC > 1 ? (int)cg::this_cluster().block_rank() : 0;
+    const int i = pr.x, b = pr.y, im = pr.z, rho = pr.w;
+    const Cell& sh = g.cells[g.node_cell[i]];
+    const double* bd = g.body + 8 * b;
+    const double a = bd[0], bb = bd[1], xc = bd[2] + sh.sx[im], yc = bd[3] + sh.sy[im], th = bd[4];
+    const int nbn = (int)bd[5], off = (int)bd[6];
+    const int nf = rho * nbn, nm = nf - nbn;
+    const double* dir = g.dtab + g.dtab_off[b] + (long long)nbn * (rho - 2);
+    const double* shp = g.bshape + 4 * b;
+    const double X = g.x[i], Y = g.y[i], n0 = g.nx[i], n1 = g.ny[i];
     double st, ct;
     sincos(th, &st, &ct);
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int k0 = blockIdx.y * kCloseAccNodes, nk = min(kCloseAccNodes, nbn - k0);
     if (nk <= 0) return;  // this body has fewer node ranges than the largest one
     for (int k = threadIdx.x; k < 3 * nk; k += blockDim.x) acc[k] = 0.0;
-    for (int f0 = 0; f0 < nf; f0 += kCloseChunk) {
-        int cnt = min(kCloseChunk, nf - f0);
+    const int gl = (int)((long long)nm * rank / NC), gh = (int)((long long)nm * (rank + 1) / NC);
+    for (int f0 = gl; f0 < gh; f0 += kCloseChunk) {
+        const int cnt = min(kCloseChunk, gh - f0);
         __syncthreads();
-        const double* shp = bshape + 4 * b;
         for (int u = threadIdx.x; u < cnt; u += blockDim.x) {
-            int f = f0 + u;
-            double t = (2.0 * kPi * f) / nf;
+            const int q = f0 + u, f = q + q / (rho - 1) + 1;  // the q-th fine node between nodes
+            const double t = (2.0 * kPi * f) / nf;
             double s, c;
             sincos(t, &s, &c);
             double px = a * c, py = bb * s;
@@ -298,25 +367,25 @@ k_close_blocks(const int4* __restrict__ pairs, const long long* __restrict__ blk
                 double ddpx, ddpy;
                 star_curve(shp, t, px, py, dpx, dpy, ddpx, ddpy);
             }
-            double yx = xc + (ct * px - st * py), yy = yc + (st * px + ct * py);
-            double dx = ct * dpx - st * dpy, dy = st * dpx + ct * dpy;
-            double wf = (2.0 * kPi / nf) * sqrt(dx * dx + dy * dy);
-            double rx = X - yx, ry = Y - yy;
-            double r2 = rx * rx + ry * ry;
-            double cc = -(rx * n0 + ry * n1) * wf / (kPi * r2 * r2);
+            const double yx = xc + (ct * px - st * py), yy = yc + (st * px + ct * py);
+            const double dx = ct * dpx - st * dpy, dy = st * dpx + ct * dpy;
+            const double wf = (2.0 * kPi / nf) * sqrt(dx * dx + dy * dy);
+            const double rx = X - yx, ry = Y - yy;
+            const double r2 = rx * rx + ry * ry;
+            const double cc = -(rx * n0 + ry * n1) * wf / (kPi * r2 * r2);
             sa[u] = cc * rx * rx;
             sb[u] = cc * rx * ry;
             sd[u] = cc * ry * ry;
         }
         __syncthreads();
         for (int kk = wid; kk < nk; kk += nw) {
-            const int k = k0 + kk;
+            const int base = rho * (k0 + kk);
             double A = 0, B = 0, D = 0;
-            int base = f0 - rho * k;
             for (int u = lane; u < cnt; u += 32) {
-                int j = base + u;
+                const int q = f0 + u;
+                int j = q + q / (rho - 1) + 1 - base;
                 j += (j < 0) ? nf : 0;
-                double dv = __ldg(dir + j);
+                const double dv = __ldg(dir + j);
                 A = fma(sa[u], dv, A);
                 B = fma(sb[u], dv, B);
                 D = fma(sd[u], dv, D);
@@ -333,26 +402,55 @@ k_close_blocks(const int4* __restrict__ pairs, const long long* __restrict__ blk
             }
         }
     }
-    __syncthreads();
-    double* out = blocks + blk_off[blockIdx.x];
-    for (int kk = threadIdx.x; kk < nk; kk += blockDim.x) {
-        // minus the smooth rule's term for node k of this body image
+    if (NC > 1)
+        cg::this_cluster().sync();
+    else
+        __syncthreads();
+    double* out = g.blocks + g.blk_off[pair];
+    for (int kk = threadIdx.x + rank * blockDim.x; kk < nk; kk += NC * blockDim.x) {
         const int k = k0 + kk;
-        double rx = X - (x[off + k] + sh.sx[im]), ry = Y - (y[off + k] + sh.sy[im]);
-        double r2 = rx * rx + ry * ry;
-        double cc = -(rx * n0 + ry * n1) * w[off + k] / (kPi * r2 * r2);
-        const double A = acc[3 * kk] - cc * rx * rx;
-        const double B = acc[3 * kk + 1] - cc * rx * ry;
-        const double D = acc[3 * kk + 2] - cc * ry * ry;
+        double A = 0, B = 0, D = 0;
+        for (int q = 0; q < NC; ++q) {
+            const double* s = NC > 1 ? cg::this_cluster().map_shared_rank(acc, q) : acc;
+            A += s[3 * kk];
+            B += s[3 * kk + 1];
+            D += s[3 * kk + 2];
+        }
+        // plus the fine rule's term at node k itself (its weight w / rho), minus the
+        // smooth rule's term for node k of this body image
+        const double rx = X - (g.x[off + k] + sh.sx[im]), ry = Y - (g.y[off + k] + sh.sy[im]);
+        const double r2 = rx * rx + ry * ry;
+        const double cc = -(rx * n0 + ry * n1) * g.w[off + k] / (kPi * r2 * r2) * (1.0 - 1.0 / rho);
+        A -= cc * rx * rx;
+        B -= cc * rx * ry;
+        D -= cc * ry * ry;
         out[3 * k] = A;
         out[3 * k + 1] = B;
         out[3 * k + 2] = D;
         // single-precision copy acting on q = sigma w (the packed sources)
-        const double iw = 1.0 / w[off + k];
-        float* o32 = blocks32 + blk_off[blockIdx.x] + 3 * k;
+        const double iw = 1.0 / g.w[off + k];
+        float* o32 = g.blocks32 + g.blk_off[pair] + 3 * k;
         o32[0] = (float)(A * iw);
         o32[1] = (float)(B * iw);
         o32[2] = (float)(D * iw);
+    }
+    // no CTA resets its sums or leaves while another reads them
+    if (NC > 1) cg::this_cluster().sync();
+}
+
+__global__ void __launch_bounds__(256) k_close_blocks(const BlockArgs g) {
+    extern __shared__ double sm[];
+    const int4 pr = g.pairs[blockIdx.x];
+    if (!close_heavy(g, pr)) close_block<1>(g, blockIdx.x, pr, sm);
+}
+
+__global__ void __cluster_dims__(kCloseCtas, 1, 1) __launch_bounds__(256)
+k_close_blocks_heavy(const BlockArgs g, int npairs) {
+    extern __shared__ double sm[];
+    cooperative_groups::this_cluster().sync();
+    for (int p = blockIdx.x / kCloseCtas; p < npairs; p += gridDim.x / kCloseCtas) {
+        const int4 pr = g.pairs[p];
+        if (close_heavy(g, pr)) close_block<kCloseCtas>(g, p, pr, sm);
     }
 }
 
@@ -637,7 +735,7 @@ int build_close(bie_ctx* c) {
                                                          c->opts.close_factor, gap_lim, kmax, c->cl.slots,
                                                          c->cl.count, c->cl.flags + 2, gap_min, c->cl.flags + 6,
                                                          c->cl.dmin, c->cl.ddir, c->utilde ? c->imc : nullptr,
-                                                         c->bimg, c->cl.flags + 7, c->bshape);
+                                                         c->bimg, c->cl.flags + 7, c->bshape, c->posdf);
     BIE_LAUNCH(c, "k_close_detect");
     int h[8];
     long long need_doubles = 0;
@@ -706,11 +804,17 @@ int build_close(bie_ctx* c) {
     const int acc = std::min(maxn, kCloseAccNodes);
     size_t shm = sizeof(double) * (3 * (size_t)kCloseChunk + 3 * (size_t)acc);
     BIE_CUDA(c, cudaFuncSetAttribute(k_close_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    BIE_CUDA(c, cudaFuncSetAttribute(k_close_blocks_heavy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
     c->cl.shm_limit = shm;
-    dim3 grid(h[0], (maxn + kCloseAccNodes - 1) / kCloseAccNodes);
-    k_close_blocks<<<grid, 256, shm, c->stream>>>(c->cl.pairs, c->cl.blk_off, c->x, c->y, c->nx, c->ny, c->w,
-                                                  c->body, c->node_cell, c->cells, c->cl.dtab, c->cl.dtab_off,
-                                                  c->cl.blocks, c->cl.blocks32, c->bshape);
+    const int ranges = (maxn + kCloseAccNodes - 1) / kCloseAccNodes;
+    const BlockArgs g{c->cl.pairs, c->cl.blk_off, c->x, c->y, c->nx, c->ny, c->w, c->body, c->node_cell, c->cells,
+                      c->cl.dtab, c->cl.dtab_off, c->cl.blocks, c->cl.blocks32, c->bshape};
+    if ((h[6] - 1LL) * maxn * maxn > kCloseHeavy) {
+        const int clusters = std::min(h[0], std::max(1, 2 * c->sms / kCloseCtas));
+        k_close_blocks_heavy<<<dim3(clusters * kCloseCtas, ranges), 256, shm, c->stream>>>(g, h[0]);
+        BIE_LAUNCH(c, "k_close_blocks_heavy");
+    }
+    k_close_blocks<<<dim3(h[0], ranges), 256, shm, c->stream>>>(g);
     BIE_LAUNCH(c, "k_close_blocks");
     return BIE_OK;
 }
@@ -1232,7 +1336,7 @@ static int finish_launch(bie_ctx* c, const double* sigma, int prec, const Worksp
     a.body = c->body;
     a.bodyF = ws.bodyF;
     a.cells = c->cells;
-    BIE_CUDA(c, launch_after(fmm_chained(c, prec), k_finish<R>, c->n_fin, kFinNodes, c->stream, a, reinterpret_cast<double2*>(yout)));
+    BIE_CUDA(c, launch_after(fmm_chained(c, prec), k_finish<R>, c->n_fin, kFinNodes, 0u, c->stream, a, reinterpret_cast<double2*>(yout)));
     ++c->launches;
     return BIE_OK;
 }

@@ -10,6 +10,8 @@
 // kernel runs over all cells of the batch at once (grid dimension "cell").
 #include <cmath>
 
+#include <cooperative_groups.h>
+
 #include "bie_internal.cuh"
 
 namespace bie {
@@ -246,6 +248,114 @@ __global__ void k_qr(double* __restrict__ Aall, int R, int C, int Qrows, double 
     }
 }
 
+// The same factorisation by a cluster of eight CTAs per cell, the columns dealt round
+// robin and kept in shared memory.  In step k the CTA with column k + 1 reflects it
+// first, forms the next reflector, writes it into every CTA's buffer and arrives at the
+// cluster's barrier; the others arrive at once, and all reflect the rest of their
+// columns before they wait.  A CTA may so be one step behind the others, which read
+// and write the other two of three buffers.  Bound by the chain of two sums over a
+// column, a square root and a division (in one warp: sixteen of them hold the FP64
+// pipe for 2 us) and the barrier: 288 x 96 in 0.42 ms against 1.8 ms on the FP64 pipe of
+// one SM.  The sums are k_qr's in its order, so that a geometry's P stays what it was
+// to the bit (solutions move by 1e-9 with the rounding of an ill-conditioned fit).
+// R <= kQrThreads.
+constexpr int kQrCtas = 8, kQrThreads = 512;
+constexpr size_t kQrShared = 200 * 1024;
+__global__ void __cluster_dims__(kQrCtas, 1, 1) __launch_bounds__(kQrThreads)
+k_qr_cluster(double* __restrict__ Aall, int R, int C, int Qrows, double lam_rel, double* __restrict__ betaall) {
+    extern __shared__ double sm[];
+    __shared__ double red[32], s_beta[3];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), cell = blockIdx.x / kQrCtas;
+    double* A = Aall + (size_t)cell * R * C;
+    double* beta = betaall + (size_t)cell * 2 * C;
+    double* cols = sm;                                      // ceil(C / 8) columns of R
+    const int mine = (C - rank + kQrCtas - 1) / kQrCtas;    // columns rank, rank + 8, ...
+    double* buf = sm + (size_t)((C + kQrCtas - 1) / kQrCtas) * R;  // 3 x R
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    constexpr int kWarps = kQrThreads / 32;
+    for (int c = 0; c < mine; ++c)
+        for (int i = tid; i < Qrows; i += kQrThreads)
+            cols[(size_t)c * R + i] = A[i + (size_t)(rank + kQrCtas * c) * R];
+    // |Q|^2, for every CTA
+    double s0 = 0.0, s1 = 0.0;
+    const int total = Qrows * C;
+    for (int idx = tid; idx < total; idx += 2 * kQrThreads) {
+        const double a = A[idx % Qrows + (size_t)(idx / Qrows) * R];
+        s0 += a * a;
+    }
+    for (int idx = tid + kQrThreads; idx < total; idx += 2 * kQrThreads) {
+        const double a = A[idx % Qrows + (size_t)(idx / Qrows) * R];
+        s1 += a * a;
+    }
+    s0 = warp_sum(s0);
+    s1 = warp_sum(s1);
+    if (lane == 0) {
+        red[wid] = s0;
+        red[wid + kWarps] = s1;
+    }
+    __syncthreads();
+    const double nrm2 = warp_sum(red[lane]);
+    // every CTA has read A, and has started before one writes into it
+    cl.sync();
+    const double lam = lam_rel * sqrt(nrm2);
+    for (int c = 0; c < mine; ++c)
+        for (int i = Qrows + tid; i < R; i += kQrThreads)
+            cols[(size_t)c * R + i] = (i - Qrows == rank + kQrCtas * c) ? lam : 0.0;
+    __syncthreads();
+    auto form = [&](int k) {  // reflector k, by the CTA that has its column
+        double* a = cols + (size_t)(k / kQrCtas) * R;
+        double s = k + tid < R ? a[k + tid] * a[k + tid] : 0.0;
+        s = warp_sum(s);
+        if (lane == 0) red[wid] = s;
+        __syncthreads();
+        if (wid == 0) {
+            s = warp_sum(lane < kWarps ? red[lane] : 0.0);
+            const double akk = a[k], n = sqrt(s), alpha = akk > 0.0 ? -n : n, v0 = akk - alpha;
+            const double vn2 = s - akk * akk + v0 * v0, bk = vn2 > 0.0 ? 2.0 / vn2 : 0.0;
+            __syncwarp();
+            if (lane == 0) {
+                a[k] = v0;
+                beta[k] = bk;
+                beta[C + k] = alpha;
+            }
+            if (lane < kQrCtas) *cl.map_shared_rank(&s_beta[k % 3], lane) = bk;
+        }
+        __syncthreads();
+        if (k + tid < R)
+            for (int q = 0; q < kQrCtas; ++q) cl.map_shared_rank(buf + (size_t)(k % 3) * R, q)[k + tid] = a[k + tid];
+    };
+    if (rank == 0) form(0);
+    cluster_arrive();
+    cluster_wait();
+    for (int k = 0; k < C; ++k) {
+        const double* v = buf + (size_t)(k % 3) * R;
+        const double bk = s_beta[k % 3];
+        auto reflect = [&](int c) {
+            double* aj = cols + (size_t)c * R;
+            double d = 0.0;
+            for (int i = k + lane; i < R; i += 32) d += v[i] * aj[i];
+            d = warp_sum(d) * bk;
+            for (int i = k + lane; i < R; i += 32) aj[i] -= d * v[i];
+        };
+        const int first = k < rank ? 0 : (k - rank) / kQrCtas + 1;
+        const int next = (k + 1 < C && (k + 1) % kQrCtas == rank) ? first : -1;
+        if (next >= 0) {
+            if (wid == 0) reflect(next);
+            __syncthreads();
+            form(k + 1);
+        }
+        cluster_arrive();
+        for (int c = first + (next >= 0) + wid; c < mine; c += kWarps) reflect(c);
+        __syncthreads();
+        cluster_wait();
+    }
+    for (int c = 0; c < mine; ++c)
+        for (int i = tid; i < R; i += kQrThreads) A[i + (size_t)(rank + kQrCtas * c) * R] = cols[(size_t)c * R + i];
+    cl.sync();  // no CTA leaves while another may still write to it
+}
+
 // Column c of P = first C rows of R^{-1} H_{C-1} ... H_0 e_c, c < Qrows, for
 // cell blockIdx.y.  P is C x Qrows per cell, stored row-major
 // (P[r * Qrows + c]) so that a warp reading one row of P in the operator
@@ -367,7 +477,14 @@ int build_proxy_fit_to(bie_ctx* c, ProxyFit& f, cudaStream_t st) {
     }
     k_build_Q<<<dim3((m * M + bs - 1) / bs, c->ncell), bs, 0, st>>>(f.A, R, m, M, c->gl_s, f.yp, c->cells, f.e2);
     BIE_LAUNCH(c, "k_build_Q");
-    k_qr<<<c->ncell, 1024, 0, st>>>(f.A, R, C, Qrows, c->opts.lam_rel, f.beta);
+    // a cluster of CTAs per cell while its columns fit their shared memory
+    const size_t shm = ((size_t)((C + kQrCtas - 1) / kQrCtas) + 3) * R * sizeof(double);
+    if (R <= kQrThreads && shm <= kQrShared) {
+        BIE_CUDA(c, cudaFuncSetAttribute(k_qr_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQrShared));
+        k_qr_cluster<<<c->ncell * kQrCtas, kQrThreads, shm, st>>>(f.A, R, C, Qrows, c->opts.lam_rel, f.beta);
+    } else {
+        k_qr<<<c->ncell, 1024, 0, st>>>(f.A, R, C, Qrows, c->opts.lam_rel, f.beta);
+    }
     BIE_LAUNCH(c, "k_qr");
     k_form_P<<<dim3(Qrows, c->ncell), 256, R * sizeof(double), st>>>(f.A, R, C, f.beta, f.P);
     BIE_LAUNCH(c, "k_form_P");

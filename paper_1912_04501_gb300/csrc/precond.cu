@@ -15,6 +15,8 @@
 #include <numeric>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "bie_internal.cuh"
 
 namespace bie {
@@ -184,20 +186,209 @@ __global__ void k_gj_elim(double* __restrict__ aug, int n, int k, const double* 
         aug[r * ld + j] -= f[r] * prow[j];
 }
 
-// z = M^-1 v: 2 v outside S ...
-__global__ void k_pc_scale(const double* __restrict__ v, const int* __restrict__ pos, double* __restrict__ z,
-                           int n2) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n2) return;
-    if (pos[e >> 1] < 0) z[e] = 2.0 * v[e];
+// The whole inversion in one launch by a cluster of NC CTAs, for blocks whose n x n
+// entries fit their shared memory (n <= kGjMost<NC>): Gauss-Jordan in place with the
+// same pivots.  Columns are dealt round robin.  In step k every CTA swaps its rows and
+// scales row k; the one with column k + 1 eliminates there first, finds the next pivot
+// row and writes it and the column into every CTA's buffer; all arrive at the cluster's
+// barrier and eliminate in the rest of their columns before they wait (three buffers,
+// as in k_qr_cluster).  In place the columns
+// come out permuted by the row swaps; the result goes to the right half of [M | I],
+// where k_pc_apply reads it.  Bound by the FP64 pipe of its SMs, n^2 / NC fma a step,
+// so by sixteen CTAs where the device takes such a cluster, and by the chain from one
+// column's pivot to the next.  (Two launches per column: n = 204 took 2.9 ms, 0.95 so;
+// 1.8 with the next pivot after the elimination instead of beside it.)
+constexpr int kGjThreads = 512;
+template <int NC>
+constexpr int kGjMost = NC == 16 ? 640 : 448;
+template <int kGjCtas>
+__global__ void __launch_bounds__(kGjThreads)
+k_gj_cluster(double* __restrict__ aug, int n, int* __restrict__ status) {
+    constexpr int kGjMax = kGjMost<kGjCtas>;
+    extern __shared__ double sm[];
+    __shared__ double sv[32], s_inv[3];
+    __shared__ int si[32], s_piv[3], s_p[kGjMax], s_cur[kGjMax];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int mine = (n - rank + kGjCtas - 1) / kGjCtas, most = (n + kGjCtas - 1) / kGjCtas;
+    const long long ld = 2LL * n;
+    double* cols = sm;                         // most columns of n
+    double* buf = sm + (size_t)most * n;       // 3 x n: column k as published
+    double* row = buf + 3 * (size_t)n;         // most: this CTA's part of row k, scaled
+    for (int i = wid; i < n; i += kGjThreads / 32)
+        for (int c = lane; c < mine; c += 32) cols[(size_t)c * n + i] = aug[i * ld + rank + kGjCtas * c];
+    __syncthreads();
+    cl.sync();  // every CTA has started before one writes into it
+    auto publish = [&](int k) {  // pivot of column k and the column, by the CTA that has it
+        const double* a = cols + (size_t)(k / kGjCtas) * n;
+        const int z = k % 3;
+        double best = -1.0;
+        int bi = n;
+        for (int r = k + tid; r < n; r += kGjThreads) {
+            const double v = fabs(a[r]);
+            if (v > best) {
+                best = v;
+                bi = r;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (ov > best || (ov == best && oi < bi)) {
+                best = ov;
+                bi = oi;
+            }
+        }
+        if (lane == 0) {
+            sv[wid] = best;
+            si[wid] = bi;
+        }
+        for (int q = 0; q < kGjCtas; ++q) {
+            double* to = cl.map_shared_rank(buf + (size_t)z * n, q);
+            for (int i = tid; i < n; i += kGjThreads) to[i] = a[i];
+        }
+        __syncthreads();
+        if (wid == 0) {  // (one warp divides: sixteen of them would hold the FP64 pipe for 2 us)
+            double bv = lane < kGjThreads / 32 ? sv[lane] : -1.0;
+            int bx = lane < kGjThreads / 32 ? si[lane] : n;
+            for (int o = 16; o > 0; o >>= 1) {
+                const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, bx, o);
+                if (ov > bv || (ov == bv && oi < bx)) {
+                    bv = ov;
+                    bx = oi;
+                }
+            }
+            const int p = (bv > 0.0 && isfinite(bv)) ? bx : -1;
+            const double inv = p >= 0 ? 1.0 / a[p] : 0.0;
+            if (lane < kGjCtas) {
+                *cl.map_shared_rank(&s_piv[z], lane) = p;
+                *cl.map_shared_rank(&s_inv[z], lane) = inv;
+            }
+        }
+    };
+    if (rank == 0) publish(0);
+    cluster_arrive();
+    cluster_wait();
+    bool bad = false;
+    for (int k = 0; k < n; ++k) {
+        const int z = k % 3, p = s_piv[z];
+        if (p < 0) {  // the same in every CTA
+            if (rank == 0 && tid == 0) *status = 1;
+            bad = true;
+            break;
+        }
+        const double inv = s_inv[z];
+        const double* f = buf + (size_t)z * n;  // column k before the swap
+        // row k of this CTA's columns after the swap, scaled; row p takes the old row k
+        for (int c = tid; c < mine; c += kGjThreads) {
+            double* a = cols + (size_t)c * n;
+            const double ap = a[p], ak = a[k];
+            a[p] = ak;
+            const bool self = rank + kGjCtas * c == k;
+            const double rk = self ? inv : ap * inv;
+            a[k] = rk;
+            row[c] = rk;
+        }
+        if (tid == 0) s_p[k] = p;
+        __syncthreads();
+        // the other rows: a_ij -= f_i row_j, and column k itself becomes -f_i / pivot
+        const double fk = f[k];
+        const int next = (k + 1 < n && (k + 1) % kGjCtas == rank) ? (k + 1) / kGjCtas : -1;
+        if (next >= 0) {
+            double* a = cols + (size_t)next * n;
+            const double rk = row[next];
+            for (int i = tid; i < n; i += kGjThreads)
+                if (i != k) a[i] = fma(-(i == p ? fk : f[i]), rk, a[i]);
+            __syncthreads();
+            publish(k + 1);
+        }
+        cluster_arrive();
+        for (int c = wid; c < mine; c += kGjThreads / 32) {
+            if (c == next) continue;
+            double* a = cols + (size_t)c * n;
+            const double rk = row[c];
+            if (rank + kGjCtas * c == k) {
+                for (int i = lane; i < n; i += 32)
+                    if (i != k) a[i] = -(i == p ? fk : f[i]) * rk;
+            } else {
+#pragma unroll 4
+                for (int i = lane; i < n; i += 32)
+                    if (i != k) a[i] = fma(-(i == p ? fk : f[i]), rk, a[i]);
+            }
+        }
+        __syncthreads();
+        cluster_wait();
+    }
+    if (bad) {
+        cl.sync();
+        return;
+    }
+    // column of the inverse that each in-place column is
+    if (tid == 0) {
+        for (int j = 0; j < n; ++j) s_cur[j] = j;
+        for (int k = n - 1; k >= 0; --k) {
+            const int p = s_p[k], q = s_cur[k];
+            s_cur[k] = s_cur[p];
+            s_cur[p] = q;
+        }
+    }
+    __syncthreads();
+    for (int j = wid; j < n; j += kGjThreads / 32) {
+        const int c = s_cur[j];
+        if (c % kGjCtas != rank) continue;
+        const double* a = cols + (size_t)(c / kGjCtas) * n;
+        for (int i = lane; i < n; i += 32) aug[i * ld + n + j] = a[i];
+    }
+    cl.sync();  // no CTA leaves while another may still write to it
 }
 
-// ... and A_SS^-1 v_S on S: one warp per row of the inverse (the right half
-// of the eliminated [M | I]).
-__global__ void k_pc_inv(const double* __restrict__ aug, int s, const int* __restrict__ nodes,
-                         const double* __restrict__ v, double* __restrict__ z) {
+// *done: whether the block fits such a cluster and the device takes it.
+template <int NC>
+static int gj_in_cluster(bie_ctx* c, int n, bool* done) {
+    if (n > kGjMost<NC>) return BIE_OK;
+    const int most = (n + NC - 1) / NC;
+    const size_t shm = ((size_t)most * n + 3 * (size_t)n + most) * sizeof(double);
+    BIE_CUDA(c, cudaFuncSetAttribute(k_gj_cluster<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    if (NC > 8) BIE_CUDA(c, cudaFuncSetAttribute(k_gj_cluster<NC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = NC;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(NC);
+    cfg.blockDim = dim3(kGjThreads);
+    cfg.dynamicSmemBytes = shm;
+    cfg.stream = c->stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, k_gj_cluster<NC>, &cfg) != cudaSuccess || clusters < 1) {
+        cudaGetLastError();
+        return BIE_OK;
+    }
+    BIE_CUDA(c, cudaLaunchKernelEx(&cfg, k_gj_cluster<NC>, c->pc.aug, n, c->pc.status));
+    ++c->launches;
+    *done = true;
+    return BIE_OK;
+}
+
+// z = M^-1 v: A_SS^-1 v_S on S, one warp per row of the inverse (the right half of
+// the eliminated [M | I]), and 2 v outside S, by the CTAs past those (one launch: in an
+// iteration of 80 us a second one was 2.4).
+__global__ void __launch_bounds__(256)
+k_pc_apply(const double* __restrict__ aug, int s, const int* __restrict__ nodes, const int* __restrict__ pos,
+           const double* v, double* z, int n2) {
+    pdl_wait();
+    pdl_trigger();
+    const int n = 2 * s, rows = (32 * n + 255) / 256;
+    if ((int)blockIdx.x >= rows) {
+        const int e = (blockIdx.x - rows) * blockDim.x + threadIdx.x;
+        if (e < n2 && pos[e >> 1] < 0) z[e] = 2.0 * v[e];
+        return;
+    }
     const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    const int n = 2 * s;
     if (row >= n) return;
     const double* a = aug + (long long)row * 2 * n + n;
     double acc = 0.0;
@@ -208,10 +399,9 @@ __global__ void k_pc_inv(const double* __restrict__ aug, int s, const int* __res
 
 int precond_apply(bie_ctx* c, const double* v, double* z) {
     const int n2 = 2 * c->N, s = c->pc.s;
-    k_pc_scale<<<(n2 + 255) / 256, 256, 0, c->stream>>>(v, c->pc.pos, z, n2);
-    BIE_LAUNCH(c, "k_pc_scale");
-    k_pc_inv<<<(2 * s * 32 + 255) / 256, 256, 0, c->stream>>>(c->pc.aug, s, c->pc.nodes, v, z);
-    BIE_LAUNCH(c, "k_pc_inv");
+    BIE_CUDA(c, launch_after(true, k_pc_apply, (64 * s + 255) / 256 + (n2 + 255) / 256, 256u, 0u, c->stream, c->pc.aug, s,
+                             c->pc.nodes, c->pc.pos, v, z, n2));
+    ++c->launches;
     return BIE_OK;
 }
 
@@ -269,14 +459,20 @@ int build_precond(bie_ctx* c) {
                                                                c->pc.aug);
         BIE_LAUNCH(c, "k_pc_close");
     }
-    for (int k = 0; k < n; ++k) {
-        const long long work = (long long)n * (2 * n - k);
-        k_gj_pivot<<<1, 1024, 0, c->stream>>>(c->pc.aug, n, k, c->pc.f, c->pc.prow, c->pc.status);
-        k_gj_elim<<<(int)((work + 255) / 256), 256, 0, c->stream>>>(c->pc.aug, n, k, c->pc.f, c->pc.prow,
-                                                                     c->pc.status);
+    bool done = false;
+    if (int rc = gj_in_cluster<16>(c, n, &done)) return rc;
+    if (!done)
+        if (int rc = gj_in_cluster<8>(c, n, &done)) return rc;
+    if (!done) {
+        for (int k = 0; k < n; ++k) {
+            const long long work = (long long)n * (2 * n - k);
+            k_gj_pivot<<<1, 1024, 0, c->stream>>>(c->pc.aug, n, k, c->pc.f, c->pc.prow, c->pc.status);
+            k_gj_elim<<<(int)((work + 255) / 256), 256, 0, c->stream>>>(c->pc.aug, n, k, c->pc.f, c->pc.prow,
+                                                                         c->pc.status);
+        }
+        BIE_LAUNCH(c, "k_gj");
+        c->launches += 2LL * n - 1;
     }
-    BIE_LAUNCH(c, "k_gj");
-    c->launches += 2LL * n - 1;
     int status = 0;
     BIE_CUDA(c, cudaMemcpyAsync(&status, c->pc.status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     BIE_CUDA(c, cudaStreamSynchronize(c->stream));
