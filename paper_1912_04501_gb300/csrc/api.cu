@@ -497,7 +497,7 @@ int bie_init_batch(bie_ctx** out, int32_t n_cells, const bie_cell* cells, const 
     rc = rc ? rc : dalloc(c, &c->sv.d, 2 * (size_t)n);
     {
         const size_t slot = (2 * (size_t)(kk + 1 + kMaxAug) + 1) * nc;
-        rc = rc ? rc : dalloc(c, &c->sv.h, 2 * slot + (size_t)(kk + kMaxAug) * nc);
+        rc = rc ? rc : dalloc(c, &c->sv.h, (size_t)(kk + kMaxAug) * nc);
         rc = rc ? rc : dalloc(c, &c->sv.fac, (4 + 3 * (size_t)kMaxAug) * nc);
         if (!rc) rc = cu(cudaMallocHost((void**)&c->sv.pinned, 2 * slot * sizeof(double)), "cudaMallocHost");
         for (int e = 0; e < 2 && !rc; ++e)

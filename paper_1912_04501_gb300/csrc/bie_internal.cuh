@@ -61,7 +61,8 @@ static_assert(kNear32Shapes == BIE_NEAR32_SHAPES, "shape count of the public hea
 constexpr int kNear32CompChunk = 2048;  // splits with more sources use compensated tile accumulation
 constexpr int kDiscSplits = 8;        // source splits per wall point of the wall-discrepancy kernel
 constexpr int kVelSplits = 8;         // source splits per body in the velocity extraction
-constexpr int kDotChunk = 256;        // vector entries per partial dot product (chunks never span cells)
+constexpr int kDotChunk = 128;        // vector entries per partial dot product: a multiple of it (chunks never
+constexpr int kDotMax = 4096;         // span cells), at most kDotMax
 constexpr int kMaxProxy = 256;
 constexpr int kMaxColl = 128;
 constexpr int kFinNodes = 128;        // nodes per CTA of the assembly (chunks never span cells)
@@ -153,11 +154,11 @@ struct Workspace {
     unsigned int* dticket = nullptr;  // ncell x 2m last-block counters of k_disc (zero between launches)
     double* xi = nullptr;       // ncell x 2M proxy strengths
     float* xif = nullptr;       // ncell x 2M the same in single precision
-    double* T = nullptr;        // 2N; alpha per cell (k_alpha32)
     double* vpart = nullptr;    // nb x kVelSplits x 3 velocity partials
     // fast image sum: sorted strengths, multipole and local expansions, and
     // the last-child counters of the upward pass (zero between launches)
     void* psum = nullptr;       // close pairs' sums (null: Close::psum)
+    double* T = nullptr;        // 2N; alpha per cell (k_alpha32)
     void *fsq = nullptr, *fmp = nullptr, *floc = nullptr;
     unsigned* ftick = nullptr;
 };
@@ -195,16 +196,16 @@ struct Solver {
     double* x = nullptr;     // 2N current solution
     double* b = nullptr;     // 2N right-hand side
     double* d = nullptr;     // 2N correction (mixed)
-    double* h = nullptr;     // 2 slots of (2 (kmax + 1 + kMaxAug) + 1) x ncell projections, then
-                             // (kmax + kMaxAug) x ncell combination coefficients
-    double* pinned = nullptr;  // host (page-locked): 2 slots, as on the device
+    double* h = nullptr;     // (kmax + kMaxAug) x ncell combination coefficients
+    double* pinned = nullptr;  // host (page-locked): 2 slots of (2 (kmax + 1 + kMaxAug) + 1) x ncell projections
     double* fac = nullptr;   // (4 + 3 kMaxAug) x ncell: normalisation factors, per-cell norms, scratch
-    cudaEvent_t ev[2] = {nullptr, nullptr};  // slot k % 2 copied to the host
+    cudaEvent_t ev[2] = {nullptr, nullptr};  // slot k % 2 written
     unsigned int* ticket = nullptr;  // last-block counter of k_dots (zero between launches)
-    double* dpart = nullptr; // (kmax + 2) x nchunks partial dot products
+    double* dpart = nullptr; // 2 x (kmax + 2 + kMaxAug) x nchunks partial dot products
     int4* chunks = nullptr;  // nchunks: (cell, first entry, end entry, 0)
     int2* cell_chunks = nullptr;  // ncell: (first chunk, chunk count)
     int nchunks = 0;
+    int chunk = 0;           // entries of a chunk
     double* sigma_prev = nullptr;  // 2N the last step's density (warm start of the next)
     double* sigma_prev2 = nullptr; // 2N the density of the step before
     bool have_prev = false, have_prev2 = false;

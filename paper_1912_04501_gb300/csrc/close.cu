@@ -1252,6 +1252,7 @@ k_finish(Finish<R> a, double2* __restrict__ out) {
         }
     }
     pdl_wait();
+    pdl_trigger();
     for (int p = t; p < a.M; p += kFinNodes) {
         if constexpr (sizeof(R) == 4) {
             const float* xi = a.xif + (size_t)ch.x * 2 * a.M;

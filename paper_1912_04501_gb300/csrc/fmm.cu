@@ -343,7 +343,7 @@ constexpr int kFmmDirect = sizeof(R) == 4 ? 128 : 256;
 
 template <typename R>
 __global__ void __launch_bounds__(128)
-k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ sigma, const double* __restrict__ w,
+k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* sigma, const double* __restrict__ w,
          int shift, C2<R>* __restrict__ sq, V4<R>* __restrict__ mp, unsigned* __restrict__ ticket, FmmTab<R> tab,
          FmmBodies bodies) {
     constexpr int P = FmmTypes<R>::P, G = kFmmItems / P, PER = 32 / G, HI = P / 4;
@@ -360,6 +360,7 @@ k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* __restrict__ 
     // children's translated series
     R* s_sum = reinterpret_cast<R*>(&sh);
     static_assert(4 * kFmmItems * 6 * sizeof(R) <= sizeof(Tables), "sums");
+    pdl_wait();
     pdl_trigger();
     if ((int)blockIdx.x >= t.nbox) {
         fmm_body(bodies, blockIdx.x - t.nbox, cells, sigma, w);
@@ -1865,10 +1866,10 @@ static int up_launch(bie_ctx* c, const double* sigma, int prec, Workspace& ws) {
     FmmBodies p{c->x, c->y, c->body, c->body_cell, nullptr, nullptr, ws.bodyF};
     if (!f.walls && prec == 0) p.src32 = c->utilde ? ws.src32n : ws.src32;
     if (!f.walls || prec != 0) p.src64 = ws.src64;
-    k_fmm_up<R><<<f.t.nbox + c->nb, 128, 0, c->stream>>>(f.t, c->cells, reinterpret_cast<const double2*>(sigma), c->w,
+    BIE_CUDA(c, launch_after(fmm_chained(c, prec), k_fmm_up<R>, f.t.nbox + c->nb, 128, 0u, c->stream, f.t, c->cells, reinterpret_cast<const double2*>(sigma), c->w,
                                                           c->utilde ? 2 : 0, (C2<R>*)ws.fsq, (V4<R>*)ws.fmp, ws.ftick,
-                                                          fmm_tab<R>(c, prec), p);
-    BIE_LAUNCH(c, "k_fmm_up");
+                                                          fmm_tab<R>(c, prec), p));
+    ++c->launches;
     return BIE_OK;
 }
 

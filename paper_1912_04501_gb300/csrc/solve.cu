@@ -38,15 +38,21 @@ __device__ inline double wsum(double v) {
     return v;
 }
 
-// Reduction chunks of kDotChunk vector entries that never span two cells.
+// Reduction chunks of the vectors, a multiple of kDotChunk entries that never spans
+// two cells: about one chunk per SM, so that the partial sums of a vector, which
+// every CTA of k_project adds up for itself, stay few (at most kDotMax entries, which
+// its shared memory holds).
 int build_dot_chunks(bie_ctx* c) {
     std::vector<int4> ch;
     std::vector<int2> cc(c->ncell);
+    const long long per = (2LL * c->N + c->sms - 1) / std::max(1, c->sms);
+    const int chunk = (int)std::min<long long>(kDotMax, std::max<long long>(1, (per + kDotChunk - 1) / kDotChunk) * kDotChunk);
+    c->sv.chunk = chunk;
     for (int ci = 0; ci < c->ncell; ++ci) {
         const Cell& cl = c->cells_h[ci];
         const int e0 = 2 * cl.node_off, e1 = 2 * (cl.node_off + cl.n_nodes);
         cc[ci] = make_int2((int)ch.size(), 0);
-        for (int e = e0; e < e1; e += kDotChunk) ch.push_back(make_int4(ci, e, std::min(e1, e + kDotChunk), 0));
+        for (int e = e0; e < e1; e += chunk) ch.push_back(make_int4(ci, e, std::min(e1, e + chunk), 0));
         cc[ci].y = (int)ch.size() - cc[ci].x;
     }
     std::vector<int4> fin;  // the assembly's chunks of nodes
@@ -60,7 +66,7 @@ int build_dot_chunks(bie_ctx* c) {
     c->sv.nchunks = (int)ch.size();
     BIE_CUDA(c, cudaMalloc((void**)&c->sv.chunks, ch.size() * sizeof(int4)));
     BIE_CUDA(c, cudaMalloc((void**)&c->sv.cell_chunks, cc.size() * sizeof(int2)));
-    BIE_CUDA(c, cudaMalloc((void**)&c->sv.dpart, (size_t)(c->sv.kmax + 2 + kMaxAug) * ch.size() * sizeof(double)));
+    BIE_CUDA(c, cudaMalloc((void**)&c->sv.dpart, 2 * (size_t)(c->sv.kmax + 2 + kMaxAug) * ch.size() * sizeof(double)));
     BIE_CUDA(c, cudaMemcpy(c->sv.chunks, ch.data(), ch.size() * sizeof(int4), cudaMemcpyHostToDevice));
     BIE_CUDA(c, cudaMemcpy(c->sv.cell_chunks, cc.data(), cc.size() * sizeof(int2), cudaMemcpyHostToDevice));
     return BIE_OK;
@@ -68,7 +74,7 @@ int build_dot_chunks(bie_ctx* c) {
 
 // Classical Gram-Schmidt building blocks for every cell at once.
 // k_dots: block (b, g) writes the partial dot products V_j . w over reduction
-// chunk b (kDotChunk entries of one cell) for the eight vectors j = 8g .. 8g+7
+// chunk b (entries of one cell) for the eight vectors j = 8g .. 8g+7
 // (one warp each); V = w with nv = 1 gives the partial squared norms.  With a
 // ticket, the last block to finish also forms the sums of k_fin (below) in
 // the same fixed order, saving a launch when there are few of them.
@@ -102,11 +108,13 @@ __device__ void fin_items(const double* __restrict__ part, int nchunks, int nv, 
 }
 
 __global__ void __launch_bounds__(256)
-k_dots(const double* __restrict__ V, size_t ld, int nv, const double* __restrict__ w,
+k_dots(const double* __restrict__ V, size_t ld, int nv, const double* w,
        const int4* __restrict__ chunks, int nchunks, double* __restrict__ part, unsigned int* __restrict__ ticket,
        const int2* __restrict__ cell_chunks, int ncell, double* __restrict__ h, const Cell* __restrict__ cells,
        double* __restrict__ fac) {
     __shared__ bool last;
+    pdl_wait();
+    pdl_trigger();
     const int j = blockIdx.y * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (j < nv) {
         const int4 ch = chunks[blockIdx.x];
@@ -169,6 +177,110 @@ static int mdots(bie_ctx* c, const double* V, size_t ld, int nv, const double* w
         BIE_LAUNCH(c, "k_fin");
     }
     return BIE_OK;
+}
+
+// One Gram-Schmidt pass, a CTA per reduction chunk: h_j = the cell's partials of
+// V_j . w (every CTA adds them for itself, in the same order; the cell's first one
+// writes them to h) and w -= sum_j h_j V_j on the chunk.  The first pass (dst null)
+// stores w and the new partials V_j . w and w . w.  The second one has
+// |w - V h|^2 = |w|^2 - |h|^2, V's vectors being orthonormal (the Pythagorean form,
+// Smoktunowicz, Barlow and Langou 2006; after a first pass h is small against w), and
+// writes the normalised vector to dst, zeros for a cell that is switched off.
+//
+// Bound by latency: V comes from L2 once, and from L1 for the new sums.  (The chunk of V
+// copied to shared memory while the launch before still ran was slower, step-wise by 5 %:
+// the SMs' split of L1 and shared memory changed with every launch.)  Orthogonalising
+// one vector of 12800 entries against 1 to 60 takes 24 us, launch by launch, against 32
+// in six launches, each of the three sums ended by one block adding everyone's partials.
+// Dynamic shared memory: chunk + kProjThreads + min(nv, kProjVecs) doubles, 45 KB at most.
+constexpr int kProjThreads = 512, kProjVecs = 1024;
+__global__ void __launch_bounds__(kProjThreads)
+k_project(const double* V, size_t ld, int nv, double* w, const double* pin, double* pout, const int4* chunks,
+          int nchunks, const int2* cell_chunks, int ncell, double* h, int chunk, const Cell* cells, double* hn,
+          double* dst) {
+    extern __shared__ double sm[];
+    __shared__ double s_f;
+    double* ws = sm;
+    double* red = ws + chunk;
+    double* hs = red + kProjThreads;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int4 ch = chunks[blockIdx.x];
+    const int2 cc = cell_chunks[ch.x];
+    const int len = ch.z - ch.y;
+    pdl_wait();
+    pdl_trigger();
+    // sums of one vector's partials by 16 threads
+    auto total = [&](int j, bool on) {
+        double s = 0;
+        if (on) {
+            const double* pp = pin + (size_t)j * nchunks + cc.x;
+#pragma unroll 8
+            for (int b = tid & 15; b < cc.y; b += 16) s += pp[b];
+        }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        return s;
+    };
+    // |w|^2 goes with the vectors' sums
+    double norm = 0;
+    if (dst && wid == 0) norm = total(nv, true);
+    // tiles of 128 entries, four threads per entry over the vectors, kProjVecs
+    // vectors at a time
+    constexpr int kT = kProjThreads / 4;
+    const int e = tid % kT, sub = tid / kT;
+    for (int jb = 0; jb < nv; jb += kProjVecs) {
+        const int je = min(nv, jb + kProjVecs);
+        for (int j0 = jb; j0 < je; j0 += kProjThreads / 16) {
+            const int j = j0 + (tid >> 4);
+            const double s = total(j, j < je);
+            if (j < je && (tid & 15) == 0) {
+                hs[j - jb] = s;
+                if (blockIdx.x == cc.x) h[(size_t)j * ncell + ch.x] = s;
+            }
+        }
+        __syncthreads();
+        if (dst && wid == 0) {
+            double q = 0;
+            for (int j = lane; j < je - jb; j += 32) q = fma(hs[j], hs[j], q);
+            norm -= wsum(q);
+            if (je == nv && lane == 0) {
+                s_f = (cells[ch.x].active && norm > 0) ? 1.0 / sqrt(norm) : 0.0;
+                // (a NaN stays one: the host looks for it)
+                if (blockIdx.x == cc.x) hn[ch.x] = norm < 0 ? 0.0 : norm;
+            }
+        }
+        for (int i0 = 0; i0 < len; i0 += kT) {
+            const int q = i0 + e;
+            const bool in = q < len;
+            double s = 0;
+            if (in) {
+                const double* v = V + ch.y + q;
+#pragma unroll 8
+                for (int j = jb + sub; j < je; j += 4) s = fma(hs[j - jb], v[(size_t)j * ld], s);
+            }
+            red[tid] = s;
+            __syncthreads();
+            if (sub == 0 && in) {
+                const double old = jb ? ws[q] : w[ch.y + q];
+                const double nw = old - ((red[e] + red[e + kT]) + (red[e + 2 * kT] + red[e + 3 * kT]));
+                ws[q] = nw;
+                if (je == nv) {
+                    if (!dst) w[ch.y + q] = nw;
+                    else dst[ch.y + q] = s_f == 0.0 ? 0.0 : s_f * nw;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    if (dst) return;
+    for (int j = wid; j <= nv; j += kProjThreads / 32) {
+        const double* v = j == nv ? ws : V + (size_t)j * ld + ch.y;
+        double s = 0;
+#pragma unroll 4
+        for (int q = lane; q < len; q += 32) s = fma(v[q], ws[q], s);
+        s = wsum(s);
+        if (lane == 0) pout[(size_t)j * nchunks + blockIdx.x] = s;
+    }
 }
 
 // dst = a[cell] src; a zero factor writes zeros (switched-off cells)
@@ -341,7 +453,7 @@ static int gmres_cycle(bie_ctx* c, int prec, double* x, const double* r, const s
     double* Ut = Vk + (size_t)(kmax + 1) * ld;
     double* w = c->sv.w;
     double* fac_d = c->sv.fac;
-    double* coef = c->sv.h + 2 * slot;  // (kmax + kMaxAug) x nc combination coefficients
+    double* coef = c->sv.h;  // (kmax + kMaxAug) x nc combination coefficients
     std::vector<double> beta = beta_in;
     std::vector<double> acoef((size_t)nu * nc, 0.0);  // C~^T r, per direction and cell
     it.assign(nc, 0);
@@ -411,24 +523,25 @@ static int gmres_cycle(bie_ctx* c, int prec, double* x, const double* r, const s
         }
         ++*n_apply;
         const int nv = nu + k + 1;
-        double* hb = c->sv.h + (size_t)(k & 1) * slot;
+        // k_project writes the projections to the page-locked slot itself
+        double* hb = c->sv.pinned + (size_t)(k & 1) * slot;
         double* h1 = hb;
         double* h2 = hb + (size_t)nv * nc;
         double* hn = hb + 2 * (size_t)nv * nc;
-        // CGS2: two projections, then the norm and the normalisation factor
-        const int gu = (int)((8LL * n + 255) / 256);
-        if (int rc = mdots(c, V, ld, nv, w, h1, nullptr)) return rc;
-        k_update<<<gu, 256, 0, c->stream>>>(V, ld, nv, h1, nc, c->node_cell, w, n);
-        BIE_LAUNCH(c, "k_update");
-        if (int rc = mdots(c, V, ld, nv, w, h2, nullptr)) return rc;
-        k_update<<<gu, 256, 0, c->stream>>>(V, ld, nv, h2, nc, c->node_cell, w, n);
-        BIE_LAUNCH(c, "k_update");
-        if (int rc = mdots(c, w, 0, 1, w, hn, fac_d)) return rc;
-        k_scale_copy<<<gs, bs, 0, c->stream>>>(w, fac_d, c->node_cell, Vk + (size_t)(k + 1) * ld, n);
-        BIE_LAUNCH(c, "k_scale_copy");
-        BIE_CUDA(c, cudaMemcpyAsync(c->sv.pinned + (size_t)(k & 1) * slot, hb,
-                                    (2 * (size_t)nv + 1) * nc * sizeof(double), cudaMemcpyDeviceToHost,
-                                    c->stream));
+        // CGS2: two projections, then the norm and the normalisation
+        const int nch = c->sv.nchunks;
+        double* p0 = c->sv.dpart;
+        double* p1 = p0 + (size_t)(kmax + 2 + kMaxAug) * nch;
+        const size_t shm = ((size_t)std::min(nv, kProjVecs) + c->sv.chunk + kProjThreads) * sizeof(double);
+        BIE_CUDA(c, launch_after(true, k_dots, dim3(nch, (nv + 7) / 8), 256u, 0u, c->stream, V, ld, nv, w, c->sv.chunks,
+                                 nch, p0, nullptr, c->sv.cell_chunks, nc, nullptr, c->cells, nullptr));
+        ++c->launches;
+        for (int pass = 0; pass < 2; ++pass) {
+            BIE_CUDA(c, launch_after(true, k_project, (unsigned)nch, (unsigned)kProjThreads, (unsigned)shm, c->stream, V, ld,
+                                     nv, w, pass ? p1 : p0, p1, c->sv.chunks, nch, c->sv.cell_chunks, nc, pass ? h2 : h1,
+                                     c->sv.chunk, c->cells, hn, pass ? Vk + (size_t)(k + 1) * ld : nullptr));
+            ++c->launches;
+        }
         BIE_CUDA(c, cudaEventRecord(c->sv.ev[k & 1], c->stream));
         return BIE_OK;
     };
