@@ -293,7 +293,8 @@ int bie_set_history(bie_ctx* ctx, const double* sigma_prev2, const double* d2, d
 
 /* bie_apply_static: the same operator application as
  * bie_apply(ctx, sigma, out, BIE_MIXED, 1), but it allocates no device memory
- * at all and does not touch the per-call buffers that bie_init allocated.  It
+ * at all and, but for the fast image sum's moments and the close pairs' sums,
+ * does not touch the per-call buffers that bie_init allocated.  It
  * has no counterpart in the paper; it exists for callers that may not call
  * cudaMalloc -- for instance code running inside a host application whose own
  * memory manager owns the device heap and forbids other allocations -- yet

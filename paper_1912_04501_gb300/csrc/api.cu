@@ -39,7 +39,7 @@ static void free_all(bie_ctx* c) {
                     c->next.ypf, c->glc, c->contour_part, c->bshape, c->near_ctr, c->fin_chunks,
                     c->gl_s, c->A, c->beta, c->P, c->wall, c->e2d, c->next.A, c->next.beta, c->next.P,
                     c->next.wall, c->next.e2, c->yp, c->ypf, c->scal, c->ws.sigma, c->ws.out, c->ws.src64, c->ws.src32,
-                    c->ws.srcdf, c->ws.bodyF, c->ws.part, c->ws.gpart, c->ws.gt, c->ws.dticket, c->sv.ticket, c->ws.xi, c->ws.xif, c->ws.T, c->ws.vpart, c->sv.V,
+                    c->ws.srcdf, c->ws.bodyF, c->ws.part, c->ws.gpart, c->ws.gt, c->ws.dticket, c->sv.ticket, c->ws.xi, c->ws.xif, c->ws.vpart, c->sv.V,
                     c->sv.w, c->sv.r, c->sv.x, c->sv.b, c->sv.d, c->sv.h, c->sv.fac, c->sv.dpart,
                     c->sv.chunks,
                     c->sv.cell_chunks, c->sv.sigma_prev, c->sv.sigma_prev2, c->sv.aug, c->sv.d2,
@@ -487,7 +487,6 @@ int bie_init_batch(bie_ctx** out, int32_t n_cells, const bie_cell* cells, const 
     rc = rc ? rc : dalloc(c, &c->sv.ticket, 1);
     if (!rc) rc = cu(cudaMemset(c->ws.dticket, 0, nc * 2 * m * sizeof(unsigned int)), "cudaMemset");
     if (!rc) rc = cu(cudaMemset(c->sv.ticket, 0, sizeof(unsigned int)), "cudaMemset");
-    rc = rc ? rc : dalloc(c, &c->ws.T, 2 * (size_t)n);
     rc = rc ? rc : dalloc(c, &c->ws.vpart, nbs * kVelSplits * 3);
     rc = rc ? rc : dalloc(c, &c->sv.V, (size_t)(kk + 1 + 2 * kMaxAug) * 2 * n);
     rc = rc ? rc : dalloc(c, &c->sv.w, 2 * (size_t)n);

@@ -15,7 +15,6 @@
 //                   g~ = g0 - g, Sec. 6.2 step 3)
 //   k_xi            (auxiliary stream) xi = P g~ per (row, cell) (Sec. 6.2 step 3)
 // then (close.cu), after the direct single-precision sum:
-//   k_alpha32       alpha = -T_0 . n_0 per cell
 //   k_assemble32    per target: T = partials + on-curve diagonal + proxy traction
 //                   (step 4) + close evaluation (Sec. 6.3) with the own-body and
 //                   close pairs redone from positions differenced in double-float;
@@ -1170,6 +1169,10 @@ static int near_ctas_per_sm(int shape32, int prec, bool ut = false) {
 // time wins: waves x (longest source chunk + a per-item overhead of
 // kItemOverhead sources).  Deterministic: no timing is involved.
 static constexpr int kItemOverhead = 32;
+// Sources of the shortest split.  A cell of few hundred nodes has one to a few
+// target tiles, and its sum then lasts as long as one item: with 64 the
+// double-precision sum at 128 nodes took 460 us on two SMs.
+static constexpr int kMinChunk = 16;
 
 // srcmul: source records per node (4 for the doubled-cell image records).
 static void choose_splits(const std::vector<Cell>& cells, int tile, int slots, std::vector<int>& splits,
@@ -1185,7 +1188,7 @@ static void choose_splits(const std::vector<Cell>& cells, int tile, int slots, s
             const int n = cells[k].n_nodes, ns = srcmul * n;
             const int tiles = (n + tile - 1) / tile;
             const double share = (double)w * slots * ((double)n * n / W) / tiles;
-            const int s = std::max(1, std::min((ns + 63) / 64, (int)share));
+            const int s = std::max(1, std::min((ns + kMinChunk - 1) / kMinChunk, (int)share));
             sp[k] = s;
             items += (long long)tiles * s;
             maxchunk = std::max(maxchunk, (ns + s - 1) / s);

@@ -1,10 +1,11 @@
 // bie_apply_static: the single-precision-pair operator application with no
 // device allocation.  Every per-call buffer (source records, near-sum
-// partials, wall-discrepancy partials, body moments, proxy strengths,
-// traction) lives in one file-scope static device array.  Of the context it
-// reads the geometry, proxy fit, close tables and work items; it writes only
-// its launch counter and, with bie_profile on, the profiler's event state, so
-// calls on one context must not overlap (as for every entry point).  See
+// partials, wall-discrepancy partials, body moments, proxy strengths) lives in one file-scope static device array, but for the moments of the
+// fast image sum and the close pairs' sums, whose space the context has had since it
+// was made.  Of the context it reads the geometry, proxy fit, close tables and work
+// items; it writes those sums, its launch counter and, with bie_profile on, the
+// profiler's event state, so calls on one context must not overlap (as for every
+// entry point).  See
 // include/bie.h for who needs this and the limits.
 #include <mutex>
 
@@ -49,15 +50,7 @@ extern "C" int bie_apply_static(bie_ctx* c, const double* sigma, double* out) {
     const size_t b_xif = round256(nc * 2 * c->M * sizeof(float));
     const size_t b_gt = round256(nc * 8 * c->m * sizeof(double));
     const size_t b_tk = round256(nc * 2 * c->m * sizeof(unsigned int));
-    const size_t b_T = round256(2 * N * sizeof(double));
-    const Fmm& fm = c->fmm[0];
-    const size_t b_ps = fm.on ? round256((size_t)c->cl.npairs * sizeof(float2)) : 0;
-    const size_t b_fsq = fm.on ? round256(fm.sq_bytes) : 0;
-    const size_t b_fmp = fm.on ? round256(fm.mp_bytes) : 0;
-    const size_t b_floc = fm.on ? round256(fm.loc_bytes) : 0;
-    const size_t b_ftk = fm.on ? round256(fm.t.nbox * sizeof(unsigned)) : 0;
-    const size_t need = b_src32 + b_src32n + b_src64 + b_part + b_body + b_gpart + b_xi + b_xif + b_gt + b_tk + b_T +
-                        b_ps + b_fsq + b_fmp + b_floc + b_ftk;
+    const size_t need = b_src32 + b_src32n + b_src64 + b_part + b_body + b_gpart + b_xi + b_xif + b_gt + b_tk;
     if (need > BIE_STATIC_SCRATCH_BYTES)
         return fail(c, BIE_EINVAL, "bie_apply_static: this context needs " + std::to_string(need) +
                                        " bytes of scratch; the static array holds " +
@@ -101,21 +94,13 @@ extern "C" int bie_apply_static(bie_ctx* c, const double* sigma, double* out) {
     ws.gt = reinterpret_cast<double*>(base + o);
     o += b_gt;
     ws.dticket = reinterpret_cast<unsigned int*>(base + o);
-    o += b_tk;
-    ws.T = reinterpret_cast<double*>(base + o);
-    o += b_T;
-    if (fm.on) {
-        if (b_ps) ws.psum = base + o;
-        o += b_ps;
-        ws.fsq = base + o;
-        o += b_fsq;
-        ws.fmp = base + o;
-        o += b_fmp;
-        ws.floc = base + o;
-        o += b_floc;
-        ws.ftick = reinterpret_cast<unsigned*>(base + o);
-        BIE_CUDA(c, cudaMemsetAsync(ws.ftick, 0, b_ftk, c->stream));
-    }
+    // the fast image sum's moments (and the close pairs' sums) stay in what the
+    // context was made with: up to some 700 bytes a box, which the array could not
+    // hold for every context it serves
+    ws.fsq = c->ws.fsq;
+    ws.fmp = c->ws.fmp;
+    ws.floc = c->ws.floc;
+    ws.ftick = c->ws.ftick;
     // the wall-discrepancy kernel's last-block counters must start at zero
     // (they return to zero when it finishes)
     BIE_CUDA(c, cudaMemsetAsync(ws.dticket, 0, b_tk, c->stream));

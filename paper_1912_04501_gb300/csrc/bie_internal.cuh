@@ -158,7 +158,6 @@ struct Workspace {
     // fast image sum: sorted strengths, multipole and local expansions, and
     // the last-child counters of the upward pass (zero between launches)
     void* psum = nullptr;       // close pairs' sums (null: Close::psum)
-    double* T = nullptr;        // 2N; alpha per cell (k_alpha32)
     void *fsq = nullptr, *fmp = nullptr, *floc = nullptr;
     unsigned* ftick = nullptr;
 };

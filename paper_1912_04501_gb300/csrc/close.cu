@@ -892,7 +892,6 @@ struct Asm32 {
     const double* body;
     const int* owner;
     const double2* sigma;
-    int N;
     const float4* tgt32;
     const float4* src32;
     const float4* posdf;
@@ -908,18 +907,15 @@ struct Asm32 {
     const double* bodyF;
 };
 
-// T_i on every thread of the calling group of NL threads (a warp, NL = 32,
-// or a whole CTA, NL = blockDim.x = 256; red: 6 NL / 32 doubles of shared
-// memory for NL > 32); fixed reduction order.
-template <int NL>
-__device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane, double* red) {
+// T_i on every lane of the calling warp; fixed reduction order.
+__device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane) {
     const int cidx = a.node_cell[i];
     const Cell& cl = a.cells[cidx];
     // near-sum partials
     float hx = 0.f, lx = 0.f, hy = 0.f, ly = 0.f, e;
     const int splits = cl.splits[0];
     const long long base = cl.part_off[0] + (i - cl.node_off);
-    for (int s = lane; s < splits; s += NL) {
+    for (int s = lane; s < splits; s += 32) {
         const float2 p = a.part[base + (long long)s * cl.n_nodes];
         two_sum(hx, p.x, hx, e);
         lx += e;
@@ -931,7 +927,7 @@ __device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane, d
     const float2* yp = a.ypf + (size_t)cidx * a.M;
     const float* xi = a.xif + (size_t)cidx * 2 * a.M;
     float cx = 0.f, cy = 0.f;
-    for (int p = lane; p < a.M; p += NL) {
+    for (int p = lane; p < a.M; p += 32) {
         const float2 q = yp[p];
         const float rx = tv.x - q.x, ry = tv.y - q.y;
         const float fx = xi[p], fy = xi[a.M + p];
@@ -985,7 +981,7 @@ __device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane, d
         const int nbn = (int)a.body[8 * b + 5], off = (int)a.body[8 * b + 6];
         const float4 p = shifted(4);
 #pragma unroll 4
-        for (int k = lane; k < nbn; k += NL)
+        for (int k = lane; k < nbn; k += 32)
             if (off + k != i) redo(off + k, 4, p);
     }
     float bx = 0.f, by = 0.f;  // close-evaluation blocks applied to q
@@ -998,7 +994,7 @@ __device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane, d
             const float* C = a.blocks32 + a.blk_off[pp];
             const float4 p = shifted(im);
 #pragma unroll 2
-            for (int k = lane; k < nbn; k += NL) {
+            for (int k = lane; k < nbn; k += 32) {
                 redo(off + k, im, p);
                 const float4 s = a.src32[a.imc ? 4 * (size_t)(off + k) : (size_t)(off + k)];  // q: the same in every record
                 const float A = C[3 * k], B = C[3 * k + 1], D = C[3 * k + 2];
@@ -1018,33 +1014,6 @@ __device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane, d
         bx += __shfl_xor_sync(0xffffffffu, bx, o);
         by += __shfl_xor_sync(0xffffffffu, by, o);
     }
-    if constexpr (NL > 32) {  // the warps' sums, added in warp order
-        constexpr int nw = NL / 32;
-        const int wid = lane >> 5;
-        if ((lane & 31) == 0) {
-            red[wid] = tx;
-            red[nw + wid] = ty;
-            red[2 * nw + wid] = fx;
-            red[3 * nw + wid] = fy;
-            red[4 * nw + wid] = bx;
-            red[5 * nw + wid] = by;
-        }
-        __syncthreads();
-        tx = ty = 0.0;
-        double sfx = 0.0, sfy = 0.0, sbx = 0.0, sby = 0.0;
-        for (int k = 0; k < nw; ++k) {
-            tx += red[k];
-            ty += red[nw + k];
-            sfx += red[2 * nw + k];
-            sfy += red[3 * nw + k];
-            sbx += red[4 * nw + k];
-            sby += red[5 * nw + k];
-        }
-        fx = (float)sfx;
-        fy = (float)sfy;
-        bx = (float)sbx;
-        by = (float)sby;
-    }
     // on-curve diagonal
     const double n0 = a.nx[i], n1 = a.ny[i];
     const double2 sg = a.sigma[i];
@@ -1054,24 +1023,28 @@ __device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane, d
     return make_double2((tx + dg * t0) + (double)bx + c * (double)fx, (ty + dg * t1) + (double)by + c * (double)fy);
 }
 
-// alpha = -T(x_1) . n_1 of every cell (x_1: node 0 of its first body), one CTA per cell.
-constexpr int kAlphaThreads = 256;
-__global__ void __launch_bounds__(kAlphaThreads, 1) k_alpha32(Asm32 a, double* __restrict__ alpha) {
-    __shared__ double red[6 * kAlphaThreads / 32];
-    const int ci = blockIdx.x;
-    const int i0 = a.cells[ci].node_off;
-    const double2 T = traction32<kAlphaThreads>(a, i0, threadIdx.x, red);
-    if (threadIdx.x == 0) alpha[ci] = -(T.x * a.nx[i0] + T.y * a.ny[i0]);
-}
-
-// y_i = sigma_i / 2 + T_i + alpha n_i + F_b + (x_i - x^c)^perp tau_b, one warp per target.
-__global__ void __launch_bounds__(256, 3) k_assemble32(Asm32 a, const double* __restrict__ alpha,
-                                                    double2* __restrict__ out) {
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (i >= a.N) return;
-    const double2 T = traction32<32>(a, i, lane, nullptr);
-    if (lane != 0) return;
-    const double al = alpha[a.node_cell[i]];
+// y_i = sigma_i / 2 + T_i + alpha n_i + F_b + (x_i - x^c)^perp tau_b, one warp per
+// target and kAsmNodes targets of one cell per CTA; one more warp forms T at the cell's
+// first node, for alpha.  (Bound by the latency of a warp's sums.  A launch of its own
+// for alpha, one CTA per cell, took another 10 us of an application of 54.)
+constexpr int kAsmNodes = 8;
+__global__ void __launch_bounds__(32 * (kAsmNodes + 1), 3)
+k_assemble32(Asm32 a, const int4* __restrict__ chunks, double2* __restrict__ out) {
+    __shared__ double s_t0[2];
+    constexpr int kParts = kFinNodes / kAsmNodes;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int4 ch = chunks[blockIdx.x / kParts];
+    const int i0 = ch.y + (int)(blockIdx.x % kParts) * kAsmNodes, head = ch.w;
+    if (i0 >= ch.z) return;
+    const int i = wid == kAsmNodes ? head : min(i0 + wid, ch.z - 1);
+    const double2 T = traction32(a, i, lane);
+    if (wid == kAsmNodes && lane == 0) {
+        s_t0[0] = T.x;
+        s_t0[1] = T.y;
+    }
+    __syncthreads();
+    if (lane != 0 || wid == kAsmNodes || i0 + wid >= ch.z) return;
+    const double al = -(s_t0[0] * a.nx[head] + s_t0[1] * a.ny[head]);
     const int b = a.owner[i];
     const double xc = a.body[8 * b + 2], yc = a.body[8 * b + 3];
     const double Fx = a.bodyF[3 * b], Fy = a.bodyF[3 * b + 1], tq = a.bodyF[3 * b + 2];
@@ -1095,7 +1068,6 @@ int assemble32(bie_ctx* c, const double* sigma, const Workspace& ws, double* you
     a.body = c->body;
     a.owner = c->owner;
     a.sigma = reinterpret_cast<const double2*>(sigma);
-    a.N = c->N;
     a.tgt32 = c->tgt32;
     a.src32 = ws.src32;
     a.posdf = c->posdf;
@@ -1109,12 +1081,8 @@ int assemble32(bie_ctx* c, const double* sigma, const Workspace& ws, double* you
     a.cells = c->cells;
     a.imc = c->utilde ? c->imc : nullptr;
     a.bodyF = ws.bodyF;
-    double* alpha = ws.T;  // the single-precision path keeps no T: its first ncell entries hold alpha
-    k_alpha32<<<c->ncell, kAlphaThreads, 0, c->stream>>>(a, alpha);
-    BIE_LAUNCH(c, "k_alpha32");
-    const int bs = 256;
-    const int gs = (int)((32LL * c->N + bs - 1) / bs);
-    k_assemble32<<<gs, bs, 0, c->stream>>>(a, alpha, reinterpret_cast<double2*>(yout));
+    k_assemble32<<<c->n_fin * (kFinNodes / kAsmNodes), 32 * (kAsmNodes + 1), 0, c->stream>>>(
+        a, c->fin_chunks, reinterpret_cast<double2*>(yout));
     BIE_LAUNCH(c, "k_assemble32");
     return BIE_OK;
 }
@@ -1209,17 +1177,22 @@ __device__ __forceinline__ void partial_sum(const Finish<R>& a, const Cell& cl, 
     }
 }
 
-template <typename R>
+template <typename R, int G>
 __global__ void __launch_bounds__(kFinNodes)
 k_finish(Finish<R> a, double2* __restrict__ out) {
     __shared__ R2<R> s_yp[kMaxProxy], s_xi[kMaxProxy];
     __shared__ double s_t0[2];
     const int t = threadIdx.x, wid = t >> 5, lane = t & 31;
-    const int4 ch = a.chunks[blockIdx.x];
-    const int i0 = ch.y, i1 = ch.z, head = ch.w;
+    const int4 ch = a.chunks[blockIdx.x / G];
+    const int i0 = ch.y + (int)(blockIdx.x % G) * (kFinNodes / G), i1 = min(ch.z, i0 + kFinNodes / G), head = ch.w;
+    const int sub = t % G;
+    if (i0 >= i1) {  // a short chunk's last part
+        pdl_wait();
+        return;
+    }
     const Cell& cl = a.cells[ch.x];
     // what only the geometry and the density decide, before the wait
-    const int i = min(i0 + t, i1 - 1);
+    const int i = min(i0 + t / G, i1 - 1);
     const double2 sg = a.sigma[i];
     const double n0 = a.nx[i], n1 = a.ny[i], wi = a.w[i], ki = a.kap[i], xi_ = a.x[i], yi = a.y[i];
     const int b = a.owner[i];
@@ -1299,11 +1272,16 @@ k_finish(Finish<R> a, double2* __restrict__ out) {
         }
     }
     double tx, ty;
-    proxy_sum(a.M, 0, 1, s_yp, s_xi, X, Y, m0, m1, tx, ty);
-    partial_sum(a, cl, i, 0, 1, tx, ty);
-    own_terms(ki, wi, n0, n1, sg, p0, p1, tx, ty);
+    proxy_sum(a.M, sub, G, s_yp, s_xi, X, Y, m0, m1, tx, ty);
+    partial_sum(a, cl, i, sub, G, tx, ty);
+#pragma unroll
+    for (int s = 1; s < G; s <<= 1) {
+        tx += __shfl_xor_sync(0xffffffffu, tx, s);
+        ty += __shfl_xor_sync(0xffffffffu, ty, s);
+    }
+    if (sub == 0) own_terms(ki, wi, n0, n1, sg, p0, p1, tx, ty);
     __syncthreads();
-    if (i0 + t >= i1) return;
+    if (sub || i0 + t / G >= i1) return;
     const double al = -(s_t0[0] * h0 + s_t0[1] * h1);
     out[i] = make_double2(0.5 * sg.x + tx + al * n0 + F0 - (yi - yc) * tq, 0.5 * sg.y + ty + al * n1 + F1 + (xi_ - xc) * tq);
 }
@@ -1337,7 +1315,12 @@ static int finish_launch(bie_ctx* c, const double* sigma, int prec, const Worksp
     a.body = c->body;
     a.bodyF = ws.bodyF;
     a.cells = c->cells;
-    BIE_CUDA(c, launch_after(fmm_chained(c, prec), k_finish<R>, c->n_fin, kFinNodes, 0u, c->stream, a, reinterpret_cast<double2*>(yout)));
+    // four threads per node where a thread per node leaves SMs idle (1024 nodes in
+    // double-float 26 us / 15, 6400 15 / 12; single precision is no faster so)
+    constexpr int G = sizeof(R) == 4 ? 1 : 4;
+    const bool few = c->n_fin < c->sms;
+    BIE_CUDA(c, launch_after(fmm_chained(c, prec), few ? k_finish<R, G> : k_finish<R, 1>, c->n_fin * (few ? (unsigned)G : 1u),
+                             (unsigned)kFinNodes, 0u, c->stream, a, reinterpret_cast<double2*>(yout)));
     ++c->launches;
     return BIE_OK;
 }

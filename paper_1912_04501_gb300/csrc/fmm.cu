@@ -1476,7 +1476,15 @@ k_fmm_down64(FmmTree t, const Cell* cells, int nimg, const C2<R>* sq, const V4<R
 static constexpr double kDirectPair[3] = {0.345e-12, 31.7e-12, 3.57e-12};
 static constexpr double kLeafPair[3] = {1.2e-12, 25e-12, 5e-12};
 static constexpr double kTranslate[3] = {0.7e-9, 26e-9, 7e-9};
-static constexpr double kFmmFixed[3] = {12e-6, 20e-6, 20e-6};
+static constexpr double kFmmFixed[3] = {5e-6, 20e-6, 20e-6};
+// What sums of few long items cost a direct application of a cell alone in its
+// context.  Measured (us, direct / fast): double-float 480 nodes 88 / 119, 1024 130 / 142,
+// 1536 192 / 153; double 480 163 / 303, 1024 470 / 383.  (Single precision: 128 nodes
+// 42 / 46, 1024 49 / 51, 1536 56 / 54, 2560 73 / 64, as the model has it.)
+static constexpr double kDirectFixed[3] = {0, 220e-6, 85e-6};
+// Boxes that any cell may have, in a batch and alone: with 64, cells below 500 nodes
+// had no leaf small enough for the walls.
+static constexpr double kFmmBoxes[2] = {64, 256};
 
 struct FmmPlanCell {
     double ox, oy, w, ht;  // rectangle (relative to the cell centre)
@@ -1673,8 +1681,8 @@ int fmm_plan(bie_ctx* c) {
             const FmmPlanCell& rc = rect[k];
             FmmCell& fc = cells[k];
             // leaf side: the modelled best of a geometric ladder, with at most
-            // one box per 8 source records (64 at least)
-            const double most = std::max(64.0, cl.n_nodes * (double)c->srcmul / 8);
+            // one box per 8 source records (kFmmBoxes at least)
+            const double most = std::max(kFmmBoxes[c->ncell == 1], cl.n_nodes * (double)c->srcmul / 8);
             const double wall = fmm_wall_side(c, k, prec);
             double best = INFINITY, bh = 0;
             for (int j = 0; j < 48; ++j) {
@@ -1713,9 +1721,11 @@ int fmm_plan(bie_ctx* c) {
             fc.off[0] = (int)nleaf;
             nleaf += (long long)fc.gx[0] * fc.gy[0];
         }
-        f.on = (t_fast < t_direct || BIE_FMM == 2) && nleaf < (1 << 26);
-        f.walls = f.on && !c->utilde;
+        f.walls = !c->utilde;
         for (const FmmCell& fc : cells) f.walls = f.walls && fc.wall >= 0;
+        if (f.walls && c->ncell == 1) t_direct += kDirectFixed[prec];
+        f.on = (t_fast < t_direct || BIE_FMM == 2) && nleaf < (1 << 26);
+        f.walls = f.walls && f.on;
         if (!f.on) continue;
         // leaves of all cells first, then the coarser levels cell by cell
         nbox = nleaf;
