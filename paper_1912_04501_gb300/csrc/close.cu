@@ -306,7 +306,8 @@ constexpr int kCloseChunk = 2048;  // fine nodes staged in shared memory at a ti
 // fine node.  A pair with more than kCloseHeavy of these is shared by a cluster of
 // kCloseCtas CTAs, each with its part of the fine nodes and the sums added through
 // distributed shared memory: one CTA for such a pair left the other SMs idle (two
-// bodies of 512 nodes 2e-3 apart: 3.6 ms, 1.7 so).  Dynamic shared memory:
+// bodies of 512 nodes 2e-3 apart: 3.6 ms, 1.5 so, two thirds
+// of the FP64 pipe's rate).  Dynamic shared memory:
 // 3 kCloseChunk + 3 min(N_b, kCloseAccNodes) doubles.
 constexpr long long kCloseHeavy = 1 << 17;
 constexpr int kCloseCtas = 8;
@@ -330,7 +331,7 @@ __device__ inline bool close_heavy(const BlockArgs& g, int4 pr) {
 }
 
 template <int NC>
-__device__ void close_block(const BlockArgs& g, int pair, int4 pr, double* sm) {
+__device__ void close_block(const BlockArgs& g, int pair, int4 pr, int per, double* sm) {
     namespace cg = cooperative_groups;
     double* sa = sm;
     double* sb = sm + kCloseChunk;
@@ -349,7 +350,7 @@ __device__ void close_block(const BlockArgs& g, int pair, int4 pr, double* sm) {
     double st, ct;
     sincos(th, &st, &ct);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int k0 = blockIdx.y * kCloseAccNodes, nk = min(kCloseAccNodes, nbn - k0);
+    const int k0 = blockIdx.y * per, nk = min(per, nbn - k0);
     if (nk <= 0) return;  // this body has fewer node ranges than the largest one
     for (int k = threadIdx.x; k < 3 * nk; k += blockDim.x) acc[k] = 0.0;
     const int gl = (int)((long long)nm * rank / NC), gh = (int)((long long)nm * (rank + 1) / NC);
@@ -441,17 +442,17 @@ __device__ void close_block(const BlockArgs& g, int pair, int4 pr, double* sm) {
 __global__ void __launch_bounds__(256) k_close_blocks(const BlockArgs g) {
     extern __shared__ double sm[];
     const int4 pr = g.pairs[blockIdx.x];
-    if (!close_heavy(g, pr)) close_block<1>(g, blockIdx.x, pr, sm);
+    if (!close_heavy(g, pr)) close_block<1>(g, blockIdx.x, pr, kCloseAccNodes, sm);
 }
 
 __global__ void __cluster_dims__(kCloseCtas, 1, 1) __launch_bounds__(256)
-k_close_blocks_heavy(const BlockArgs g, int npairs) {
+k_close_blocks_heavy(const BlockArgs g, int per) {
     extern __shared__ double sm[];
-    cooperative_groups::this_cluster().sync();
-    for (int p = blockIdx.x / kCloseCtas; p < npairs; p += gridDim.x / kCloseCtas) {
-        const int4 pr = g.pairs[p];
-        if (close_heavy(g, pr)) close_block<kCloseCtas>(g, p, pr, sm);
-    }
+    const int p = blockIdx.x / kCloseCtas;
+    const int4 pr = g.pairs[p];
+    if (!close_heavy(g, pr)) return;
+    cooperative_groups::this_cluster().sync();  // its CTAs have started
+    close_block<kCloseCtas>(g, p, pr, per, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -810,8 +811,11 @@ int build_close(bie_ctx* c) {
     const BlockArgs g{c->cl.pairs, c->cl.blk_off, c->x, c->y, c->nx, c->ny, c->w, c->body, c->node_cell, c->cells,
                       c->cl.dtab, c->cl.dtab_off, c->cl.blocks, c->cl.blocks32, c->bshape};
     if ((h[6] - 1LL) * maxn * maxn > kCloseHeavy) {
-        const int clusters = std::min(h[0], std::max(1, 2 * c->sms / kCloseCtas));
-        k_close_blocks_heavy<<<dim3(clusters * kCloseCtas, ranges), 256, shm, c->stream>>>(g, h[0]);
+        // few pairs, fewer nodes of one per cluster: the fine nodes' values are
+        // formed again for every range, some 150 operations against 3 per node
+        int per = kCloseAccNodes;
+        while (per > 128 && (long long)h[0] * ((maxn + per - 1) / per) * kCloseCtas < 8LL * c->sms) per /= 2;
+        k_close_blocks_heavy<<<dim3(h[0] * kCloseCtas, (maxn + per - 1) / per), 256, shm, c->stream>>>(g, per);
         BIE_LAUNCH(c, "k_close_blocks_heavy");
     }
     k_close_blocks<<<dim3(h[0], ranges), 256, shm, c->stream>>>(g);
