@@ -306,9 +306,8 @@ constexpr int kCloseChunk = 2048;  // fine nodes staged in shared memory at a ti
 // fine node.  A pair with more than kCloseHeavy of these is shared by a cluster of
 // kCloseCtas CTAs, each with its part of the fine nodes and the sums added through
 // distributed shared memory: one CTA for such a pair left the other SMs idle (two
-// bodies of 512 nodes 2e-3 apart: 3.6 ms, 1.5 so, two thirds
-// of the FP64 pipe's rate).  Dynamic shared memory:
-// 3 kCloseChunk + 3 min(N_b, kCloseAccNodes) doubles.
+// bodies of 512 nodes 2e-3 apart: 3.6 ms, 1.5 so, at two thirds of the FP64 pipe's
+// rate).  Dynamic shared memory: 3 kCloseChunk + 3 min(N_b, kCloseAccNodes) doubles.
 constexpr long long kCloseHeavy = 1 << 17;
 constexpr int kCloseCtas = 8;
 
@@ -1028,27 +1027,29 @@ __device__ __forceinline__ double2 traction32(const Asm32& a, int i, int lane) {
 }
 
 // y_i = sigma_i / 2 + T_i + alpha n_i + F_b + (x_i - x^c)^perp tau_b, one warp per
-// target and kAsmNodes targets of one cell per CTA; one more warp forms T at the cell's
-// first node, for alpha.  (Bound by the latency of a warp's sums.  A launch of its own
-// for alpha, one CTA per cell, took another 10 us of an application of 54.)
-constexpr int kAsmNodes = 8;
-__global__ void __launch_bounds__(32 * (kAsmNodes + 1), 3)
-k_assemble32(Asm32 a, const int4* __restrict__ chunks, double2* __restrict__ out) {
-    __shared__ double s_t0[2];
-    constexpr int kParts = kFinNodes / kAsmNodes;
+// target; a CTA of nine takes 8 `rounds` targets of one cell and the cell's first node,
+// whose T gives alpha.  (Bound by the latency of a warp's sums where targets are few,
+// two bodies of 512 nodes: 16 us; a launch of its own for alpha, one CTA per cell, took
+// another 10.  Two rounds from kAsmMany nodes on, where the first node's repeated sums
+// count: 64 cells of 480 nodes 346 us an application with one, 322 with two.)
+constexpr int kAsmWarps = 9, kAsmRounds = 2, kAsmMany = 8192;
+__global__ void __launch_bounds__(32 * kAsmWarps, 3)
+k_assemble32(Asm32 a, const int4* __restrict__ chunks, int rounds, double2* __restrict__ out) {
+    __shared__ double2 s_t[8 * kAsmRounds + 1];  // T of the first node, then of the targets
+    const int nt = 8 * rounds, parts = kFinNodes / nt;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int4 ch = chunks[blockIdx.x / kParts];
-    const int i0 = ch.y + (int)(blockIdx.x % kParts) * kAsmNodes, head = ch.w;
-    if (i0 >= ch.z) return;
-    const int i = wid == kAsmNodes ? head : min(i0 + wid, ch.z - 1);
-    const double2 T = traction32(a, i, lane);
-    if (wid == kAsmNodes && lane == 0) {
-        s_t0[0] = T.x;
-        s_t0[1] = T.y;
+    const int4 ch = chunks[blockIdx.x / parts];
+    const int i0 = ch.y + (int)(blockIdx.x % parts) * nt, n = min(nt, ch.z - i0), head = ch.w;
+    if (n <= 0) return;
+    for (int t = wid; t <= n; t += kAsmWarps) {
+        const double2 T = traction32(a, t ? i0 + t - 1 : head, lane);
+        if (lane == 0) s_t[t] = T;
     }
     __syncthreads();
-    if (lane != 0 || wid == kAsmNodes || i0 + wid >= ch.z) return;
-    const double al = -(s_t0[0] * a.nx[head] + s_t0[1] * a.ny[head]);
+    if (threadIdx.x >= n) return;
+    const int i = i0 + threadIdx.x;
+    const double2 T = s_t[threadIdx.x + 1];
+    const double al = -(s_t[0].x * a.nx[head] + s_t[0].y * a.ny[head]);
     const int b = a.owner[i];
     const double xc = a.body[8 * b + 2], yc = a.body[8 * b + 3];
     const double Fx = a.bodyF[3 * b], Fy = a.bodyF[3 * b + 1], tq = a.bodyF[3 * b + 2];
@@ -1085,8 +1086,9 @@ int assemble32(bie_ctx* c, const double* sigma, const Workspace& ws, double* you
     a.cells = c->cells;
     a.imc = c->utilde ? c->imc : nullptr;
     a.bodyF = ws.bodyF;
-    k_assemble32<<<c->n_fin * (kFinNodes / kAsmNodes), 32 * (kAsmNodes + 1), 0, c->stream>>>(
-        a, c->fin_chunks, reinterpret_cast<double2*>(yout));
+    const int rounds = c->N < kAsmMany ? 1 : kAsmRounds;
+    k_assemble32<<<c->n_fin * (kFinNodes / (8 * rounds)), 32 * kAsmWarps, 0, c->stream>>>(
+        a, c->fin_chunks, rounds, reinterpret_cast<double2*>(yout));
     BIE_LAUNCH(c, "k_assemble32");
     return BIE_OK;
 }
