@@ -57,6 +57,9 @@ FLOPS_PER_PAIR_ROWS = 14.0 + 4.0 / 3.0
 # FP32 instructions per pair of k_near32r (an FMA counts once): the FP32
 # pipe's issue limit is half the FMA flop peak in these units
 OPS_PER_PAIR_ROWS = 9.0 + 4.0 / 3.0
+# a translation of a multipole expansion of P coefficients to a local one, two complex
+# series with real weights: 4 fma per pair of coefficients
+FLOPS_PER_TRANSLATION = 8.0  # times P^2
 # the doubled-cell kernel shares the r_y terms between a node's two images
 # at one lattice row (dm = 0, 1): 14 per pair + 4 per two pairs
 FLOPS_PER_PAIR_UROWS = 14.0 + 4.0 / 2.0
@@ -192,6 +195,15 @@ def kernel_source(kernel):
 
 def source_hash(kernel):
     return hashlib.sha256(kernel_source(kernel).encode()).hexdigest()[:16]
+
+
+def near_flops(ctx, precision, direct_flops):
+    """Algorithmic flops of one near image sum and whether it runs by expansions."""
+    pairs, translations, order = ctx.near_work(precision)
+    if not translations:
+        return {"flops": direct_flops * pairs, "fast": False, "pairs": pairs}
+    return {"flops": FLOPS_PER_PAIR * pairs + FLOPS_PER_TRANSLATION * order ** 2 * translations, "fast": True,
+            "pairs": pairs, "translations": translations, "order": order}
 
 
 def profiled_traffic(kernel, workload):
@@ -446,6 +458,7 @@ def main():
     clk = clocks.stop()
     prof = ctx.profile_read()
     ctx.profile(False)
+    work32, workdf = near_flops(ctx, bie.BIE_MIXED, fpp32), near_flops(ctx, bie.BIE_DF64, fpp32)
     total_ms = sum(run["ms"])
     applies32, applies64 = run["applies32"], run["applies64"]
     pairs = pairs_per_apply * (applies32 + applies64)  # applies64: FP64-class (double-float) residuals
@@ -515,6 +528,7 @@ def main():
     ru = timed_steps(cu, stream, dt, max(3, args.steps // 4), flush)
     pu = cu.profile_read()
     cu.profile(False)
+    worku = near_flops(cu, bie.BIE_MIXED, FLOPS_PER_PAIR_UROWS if cell["e1"][1] == 0.0 else FLOPS_PER_PAIR)
     if net is not None:
         cu.set_warm_net(None)
     cu.close()
@@ -528,8 +542,9 @@ def main():
               "iterations_mean": statistics.mean(ru["iters"]), "mu_eff_last": ru["mu"][-1],
               "near32_ms_per_launch": pu["near32_ms"] / max(1, pu["near32_launches"]),
               "neardf_ms_per_launch": pu["neardf_ms"] / max(1, pu["neardf_launches"]),
-              "near32_tflops": (FLOPS_PER_PAIR_UROWS if cell["e1"][1] == 0.0 else FLOPS_PER_PAIR) * pairs_u
-              / (pu["near32_ms"] / max(1, pu["near32_launches"]) / 1e3) / 1e12 if pu["near32_launches"] else None}
+              "near_work": worku,
+              "near32_tflops": worku["flops"] / (pu["near32_ms"] / max(1, pu["near32_launches"]) / 1e3) / 1e12
+              if pu["near32_launches"] else None}
 
     # plain FP64 solve (zero start, double-precision pair sums): one operator
     # application timed on the device, times the plain GMRES iterations plus
@@ -549,6 +564,7 @@ def main():
     ev1.record(stream)
     ev1.synchronize()
     ms64_apply = ev0.elapsed_time(ev1)
+    work64 = near_flops(ctx64, bie.BIE_FP64, FLOPS_PER_PAIR)
     fp64 = None
     if N > 20000:
         cdf = bie.Context(cell, precision=bie.BIE_DF64, device=local, warm_start=0)
@@ -661,6 +677,7 @@ def main():
         e1.synchronize()
         p4 = cb.profile_read()
         cb.profile(False)
+        work4 = near_flops(cb, bie.BIE_MIXED, FLOPS_PER_PAIR)
         cb.set_warm_net(None)
         cb.close()
         ms4 = statistics.mean(r4["ms"])
@@ -672,8 +689,8 @@ def main():
                  "apply_ms": e0.elapsed_time(e1) / 10, "near32_ms_per_launch": ms4_near,
                  "value": pairs4 / (ms4_near / 1e3) / 1e9 if p4["near32_launches"] else None,
                  "unit": "Gpairs/s (near sum of a full application, every cell active)",
-                 "near_sum": "persistent work queue (k_near32r_queue), items sorted longest first",
-                 "graph": True, "tile_shape": {"chosen": shape4, "ms_per_shape": ms_shapes4}}
+                 "near_sum": "by expansions" if work4["fast"] else "direct", "near_work": work4,
+                 "tile_shape": {"chosen": shape4, "ms_per_shape": ms_shapes4}}
 
     # rooflines: measured CUDA-core FMA throughput of this device
     peak = bie.alu_peak(local, stream.cuda_stream)
@@ -683,23 +700,24 @@ def main():
     n32, n64, ndf = prof["near32_launches"], prof["near64_launches"], prof["neardf_launches"]
     ms32 = prof["near32_ms"] / max(1, n32)
     msdf = prof["neardf_ms"] / max(1, ndf)
-    roof32 = {"kernel": near32, "bound": "alu", "unit": "TFLOP/s", "peak": fp32_peak,
-              "achieved": fpp32 * pairs_per_apply / (ms32 / 1e3) / 1e12 if n32 else None,
-              "flops_per_pair": fpp32, "launch_ms": ms32, "launches": n32, "device_ms_total": prof["near32_ms"],
-              "peak_source": fp32_src, "traffic": profiled_traffic(near32, name)}
-    if rows and n32:
-        # the same launches as a fraction of the FP32 pipe's instruction rate
-        roof32["fp32_issue_frac"] = OPS_PER_PAIR_ROWS * pairs_per_apply / (ms32 / 1e3) / 1e12 / (fp32_peak / 2)
+    # achieved: the algorithmic flops of the near sum as it runs -- the pairs summed one
+    # by one and, by expansions, the translations (bie_near_work); the value's pairs are
+    # those of the direct sum that an application stands for
+    name32 = "k_fmm_m2l + k_fmm_down32" if work32["fast"] else near32
+    roof32 = {"kernel": name32, "bound": "alu", "unit": "TFLOP/s", "peak": fp32_peak,
+              "achieved": work32["flops"] / (ms32 / 1e3) / 1e12 if n32 else None,
+              "work": work32, "launch_ms": ms32, "launches": n32, "device_ms_total": prof["near32_ms"],
+              "peak_source": fp32_src, "traffic": profiled_traffic(near32, name) if not work32["fast"] else None}
     # double-float pairs run on the FP32 pipe: measured against the FP32 peak,
-    # counting the same algorithmic flops per pair as the single-precision
-    # kernel (the extra ~100 FP32 instructions per pair are the price of the
-    # 48-bit arithmetic)
-    roofdf = {"kernel": "k_near_df", "bound": "alu", "unit": "TFLOP/s", "peak": fp32_peak,
-              "achieved": fpp32 * pairs_per_apply / (msdf / 1e3) / 1e12 if ndf else None,
-              "launch_ms": msdf, "launches": ndf, "device_ms_total": prof["neardf_ms"],
-              "peak_source": fp32_src, "traffic": profiled_traffic("k_near_df", name)}
-    roof64 = {"kernel": "k_near64 (plain FP64 operator, whole application)", "bound": "alu", "unit": "TFLOP/s",
-              "peak": peak["dfma"], "achieved": FLOPS_PER_PAIR * pairs_per_apply / (ms64_apply / 1e3) / 1e12,
+    # counting the same algorithmic flops per pair and translation as in single
+    # precision (the other FP32 instructions are the price of 48-bit arithmetic)
+    roofdf = {"kernel": "k_fmm_m2l + k_fmm_down64 (double-float)" if workdf["fast"] else "k_near_df", "bound": "alu",
+              "unit": "TFLOP/s", "peak": fp32_peak,
+              "achieved": workdf["flops"] / (msdf / 1e3) / 1e12 if ndf else None,
+              "work": workdf, "launch_ms": msdf, "launches": ndf, "device_ms_total": prof["neardf_ms"],
+              "peak_source": fp32_src, "traffic": None}
+    roof64 = {"kernel": "plain FP64 operator, whole application", "bound": "alu", "unit": "TFLOP/s",
+              "peak": peak["dfma"], "achieved": work64["flops"] / (ms64_apply / 1e3) / 1e12, "work": work64,
               "launch_ms": ms64_apply, "launches": 1, "device_ms_total": ms64_apply,
               "peak_source": f"measured FP64 FMA throughput of this GPU (bie_alu_peak: {peak['dfma']:.2f} TFLOP/s)",
               "traffic": None}
@@ -718,7 +736,9 @@ def main():
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "strong",
             "vs_baseline": None, "dtype": "f32+f64", "data": "synthetic",
             "config": {"workload": WORKLOADS[name], "N": N, "bodies": nb,
-                       "precision": "FP32 pair sums; refinement residual with double-float pair sums",
+                       "precision": "FP32 image sums; refinement residual with double-float image sums",
+                       "pairs": "9 N^2 of the direct near image sum per application; the sum runs "
+                                + ("by expansions (roofline: its own work)" if work32["fast"] else "directly"),
                        "gmres_tol": 1e-10,
                        "warm_start": ("learned: first GMRES cycle augmented with the previous density, its last "
                                       "change and the shipped network's predicted change; second refinement sweep "

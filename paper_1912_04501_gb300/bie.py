@@ -9,7 +9,7 @@ call raises -- there is no fallback implementation.
 The functions carry the C names:
     bie_default_opts, bie_init, bie_destroy, bie_size, bie_nodes, bie_apply,
     bie_rhs, bie_solve, bie_velocities, bie_step, bie_get_state,
-    bie_set_state, bie_set_stream, bie_close_info, bie_near_shape, bie_profile, bie_profile_read,
+    bie_set_state, bie_set_stream, bie_close_info, bie_near_shape, bie_near_work, bie_profile, bie_profile_read,
     bie_apply_static, bie_init_batch, bie_cells, bie_features, bie_set_warm_net,
     bie_get_history, bie_set_history,
     bie_net_init, bie_net_destroy, bie_net_last_error, bie_net_size,
@@ -118,6 +118,8 @@ def library():
         "bie_set_state": (c_int32, [vp, c_double, vp, vp, vp, vp]),
         "bie_close_info": (c_int32, [vp, ctypes.POINTER(c_int32), ctypes.POINTER(c_int32)]),
         "bie_near_shape": (c_int32, [vp, ctypes.POINTER(c_int32), vp]),
+        "bie_near_work": (c_int32, [vp, c_int32, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64),
+                                    ctypes.POINTER(c_int32)]),
         "bie_apply_static": (c_int32, [vp, vp, vp]),
         "bie_device_sms": (c_int32, [vp, ctypes.POINTER(c_int32)]),
         "bie_mu_eff_contour": (c_int32, [vp, vp, vp, c_int32]),
@@ -159,7 +161,7 @@ def exported_symbols():
                         "bie_set_warm_net", "bie_net_init", "bie_net_destroy", "bie_net_last_error",
                         "bie_net_size", "bie_net_set_stream", "bie_net_set_params", "bie_net_get_params",
                         "bie_net_forward", "bie_net_loss_grad", "bie_net_adam_step", "bie_get_history",
-                        "bie_set_history", "bie_near_shape", "bie_device_sms", "bie_alu_peak", "bie_mu_eff_contour", "bie_set_partition")
+                        "bie_set_history", "bie_near_shape", "bie_near_work", "bie_device_sms", "bie_alu_peak", "bie_mu_eff_contour", "bie_set_partition")
             if hasattr(L, n)]
 
 
@@ -390,6 +392,13 @@ class Context:
         ms = (ctypes.c_float * BIE_NEAR32_SHAPES)()
         self._check(library().bie_near_shape(self.h, ctypes.byref(sh), ms))
         return sh.value, list(ms)
+
+    def near_work(self, precision=BIE_MIXED):
+        """(pairs, translations, coefficients per series) of one near image sum:
+        the work a roofline counts."""
+        p, t, o = ctypes.c_int64(), ctypes.c_int64(), c_int32()
+        self._check(library().bie_near_work(self.h, precision, ctypes.byref(p), ctypes.byref(t), ctypes.byref(o)))
+        return p.value, t.value, o.value
 
     def device_sms(self):
         """Streaming multiprocessors of the context's device (queried at init)."""

@@ -989,6 +989,14 @@ int bie_device_sms(const bie_ctx* c, int32_t* sms) {
     return BIE_OK;
 }
 
+int bie_near_work(bie_ctx* c, int32_t precision, int64_t* pairs, int64_t* translations, int32_t* order) {
+    if (!c || !pairs || !translations || !order) return BIE_EINVAL;
+    if (precision != BIE_FP64 && precision != BIE_MIXED && precision != BIE_DF64)
+        return fail(c, BIE_EINVAL, "bie_near_work: unknown precision");
+    BIE_CUDA(c, cudaSetDevice(c->device));
+    return fmm_work(c, precision == BIE_MIXED ? 0 : (precision == BIE_DF64 ? 2 : 1), pairs, translations, order);
+}
+
 int bie_near_shape(bie_ctx* c, int32_t* shape, float* ms) {
     if (!c) return BIE_EINVAL;
     if (shape) *shape = c->shape32;

@@ -459,6 +459,8 @@ __device__ inline double block_sum_d(double v, double* red) {
 }
 
 // fmm.cu --------------------------------------------------------------------
+// pairs and translations of one near sum, for rooflines
+int fmm_work(bie_ctx* c, int prec, int64_t* pairs, int64_t* translations, int32_t* order);
 int fmm_plan(bie_ctx* c);             // boxes for the bodies' current places (host mirror)
 int fmm_build(bie_ctx* c, int prec);  // sorts the current geometry if it is not
 int fmm_up(bie_ctx* c, const double* sigma, int prec, Workspace& ws);      // moments of every box, and of every body

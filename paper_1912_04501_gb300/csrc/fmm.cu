@@ -1550,6 +1550,33 @@ static FmmPlanCell fmm_rect(const bie_ctx* c, int k) {
     return p;
 }
 
+int fmm_work(bie_ctx* c, int prec, int64_t* pairs, int64_t* translations, int32_t* order) {
+    *pairs = *translations = 0;
+    *order = prec == 0 ? kFmmP32 : kFmmP64;
+    const Fmm& f = c->fmm[prec];
+    if (!f.on) {
+        for (const Cell& cl : c->cells_h) *pairs += (int64_t)cl.n_nodes * cl.n_nodes * (c->utilde ? 4 : 9);
+        return BIE_OK;
+    }
+    if (int rc = fmm_build(c, prec)) return rc;
+    std::vector<int> count(f.t.nleaf), nnear(f.t.nleaf), nfar(f.t.nbox);
+    std::vector<FmmRange> near((size_t)f.t.nleaf * kFmmRanges);
+    BIE_CUDA(c, cudaStreamSynchronize(c->stream));
+    BIE_CUDA(c, cudaMemcpy(count.data(), f.t.tcount, count.size() * sizeof(int), cudaMemcpyDeviceToHost));
+    BIE_CUDA(c, cudaMemcpy(nnear.data(), f.t.nnear, nnear.size() * sizeof(int), cudaMemcpyDeviceToHost));
+    BIE_CUDA(c, cudaMemcpy(nfar.data(), f.t.nfar, nfar.size() * sizeof(int), cudaMemcpyDeviceToHost));
+    BIE_CUDA(c, cudaMemcpy(near.data(), f.t.near, near.size() * sizeof(FmmRange), cudaMemcpyDeviceToHost));
+    for (int b = 0; b < f.t.nleaf; ++b) {
+        if (!count[b]) continue;
+        for (int r = 0; r < nnear[b]; ++r) {
+            const FmmRange& g = near[(size_t)b * kFmmRanges + r];
+            *pairs += (int64_t)count[b] * (g.s1 - g.s0);
+        }
+    }
+    for (int n : nfar) *translations += n;
+    return BIE_OK;
+}
+
 void free_fmm(bie_ctx* c) {
     for (Fmm& f : c->fmm) {
         if (f.arena) cudaFree(f.arena);
