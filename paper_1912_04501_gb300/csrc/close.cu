@@ -803,8 +803,10 @@ int build_close(bie_ctx* c) {
     for (int n : c->n_nodes) maxn = std::max(maxn, n);
     const int acc = std::min(maxn, kCloseAccNodes);
     size_t shm = sizeof(double) * (3 * (size_t)kCloseChunk + 3 * (size_t)acc);
-    BIE_CUDA(c, cudaFuncSetAttribute(k_close_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    BIE_CUDA(c, cudaFuncSetAttribute(k_close_blocks_heavy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    // (the limit is the kernels', whichever thread sets it: always the same value)
+    constexpr int kShm = (int)(sizeof(double) * (3 * (size_t)kCloseChunk + 3 * (size_t)kCloseAccNodes));
+    BIE_CUDA(c, cudaFuncSetAttribute(k_close_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize, kShm));
+    BIE_CUDA(c, cudaFuncSetAttribute(k_close_blocks_heavy, cudaFuncAttributeMaxDynamicSharedMemorySize, kShm));
     c->cl.shm_limit = shm;
     const int ranges = (maxn + kCloseAccNodes - 1) / kCloseAccNodes;
     const BlockArgs g{c->cl.pairs, c->cl.blk_off, c->x, c->y, c->nx, c->ny, c->w, c->body, c->node_cell, c->cells,

@@ -350,7 +350,10 @@ static int gj_in_cluster(bie_ctx* c, int n, bool* done) {
     if (n > kGjMost<NC>) return BIE_OK;
     const int most = (n + NC - 1) / NC;
     const size_t shm = ((size_t)most * n + 3 * (size_t)n + most) * sizeof(double);
-    BIE_CUDA(c, cudaFuncSetAttribute(k_gj_cluster<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    // the limit is the kernel's, whichever thread sets it: always the same value
+    constexpr size_t kCols = (kGjMost<NC> + NC - 1) / NC;
+    constexpr int kShm = (int)((kCols * kGjMost<NC> + 3 * (size_t)kGjMost<NC> + kCols) * sizeof(double));
+    BIE_CUDA(c, cudaFuncSetAttribute(k_gj_cluster<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kShm));
     if (NC > 8) BIE_CUDA(c, cudaFuncSetAttribute(k_gj_cluster<NC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;
