@@ -878,10 +878,8 @@ int bie_set_state(bie_ctx* c, double t, const double* e2, const double* xc, cons
         cell_set_lattice(cl, e1, e2 + 2 * k);
     }
     c->body_host = h;
-    const unsigned long long epoch = c->epoch;
-    int rc = fmm_plan(c);
+    int rc = fmm_fit(c);
     if (rc) return rc;
-    if (c->epoch != epoch && (rc = build_near_items(c))) return rc;  // other boxes: the image sums' layout may change
     rc = upload_cells(c, c->stream);
     if (rc) return rc;
     rc = upload_e2(c, c->e2d, current_e2(c), c->stream);

@@ -223,7 +223,7 @@ struct FmmCell {
     double ox, oy, h, inv_h;
     int nlev;
     int gx[kFmmLevels], gy[kFmmLevels], off[kFmmLevels];  // off: the level's first box
-    int wall;  // level whose boxes the walls' far images are well away from
+    int wall;  // level whose boxes the walls' far images are well away from; -1: none, node by node
 };
 
 // Node data the sorting reads.
@@ -262,6 +262,7 @@ struct FmmTree {
 struct Fmm {
     bool on = false;
     FmmTree t;
+    std::vector<FmmCell> plan, now;    // the cells' boxes as laid out, and as placed for the current bodies
     FmmCell* cells = nullptr;
     int4* box = nullptr;
     bool walls = false;                // the wall discrepancy runs by expansions too
@@ -343,7 +344,6 @@ struct bie_ctx {
     int* near_ctr = nullptr;    // work-queue counter of the persistent near sum (batches)
     bie::Fmm fmm[3];            // fast image sum per precision (0 single, 1 double, 2 double-float)
     void* fmm_ws = nullptr;     // its part of the workspace
-    std::vector<double> fmm_rects;          // 4 x ncell: the rectangles its boxes cover
     unsigned long long geometry = 0;        // bumped by build_geometry
     unsigned long long epoch = 0;  // bumped whenever a kernel argument of the operator application changes
     // contact-block right preconditioner (opts.precond, precond.cu)
@@ -461,7 +461,8 @@ __device__ inline double block_sum_d(double v, double* red) {
 // fmm.cu --------------------------------------------------------------------
 // pairs and translations of one near sum, for rooflines
 int fmm_work(bie_ctx* c, int prec, int64_t* pairs, int64_t* translations, int32_t* order);
-int fmm_plan(bie_ctx* c);             // boxes for the bodies' current places (host mirror)
+int fmm_plan(bie_ctx* c);             // boxes for the bodies' first places (host mirror)
+int fmm_fit(bie_ctx* c);              // the same boxes moved to where the bodies are now
 int fmm_build(bie_ctx* c, int prec);  // sorts the current geometry if it is not
 int fmm_up(bie_ctx* c, const double* sigma, int prec, Workspace& ws);      // moments of every box, and of every body
 // partials of every target from them; the close pairs' sums and, with

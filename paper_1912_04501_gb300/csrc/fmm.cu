@@ -603,6 +603,7 @@ constexpr int kWallImages = 6;
 struct SideArgs {
     int ncell, m, walls, npairs, ctas;  // ctas: four tasks each
     const double *wall, *bodyF;
+    const double *x, *y;
     double* gpart;
     const int4* pairs;
     const int* node_cell;
@@ -650,6 +651,27 @@ __global__ void __launch_bounds__(128) k_close_pairs(SideArgs a, const Cell* __r
     if (p < a.npairs) close_pair<B>(a, cells, p, threadIdx.x & 31);
 }
 
+// The same for one far image node by node, for a cell whose bodies reach so near to the
+// walls' images that no box is well away from them (FmmCell::wall -1: centres set far
+// outside the cell): velocity times 4 pi mu and traction times -pi, by k_disc's formulas,
+// in single precision (cell-centred) or double.
+template <typename S>
+__device__ __forceinline__ void wall_nodes(const SideArgs& a, const Cell& cl, S px, S py, S n0, S n1, int lane, S* v) {
+    constexpr bool F32 = sizeof(S) == 4;
+    for (int j = cl.node_off + lane; j < cl.node_off + cl.n_nodes; j += 32) {
+        const double2 sg = a.sigma[j];
+        const double w = a.w[j];
+        const S qx = (S)(sg.x * w), qy = (S)(sg.y * w);
+        const S rx = px - (F32 ? (S)(a.x[j] - cl.C[0]) : (S)a.x[j]), ry = py - (F32 ? (S)(a.y[j] - cl.C[1]) : (S)a.y[j]);
+        const S r2 = rx * rx + ry * ry, inv = S(1) / r2, rq = (rx * qx + ry * qy) * inv, l = S(-0.5) * log(r2);
+        const S cc = (rx * n0 + ry * n1) * rq * inv;
+        v[0] += l * qx + rx * rq;
+        v[1] += l * qy + ry * rq;
+        v[2] += cc * rx;
+        v[3] += cc * ry;
+    }
+}
+
 template <typename R>
 __device__ void side_tasks(const SideArgs& a, const FmmTree& t, const Cell* cells, const V4<R>* mp, int cta) {
     constexpr int P = FmmTypes<R>::P;
@@ -679,10 +701,17 @@ __device__ void side_tasks(const SideArgs& a, const FmmTree& t, const Cell* cell
             }
             const int wp = q / kWallImages, im = q % kWallImages;
             const FmmCell& f = t.cells[ci];
-            const int lv = f.wall, gx = f.gx[lv], n = gx * f.gy[lv];
+            const int lv = f.wall, gx = f.gx[max(lv, 0)], n = gx * f.gy[max(lv, 0)];
             const double* wt = a.wall + ((size_t)ci * 2 * a.m + wp) * kWallStride;
             S v[4] = {0, 0, 0, 0};
-            if constexpr (sizeof(R) == 4) {  // cell-centred single precision
+            if (lv < 0) {
+                if constexpr (sizeof(R) == 4) {
+                    const float* wf = reinterpret_cast<const float*>(wt + 16);
+                    wall_nodes<float>(a, cl, wf[2 * im], wf[2 * im + 1], wf[12], wf[13], lane, v);
+                } else {
+                    wall_nodes<double>(a, cl, wt[2 * im], wt[2 * im + 1], wt[12], wt[13], lane, v);
+                }
+            } else if constexpr (sizeof(R) == 4) {  // cell-centred single precision
                 const float* wf = reinterpret_cast<const float*>(wt + 16);
                 const float H = (float)f.h * (1 << lv), iH = 1.f / H;
                 const float px = wf[2 * im] - (float)f.ox, py = wf[2 * im + 1] - (float)f.oy, n0 = wf[12], n1 = wf[13];
@@ -717,7 +746,8 @@ __device__ void side_tasks(const SideArgs& a, const FmmTree& t, const Cell* cell
                 for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
             if (lane < 4) {
                 const double sg = im < 3 ? 1.0 : -1.0;
-                const double g = lane < 2 ? sg / (4.0 * kPi * cl.mu) : sg * f.inv_h / (4.0 * kPi * (1 << lv));
+                const double g = lane < 2 ? sg / (4.0 * kPi * cl.mu)
+                                          : (lv < 0 ? -sg / kPi : sg * f.inv_h / (4.0 * kPi * (1 << lv)));
                 gp[(size_t)im * 8 * a.m + 4 * wp + lane] =
                     g * (double)(lane == 0 ? v[0] : (lane == 1 ? v[1] : (lane == 2 ? v[2] : v[3])));
             }
@@ -1667,31 +1697,70 @@ static double fmm_wall_side(const bie_ctx* c, int k, int prec) {
     return (prec == 0 ? 0.3 : 0.45) * d * std::sqrt(2.0);
 }
 
+// The boxes of one cell for where its bodies are now: the grid as planned while it
+// covers their rectangle, and else moved and its side stretched until it does; then the
+// coarsest level that the walls' far images are well away from, which depends on the
+// lattice and the centres too.  The counts of boxes never change, so neither do any
+// kernel's arguments (a captured application stays right), and nothing is allocated.
+// Stretched leaves cost pairs (side times 1.6 for bodies listed a lattice vector away).
+static FmmCell fmm_place(const bie_ctx* c, int k, int prec) {
+    FmmCell f = c->fmm[prec].plan[k];
+    const FmmPlanCell r = fmm_rect(c, k);
+    const double x1 = std::max(f.ox + f.gx[0] * f.h, r.ox + r.w), y1 = std::max(f.oy + f.gy[0] * f.h, r.oy + r.ht);
+    if (r.ox < f.ox || r.oy < f.oy || r.ox + r.w > f.ox + f.gx[0] * f.h || r.oy + r.ht > f.oy + f.gy[0] * f.h) {
+        f.ox = std::min(f.ox, r.ox);
+        f.oy = std::min(f.oy, r.oy);
+        f.h = std::max((x1 - f.ox) / f.gx[0], (y1 - f.oy) / f.gy[0]);
+        f.inv_h = 1.0 / f.h;
+    }
+    const double wall = fmm_wall_side(c, k, prec);
+    f.wall = -1;
+    for (int l = 0; l < f.nlev; ++l)
+        if (f.h * (1 << l) <= wall) f.wall = l;
+    return f;
+}
+
+static void fmm_centres(const std::vector<FmmCell>& cells, float4* centre) {
+    for (const FmmCell& f : cells)
+        for (int l = 0; l < f.nlev; ++l)
+            for (int y = 0; y < f.gy[l]; ++y)
+                for (int x = 0; x < f.gx[l]; ++x) {
+                    const double2 p = fmm_centre(f, l, x, y);
+                    float4& o = centre[f.off[l] + (size_t)y * f.gx[l] + x];
+                    o.x = (float)p.x;
+                    o.y = (float)(p.x - (double)o.x);
+                    o.z = (float)p.y;
+                    o.w = (float)(p.y - (double)o.z);
+                }
+}
+
+// Called when a configuration is set (host mirrors of bodies and lattices).
+int fmm_fit(bie_ctx* c) {
+    for (int prec = 0; prec < 3; ++prec) {
+        Fmm& f = c->fmm[prec];
+        if (!f.on) continue;
+        bool moved = false;
+        for (int k = 0; k < c->ncell; ++k) {
+            const FmmCell q = fmm_place(c, k, prec);
+            FmmCell& o = f.now[k];
+            moved = moved || q.ox != o.ox || q.oy != o.oy || q.h != o.h || q.wall != o.wall;
+            o = q;
+        }
+        if (!moved) continue;
+        std::vector<float4> centre(f.t.nbox);
+        fmm_centres(f.now, centre.data());
+        BIE_CUDA(c, cudaMemcpyAsync(f.cells, f.now.data(), f.now.size() * sizeof(FmmCell), cudaMemcpyHostToDevice, c->stream));
+        BIE_CUDA(c, cudaMemcpyAsync(f.t.centre, centre.data(), centre.size() * sizeof(float4), cudaMemcpyHostToDevice,
+                                    c->stream));
+    }
+    return BIE_OK;
+}
+
 // Boxes of every precision whose near sums run faster this way.  Called when
-// a context is made and when a configuration is set; a plan whose rectangles
-// still hold every body is kept.
+// a context is made.
 int fmm_plan(bie_ctx* c) {
     std::vector<FmmPlanCell> rect(c->ncell);
     for (int k = 0; k < c->ncell; ++k) rect[k] = fmm_rect(c, k);
-    if (!c->fmm_rects.empty()) {
-        bool holds = true;
-        for (int k = 0; k < c->ncell; ++k) {
-            const double* o = &c->fmm_rects[4 * (size_t)k];
-            holds = holds && rect[k].ox >= o[0] && rect[k].oy >= o[1] && rect[k].ox + rect[k].w <= o[0] + o[2] &&
-                    rect[k].oy + rect[k].ht <= o[1] + o[3];
-        }
-        if (holds) return BIE_OK;
-        ++c->epoch;
-        free_fmm(c);
-    }
-    c->fmm_rects.resize(4 * (size_t)c->ncell);
-    for (int k = 0; k < c->ncell; ++k) {
-        double* o = &c->fmm_rects[4 * (size_t)k];
-        o[0] = rect[k].ox;
-        o[1] = rect[k].oy;
-        o[2] = rect[k].w;
-        o[3] = rect[k].ht;
-    }
     if (!BIE_FMM) return BIE_OK;
     std::vector<double> per(c->nb);
     for (int b = 0; b < c->nb; ++b) per[b] = body_perimeter(c, b);
@@ -1797,21 +1866,15 @@ int fmm_plan(bie_ctx* c) {
                             make_int4(k, l, x | (y << 16),
                                       l + 1 < fc.nlev ? fc.off[l + 1] + (y / 2) * fc.gx[l + 1] + x / 2 : -1);
         }
-        float4* centre = (float4*)&host[o_centre];
+        fmm_centres(cells, (float4*)&host[o_centre]);
         int4* grid = (int4*)&host[o_grid];
-        for (long long b = 0; b < nbox; ++b) {
-            const FmmCell& fc = cells[box[b].x];
-            grid[b] = make_int4(fc.off[box[b].y], fc.gx[box[b].y], 0, 0);
-            const double2 p = fmm_centre(fc, box[b].y, fmm_ix(box[b]), fmm_iy(box[b]));
-            centre[b].x = (float)p.x;
-            centre[b].y = (float)(p.x - (double)centre[b].x);
-            centre[b].z = (float)p.y;
-            centre[b].w = (float)(p.y - (double)centre[b].z);
-        }
+        for (long long b = 0; b < nbox; ++b)
+            grid[b] = make_int4(cells[box[b].x].off[box[b].y], cells[box[b].x].gx[box[b].y], 0, 0);
         if (prec == 0) fmm_tables<float>(&host[o_tab]);
         else if (prec == 1) fmm_tables<double>(&host[o_tab]);
         else fmm_tables<df>(&host[o_tab]);
         BIE_CUDA(c, cudaMemcpy(f.arena, host.data(), written, cudaMemcpyHostToDevice));
+        f.plan = f.now = cells;
         unsigned char* a = (unsigned char*)f.arena;
         FmmTree& t = f.t;
         t.nleaf = (int)nleaf;
@@ -1925,6 +1988,8 @@ static SideArgs side_args(bie_ctx* c, const double* sigma, int prec, bool walls,
     a.ctas = (int)((tasks + 3) / 4);
     a.wall = c->wall;
     a.bodyF = ws.bodyF;
+    a.x = c->x;
+    a.y = c->y;
     a.gpart = ws.gpart;
     a.pairs = c->cl.pairs;
     a.node_cell = c->node_cell;
