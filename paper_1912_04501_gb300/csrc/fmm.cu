@@ -531,8 +531,8 @@ k_fmm_up(FmmTree t, const Cell* __restrict__ cells, const double2* sigma, const 
 // beside the translations: wall discrepancy and close pairs
 // ---------------------------------------------------------------------------
 // The wall discrepancy (Sec. 6.2 step 2, the far-image form of k_disc) from the
-// moments of the boxes of one level: the six far images of a wall point lie a
-// cell away from every box, so the series converge by 0.3 per order or better.
+// moments of the boxes of one level, which the six far images of a wall point are well
+// away from (fmm_wall_side).
 // With u = 1 / W, W = (p - c) / H, per box
 //   velocity   4 pi mu u = -a_0 log|w| + (sum_{k>0} a_k u^k / k + conj(sum_{k>0} e_k u^k / k)
 //                          + conj(conj(W) A) + a_0) / 2,
@@ -1672,11 +1672,15 @@ static void fmm_tables(void* out) {
     }
 }
 
-// The largest box side from whose corners the walls' far images are so far that
-// the moments converge there by a factor of 0.3 per order (24 orders reach
-// 3e-13) or 0.45 (48 orders, 2e-17); <= 0: none.  The images of L and R lie on the
-// lines lattice coordinate s = +-3/2, those of D and U on t = +-3/2; nodes lie
-// within a bounding radius of their centres.
+// The largest box side that the walls' far images are well away from; <= 0: none.  The
+// images of L and R lie on the lines lattice coordinate s = +-3/2, those of D and U on
+// t = +-3/2; nodes lie within a bounding radius of their centres, so at least d from any
+// image.  A source at a box's corner is e = side / sqrt 2 from its centre, and an image may
+// be as near as d - e to that, so the moments converge by e / (d - e) per order at worst:
+// 3/7 in single precision (e = 0.3 d; 24 orders reach 1.5e-9) and 1/2 in double (e = d / 3;
+// 48 orders reach 3.6e-15, and sources elsewhere far less).  With e = 0.45 d, 0.45 per order
+// as the source sees it but 9/11 from the centre, the first terms left out added up to
+// 8e-12 on 25 bodies in a cell sheared by half.
 static double fmm_wall_side(const bie_ctx* c, int k, int prec) {
     const Cell& cl = c->cells_h[k];
     const double det = cl.e1[0] * cl.e2[1] - cl.e1[1] * cl.e2[0];
@@ -1694,7 +1698,7 @@ static double fmm_wall_side(const bie_ctx* c, int k, int prec) {
     if (cl.e1[1] == 0.0) e2x = std::max(e2x, 0.5 * std::fabs(cl.e1[0]));
     const double l2 = std::hypot(e2x, cl.e2[1]), l1 = std::hypot(cl.e1[0], cl.e1[1]);
     const double d = (1.5 - far) * std::fabs(det) / std::max(l1, l2) - R;
-    return (prec == 0 ? 0.3 : 0.45) * d * std::sqrt(2.0);
+    return (prec == 0 ? 0.3 : 1.0 / 3.0) * d * std::sqrt(2.0);
 }
 
 // The boxes of one cell for where its bodies are now: the grid as planned while it

@@ -129,3 +129,20 @@ def test_boxes_follow_a_configuration(program, skew, bodies, nodes):
             assert _tail(cell, e2, xc, box, ORDERS[prec]) < (6e-8 if prec == 0 else 1e-12), (prec, e2)
     # back where it began: the boxes as planned
     assert res[len(states)][1] == res[0][1]
+
+
+@pytest.mark.parametrize("seed", [1, 2, 3])
+@pytest.mark.parametrize("bodies,nodes", [(3, 1024), (25, 256), (100, 160)])
+def test_walls_series_of_sheared_cells(program, bodies, nodes, seed):
+    """The double series leave out less than a rounding for every source, whatever the
+    shear, where a box's corner nearest to an image holds the source farthest from the
+    box's centre."""
+    for skew in (0.3, 0.45, 0.5):
+        cell = workloads.random_cell(bodies, 0.3, (1.0, 3.0), 1e-2 if bodies < 60 else 2e-3, nodes, 1000 + seed,
+                                     e2=(skew, 1.0), equal_area=seed != 2, max_tries=2000000)
+        precs = _run(program, cell, ("plan", 0))[0][1]
+        home = np.array([b["xc"] for b in cell["bodies"]])
+        for prec in (1, 2):
+            on, walls, _, box = precs[prec]
+            assert on and walls
+            assert _tail(cell, cell["e2"], home, box, ORDERS[prec]) < 1e-16, (prec, skew)
