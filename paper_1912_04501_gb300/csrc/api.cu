@@ -587,11 +587,12 @@ int bie_init_batch(bie_ctx** out, int32_t n_cells, const bie_cell* cells, const 
         rc = rc ? rc : up(c->next.ypf, ypf.data(), ypf.size() * sizeof(float2));
     }
     rc = rc ? rc : up(c->e2d, c->e2_0.data(), c->e2_0.size() * sizeof(double));
-    rc = rc ? rc : fmm_plan(c);
-    rc = rc ? rc : build_near_items(c);
+    rc = rc ? rc : upload_cells(c, c->stream);
     rc = rc ? rc : build_dot_chunks(c);
     rc = rc ? rc : build_dirichlet_tables(c, 64);
     rc = rc ? rc : rebuild(c);
+    rc = rc ? rc : fmm_plan(c);
+    rc = rc ? rc : build_near_items(c);
     if (o.autotune) rc = rc ? rc : autotune_near32(c);
     rc = rc ? rc : cu(cudaStreamSynchronize(c->stream), "init sync");
     if (rc) {

@@ -1761,7 +1761,9 @@ int fmm_fit(bie_ctx* c) {
 }
 
 // Boxes of every precision whose near sums run faster this way.  Called when
-// a context is made.
+// a context is made, after all else has its memory: a precision whose boxes do not fit
+// beside it keeps the direct sum (all of them, where the moments do not fit).  Nothing
+// of the context refers to the boxes before they are complete.
 int fmm_plan(bie_ctx* c) {
     std::vector<FmmPlanCell> rect(c->ncell);
     for (int k = 0; k < c->ncell; ++k) rect[k] = fmm_rect(c, k);
@@ -1771,8 +1773,17 @@ int fmm_plan(bie_ctx* c) {
     const int N = c->N, nsrc = N * c->srcmul;
     size_t mp_bytes = 0, loc_bytes = 0, sq_bytes = 0;
     int max_box = 0;
+    Fmm made[3];
+    auto drop = [&](cudaError_t e, const char* what) {  // nothing kept; BIE_OK if memory was short
+        for (Fmm& f : made)
+            if (f.arena) cudaFree(f.arena);
+        if (c->fmm_ws) cudaFree(c->fmm_ws);
+        c->fmm_ws = nullptr;
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? BIE_OK : cuda_check(c, e, what);
+    };
     for (int prec = 0; prec < 3; ++prec) {
-        Fmm& f = c->fmm[prec];
+        Fmm f;
         std::vector<FmmCell> cells(c->ncell);
         double t_fast = kFmmFixed[prec], t_direct = 0;
         long long nleaf = 0, nbox = 0;
@@ -1857,7 +1868,12 @@ int fmm_plan(bie_ctx* c) {
         const size_t o_tcount = ut ? place(nbox * sizeof(int)) : 0, o_tstart = ut ? place((nleaf + 1) * sizeof(int)) : 0,
                      o_tperm = ut ? place(N * sizeof(int)) : 0,
                      o_tpos = ut ? place(N * (dbl ? sizeof(double2) : sizeof(float4))) : 0;
-        BIE_CUDA(c, cudaMalloc(&f.arena, total));
+        if (const cudaError_t e = cudaMalloc(&f.arena, total)) {
+            f.arena = nullptr;
+            if (e != cudaErrorMemoryAllocation) return drop(e, "cudaMalloc");
+            cudaGetLastError();
+            continue;
+        }
         std::vector<unsigned char> host(written);
         std::memcpy(&host[o_cells], cells.data(), cells.size() * sizeof(FmmCell));
         int4* box = (int4*)&host[o_box];
@@ -1877,7 +1893,10 @@ int fmm_plan(bie_ctx* c) {
         if (prec == 0) fmm_tables<float>(&host[o_tab]);
         else if (prec == 1) fmm_tables<double>(&host[o_tab]);
         else fmm_tables<df>(&host[o_tab]);
-        BIE_CUDA(c, cudaMemcpy(f.arena, host.data(), written, cudaMemcpyHostToDevice));
+        if (const cudaError_t e = cudaMemcpy(f.arena, host.data(), written, cudaMemcpyHostToDevice)) {
+            cudaFree(f.arena);
+            return drop(e, "cudaMemcpy");
+        }
         f.plan = f.now = cells;
         unsigned char* a = (unsigned char*)f.arena;
         FmmTree& t = f.t;
@@ -1919,18 +1938,23 @@ int fmm_plan(bie_ctx* c) {
         loc_bytes = std::max(loc_bytes, f.loc_bytes);
         sq_bytes = std::max(sq_bytes, f.sq_bytes);
         max_box = std::max(max_box, (int)nbox);
+        made[prec] = f;
     }
     if (max_box) {
         auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
         const size_t tick = up(max_box * sizeof(unsigned));
-        BIE_CUDA(c, cudaMalloc(&c->fmm_ws, tick + up(sq_bytes) + up(mp_bytes) + up(loc_bytes)));
+        if (const cudaError_t e = cudaMalloc(&c->fmm_ws, tick + up(sq_bytes) + up(mp_bytes) + up(loc_bytes))) {
+            c->fmm_ws = nullptr;
+            return drop(e, "cudaMalloc");
+        }
+        if (const cudaError_t e = cudaMemset(c->fmm_ws, 0, tick)) return drop(e, "cudaMemset");
         unsigned char* a = (unsigned char*)c->fmm_ws;
         c->ws.ftick = (unsigned*)a;
         c->ws.fsq = a + tick;
         c->ws.fmp = a + tick + up(sq_bytes);
         c->ws.floc = a + tick + up(sq_bytes) + up(mp_bytes);
-        BIE_CUDA(c, cudaMemset(c->ws.ftick, 0, tick));
     }
+    for (int prec = 0; prec < 3; ++prec) c->fmm[prec] = made[prec];
     return BIE_OK;
 }
 

@@ -146,3 +146,22 @@ def test_walls_series_of_sheared_cells(program, bodies, nodes, seed):
             on, walls, _, box = precs[prec]
             assert on and walls
             assert _tail(cell, cell["e2"], home, box, ORDERS[prec]) < 1e-16, (prec, skew)
+
+
+@pytest.mark.parametrize("doubled", [0, 1])
+def test_short_memory_leaves_the_direct_sum(program, doubled):
+    """An allocation that fails costs its precision the boxes (the moments', all three),
+    never the context: no error is left, nothing half made stays, and a configuration can
+    be set all the same."""
+    cell = workloads.random_cell(40, 0.25, (1.0, 2.0), 5e-3, 256, 2, e2=(0.2, 1.0))
+    home = np.array([b["xc"] for b in cell["bodies"]])
+    for fail in range(0, 5):
+        plan, state, end = _run(program, cell, ("plan", fail), ("set", cell["e2"], home + [0.4, 0.0]), doubled=doubled)
+        off = {0: (), 1: (0,), 2: (1,), 3: (2,), 4: (0, 1, 2)}[fail]
+        for status, precs in (plan, state):
+            assert status["rc"] == 0 and status["error"] == 0
+            assert status["calls"] == 4
+            assert status["live"] == (0 if fail == 4 else 4 - len(off)) and status["work"] == (fail != 4)
+            for prec, (on, _, held, _) in precs.items():
+                assert (on, held) == ((0, 0) if prec in off else (1, 1))
+        assert end[0]["live"] == 0
