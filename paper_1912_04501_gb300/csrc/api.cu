@@ -243,6 +243,8 @@ int prof_fold(bie_ctx* c) {
 static int rebuild(bie_ctx* c) {
     int rc = build_geometry(c);
     if (rc) return rc;
+    rc = fmm_build_static(c);
+    if (rc) return rc;
     rc = build_proxy_fit(c);
     if (rc) return rc;
     rc = build_close(c);
@@ -593,6 +595,7 @@ int bie_init_batch(bie_ctx** out, int32_t n_cells, const bie_cell* cells, const 
     rc = rc ? rc : rebuild(c);
     rc = rc ? rc : fmm_plan(c);
     rc = rc ? rc : build_near_items(c);
+    rc = rc ? rc : fmm_build_static(c);
     if (o.autotune) rc = rc ? rc : autotune_near32(c);
     rc = rc ? rc : cu(cudaStreamSynchronize(c->stream), "init sync");
     if (rc) {
@@ -816,6 +819,7 @@ int bie_step(bie_ctx* c, double dt, int32_t n_steps, double* mu_eff_out, bie_sol
         std::swap(c->yp, c->next.yp);
         std::swap(c->ypf, c->next.ypf);
         if ((rc = build_geometry(c))) return rc;
+        if ((rc = fmm_build_static(c))) return rc;
         std::swap(c->cl.dmin, c->cl.dmin_prev);
         c->cl.have_dprev = true;
         if ((rc = build_close(c))) return rc;

@@ -13,7 +13,6 @@
 
 // 4 MiB, held by every GPU that loads the library until the process exits.
 #define BIE_STATIC_SCRATCH_BYTES (4u << 20)
-#define BIE_STATIC_MAX_NODES 8192
 #define BIE_STATIC_MAX_DEVICES 64
 
 static __device__ __align__(256) unsigned char bie_static_scratch[BIE_STATIC_SCRATCH_BYTES];
@@ -31,10 +30,10 @@ extern "C" int bie_apply_static(bie_ctx* c, const double* sigma, double* out) {
     using namespace bie;
     if (!c || !sigma || !out) return BIE_EINVAL;
     const size_t N = (size_t)c->N;
-    if (c->N > BIE_STATIC_MAX_NODES)
+    if (c->N > kStaticMaxNodes)
         return fail(c, BIE_EINVAL, "bie_apply_static: the context has " + std::to_string(c->N) +
                                        " nodes; the static scratch serves at most " +
-                                       std::to_string(BIE_STATIC_MAX_NODES));
+                                       std::to_string(kStaticMaxNodes));
     if (c->device < 0 || c->device >= BIE_STATIC_MAX_DEVICES)
         return fail(c, BIE_EINVAL, "bie_apply_static: device ordinal out of range");
     // layout of the per-call buffers inside the static array (the doubled-cell

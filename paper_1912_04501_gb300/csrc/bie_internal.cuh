@@ -72,6 +72,7 @@ constexpr int kCloseAccNodes = 4096;  // source nodes per CTA of k_close_blocks 
 constexpr int kMaxBodyNodes = 16384;  // nodes per body
 constexpr int kPcMaxNodes = 1024;     // nodes of the contact-block preconditioner: [A_SS | I] (67 MB) stays in L2
 constexpr int kMaxCells = 4096;
+constexpr int kStaticMaxNodes = 8192; // nodes of the contexts that bie_apply_static takes
 constexpr int kWallStride = 24;       // doubles per wall point of the wall table (see k_wall_table)
 constexpr int kNetHidden = 64;        // hidden width of the warm-start network
 constexpr int kNetMaxIn = 16;         // its maximum number of inputs per node
@@ -464,6 +465,7 @@ int fmm_work(bie_ctx* c, int prec, int64_t* pairs, int64_t* translations, int32_
 int fmm_plan(bie_ctx* c);             // boxes for the bodies' first places (host mirror)
 int fmm_fit(bie_ctx* c);              // the same boxes moved to where the bodies are now
 int fmm_build(bie_ctx* c, int prec);  // sorts the current geometry if it is not
+int fmm_build_static(bie_ctx* c);     // the same with every geometry, for bie_apply_static
 int fmm_up(bie_ctx* c, const double* sigma, int prec, Workspace& ws);      // moments of every box, and of every body
 // partials of every target from them; the close pairs' sums and, with
 // Fmm::walls, the wall discrepancy and the proxy strengths

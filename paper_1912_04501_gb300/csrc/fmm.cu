@@ -601,7 +601,8 @@ constexpr int kWallImages = 6;
 // gpart[((cell 7) + image) 8m + 4 wp + component]; then one per cell for its
 // total force (slot 6); then the close pairs (Sec. 6.3), C_p sigma into psum[p].
 struct SideArgs {
-    int ncell, m, walls, npairs, ctas;  // ctas: four tasks each
+    int ncell, m, walls, ctas;  // ctas: four tasks each
+    const int* npairs;          // on the device (a replayed capture meets later geometries), or null: none
     const double *wall, *bodyF;
     const double *x, *y;
     double* gpart;
@@ -647,8 +648,8 @@ __device__ __forceinline__ void close_pair(const SideArgs& a, const Cell* cells,
 
 template <typename B>
 __global__ void __launch_bounds__(128) k_close_pairs(SideArgs a, const Cell* __restrict__ cells) {
-    const int p = blockIdx.x * 4 + (threadIdx.x >> 5);
-    if (p < a.npairs) close_pair<B>(a, cells, p, threadIdx.x & 31);
+    for (int p = blockIdx.x * 4 + (threadIdx.x >> 5); p < *a.npairs; p += 4 * a.ctas)
+        close_pair<B>(a, cells, p, threadIdx.x & 31);
 }
 
 // The same for one far image node by node, for a cell whose bodies reach so near to the
@@ -678,7 +679,7 @@ __device__ void side_tasks(const SideArgs& a, const FmmTree& t, const Cell* cell
     typedef typename WallReal<R>::T S;
     __shared__ R s_inv[P];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int task = cta * 4 + wid;
+    int task = cta * 4 + wid, step = 4 * a.ctas;
     if (a.walls) {
         for (int k = threadIdx.x; k < P; k += 128) s_inv[k] = R(k ? 1.0 / k : 0.0);
         __syncthreads();
@@ -754,10 +755,13 @@ __device__ void side_tasks(const SideArgs& a, const FmmTree& t, const Cell* cell
             return;
         }
         task -= a.ncell * per;
+        step -= a.ncell * per;
     }
-    if (task >= a.npairs) return;
-    if constexpr (sizeof(R) == 4) close_pair<float>(a, cells, task, lane);
-    else close_pair<double>(a, cells, task, lane);
+    if (!a.npairs) return;
+    for (const int n = *a.npairs; task < n; task += step) {
+        if constexpr (sizeof(R) == 4) close_pair<float>(a, cells, task, lane);
+        else close_pair<double>(a, cells, task, lane);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1959,7 +1963,8 @@ int fmm_plan(bie_ctx* c) {
 }
 
 // Sorts the current geometry's records into the boxes (once per geometry and
-// precision, when an application first needs it).
+// precision, when an application first needs it; work that is only recorded by a stream
+// capture has not sorted anything yet).
 int fmm_build(bie_ctx* c, int prec) {
     Fmm& f = c->fmm[prec];
     if (!f.on || f.built == c->geometry) return BIE_OK;
@@ -1982,9 +1987,17 @@ int fmm_build(bie_ctx* c, int prec) {
     }
     k_fmm_lists<<<t.nbox, 128, 0, c->stream>>>(t, c->cells, c->utilde ? 1 : 9);
     BIE_LAUNCH(c, "k_fmm_lists");
-    f.built = c->geometry;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture == cudaStreamCaptureStatusNone) f.built = c->geometry;
     return BIE_OK;
 }
+
+// bie_apply_static may be captured by the caller and replayed for later geometries: the
+// contexts that it takes have their boxes sorted with every geometry, so that no capture
+// holds the sorting and every replay finds the current one.  (All other applications end
+// in a wait and cannot be captured.)
+int fmm_build_static(bie_ctx* c) { return c->N <= kStaticMaxNodes ? fmm_build(c, 0) : BIE_OK; }
 
 template <typename R>
 static int up_launch(bie_ctx* c, const double* sigma, int prec, Workspace& ws) {
@@ -2011,8 +2024,8 @@ static SideArgs side_args(bie_ctx* c, const double* sigma, int prec, bool walls,
     a.ncell = c->ncell;
     a.m = c->m;
     a.walls = walls ? 1 : 0;
-    a.npairs = c->cl.npairs;
-    const long long tasks = (walls ? (long long)c->ncell * (2 * c->m * kWallImages + 1) : 0) + a.npairs;
+    a.npairs = c->cl.npairs > 0 ? c->cl.pair_base + c->N : nullptr;
+    const long long tasks = (walls ? (long long)c->ncell * (2 * c->m * kWallImages + 1) : 0) + c->cl.npairs;
     a.ctas = (int)((tasks + 3) / 4);
     a.wall = c->wall;
     a.bodyF = ws.bodyF;
@@ -2032,7 +2045,7 @@ static SideArgs side_args(bie_ctx* c, const double* sigma, int prec, bool walls,
 
 int close_pairs(bie_ctx* c, const double* sigma, int prec, Workspace& ws, cudaStream_t st) {
     const SideArgs a = side_args(c, sigma, prec, false, ws);
-    if (a.npairs == 0) return BIE_OK;
+    if (!a.npairs) return BIE_OK;
     if (prec == 0) k_close_pairs<float><<<a.ctas, 128, 0, st>>>(a, c->cells);
     else k_close_pairs<double><<<a.ctas, 128, 0, st>>>(a, c->cells);
     BIE_LAUNCH(c, "k_close_pairs");

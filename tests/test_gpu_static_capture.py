@@ -1,0 +1,82 @@
+"""GPU tests of bie_apply_static on a stream of the caller's own, captured into a CUDA graph
+between configurations: an application before the first replay, replays after later
+configurations (inside and outside the boxes as laid out, with more close pairs and with
+fewer) and plain calls all equal a context that never saw a capture, bit for bit (the same
+kernels on the same numbers)."""
+import numpy as np
+import pytest
+
+from paper_1912_04501_gb300 import workloads
+
+pytestmark = pytest.mark.gpu
+
+bie = pytest.importorskip("paper_1912_04501_gb300.bie")
+torch = pytest.importorskip("torch")
+
+
+def _placed(cell, dx=0.0, dy=0.0, tall=1.0):
+    c = cell["centre"]
+    return [[b["xc"][0] + dx, c[1] + tall * (b["xc"][1] - c[1]) + dy] for b in cell["bodies"]]
+
+
+@pytest.mark.parametrize("which", ["fast", "direct", "doubled"])
+def test_capture_between_configurations(which):
+    cell = workloads.random_cell(*((4, 0.2, (1.0, 2.0), 1e-2, 64, 3) if which == "direct" else
+                                   (40, 0.25, (1.0, 2.0), 1.2e-2, 160, 5)))
+    cell.update(solver=dict(n_proxy=48, proxy_radius=1.5, n_coll=24, gmres_tol=1e-10))
+    kw = dict(n_images=4, n_proxy=128, n_coll=32) if which == "doubled" else {}
+    ctx = bie.Context(cell, precision=bie.BIE_MIXED, **kw)
+    ref = bie.Context(cell, precision=bie.BIE_MIXED, **kw)
+    assert (ctx.near_work(bie.BIE_MIXED)[1] > 0) == (which != "direct")
+    # the close pairs' storage holds this many: no later configuration may have more (it
+    # would be moved, and a captured application with it left behind)
+    most, room = ctx.close_info()[0], min(ctx.N, 1024)
+    assert most + 8 < room or most > room
+    theta = [b["theta"] for b in cell["bodies"]]
+    sigma = torch.tensor(np.random.default_rng(3).standard_normal(2 * ctx.N), device="cuda")
+    out, eager, want = torch.empty_like(sigma), torch.empty_like(sigma), torch.empty_like(sigma)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ctx.set_stream(stream.cuda_stream)
+    ctx.apply_static(sigma, out)  # looks up the array's address, before any capture
+    stream.synchronize()
+
+    def at(e2, xc):
+        ctx.set_state(0.0, e2, xc, theta)
+        ref.set_state(0.0, e2, xc, theta)
+        ref.apply(sigma, want, precision=bie.BIE_MIXED)
+        torch.cuda.synchronize()
+        n = ctx.close_info()[0]
+        assert n <= most + 8
+        return n
+
+    # a taller cell: the bodies farther apart, fewer close pairs
+    few = at((0.0, 1.06), _placed(cell, tall=1.06))
+    assert 0 < few < most
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        ctx.apply_static(sigma, out)
+    # the capture ran nothing: an application before its first replay
+    ctx.apply(sigma, eager, precision=bie.BIE_MIXED)
+    assert torch.equal(eager, want)
+
+    def replay():
+        out.fill_(float("nan"))
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            graph.replay()
+        stream.synchronize()
+        assert torch.equal(out, want)
+
+    replay()
+    states = [((0.0, 1.0), _placed(cell)), ((0.0, 1.06), _placed(cell, 0.03, 0.04, 1.06))]
+    if which != "doubled":  # past the cell, and the same lattice by another second vector
+        states += [((0.0, 1.0), _placed(cell, 1.1)), ((1.0, 1.0), _placed(cell)), ((0.0, 1.0), _placed(cell))]
+    for e2, xc in states:
+        at(e2, xc)
+        replay()
+        ctx.apply_static(sigma, eager)
+        stream.synchronize()
+        assert torch.equal(eager, want)
+    ctx.close()
+    ref.close()
