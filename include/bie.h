@@ -293,8 +293,8 @@ int bie_set_history(bie_ctx* ctx, const double* sigma_prev2, const double* d2, d
 
 /* bie_apply_static: the same operator application as
  * bie_apply(ctx, sigma, out, BIE_MIXED, 1), but it allocates no device memory
- * at all and, but for the fast image sum's moments and the close pairs' sums,
- * does not touch the per-call buffers that bie_init allocated.  It
+ * at all and does not touch the per-call buffers that bie_init allocated for
+ * the other calls.  It
  * has no counterpart in the paper; it exists for callers that may not call
  * cudaMalloc -- for instance code running inside a host application whose own
  * memory manager owns the device heap and forbids other allocations -- yet
@@ -309,7 +309,8 @@ int bie_set_history(bie_ctx* ctx, const double* sigma_prev2, const double* d2, d
  *   reaches the end of it.
  * Its per-call scratch is one static device array of 4 MiB inside the
  * library, which every GPU that loads the library keeps until the process
- * exits.  Contexts with more than 8192 nodes (or whose buffers would not fit
+ * exits, and, for the fast image sum's moments and the close pairs' sums, a
+ * few MiB of the context's that bie_init allocated for this call alone.  Contexts with more than 8192 nodes (or whose buffers would not fit
  * the 4 MiB) are rejected with BIE_EINVAL and a message.  All calls share
  * that array and it keeps the last call's contents; each call writes every
  * buffer it reads, so nothing needs clearing, but calls that overlap on the

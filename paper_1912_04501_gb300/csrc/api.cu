@@ -43,7 +43,7 @@ static void free_all(bie_ctx* c) {
                     c->sv.w, c->sv.r, c->sv.x, c->sv.b, c->sv.d, c->sv.h, c->sv.fac, c->sv.dpart,
                     c->sv.chunks,
                     c->sv.cell_chunks, c->sv.sigma_prev, c->sv.sigma_prev2, c->sv.aug, c->sv.d2,
-                    c->sv.feat, c->sv.pred, c->cl.dmin, c->cl.dmin_prev, c->cl.ddir, c->cl.slots, c->cl.count, c->cl.pair_base, c->cl.pairs, c->cl.psum,
+                    c->sv.feat, c->sv.pred, c->cl.dmin, c->cl.dmin_prev, c->cl.ddir, c->cl.slots, c->cl.count, c->cl.pair_base, c->cl.pairs, c->cl.psum, c->cl.psum_static,
                     c->cl.blk_off, c->cl.blocks, c->cl.blocks32, c->cl.flags, c->cl.dtab, c->cl.dtab_off,
                     c->cl.bkd, c->cl.bcot, c->cl.bary, c->near[0].items,
                     c->near[1].items, c->near[2].items};
@@ -531,6 +531,7 @@ int bie_init_batch(bie_ctx** out, int32_t n_cells, const bie_cell* cells, const 
         rc = rc ? rc : dalloc(c, &c->cl.pairs, c->cl.cap_pairs);
         rc = rc ? rc : dalloc(c, &c->cl.blk_off, c->cl.cap_pairs);
         rc = rc ? rc : dalloc(c, &c->cl.psum, c->cl.cap_pairs);
+        if (n <= kStaticMaxNodes) rc = rc ? rc : dalloc(c, &c->cl.psum_static, c->cl.cap_pairs);
         rc = rc ? rc : dalloc(c, &c->cl.blocks, (size_t)c->cl.cap_doubles);
         rc = rc ? rc : dalloc(c, &c->cl.blocks32, (size_t)c->cl.cap_doubles);
         rc = rc ? rc : dalloc(c, &c->cl.flags, 10);

@@ -1,11 +1,11 @@
 // bie_apply_static: the single-precision-pair operator application with no
 // device allocation.  Every per-call buffer (source records, near-sum
-// partials, wall-discrepancy partials, body moments, proxy strengths) lives in one file-scope static device array, but for the moments of the
-// fast image sum and the close pairs' sums, whose space the context has had since it
-// was made.  Of the context it reads the geometry, proxy fit, close tables and work
-// items; it writes those sums, its launch counter and, with bie_profile on, the
-// profiler's event state, so calls on one context must not overlap (as for every
-// entry point).  See
+// partials, wall-discrepancy partials, body moments, proxy strengths) lives in
+// one file-scope static device array, but for the moments of the fast image sum and
+// the close pairs' sums, which the context has a second set of, for this call alone.
+// Of the context it reads the geometry, proxy fit, close tables and work items; it
+// writes that set, its launch counter and, with bie_profile on, the profiler's event
+// state, so calls on one context must not overlap (as for every entry point).  See
 // include/bie.h for who needs this and the limits.
 #include <mutex>
 
@@ -93,13 +93,14 @@ extern "C" int bie_apply_static(bie_ctx* c, const double* sigma, double* out) {
     ws.gt = reinterpret_cast<double*>(base + o);
     o += b_gt;
     ws.dticket = reinterpret_cast<unsigned int*>(base + o);
-    // the fast image sum's moments (and the close pairs' sums) stay in what the
-    // context was made with: up to some 700 bytes a box, which the array could not
-    // hold for every context it serves
-    ws.fsq = c->ws.fsq;
-    ws.fmp = c->ws.fmp;
-    ws.floc = c->ws.floc;
-    ws.ftick = c->ws.ftick;
+    // the fast image sum's moments and the close pairs' sums have space of this call's own,
+    // made with the context: up to some 700 bytes a box, which the array could not hold
+    // for every context it serves
+    ws.fsq = c->fmm_static.fsq;
+    ws.fmp = c->fmm_static.fmp;
+    ws.floc = c->fmm_static.floc;
+    ws.ftick = c->fmm_static.ftick;
+    ws.of_static = true;
     // the wall-discrepancy kernel's last-block counters must start at zero
     // (they return to zero when it finishes)
     BIE_CUDA(c, cudaMemsetAsync(ws.dticket, 0, b_tk, c->stream));

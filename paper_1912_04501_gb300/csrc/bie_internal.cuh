@@ -115,6 +115,7 @@ struct Close {
                                   //  violations (bit 0: a node beyond the doubled cell, bit 1: a close
                                   //  pair's body image not wholly among its nodes' images), block doubles (8 bytes)]
     double2* psum = nullptr;      // cap_pairs: the pairs' sums of one application
+    float2* psum_static = nullptr;  // cap_pairs: the same for bie_apply_static (contexts that it takes)
     int cap_pairs = 0;
     long long cap_doubles = 0;
     bool grow = true;             // storage grows on demand (no close_capacity given)
@@ -158,7 +159,7 @@ struct Workspace {
     double* vpart = nullptr;    // nb x kVelSplits x 3 velocity partials
     // fast image sum: sorted strengths, multipole and local expansions, and
     // the last-child counters of the upward pass (zero between launches)
-    void* psum = nullptr;       // close pairs' sums (null: Close::psum)
+    bool of_static = false;     // bie_apply_static's: the close pairs' sums are Close::psum_static
     void *fsq = nullptr, *fmp = nullptr, *floc = nullptr;
     unsigned* ftick = nullptr;
 };
@@ -344,7 +345,8 @@ struct bie_ctx {
     int n_fin = 0;
     int* near_ctr = nullptr;    // work-queue counter of the persistent near sum (batches)
     bie::Fmm fmm[3];            // fast image sum per precision (0 single, 1 double, 2 double-float)
-    void* fmm_ws = nullptr;     // its part of the workspace
+    void* fmm_ws = nullptr;     // its part of the workspace, and bie_apply_static's
+    bie::Workspace fmm_static;  // the latter's fsq, fmp, floc and ftick (contexts that it takes)
     unsigned long long geometry = 0;        // bumped by build_geometry
     unsigned long long epoch = 0;  // bumped whenever a kernel argument of the operator application changes
     // contact-block right preconditioner (opts.precond, precond.cu)

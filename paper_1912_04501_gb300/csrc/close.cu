@@ -765,6 +765,7 @@ int build_close(bie_ctx* c) {
             int rc = regrow(c, &c->cl.pairs, cap);
             rc = rc ? rc : regrow(c, &c->cl.blk_off, cap);
             rc = rc ? rc : regrow(c, &c->cl.psum, cap);
+            if (c->N <= kStaticMaxNodes) rc = rc ? rc : regrow(c, &c->cl.psum_static, cap);
             if (rc) return rc;
             c->cl.cap_pairs = cap;
         }
@@ -1308,7 +1309,7 @@ static int finish_launch(bie_ctx* c, const double* sigma, int prec, const Worksp
     a.xi = ws.xi;
     a.xif = ws.xif;
     a.pair_base = c->cl.pair_base;
-    a.psum = ws.psum ? ws.psum : c->cl.psum;
+    a.psum = ws.of_static ? (const void*)c->cl.psum_static : (const void*)c->cl.psum;
     a.sigma = reinterpret_cast<const double2*>(sigma);
     a.tgt32 = c->tgt32;
     a.xw = c->xw;

@@ -1620,6 +1620,7 @@ void free_fmm(bie_ctx* c) {
     c->fmm_ws = nullptr;
     c->ws.fsq = c->ws.fmp = c->ws.floc = nullptr;
     c->ws.ftick = nullptr;
+    c->fmm_static = Workspace{};
 }
 
 // Table sizes in numbers of R: hankel, binom, then the child powers.
@@ -1946,17 +1947,27 @@ int fmm_plan(bie_ctx* c) {
     }
     if (max_box) {
         auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+        // counters (a set for bie_apply_static's single-precision sum after the context's),
+        // then sorted strengths and expansions, again for the context and for that call
         const size_t tick = up(max_box * sizeof(unsigned));
-        if (const cudaError_t e = cudaMalloc(&c->fmm_ws, tick + up(sq_bytes) + up(mp_bytes) + up(loc_bytes))) {
+        const Fmm& s = made[0];
+        const bool own = s.on && N <= kStaticMaxNodes;
+        const size_t whole = up(sq_bytes) + up(mp_bytes) + up(loc_bytes),
+                     second = own ? up(s.sq_bytes) + up(s.mp_bytes) + up(s.loc_bytes) : 0;
+        if (const cudaError_t e = cudaMalloc(&c->fmm_ws, 2 * tick + whole + second)) {
             c->fmm_ws = nullptr;
             return drop(e, "cudaMalloc");
         }
-        if (const cudaError_t e = cudaMemset(c->fmm_ws, 0, tick)) return drop(e, "cudaMemset");
+        if (const cudaError_t e = cudaMemset(c->fmm_ws, 0, 2 * tick)) return drop(e, "cudaMemset");
         unsigned char* a = (unsigned char*)c->fmm_ws;
-        c->ws.ftick = (unsigned*)a;
-        c->ws.fsq = a + tick;
-        c->ws.fmp = a + tick + up(sq_bytes);
-        c->ws.floc = a + tick + up(sq_bytes) + up(mp_bytes);
+        auto lay = [&](Workspace& ws, unsigned char* ticks, unsigned char* at, size_t sq, size_t mp) {
+            ws.ftick = (unsigned*)ticks;
+            ws.fsq = at;
+            ws.fmp = at + up(sq);
+            ws.floc = at + up(sq) + up(mp);
+        };
+        lay(c->ws, a, a + 2 * tick, sq_bytes, mp_bytes);
+        if (own) lay(c->fmm_static, a + tick, a + 2 * tick + whole, s.sq_bytes, s.mp_bytes);
     }
     for (int prec = 0; prec < 3; ++prec) c->fmm[prec] = made[prec];
     return BIE_OK;
@@ -2039,7 +2050,7 @@ static SideArgs side_args(bie_ctx* c, const double* sigma, int prec, bool walls,
     a.body = c->body;
     a.sigma = reinterpret_cast<const double2*>(sigma);
     a.w = c->w;
-    a.psum = ws.psum ? ws.psum : c->cl.psum;
+    a.psum = ws.of_static ? (void*)c->cl.psum_static : (void*)c->cl.psum;
     return a;
 }
 

@@ -80,3 +80,28 @@ def test_capture_between_configurations(which):
         assert torch.equal(eager, want)
     ctx.close()
     ref.close()
+
+
+def test_beside_the_context_s_other_calls():
+    """The allocation-free application on one stream while the context's own application
+    runs on another: neither writes what the other reads."""
+    cell = workloads.random_cell(40, 0.25, (1.0, 2.0), 1.2e-2, 160, 5)
+    cell.update(solver=dict(n_proxy=48, proxy_radius=1.5, n_coll=24, gmres_tol=1e-10))
+    ctx = bie.Context(cell, precision=bie.BIE_MIXED)
+    assert ctx.near_work(bie.BIE_MIXED)[1] > 0 and ctx.close_info()[0] > 0
+    rng = np.random.default_rng(4)
+    a, b = (torch.tensor(rng.standard_normal(2 * ctx.N), device="cuda") for _ in range(2))
+    want_a, want_b, got_a, got_b = (torch.empty_like(a) for _ in range(4))
+    ctx.apply(a, want_a, precision=bie.BIE_MIXED)
+    ctx.apply(b, want_b, precision=bie.BIE_MIXED)
+    one, two = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(100):
+        ctx.set_stream(one.cuda_stream)
+        for _ in range(3):
+            ctx.apply_static(a, got_a)
+        ctx.set_stream(two.cuda_stream)
+        ctx.apply(b, got_b, precision=bie.BIE_MIXED)  # waits for the second stream only
+        one.synchronize()
+        assert torch.equal(got_a, want_a) and torch.equal(got_b, want_b)
+    ctx.close()
