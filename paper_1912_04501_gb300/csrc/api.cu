@@ -981,8 +981,10 @@ int bie_set_partition(bie_ctx* c, int32_t body_begin, int32_t body_end,
     c->shard.n1 = c->offsets[body_end];
     c->shard.exchange = whole ? nullptr : exchange;
     c->shard.user = whole ? nullptr : user;
+    for (Fmm& f : c->fmm) f.built = 0;  // the boxes' counts of wanted targets change
     int rc = build_near_items(c);
     if (rc) return rc;
+    if ((rc = fmm_build_static(c))) return rc;
     BIE_CUDA(c, cudaStreamSynchronize(c->stream));
     return BIE_OK;
 }

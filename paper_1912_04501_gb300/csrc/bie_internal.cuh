@@ -255,6 +255,7 @@ struct FmmTree {
     int* nnear = nullptr;
     float4* shift = nullptr;       // 9 per cell: image shifts in leaf sides, float pairs
     int *scount = nullptr, *tcount = nullptr;  // nbox: records in the box
+    int* wanted = nullptr;         // nbox: targets to evaluate in the box (tcount, but for a target partition)
     int *sstart = nullptr, *tstart = nullptr;  // nleaf + 1: first sorted record
     int *sperm = nullptr, *tperm = nullptr;    // sorted record -> record (sources: node, or 4 node + image)
     float4 *spos = nullptr, *tpos = nullptr;   // sorted positions from the cell centre, double-float
@@ -269,6 +270,7 @@ struct Fmm {
     int4* box = nullptr;
     bool walls = false;                // the wall discrepancy runs by expansions too
     int *cursor = nullptr, *leaf = nullptr, *raw = nullptr;  // sorting scratch
+    int* owned = nullptr;              // nbox: a partition's counts (single cells)
     unsigned long long built = 0;      // geometry the records are sorted for (0: none)
     int shares = 1;                    // CTAs a box's list is split over
     size_t mp_bytes = 0, loc_bytes = 0, sq_bytes = 0;  // multipole and local expansions, sorted strengths

@@ -158,25 +158,33 @@ __device__ __forceinline__ int fmm_leaf(const FmmCell& f, double2 p) {
 }
 
 // Leaf of every record, and the record counts of its box and the box's ancestors.
-// set 0: sources, set 1: targets (doubled cell only).  Bound by the atomics of the
+// set 0: sources, set 1: targets (doubled cell only).  With `owned` also the counts of the
+// nodes n0 <= i < n1 and of the cell's first: a target partition's own targets.
+// Bound by the atomics of the
 // coarse boxes, which every record adds to: a warp's records of one box (neighbours on
 // a curve, mostly) go as one, 102400 records in 9 us against 148.
 __global__ void k_fmm_bin(FmmGeom g, const Cell* __restrict__ cells, const FmmCell* __restrict__ fc,
                           const int4* __restrict__ box, int n, int mul, int targets, int* __restrict__ leaf,
-                          int* __restrict__ count) {
+                          int* __restrict__ count, int n0, int n1, int* __restrict__ owned) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     int b = -1;
+    bool own = false;
     if (r < n) {
         const int c = g.node_cell[mul == 1 ? r : r >> 2];
         const Cell& cl = cells[c];
         const double2 p = targets ? make_double2(g.xw[r] - cl.C[0], g.yw[r] - cl.C[1]) : fmm_source(g, cl, r, mul);
         b = fmm_leaf(fc[c], p);
         leaf[r] = b;
+        own = owned && ((r >= n0 && r < n1) || r == cl.node_off);
     }
+    const unsigned mine = __ballot_sync(0xffffffffu, own);
     while (__any_sync(0xffffffffu, b >= 0)) {
         const unsigned same = __match_any_sync(0xffffffffu, b);
         if (b >= 0) {
-            if ((threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(count + b, __popc(same));
+            if ((threadIdx.x & 31) == __ffs(same) - 1) {
+                atomicAdd(count + b, __popc(same));
+                if (same & mine) atomicAdd(owned + b, __popc(same & mine));
+            }
             b = box[b].w;
         }
     }
@@ -842,7 +850,7 @@ k_fmm_lists(FmmTree t, const Cell* __restrict__ cells, int nimg) {
         }
     }
     __syncthreads();
-    if (t.tcount[b] == 0) {
+    if (t.wanted[b] == 0) {
         if (threadIdx.x == 0) t.nfar[b] = 0;
         if (threadIdx.x == 0 && level == 0) t.nnear[b] = 0;
         return;
@@ -920,7 +928,7 @@ k_fmm_m2l(FmmTree t, const Cell* cells, int nimg, const V4<R>* mp, V4<R>* loc, F
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int4 bx = t.box[b];
     const Cell& cl = cells[bx.x];
-    if (t.tcount[b] == 0 || !cl.active) {
+    if (t.wanted[b] == 0 || !cl.active) {
         pdl_wait();
         return;
     }
@@ -1257,7 +1265,7 @@ k_fmm_down32(FmmTree t, const Cell* cells, int nimg, const C2<float>* sq, const 
     const int4 bx = t.box[b];
     const FmmCell& f = t.cells[bx.x];
     const Cell& cl = cells[bx.x];
-    if (t0 + 64 * tile >= t1 || !cl.active) {
+    if (t0 + 64 * tile >= t1 || t.wanted[b] == 0 || !cl.active) {
         pdl_wait();
         return;
     }
@@ -1383,7 +1391,7 @@ k_fmm_down64(FmmTree t, const Cell* cells, int nimg, const C2<R>* sq, const V4<R
     const int4 bx = t.box[b];
     const FmmCell& f = t.cells[bx.x];
     const Cell& cl = cells[bx.x];
-    if (t0 + 32 * tile >= t1 || !cl.active) {
+    if (t0 + 32 * tile >= t1 || t.wanted[b] == 0 || !cl.active) {
         pdl_wait();
         return;
     }
@@ -1589,14 +1597,17 @@ int fmm_work(bie_ctx* c, int prec, int64_t* pairs, int64_t* translations, int32_
     *order = prec == 0 ? kFmmP32 : kFmmP64;
     const Fmm& f = c->fmm[prec];
     if (!f.on) {
-        for (const Cell& cl : c->cells_h) *pairs += (int64_t)cl.n_nodes * cl.n_nodes * (c->utilde ? 4 : 9);
+        for (const Cell& cl : c->cells_h) {
+            const int own = c->shard.on ? c->shard.n1 - c->shard.n0 + (c->shard.n0 > 0) : cl.n_nodes;
+            *pairs += (int64_t)own * cl.n_nodes * (c->utilde ? 4 : 9);
+        }
         return BIE_OK;
     }
     if (int rc = fmm_build(c, prec)) return rc;
     std::vector<int> count(f.t.nleaf), nnear(f.t.nleaf), nfar(f.t.nbox);
     std::vector<FmmRange> near((size_t)f.t.nleaf * kFmmRanges);
     BIE_CUDA(c, cudaStreamSynchronize(c->stream));
-    BIE_CUDA(c, cudaMemcpy(count.data(), f.t.tcount, count.size() * sizeof(int), cudaMemcpyDeviceToHost));
+    BIE_CUDA(c, cudaMemcpy(count.data(), f.t.wanted, count.size() * sizeof(int), cudaMemcpyDeviceToHost));
     BIE_CUDA(c, cudaMemcpy(nnear.data(), f.t.nnear, nnear.size() * sizeof(int), cudaMemcpyDeviceToHost));
     BIE_CUDA(c, cudaMemcpy(nfar.data(), f.t.nfar, nfar.size() * sizeof(int), cudaMemcpyDeviceToHost));
     BIE_CUDA(c, cudaMemcpy(near.data(), f.t.near, near.size() * sizeof(FmmRange), cudaMemcpyDeviceToHost));
@@ -1873,6 +1884,7 @@ int fmm_plan(bie_ctx* c) {
         const size_t o_tcount = ut ? place(nbox * sizeof(int)) : 0, o_tstart = ut ? place((nleaf + 1) * sizeof(int)) : 0,
                      o_tperm = ut ? place(N * sizeof(int)) : 0,
                      o_tpos = ut ? place(N * (dbl ? sizeof(double2) : sizeof(float4))) : 0;
+        const size_t o_owned = c->ncell == 1 ? place(nbox * sizeof(int)) : 0;
         if (const cudaError_t e = cudaMalloc(&f.arena, total)) {
             f.arena = nullptr;
             if (e != cudaErrorMemoryAllocation) return drop(e, "cudaMalloc");
@@ -1917,6 +1929,7 @@ int fmm_plan(bie_ctx* c) {
         t.nnear = (int*)(a + o_nnear);
         t.shift = (float4*)(a + o_shift);
         f.tables = a + o_tab;
+        f.owned = c->ncell == 1 ? (int*)(a + o_owned) : nullptr;
         t.tcount = t.scount = (int*)(a + o_scount);
         t.tstart = t.sstart = (int*)(a + o_sstart);
         t.tperm = t.sperm = (int*)(a + o_sperm);
@@ -1932,6 +1945,7 @@ int fmm_plan(bie_ctx* c) {
             t.tpos = dbl ? nullptr : (float4*)(a + o_tpos);
             t.tpos64 = dbl ? (double2*)(a + o_tpos) : nullptr;
         }
+        t.wanted = t.tcount;
         f.built = 0;
         f.mp_bytes = (size_t)nbox * (dbl ? kFmmP64 * sizeof(V4<double>) : kFmmP32 * sizeof(V4<float>));
         // lists split into shares until the boxes (about half of them occupied)
@@ -1981,12 +1995,21 @@ int fmm_build(bie_ctx* c, int prec) {
     if (!f.on || f.built == c->geometry) return BIE_OK;
     const FmmGeom g{c->x, c->y, c->xw, c->yw, c->imc, c->node_cell};
     FmmTree& t = f.t;
+    t.wanted = t.tcount;
+    if (c->shard.on) {
+        // (the kernels pass over the boxes without a target of the partition's own; whole
+        // leaves, so that an owned target's sums stay what they are without it, bit for bit)
+        t.wanted = f.owned;
+        BIE_CUDA(c, cudaMemsetAsync(f.owned, 0, t.nbox * sizeof(int), c->stream));
+    }
     for (int set = 0; set < (c->utilde ? 2 : 1); ++set) {
         const int mul = set ? 1 : c->srcmul, n = c->N * mul;
         int* count = set ? t.tcount : t.scount;
         int* start = set ? t.tstart : t.sstart;
         BIE_CUDA(c, cudaMemsetAsync(count, 0, t.nbox * sizeof(int), c->stream));
-        k_fmm_bin<<<(n + 255) / 256, 256, 0, c->stream>>>(g, c->cells, f.cells, f.box, n, mul, set, f.leaf, count);
+        k_fmm_bin<<<(n + 255) / 256, 256, 0, c->stream>>>(g, c->cells, f.cells, f.box, n, mul, set, f.leaf, count,
+                                                             c->shard.n0, c->shard.n1,
+                                                             c->shard.on && (set || !c->utilde) ? f.owned : nullptr);
         BIE_LAUNCH(c, "k_fmm_bin");
         k_fmm_scan<<<1, 1024, 0, c->stream>>>(count, t.nleaf, start, f.cursor);
         BIE_LAUNCH(c, "k_fmm_scan");
