@@ -1585,7 +1585,11 @@ int autotune_near32(bie_ctx* c) {
     k_rhs<<<(N + 255) / 256, 256, 0, c->stream>>>(c->nx, c->ny, c->node_cell, c->cells, N,
                                                   reinterpret_cast<double2*>(c->sv.r));
     BIE_LAUNCH(c, "k_rhs");
-    if (int rc = apply_impl(c, c->sv.r, c->sv.d, BIE_MIXED, c->ws)) return rc;  // packs ws.src32
+    // (an application whose sum runs by expansions does not pack the direct sum's sources)
+    c->ws_x = nullptr;
+    k_pack_moments<<<c->nb, 256, 0, c->stream>>>(reinterpret_cast<const double2*>(c->sv.r), c->x, c->y, c->w, c->body,
+                                                 c->body_cell, c->cells, c->ws.src32, c->ws.src64, nullptr, c->ws.bodyF);
+    BIE_LAUNCH(c, "k_pack_moments");
     cudaEvent_t ev[2];
     BIE_CUDA(c, cudaEventCreate(&ev[0]));
     BIE_CUDA(c, cudaEventCreate(&ev[1]));
