@@ -352,7 +352,8 @@ k_net_grad(const __nv_bfloat16* __restrict__ wb, int n_in, const float* __restri
             if ((f >= kK1 / 2) == (half == 1)) st_column(sm + kSmBS, H + f, t, pack_bf16(x[f], x[f + 1]));
         const bool valid = tile * kTcTile + t < N;
         const float w = wi, g0 = ti0, g1 = ti1;
-        read((tile + gridDim.x) * kTcTile + t);
+        const long long ahead = (long long)(tile + gridDim.x) * kTcTile + t;  // (past 2^31 for the last rows that an int counts)
+        read(ahead < N ? (int)ahead : N);
         if (!tc_step(S, phase, [&] { issue_layer1(sbase, dZ); })) break;
         tc_layer1_out(dZ + lane, S, sm, t, c0, NC, true);
         if (!tc_step(S, phase, [&] { issue_layer2(sbase, dZ2); })) break;
