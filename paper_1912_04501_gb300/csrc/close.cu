@@ -1099,7 +1099,7 @@ int assemble32(bie_ctx* c, const double* sigma, const Workspace& ws, double* you
 // ---------------------------------------------------------------------------
 // Assembly after the fast image sum (single precision) and after every FP64 or
 // double-float sum: T_i = partials + proxy traction + on-curve diagonal + close
-// pairs' sums (k_side), y_i = sigma_i / 2 + T_i + alpha n_i + F_b +
+// pairs' sums (close_pair, fmm.cu), y_i = sigma_i / 2 + T_i + alpha n_i + F_b +
 // (x_i - x^c)^perp tau_b.  One thread per node, a CTA per chunk of one cell's
 // nodes: the double-precision epilogue then costs one instruction per 32 nodes.
 // (A warp per node spent 340 us on it at 102400 nodes, the FP64 pipe issuing a

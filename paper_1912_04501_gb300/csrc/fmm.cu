@@ -910,7 +910,7 @@ k_fmm_lists(FmmTree t, const Cell* __restrict__ cells, int nimg) {
 // shares the longest lists (90 boxes, at the coarse levels) held up the launch.
 template <typename R>
 __global__ void __launch_bounds__(128)
-k_fmm_m2l(FmmTree t, const Cell* cells, int nimg, const V4<R>* mp, V4<R>* loc, FmmTab<R> tab, int shares,
+k_fmm_m2l(FmmTree t, const Cell* cells, const V4<R>* mp, V4<R>* loc, FmmTab<R> tab, int shares,
           SideArgs side) {
     constexpr int P = FmmTypes<R>::P;
     constexpr bool F32 = sizeof(R) == 4;
@@ -1245,8 +1245,8 @@ __device__ __forceinline__ int fmm_split(int n) { return n > 16 ? 1 : (n > 8 ? 2
 // double-float positions make every difference exact to single precision, so no
 // later pass has to redo near pairs.
 __global__ void __launch_bounds__(128, 6)
-k_fmm_down32(FmmTree t, const Cell* cells, int nimg, const C2<float>* sq, const V4<float>* loc, int shares, FmmTab<float> tab, const float4* __restrict__ tgt32,
-             int n0, int n1, float2* __restrict__ part, XiArgs xi, int tiles) {
+k_fmm_down32(FmmTree t, const Cell* cells, const C2<float>* sq, const V4<float>* loc, int shares, FmmTab<float> tab,
+             const float4* __restrict__ tgt32, int n0, int n1, float2* __restrict__ part, XiArgs xi, int tiles) {
     constexpr int P = kFmmP32;
     __shared__ V4<float> s_l[4][P];
     __shared__ C2<float> s_pw[4][2][kPowTab];
@@ -1369,8 +1369,8 @@ k_fmm_down32(FmmTree t, const Cell* cells, int nimg, const C2<float>* sq, const 
 // the near sources, then four lanes per target split the local expansion.
 template <typename R>
 __global__ void __launch_bounds__(128, 4)
-k_fmm_down64(FmmTree t, const Cell* cells, int nimg, const C2<R>* sq, const V4<R>* loc, int shares, FmmTab<R> tab, const double* __restrict__ nxv,
-             const double* __restrict__ nyv, int prec, int n0, int n1, double2* __restrict__ part,
+k_fmm_down64(FmmTree t, const Cell* cells, const C2<R>* sq, const V4<R>* loc, int shares, FmmTab<R> tab,
+             const double* __restrict__ nxv, const double* __restrict__ nyv, int prec, int n0, int n1, double2* __restrict__ part,
              XiArgs xi, int tiles) {
     constexpr int P = FmmTypes<R>::P;
     constexpr bool DF = std::is_same<R, df>::value;
@@ -2091,22 +2091,22 @@ static int across_launch(bie_ctx* c, const double* sigma, int prec, Workspace& w
     const Fmm& f = c->fmm[prec];
     const FmmTree& t = f.t;
     const FmmTab<R> tab = fmm_tab<R>(c, prec);
-    const int nimg = c->utilde ? 1 : 9, tiles = 2;
+    const int tiles = 2;
     const int n0 = c->shard.on ? c->shard.n0 : 0, n1 = c->shard.on ? c->shard.n1 : c->N;
     const V4<R>* loc = (const V4<R>*)ws.floc;
     const SideArgs side = side_args(c, sigma, prec, f.walls, ws);
     const bool early = fmm_chained(c, prec);
-    BIE_CUDA(c, launch_after(early, k_fmm_m2l<R>, side.ctas + t.nbox * f.shares, 128, 0u, c->stream, t, c->cells, nimg,
+    BIE_CUDA(c, launch_after(early, k_fmm_m2l<R>, side.ctas + t.nbox * f.shares, 128, 0u, c->stream, t, c->cells,
                              (const V4<R>*)ws.fmp, (V4<R>*)ws.floc, tab, f.shares, side));
     ++c->launches;
     XiArgs xi{c->m, c->M, 0, (2 * c->M + 3) / 4, ws.gpart, c->P, ws.xi, ws.xif};
     if (f.walls) xi.ctas = xi.per_cell * c->ncell;
     const unsigned down = xi.ctas + t.nleaf * tiles;
     if constexpr (sizeof(R) == 4)
-        BIE_CUDA(c, launch_after(early, k_fmm_down32, down, 128, 0u, c->stream, t, c->cells, nimg, (const C2<float>*)ws.fsq, loc,
+        BIE_CUDA(c, launch_after(early, k_fmm_down32, down, 128, 0u, c->stream, t, c->cells, (const C2<float>*)ws.fsq, loc,
                                  f.shares, tab, c->tgt32, n0, n1, (float2*)ws.part, xi, tiles));
     else
-        BIE_CUDA(c, launch_after(early, k_fmm_down64<R>, down, 128, 0u, c->stream, t, c->cells, nimg, (const C2<R>*)ws.fsq, loc,
+        BIE_CUDA(c, launch_after(early, k_fmm_down64<R>, down, 128, 0u, c->stream, t, c->cells, (const C2<R>*)ws.fsq, loc,
                                  f.shares, tab, c->nx, c->ny, prec, n0, n1, (double2*)ws.part, xi, tiles));
     ++c->launches;
     return BIE_OK;
