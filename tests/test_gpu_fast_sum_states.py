@@ -1,6 +1,6 @@
 """GPU tests of the near image sum by expansions in a context whose configuration is
 set after the boxes were laid out: centres past a skewed cell (inside and outside the
-rectangle of before), a flatter lattice, and back.
+rectangle of before), a flatter lattice, and back; on a stream of its own; and in a batch.
 
 A context made in the configuration itself sums the walls with boxes chosen for it, on the
 same proxy fit bit for bit; the two agree to the rounding of the sums times the fit's gain:
@@ -23,8 +23,8 @@ bie = pytest.importorskip("paper_1912_04501_gb300.bie")
 PRECS = ((bie.BIE_FP64, 1e-11), (bie.BIE_DF64, 1e-10), (bie.BIE_MIXED, 5e-6))
 
 
-def _cell(bodies, nodes, e2, seed=1001):
-    c = workloads.random_cell(bodies, 0.3, (1.0, 3.0), 5e-3, nodes, seed, e2=e2)
+def _cell(bodies, nodes, e2, seed=1001, phi=0.3):
+    c = workloads.random_cell(bodies, phi, (1.0, 3.0), 5e-3, nodes, seed, e2=e2)
     c.update(solver=dict(n_proxy=48, proxy_radius=1.5, n_coll=24, gmres_tol=1e-10), dt=1e-3, steps=1)
     return c
 
@@ -83,4 +83,56 @@ def test_centres_outside_and_a_flatter_lattice():
                               for k, b in enumerate(tall["bodies"])])
     _set(ctx, away)
     _compare(ctx, away, 1e-7)
+    ctx.close()
+
+
+def test_stream_of_its_own():
+    """On a stream of its own a context's launches begin before the ones ahead have ended;
+    the results are those of the default stream, bit for bit, and so they are with the
+    profiler on."""
+    torch = pytest.importorskip("torch")
+    cell = _cell(25, 200, (0.2, 1.0), seed=5)
+    stream = torch.cuda.Stream()
+    got = []
+    for own, prof in ((False, False), (True, False), (True, True)):
+        ctx = bie.Context(cell, precision=bie.BIE_MIXED)
+        assert _fast(ctx)
+        if own:
+            ctx.set_stream(stream.cuda_stream)
+        ctx.profile(prof)
+        sigma = np.random.default_rng(1).standard_normal(2 * ctx.N)
+        out = [ctx.apply(sigma, precision=p) for p, _ in PRECS for _ in range(3)]
+        s, _ = ctx.solve()
+        v, om, mu = ctx.velocities(s)
+        mus, _ = ctx.step(1e-3, 2)
+        st = ctx.get_state()
+        got.append([*out, s, v, om, mu, mus, st["xc"], st["theta"], st["sigma"]])
+        ctx.close()
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert np.array_equal(a, b)
+
+
+def test_batch_by_expansions_with_cells_switched_off():
+    """A batch whose sums all run by expansions: every cell's application against the
+    oracle, and a lockstep solve in which cells drop out at different iterations, against
+    each cell's own solve (two solutions of a 1e-10 residual: 1e-8)."""
+    cells = [_cell(30, 150, (0.0, 1.0), seed=11), _cell(12, 230, (0.2, 1.0), seed=12, phi=0.1), _cell(25, 160, (-0.4, 1.0), seed=13)]
+    ctx = bie.Context(cells, precision=bie.BIE_MIXED)
+    assert _fast(ctx)
+    sigma = np.random.default_rng(3).standard_normal(2 * ctx.N)
+    cut = [slice(2 * a, 2 * b) for a, b in zip(ctx.node_offsets[:-1], ctx.node_offsets[1:])]
+    ref = [oracle_operator(c).apply(sigma[sl].reshape(-1, 2)).ravel() for c, sl in zip(cells, cut)]
+    for prec, tol in ((bie.BIE_FP64, 1e-10), (bie.BIE_DF64, 1e-10), (bie.BIE_MIXED, 5e-6)):
+        y = ctx.apply(sigma, precision=prec)
+        for r, sl in zip(ref, cut):
+            assert np.abs(y[sl] - r).max() < tol * np.abs(r).max(), prec
+    s, info = ctx.solve()
+    assert info["rel_residual"] <= 1e-10
+    assert len({c["iterations"] for c in ctx.cell_info()}) > 1  # some ended before others
+    for c, sl in zip(cells, cut):
+        one = bie.Context(c, precision=bie.BIE_MIXED)
+        t, _ = one.solve()
+        one.close()
+        assert np.abs(s[sl] - t).max() < 1e-8 * np.abs(t).max()
     ctx.close()
