@@ -884,8 +884,12 @@ int bie_set_state(bie_ctx* c, double t, const double* e2, const double* xc, cons
         cell_set_lattice(cl, e1, e2 + 2 * k);
     }
     c->body_host = h;
+    const unsigned long long epoch = c->epoch;
     int rc = fmm_fit(c);
     if (rc) return rc;
+    bool items = c->epoch != epoch;
+    for (int prec = 0; prec < 3; ++prec) items = items || (!c->fmm[prec].on && c->near[prec].count == 0);
+    if (items && (rc = build_near_items(c))) return rc;
     rc = upload_cells(c, c->stream);
     if (rc) return rc;
     rc = upload_e2(c, c->e2d, current_e2(c), c->stream);

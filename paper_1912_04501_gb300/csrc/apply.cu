@@ -1250,6 +1250,7 @@ static int build_near_items_prec(bie_ctx* c, int prec, bool direct = false) {
     if (bytes > c->ws.part_bytes) return fail(c, BIE_EINVAL, "near-sum partial buffer too small");
     if (c->near[prec].items) BIE_CUDA(c, cudaFree(c->near[prec].items));
     c->near[prec].items = nullptr;
+    c->near[prec].count = 0;  // (no application and another attempt by the next bie_set_state, should the list not be made)
     BIE_CUDA(c, cudaMalloc((void**)&c->near[prec].items, items.size() * sizeof(int4)));
     BIE_CUDA(c, cudaMemcpy(c->near[prec].items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice));
     c->near[prec].count = (int)items.size();
@@ -1415,6 +1416,7 @@ static int apply_part(bie_ctx* c, int part, const double* sigma, double* yout, i
     }
     if (part == 1) {
         if (fast) return fmm_across(c, sigma, prec, ws);
+        if (c->near[prec].count == 0) return fail(c, BIE_ENOMEM, "the near sum's work list was not made: memory was short");
         if (f32) return launch_near32(c, ws.src32, (float2*)ws.part);
         if (c->utilde) {
             if (df)

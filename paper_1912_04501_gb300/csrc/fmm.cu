@@ -1720,9 +1720,7 @@ static double fmm_wall_side(const bie_ctx* c, int k, int prec) {
 // The boxes of one cell for where its bodies are now: the grid as planned while it
 // covers their rectangle, and else moved and its side stretched until it does; then the
 // coarsest level that the walls' far images are well away from, which depends on the
-// lattice and the centres too.  The counts of boxes never change, so neither do any
-// kernel's arguments (a captured application stays right), and nothing is allocated.
-// Stretched leaves cost pairs (side times 1.6 for bodies listed a lattice vector away).
+// lattice and the centres too.
 static FmmCell fmm_place(const bie_ctx* c, int k, int prec) {
     FmmCell f = c->fmm[prec].plan[k];
     const FmmPlanCell r = fmm_rect(c, k);
@@ -1730,7 +1728,7 @@ static FmmCell fmm_place(const bie_ctx* c, int k, int prec) {
     if (r.ox < f.ox || r.oy < f.oy || r.ox + r.w > f.ox + f.gx[0] * f.h || r.oy + r.ht > f.oy + f.gy[0] * f.h) {
         f.ox = std::min(f.ox, r.ox);
         f.oy = std::min(f.oy, r.oy);
-        f.h = std::max((x1 - f.ox) / f.gx[0], (y1 - f.oy) / f.gy[0]);
+        f.h = std::max(std::max((x1 - f.ox) / f.gx[0], (y1 - f.oy) / f.gy[0]), f.h * (1 + 1e-15));
         f.inv_h = 1.0 / f.h;
     }
     const double wall = fmm_wall_side(c, k, prec);
@@ -1754,19 +1752,36 @@ static void fmm_centres(const std::vector<FmmCell>& cells, float4* centre) {
                 }
 }
 
-// Called when a configuration is set (host mirrors of bodies and lattices).
+// Called when a configuration is set (host mirrors of bodies and lattices).  A context
+// that bie_apply_static takes keeps its counts of boxes, and with them every kernel's
+// arguments, so that an application captured before stays right; stretched leaves cost
+// it pairs (a side 1.6 times as long for bodies listed a lattice vector away).  Larger
+// ones are planned anew when their bodies leave the grid: leaves of many more targets than
+// planned would leave the chip to a few CTAs.  (The epoch then tells that the layout
+// of the sums may have changed.)
 int fmm_fit(bie_ctx* c) {
+    std::vector<FmmCell> place[3];
+    bool left = false;
+    for (int prec = 0; prec < 3; ++prec)
+        for (int k = 0; k < c->ncell && c->fmm[prec].on; ++k) {
+            place[prec].push_back(fmm_place(c, k, prec));
+            left = left || place[prec][k].h > c->fmm[prec].plan[k].h;
+        }
+    if (left && c->N > kStaticMaxNodes) {
+        ++c->epoch;
+        free_fmm(c);
+        return fmm_plan(c);
+    }
     for (int prec = 0; prec < 3; ++prec) {
         Fmm& f = c->fmm[prec];
         if (!f.on) continue;
         bool moved = false;
         for (int k = 0; k < c->ncell; ++k) {
-            const FmmCell q = fmm_place(c, k, prec);
-            FmmCell& o = f.now[k];
+            const FmmCell &q = place[prec][k], &o = f.now[k];
             moved = moved || q.ox != o.ox || q.oy != o.oy || q.h != o.h || q.wall != o.wall;
-            o = q;
         }
         if (!moved) continue;
+        f.now = place[prec];
         std::vector<float4> centre(f.t.nbox);
         fmm_centres(f.now, centre.data());
         BIE_CUDA(c, cudaMemcpyAsync(f.cells, f.now.data(), f.now.size() * sizeof(FmmCell), cudaMemcpyHostToDevice, c->stream));
@@ -1777,7 +1792,7 @@ int fmm_fit(bie_ctx* c) {
 }
 
 // Boxes of every precision whose near sums run faster this way.  Called when
-// a context is made, after all else has its memory: a precision whose boxes do not fit
+// a context is made, after all else has its memory (and by fmm_fit): a precision whose boxes do not fit
 // beside it keeps the direct sum (all of them, where the moments do not fit).  Nothing
 // of the context refers to the boxes before they are complete.
 int fmm_plan(bie_ctx* c) {

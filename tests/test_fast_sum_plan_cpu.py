@@ -106,10 +106,11 @@ def relisted(cell, past):
 
 
 @pytest.mark.parametrize("skew", [0.0, -0.3, -0.45, 0.45])
-@pytest.mark.parametrize("bodies,nodes", [(25, 256), (60, 160)])
+@pytest.mark.parametrize("bodies,nodes", [(25, 256), (60, 130)])
 def test_boxes_follow_a_configuration(program, skew, bodies, nodes):
     """Whatever configuration is set, the boxes hold every node and the walls' series
-    leave out less than single precision's or double's rounding."""
+    leave out less than single precision's or double's rounding (sizes that
+    bie_apply_static takes: the boxes' counts never change)."""
     cell = workloads.random_cell(bodies, 0.3, (1.0, 3.0), 5e-3, nodes, 1001, e2=(skew, 1.0))
     home = np.array([b["xc"] for b in cell["bodies"]])
     rng = np.random.default_rng(3)
@@ -153,7 +154,7 @@ def test_short_memory_leaves_the_direct_sum(program, doubled):
     """An allocation that fails costs its precision the boxes (the moments', all three),
     never the context: no error is left, nothing half made stays, and a configuration can
     be set all the same."""
-    cell = workloads.random_cell(40, 0.25, (1.0, 2.0), 5e-3, 256, 2, e2=(0.2, 1.0))
+    cell = workloads.random_cell(40, 0.25, (1.0, 2.0), 5e-3, 200, 2, e2=(0.2, 1.0))
     home = np.array([b["xc"] for b in cell["bodies"]])
     for fail in range(0, 5):
         plan, state, end = _run(program, cell, ("plan", fail), ("set", cell["e2"], home + [0.4, 0.0]), doubled=doubled)
@@ -164,4 +165,28 @@ def test_short_memory_leaves_the_direct_sum(program, doubled):
             assert status["live"] == (0 if fail == 4 else 4 - len(off)) and status["work"] == (fail != 4)
             for prec, (on, _, held, _) in precs.items():
                 assert (on, held) == ((0, 0) if prec in off else (1, 1))
+        assert end[0]["live"] == 0
+
+
+def test_large_cells_are_planned_anew(program):
+    """Beyond the sizes that bie_apply_static takes, a configuration that leaves the grid
+    gets another one (the leaves stay as small as they were), memory permitting."""
+    cell = workloads.random_cell(60, 0.25, (1.0, 2.0), 5e-3, 200, 2, e2=(0.2, 1.0))
+    home = np.array([b["xc"] for b in cell["bodies"]])
+    away = home + np.array([[4.0 * (k == 5), 0.0] for k in range(len(home))])
+    for fail in (0, 6, 8):
+        plan, inside, out, back, end = _run(program, cell, ("plan", fail), ("set", cell["e2"], home),
+                                            ("set", cell["e2"], away), ("set", cell["e2"], home))
+        assert inside[1] == plan[1] and (inside[0]["calls"], out[0]["calls"], back[0]["calls"]) == (4, 8, 8)
+        off = {0: (), 6: (1,), 8: (0, 1, 2)}[fail]
+        X = _nodes(cell, away)[0]
+        for status, precs in (out, back):
+            assert status["rc"] == 0 and status["error"] == 0
+            assert status["live"] == (0 if fail == 8 else 4 - len(off)) and status["work"] == (fail != 8)
+            for prec, (on, _, held, box) in precs.items():
+                assert (on, held) == ((0, 0) if prec in off else (1, 1))
+                if on:
+                    ox, oy, h, gx, gy = box[:5]
+                    assert h < 1.5 * plan[1][prec][3][2]
+                    assert (X >= [ox, oy]).all() and (X <= [ox + gx * h, oy + gy * h]).all()
         assert end[0]["live"] == 0

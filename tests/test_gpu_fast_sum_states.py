@@ -70,10 +70,12 @@ def test_centres_past_a_skewed_cell(skew):
     ctx.close()
 
 
-def test_centres_outside_and_a_flatter_lattice():
+@pytest.mark.parametrize("bodies", [24, 40])
+def test_centres_outside_and_a_flatter_lattice(bodies):
     """Bodies a whole lattice vector away (the walls' images are then among them: no box is
-    well away), and a lattice of 0.6 of the height."""
-    flat = _cell(24, 256, (0.3, 0.6), seed=7)
+    well away), and a lattice of 0.6 of the height; 6144 nodes keep their boxes, 10240
+    get others."""
+    flat = _cell(bodies, 256, (0.3, 0.6), seed=7)
     tall = dict(flat, e2=[0.3, 1.0])
     ctx = bie.Context(tall, precision=bie.BIE_FP64)
     assert _fast(ctx)
@@ -83,6 +85,8 @@ def test_centres_outside_and_a_flatter_lattice():
                               for k, b in enumerate(tall["bodies"])])
     _set(ctx, away)
     _compare(ctx, away, 1e-7)
+    _set(ctx, tall)
+    _compare(ctx, tall, 1e-10)
     ctx.close()
 
 
