@@ -1252,7 +1252,9 @@ static int build_near_items_prec(bie_ctx* c, int prec, bool direct = false) {
     c->near[prec].items = nullptr;
     c->near[prec].count = 0;  // (no application and another attempt by the next bie_set_state, should the list not be made)
     BIE_CUDA(c, cudaMalloc((void**)&c->near[prec].items, items.size() * sizeof(int4)));
-    BIE_CUDA(c, cudaMemcpy(c->near[prec].items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    BIE_CUDA(c, cudaMemcpyAsync(c->near[prec].items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice,
+                                c->stream));
+    BIE_CUDA(c, cudaStreamSynchronize(c->stream));
     c->near[prec].count = (int)items.size();
     return BIE_OK;
 }

@@ -21,8 +21,8 @@
 // when the centres differ by less than two sides in both coordinates.  Far
 // triples whose parents are near (every far triple at the top) pass by
 // expansions; near triples of the finest level are evaluated pair by pair.
-// Truncation: worst case (two box corners) 0.547^P, typically 1e-2 of that:
-// P = 24 in single precision, P = 48 in double.
+// Truncation: 0.547^P for two box corners that face each other, P = 24 in single
+// precision, P = 48 in double; of a corner's whole far sum 2e-16 in double.
 //
 // Three arithmetics: float, double, and double-float (df, bie_internal.cuh) for
 // the double-float application, all of it on the FP32 pipe.
@@ -31,11 +31,13 @@
 // pair sum (about 20 instructions per pair, a few hundred pairs per target);
 // double: the FP64 pipe in the translations (a warp DFMA per 19 cycles and SM).
 // Whole applications on GB300, direct sum before and this now: single precision
-// 32.8 -> 0.20 ms on the 400-ellipse cell (102400 nodes), 0.94 -> 0.105 ms at
-// 16000 nodes, 0.21 -> 0.092 ms at 6400; double-float 340 -> 1.12 ms at 102400;
-// FP64 12.2 -> 0.86 ms at 6400.  The single-precision application's error
-// against 64 bits falls (4.2e-7 -> 1.2e-7 at 6400 nodes): near pairs are
-// differenced exactly.
+// 32.8 -> 0.185 ms on the 400-ellipse cell (102400 nodes), 0.94 -> 0.095 ms at
+// 16000 nodes, 0.21 -> 0.077 ms at 6400; double-float 340 -> 1.10 ms at 102400;
+// FP64 12.2 -> 0.85 ms at 6400.  The single-precision application's error
+// against 64 bits falls (5.0e-7 -> 1.9e-7 in the 2-norm at 6400 nodes): near pairs are
+// differenced exactly.  So does the double-float application's against FP64
+// (4.1e-13 -> 8.5e-14; 1 to 400 bodies, shear to 0.45), whose walls and proxies were
+// summed in FP64 before.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -343,9 +345,9 @@ __device__ void fmm_body(const FmmBodies& p, int b, const Cell* cells, const dou
     }
 }
 
-// Measured (whole application, us): single precision at 6400 / 102400 nodes 64.4 /
-// 167 with 128, 67.1 / 170 with 512, 80.9 / 188 with 2048; double-float 270 / 1119
-// with 64, 262 / 1132 with 256, 278 / 1178 with 512.
+// Measured (whole application, us, on a stream of the context's own): single precision
+// at 6400 / 102400 nodes 64.4 / 167 with 128, 67.1 / 170 with 512, 80.9 / 188 with 2048;
+// double-float 270 / 1119 with 64, 262 / 1132 with 256, 278 / 1178 with 512.
 template <typename R>
 constexpr int kFmmDirect = sizeof(R) == 4 ? 128 : 256;
 
@@ -1787,6 +1789,7 @@ int fmm_fit(bie_ctx* c) {
         BIE_CUDA(c, cudaMemcpyAsync(f.cells, f.now.data(), f.now.size() * sizeof(FmmCell), cudaMemcpyHostToDevice, c->stream));
         BIE_CUDA(c, cudaMemcpyAsync(f.t.centre, centre.data(), centre.size() * sizeof(float4), cudaMemcpyHostToDevice,
                                     c->stream));
+        BIE_CUDA(c, cudaStreamSynchronize(c->stream));
     }
     return BIE_OK;
 }
@@ -1925,9 +1928,11 @@ int fmm_plan(bie_ctx* c) {
         if (prec == 0) fmm_tables<float>(&host[o_tab]);
         else if (prec == 1) fmm_tables<double>(&host[o_tab]);
         else fmm_tables<df>(&host[o_tab]);
-        if (const cudaError_t e = cudaMemcpy(f.arena, host.data(), written, cudaMemcpyHostToDevice)) {
+        cudaError_t e = cudaMemcpyAsync(f.arena, host.data(), written, cudaMemcpyHostToDevice, c->stream);
+        if (!e) e = cudaStreamSynchronize(c->stream);  // (the copy in host memory goes)
+        if (e) {
             cudaFree(f.arena);
-            return drop(e, "cudaMemcpy");
+            return drop(e, "cudaMemcpyAsync");
         }
         f.plan = f.now = cells;
         unsigned char* a = (unsigned char*)f.arena;
@@ -1987,7 +1992,8 @@ int fmm_plan(bie_ctx* c) {
             c->fmm_ws = nullptr;
             return drop(e, "cudaMalloc");
         }
-        if (const cudaError_t e = cudaMemset(c->fmm_ws, 0, 2 * tick)) return drop(e, "cudaMemset");
+        // (on the context's stream, which need not wait for the default one)
+        if (const cudaError_t e = cudaMemsetAsync(c->fmm_ws, 0, 2 * tick, c->stream)) return drop(e, "cudaMemsetAsync");
         unsigned char* a = (unsigned char*)c->fmm_ws;
         auto lay = [&](Workspace& ws, unsigned char* ticks, unsigned char* at, size_t sq, size_t mp) {
             ws.ftick = (unsigned*)ticks;

@@ -1,5 +1,5 @@
 // Host side of the fast image sum without a GPU: the allocations and copies that
-// fmm_plan and fmm_fit make land in host memory (linked with --wrap for the five
+// fmm_plan and fmm_fit make land in host memory (linked with --wrap for the
 // calls below), and the n-th allocation can be made to fail.
 //
 // Input: doubled n_coll n_cells, then per cell e1 e2 C n_bodies and per body n a b x y;
@@ -32,18 +32,15 @@ cudaError_t __wrap_cudaFree(void* p) {
     std::free(p);
     return cudaSuccess;
 }
-cudaError_t __wrap_cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
-    std::memcpy(d, s, n);
-    return cudaSuccess;
-}
 cudaError_t __wrap_cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
     std::memcpy(d, s, n);
     return cudaSuccess;
 }
-cudaError_t __wrap_cudaMemset(void* d, int v, size_t n) {
+cudaError_t __wrap_cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) {
     std::memset(d, v, n);
     return cudaSuccess;
 }
+cudaError_t __wrap_cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t __wrap_cudaGetLastError() {
     const cudaError_t e = g_last;
     g_last = cudaSuccess;

@@ -19,7 +19,7 @@ def program(tmp_path_factory):
     _build.build()
     exe = str(tmp_path_factory.mktemp("plan") / "fast_sum_plan")
     objs = [os.path.join(_build.BUILD, os.path.splitext(s)[0] + ".o") for s in _build.SOURCES]
-    wrap = [a for f in ("Malloc", "Free", "Memcpy", "MemcpyAsync", "Memset", "GetLastError")
+    wrap = [a for f in ("Malloc", "Free", "MemcpyAsync", "MemsetAsync", "StreamSynchronize", "GetLastError")
             for a in ("-Xlinker", "--wrap=cuda" + f)]
     subprocess.run([_build.nvcc(), *_build.ARCH, "-std=c++17", "-O1", "-o", exe,
                     os.path.join(HERE, "native", "fast_sum_plan.cu"), *objs, *wrap], check=True)
