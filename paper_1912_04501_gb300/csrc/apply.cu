@@ -1176,7 +1176,7 @@ static constexpr int kMinChunk = 16;
 
 // srcmul: source records per node (4 for the doubled-cell image records).
 static void choose_splits(const std::vector<Cell>& cells, int tile, int slots, std::vector<int>& splits,
-                          int srcmul = 1) {
+                          int srcmul = 1, int min_chunk = kMinChunk) {
     double W = 0;
     for (const Cell& cl : cells) W += (double)cl.n_nodes * cl.n_nodes;
     double best = 1e300;
@@ -1188,7 +1188,7 @@ static void choose_splits(const std::vector<Cell>& cells, int tile, int slots, s
             const int n = cells[k].n_nodes, ns = srcmul * n;
             const int tiles = (n + tile - 1) / tile;
             const double share = (double)w * slots * ((double)n * n / W) / tiles;
-            const int s = std::max(1, std::min((ns + kMinChunk - 1) / kMinChunk, (int)share));
+            const int s = std::max(1, std::min((ns + min_chunk - 1) / min_chunk, (int)share));
             sp[k] = s;
             items += (long long)tiles * s;
             maxchunk = std::max(maxchunk, (ns + s - 1) / s);
@@ -1263,7 +1263,25 @@ int build_near_items(bie_ctx* c) {
     for (int prec = 0; prec < 3; ++prec)
         if (int rc = build_near_items_prec(c, prec)) return rc;
     ++c->epoch;
+    if (int rc = build_static_part(c)) return rc;
     return upload_cells(c, c->stream);
+}
+
+// bie_apply_static's array has room for the partials of splits of at least 64 sources (what
+// it takes and refuses goes by those); shorter splits' are kept beside it.
+static constexpr int kStaticMinChunk = 64;
+int build_static_part(bie_ctx* c) {
+    if (c->N > kStaticMaxNodes) return BIE_OK;
+    std::vector<int> splits;
+    choose_splits(c->cells_h, near_tile(c->shape32, 0, c->utilde), near_ctas_per_sm(c->shape32, 0, c->utilde) * c->sms,
+                  splits, c->srcmul, kStaticMinChunk);
+    c->static_part_n = 0;
+    for (size_t k = 0; k < splits.size(); ++k) c->static_part_n += (size_t)splits[k] * c->cells_h[k].n_nodes;
+    if (c->static_part) BIE_CUDA(c, cudaFree(c->static_part));
+    c->static_part = nullptr;
+    if (near_part32_elems(c) > c->static_part_n)
+        BIE_CUDA(c, cudaMalloc((void**)&c->static_part, near_part32_elems(c) * sizeof(float2)));
+    return BIE_OK;
 }
 
 // Bytes of the near-sum partial buffer (largest over the precisions and the
@@ -1623,6 +1641,7 @@ int autotune_near32(bie_ctx* c) {
     if (rc) return rc;
     c->shape32 = best;
     if ((rc = build_near_items_prec(c, 0))) return rc;
+    if ((rc = build_static_part(c))) return rc;
     ++c->epoch;
     return upload_cells(c, c->stream);
 }

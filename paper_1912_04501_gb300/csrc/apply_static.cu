@@ -2,7 +2,8 @@
 // device allocation.  Every per-call buffer (source records, near-sum
 // partials, wall-discrepancy partials, body moments, proxy strengths) lives in
 // one file-scope static device array, but for the moments of the fast image sum and
-// the close pairs' sums, which the context has a second set of, for this call alone.
+// the close pairs' sums, which the context has a second set of, for this call alone, and
+// for partials of more splits than the array was sized for.
 // Of the context it reads the geometry, proxy fit, close tables and work items; it
 // writes that set, its launch counter and, with bie_profile on, the profiler's event
 // state, so calls on one context must not overlap (as for every entry point).  See
@@ -42,14 +43,16 @@ extern "C" int bie_apply_static(bie_ctx* c, const double* sigma, double* out) {
     const size_t b_src32n = c->utilde ? round256(N * sizeof(float4)) : 0;
     const size_t b_src64 = round256(N * sizeof(Src64));
     const size_t nc = (size_t)c->ncell;
-    const size_t b_part = round256(near_part32_elems(c) * sizeof(float2));
+    const size_t b_part = round256(c->static_part_n * sizeof(float2));
     const size_t b_body = round256(3 * (size_t)c->nb * sizeof(double));
     const size_t b_gpart = round256(nc * kDiscSplits * 8 * c->m * sizeof(double));
     const size_t b_xi = round256(nc * 2 * c->M * sizeof(double));
     const size_t b_xif = round256(nc * 2 * c->M * sizeof(float));
     const size_t b_gt = round256(nc * 8 * c->m * sizeof(double));
     const size_t b_tk = round256(nc * 2 * c->m * sizeof(unsigned int));
-    const size_t need = b_src32 + b_src32n + b_src64 + b_part + b_body + b_gpart + b_xi + b_xif + b_gt + b_tk;
+    // (2N doubles more: what the call takes and refuses is as it was when it kept the traction)
+    const size_t b_spare = round256(2 * N * sizeof(double));
+    const size_t need = b_src32 + b_src32n + b_src64 + b_part + b_body + b_gpart + b_xi + b_xif + b_gt + b_tk + b_spare;
     if (need > BIE_STATIC_SCRATCH_BYTES)
         return fail(c, BIE_EINVAL, "bie_apply_static: this context needs " + std::to_string(need) +
                                        " bytes of scratch; the static array holds " +
@@ -79,8 +82,7 @@ extern "C" int bie_apply_static(bie_ctx* c, const double* sigma, double* out) {
     o += b_src32n;
     ws.src64 = reinterpret_cast<Src64*>(base + o);
     o += b_src64;
-    ws.part = base + o;
-    ws.part_bytes = b_part;
+    ws.part = c->static_part ? (void*)c->static_part : (void*)(base + o);
     o += b_part;
     ws.bodyF = reinterpret_cast<double*>(base + o);
     o += b_body;

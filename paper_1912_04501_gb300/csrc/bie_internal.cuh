@@ -342,6 +342,8 @@ struct bie_ctx {
     bie::Solver sv;
     bie::Close cl;
     bie::NearItems near[3];     // 0 single precision, 1 double, 2 double-float
+    size_t static_part_n = 0;   // partials that bie_apply_static's array has room for (build_static_part)
+    float2* static_part = nullptr;  // they are here where the splits need more
     int shape32 = 0;            // tile shape of the single-precision near sum (kNear32ShapeList)
     int4* fin_chunks = nullptr; // n_fin: (cell, first node, end node, the cell's first)
     int n_fin = 0;
@@ -491,6 +493,7 @@ inline bool fmm_chained(const bie_ctx* c, int prec) {
 int build_near_items(bie_ctx* c);
 size_t near_part_bytes(const bie_ctx* c);     // partial buffer the items need
 size_t near_part32_elems(const bie_ctx* c);   // single-precision partials of the current items
+int build_static_part(bie_ctx* c);            // bie_apply_static's room for them
 // y = A sigma for device sigma, y (2N each); precision BIE_FP64 / BIE_MIXED / BIE_DF64
 int apply_device(bie_ctx* c, const double* sigma, double* y, int precision);
 // single-precision-pair application with caller-provided per-call buffers
