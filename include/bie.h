@@ -387,7 +387,8 @@ int bie_near_shape(bie_ctx* ctx, int32_t* shape, float* ms);
 /* Work of one near image sum in a precision (BIE_FP64 / BIE_MIXED / BIE_DF64) for
  * the current geometry: pairs (target, source, image) summed one by one, and
  * translations of a box's multipole expansion to another box's local one (0 where
- * the sum is direct), with *order complex coefficients per series.  The counts that a
+ * the sum is direct), with *order complex coefficients per series; with a target
+ * partition (bie_set_partition) for its own targets.  The counts that a
  * roofline divides by; they wait for the context's stream.  Errors: BIE_EINVAL,
  * BIE_ECUDA. */
 int bie_near_work(bie_ctx* ctx, int32_t precision, int64_t* pairs, int64_t* translations, int32_t* order);
